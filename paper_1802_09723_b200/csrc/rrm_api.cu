@@ -202,7 +202,7 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
         net->layer_switch = all_auto && n_layers <= 64;
         {
             bool all_tc = true;
-            for (auto& L : net->layers) all_tc = all_tc && L.tc_ready;
+            for (auto& L : net->layers) all_tc = all_tc && L.on_tensor() && L.d.dtype != RRM_F32;
             net->chunk_switch = all_auto && all_tc && n_layers <= 64;
         }
         // an all-ones bitmap stands in for a layer's update bitmap when the layer is evaluated densely inside a delta step
@@ -1290,7 +1290,7 @@ static int stats_fill(rrm_net* net, int layer, rrm_stats* h)
     h->active_macs = (int64_t)m;
     h->active_out_pixels = oc;
     // (a layer that was evaluated densely inside the delta step keeps its counters: the deltas were still formed and counted)
-    h->variant = L.ran_dense ? RRM_VARIANT_DENSE : (L.tc_ready ? RRM_VARIANT_TENSOR : RRM_VARIANT_GATHER);
+    h->variant = L.ran_dense ? RRM_VARIANT_DENSE : (L.on_tensor() ? RRM_VARIANT_TENSOR : RRM_VARIANT_GATHER);
     return RRM_OK;
 }
 int rrm_get_stats(rrm_layer* layer, rrm_stats* host_out) { return rrm_net_get_stats(layer, 0, host_out); }

@@ -195,6 +195,11 @@ struct Layer {
     int8_t* tc_Wimg = nullptr;              // [n_tiles][slabs][bn * 128] shared-memory images of the filter tiles
     int tc_kpp = 0;                         // K bytes per tap (padded channels per pixel)
     int tc_bn = 0, tc_ntiles = 0, tc_slabs = 0;
+    // window kernel (rrm_conv_win.cu)
+    bool win_ready = false;
+    void* win_Wimg = nullptr;               // [n_tiles][tap][K group][pieces][2][bn][16 bytes] operand tiles of the filters
+    int win_bn = 0, win_ntiles = 0;
+    bool on_tensor() const { return tc_ready || win_ready; }
     // few-row dense FC on the tensor cores (weights as the M operand, K split over CTAs)
     int32_t* ft_acc = nullptr;              // [rows][tiles * 128] partial sums, zero between launches
     unsigned* ft_arrive = nullptr;          // [tiles] arrival counters, zero between launches
@@ -347,6 +352,11 @@ int conv_tc_create(rrm_net* net, Layer& L, const void* W_dev);
 int launch_conv_tc(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
                    const uint32_t* count_bitmap = nullptr, void* P_dst = nullptr, int frames = 1, long long arena_stride = 0);
 int zero_projection(void* P, long long words, cudaStream_t st);
+
+// ---- rrm_conv_win.cu
+int conv_win_create(rrm_net* net, Layer& L, const void* W_dev);
+int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
+                    const uint32_t* count_bitmap = nullptr, void* P_dst = nullptr, int frames = 1, long long arena_stride = 0);
 
 // ---- rrm_conv.cu
 int conv_layer_create(rrm_net* net, Layer& L, const void* W_dev, const void* bias_dev);

@@ -1321,21 +1321,25 @@ int conv_layer_create(rrm_net* net, Layer& L, const void* W_dev, const void* bia
     L.ku = d.kh * d.kw * L.u_in;
     L.kup = round_up(L.ku, TK);
     L.np = round_up(d.c_out, TN);
-    RRM_TRY(dev_alloc(net, &L.Wk, (size_t)L.kup * L.np * 4));
     RRM_TRY(dev_alloc(net, &L.bias, (size_t)d.c_out * 4));
     RRM_TRY(dev_alloc(net, &L.P, (size_t)L.opixels() * d.c_out * 4));
     if (bias_dev) RRM_CUDA_TRY(cudaMemcpy(L.bias, bias_dev, (size_t)d.c_out * 4, cudaMemcpyDeviceToDevice));
+    if (d.kh * d.kw > 128) return RRM_ERR_UNSUPPORTED;       // the kernels keep a row's usable taps in a 128-bit mask
+    if (d.variant != RRM_VARIANT_GATHER) {
+        // the window kernel where it takes the layer, else the kernel that gathers compacted rows (int8 and binary)
+        const int s = conv_win_create(net, L, W_dev);
+        if (s != RRM_ERR_UNSUPPORTED) return s;
+        if (conv_tc_eligible(net, L)) return conv_tc_create(net, L, W_dev);
+    }
+    RRM_TRY(dev_alloc(net, &L.Wk, (size_t)L.kup * L.np * 4));
     const int tot = L.kup * L.np;
     pack_weights_kernel<<<ceil_div(tot, 256), 256>>>(W_dev, reinterpret_cast<uint32_t*>(L.Wk),
                                                     d.dtype == RRM_F32 ? T_F32 : (d.dtype == RRM_I8 ? T_I8 : T_BIN),
                                                     d.c_in, d.c_out, d.kh, d.kw, L.u_in, L.kup, L.np);
     RRM_CUDA_TRY(cudaGetLastError());
-    if (d.kh * d.kw > 128) return RRM_ERR_UNSUPPORTED;       // the kernels keep a row's usable taps in a 128-bit mask
-
     RRM_TRY(gemm_allow_smem<T_F32>());
     RRM_TRY(gemm_allow_smem<T_I8>());
     RRM_TRY(gemm_allow_smem<T_BIN>());
-    if (d.variant != RRM_VARIANT_GATHER && conv_tc_eligible(net, L)) RRM_TRY(conv_tc_create(net, L, W_dev));
     return RRM_OK;
 }
 
@@ -1506,9 +1510,10 @@ int launch_layer(rrm_net* net, int l, bool dense, bool stateless, cudaStream_t s
         p.ksplit = ks;
         grid.z = ks;
         // (integer shares add onto a zeroed projection; fp32 shares meet in their cluster's shared memory, in a fixed order)
-        if (!L.tc_ready && conv_dense && ks > 1 && d.dtype != RRM_F32) RRM_TRY(zero_projection(p.P, (long long)L.opixels() * d.c_out, st));
+        if (!L.on_tensor() && conv_dense && ks > 1 && d.dtype != RRM_F32) RRM_TRY(zero_projection(p.P, (long long)L.opixels() * d.c_out, st));
     }
-    if (L.tc_ready) RRM_TRY(launch_conv_tc(net, L, in, conv_dense, stateless, st, p.count_bitmap, split ? split->dP : nullptr));
+    if (L.win_ready) RRM_TRY(launch_conv_win(net, L, in, conv_dense, stateless, st, p.count_bitmap, split ? split->dP : nullptr));
+    else if (L.tc_ready) RRM_TRY(launch_conv_tc(net, L, in, conv_dense, stateless, st, p.count_bitmap, split ? split->dP : nullptr));
     else if (d.dtype == RRM_F32) { if (conv_dense) launch_gemm<T_F32, true>(p, grid, st); else launch_gemm<T_F32, false>(p, grid, st); }
     else if (d.dtype == RRM_I8) { if (conv_dense) launch_gemm<T_I8, true>(p, grid, st); else launch_gemm<T_I8, false>(p, grid, st); }
     else { if (conv_dense) launch_gemm<T_BIN, true>(p, grid, st); else launch_gemm<T_BIN, false>(p, grid, st); }
@@ -1719,7 +1724,8 @@ int launch_layer_seq(rrm_net* net, int l, int frames, long long arena_stride, cu
     const rrm_layer_desc& d = L.d;
     Tensor& in = net->tensors[d.src];
     if (!L.dPall || frames < 1) return RRM_ERR_INVALID_ARG;
-    if (L.tc_ready) RRM_TRY(launch_conv_tc(net, L, in, false, false, st, nullptr, L.dPall, frames, arena_stride));
+    if (L.win_ready) RRM_TRY(launch_conv_win(net, L, in, false, false, st, nullptr, L.dPall, frames, arena_stride));
+    else if (L.tc_ready) RRM_TRY(launch_conv_tc(net, L, in, false, false, st, nullptr, L.dPall, frames, arena_stride));
     else {
         ConvParams p{};
         p.D = in.D; p.X = in.Xn_cur ? in.Xn_cur : in.X; p.in_act = in.act; p.oact = L.oact; p.ocount = L.ocount;

@@ -1,0 +1,1008 @@
+// Convolution on the tensor cores through windows of the input kept in shared memory (int8, binary and fp32 layers,
+// delta and dense; tcgen05.mma kind::i8 and kind::f16).
+//
+// What bounds a convolution as an implicit GEMM here is not the tensor core but the way of its A operand into shared
+// memory: gathered tap by tap, every input pixel is copied kh * kw times.  This kernel copies it once:
+//   - the output pixels of all images are numbered in one linear space with row pitch Wq and image pitch Hq * Wq, so
+//     much wider than the image that the zero padding of a row is the start of the next one.  In that space the input
+//     pixel under tap (ky, kx) of output pixel i is pixel i + shift(ky, kx): an accumulator tile of 128 consecutive
+//     output pixels reads 128 consecutive input pixels for every tap, from `shift` on;
+//   - the window of input pixels that the tile's taps touch is laid out in shared memory as [16 bytes of K][pixel], the
+//     K-major layout without swizzle whose row groups are 128 bytes apart, so a tap's operand is the same window read
+//     from a start address 16 * shift bytes further on: no copy per tap at all;
+//   - a stride s splits the input into s * s planes (pixels of equal remainders), each with taps of its own that are
+//     again shifts within the plane; a block of the K loop is one plane and some channels;
+//   - first layers (at most 4 channels) have too few K bytes per pixel: their windows hold, per output column, the kw
+//     pixels of a filter row side by side (a copy per column instead of one per tap), and the taps are the filter rows.
+// Pixels that did not change (delta) or lie outside the image are zero in the window.  A tile none of whose projection
+// pixels has to be updated leaves at once; there is no compaction of rows below that (a tile's MMAs cost less than
+// finding its rows did).
+//
+// fp32 layers: every operand is split into three bf16 pieces (8 + 8 + 8 bits: all 24 bits of the significand), and six
+// of the nine products of pieces are formed; what the other three would add is below 2^-25 of a product, less than the
+// rounding of one fp32 multiplication.  The tensor core adds in fp32 but truncates, so the leading product has an
+// accumulator that is added to registers (round to nearest) after at most WN_PROMOTE K steps of 16, and the five
+// small ones have one of their own.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
+// a chain of fmaf 6e-7; without the promotion 1.7e-6, with everything in one accumulator 1.5e-5.
+//
+// Roles: warps 0-7 fill windows and drain accumulators, warp 8 issues the MMAs, warp 9 the bulk copies of the filters
+// (packed at create time as the operand tiles they are).  K can be split over the CTAs of a cluster by blocks: the
+// partial tiles are added through distributed shared memory in a fixed order (fp32 results are reproducible bit for bit,
+// and a dense pass needs no zeroed projection).  Every wait on an mbarrier is bounded; one that runs out sets
+// ERRW_TIMEOUT and the CTA leaves through the common exit.
+//
+// Measured, AlexNet-shaped stack at 227 x 227, against the kernels that gathered rows tap by tap (fp32: on the CUDA cores):
+// fp32, 32 frames of one stream 1700 -> 818 us (conv2: 351 -> 195, conv4: 412 -> 167), 8 streams 546 -> 269; int8, one
+// frame 84 -> 70, 32 dense frames 266 -> 212 (conv1: 62 -> 44, conv2: 43 -> 28); ResNet-18 shape, 4 streams 344 -> 278.
+// A launch of a few tiles is a chain of ~7 us: rows and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7.
+#include "rrm_common.cuh"
+#include "rrm_tc.cuh"
+#include "rrm_dev.cuh"
+#include <type_traits>
+
+namespace rrm {
+
+constexpr int WN_FILL = 256;                  // threads that fill windows and drain accumulators: two warpgroups
+constexpr int WN_THREADS = WN_FILL + 64;
+constexpr int WN_MAX_STAGES = 8, WN_MAX_ABUF = 4, WN_MAX_MT = 2;
+constexpr int WN_MAX_SPAN = 1152;             // pixels of one plane of a window
+constexpr int WN_PROMOTE = 32;                // fp32: K steps the leading product accumulates before it is promoted
+constexpr size_t WN_SMEM_LIMIT = 227 * 1024;
+
+// One plane's taps: first filter row / column and their numbers, the remainders of its pixels, the first tap's shift.
+struct WinPlane { int ky0, kx0, ny, nx, ry, rx, shift0; };
+constexpr int WN_MAX_PLANES = 16;
+
+// x / d for 0 <= x < 2^31 as a 64-bit product and a shift
+struct WinDiv { unsigned m, sh; };
+
+struct WinParams {
+    const void* A;            // int8 / fp32: delta rows (delta) or values (dense); binary: changed bits (delta) / unused
+    const void* Anew;         // binary: current sign bits
+    const uint32_t* in_act;   // input activity bitmap (delta mode)
+    const uint32_t* oact;     // projection pixels to update (delta mode)
+    int* ocount;              // their number is added here
+    const unsigned char* Wimg;      // [n tile][tap][group][pieces][2][bn][16 bytes]
+    const void* bias;
+    void* P;                  // [opixels][c_out]
+    int* errw;
+    const uint32_t* count_bitmap;   // dense evaluation inside a delta step: the layer's update bitmap, whose bits are counted
+    int n, h, w, oh, ow, kh, kw, stride, pad, c_in, c_out;
+    int row_units;            // units per input pixel: bytes, words or floats
+    int Wq, Hq;               // pitches of the linear output space
+    int min_shift, span, L;   // window: first pixel relative to the tile's first, pixels, 16-byte slots per K chunk
+    int planes;
+    WinPlane plane[WN_MAX_PLANES];
+    WinDiv div_img, div_row;  // by Hq * Wq and by Wq
+    int groups, gblk, nchb, nblk;   // 32-byte K groups per tap, groups per block, channel blocks per plane, blocks
+    int ks, per;              // CTAs that share a tile's blocks, blocks of each
+    int tsplit;               // > 1: a share is one block's taps, cut into so many parts (ks = nblk * tsplit)
+    int cluster;              // the shares of a tile form a cluster that adds them up (0: each adds onto the projection by itself)
+    int eager;                // filter copies start before it is known whether the tile has anything to update
+    int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
+    int tps, stages, abuf;    // taps per filter stage, stages, window buffers
+    unsigned stage_bytes, abytes, tail_off, tmem_cols;    // (tail_off: barriers and tables, behind windows, stages and drained rows)
+    unsigned wait_limit;
+    int frames;               // several frames in one launch (delta only; gridDim.z = frames x ks), distances as in TcParams
+    long long row_stride, arena_stride, p_stride;
+    int store;                // delta: the product is stored, not added
+};
+
+struct WinTail {
+    unsigned long long afull[WN_MAX_ABUF], aempty[WN_MAX_ABUF], bfull[WN_MAX_STAGES], bempty[WN_MAX_STAGES], dfull[2], dempty[2], done;
+    uint32_t tmem_base;
+    int fail;
+    int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
+    int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
+    int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row
+};
+
+// ---- small device helpers
+// Low half of an operand descriptor: start address and the distance between the two 16-byte K chunks of an MMA, both in
+// units of 16 bytes; the high half is the same for all (row groups 128 bytes apart, no swizzle).
+__device__ __forceinline__ uint32_t wn_desc_lo(uint32_t addr, uint32_t k_slots) { return ((addr & 0x3ffffu) >> 4) | k_slots << 16; }
+constexpr uint32_t WN_DESC_HI = (128u >> 4) | 1u << 14;
+// One MMA (kind::i8 or kind::f16) of the lane with e != 0, in code the whole warp runs.  The descriptors come as 32-bit
+// halves of which only the low one changes from MMA to MMA.
+template <bool F16>
+__device__ __forceinline__ void wn_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate, uint32_t e)
+{
+    if (F16)
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+            "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+            "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
+            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+            "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+            "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+            "@q tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
+            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
+}
+__device__ __forceinline__ void wn_commit(uint32_t bar, uint32_t e)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(e) : "memory");
+}
+__device__ __forceinline__ uint32_t wn_elect()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+__device__ __forceinline__ void wn_ld32(uint32_t taddr, uint32_t (&v)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// the filling warps agree (and meet): true only if all of them say so
+__device__ __forceinline__ bool wn_agree(bool ok)
+{
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "barrier.cta.red.and.pred q, 1, 256, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(r) : "r"((int)ok) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void wn_meet() { asm volatile("barrier.cta.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void wn_cluster_meet()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint4 wn_ld_remote(uint32_t addr, uint32_t rank)
+{
+    uint4 v;
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %4, %5;\n\t"
+        "ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [r];\n\t}"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+// two floats -> their three bf16 pieces, packed (low half: the first float)
+__device__ __forceinline__ void wn_split(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2)
+{
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(b), "f"(a));
+    a -= __uint_as_float(p0 << 16); b -= __uint_as_float(p0 & 0xffff0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(b), "f"(a));
+    a -= __uint_as_float(p1 << 16); b -= __uint_as_float(p1 & 0xffff0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(b), "f"(a));
+}
+__device__ __forceinline__ uint32_t wn_spread4(uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; }
+__device__ __forceinline__ int wn_div(int x, const WinDiv& d) { return (int)((unsigned long long)(unsigned)x * d.m >> d.sh); }
+
+// The windows' table for one plane: where each window pixel lies in the input.
+template <bool DENSE, bool XCOL>
+__device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_act, WinTail* S, int lin0, int plane)
+{
+    const int ry = p.plane[plane].ry, rx = p.plane[plane].rx;
+    const int hwq = p.Hq * p.Wq;
+    #pragma unroll 2
+    for (int i = threadIdx.x; i < p.span; i += WN_FILL) {
+        const int lin = lin0 + p.min_shift + i;
+        int off = -1, x0 = 0;
+        if (lin >= 0) {
+            const int img = wn_div(lin, p.div_img), rem = lin - img * hwq, Y = wn_div(rem, p.div_row), X = rem - Y * p.Wq;
+            const int iy = Y * p.stride + ry;
+            if (XCOL) {
+                x0 = X * p.stride - p.pad;
+                if (img < p.n && iy < p.h) off = (img * p.h + iy) * p.w;
+            } else {
+                const int ix = X * p.stride + rx;
+                if (img < p.n && iy < p.h && ix < p.w) {
+                    const int pix = (img * p.h + iy) * p.w + ix;
+                    if (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u)) off = pix * p.row_units;
+                }
+            }
+        }
+        S->src[i] = off;
+        if (XCOL) S->x0[i] = x0;
+    }
+}
+
+// DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.
+template <int DT, bool DENSE, bool XCOL>
+__global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kernel(const __grid_constant__ WinParams p)
+{
+    constexpr int PIECES = DT == T_F32 ? 3 : 1;
+    extern __shared__ unsigned char wn_smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tile = blockIdx.x, ntile = blockIdx.y;
+    const int frame = (!DENSE && p.frames > 1) ? blockIdx.z / p.ks : 0, split = blockIdx.z - frame * p.ks;
+    // (the frame's data; the parameters themselves stay in constant memory)
+    const long long row_off = frame * p.row_stride, arena_off = frame * p.arena_stride;
+    const char* const A = (const char*)p.A + row_off;
+    const char* const Anew = (const char*)p.Anew + row_off;
+    const uint32_t* const in_act = shift_bytes(p.in_act, arena_off);
+    const uint32_t* const oact = shift_bytes(p.oact, arena_off);
+    char* const P = (char*)p.P + frame * p.p_stride * 4;
+    unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)wn_smem_raw + 127) & ~(uintptr_t)127);
+    const uint32_t base_u32 = smem_u32(base), bstage_u32 = base_u32 + p.abuf * p.abytes;
+    WinTail* S = reinterpret_cast<WinTail*>(base + p.tail_off);
+    const int lin0 = tile * p.mt * TC_M;
+    const int b0 = p.tsplit > 1 ? split / p.tsplit : split * p.per, b1 = min(p.nblk, b0 + p.per);
+    const int part = p.tsplit > 1 ? split - b0 * p.tsplit : 0;
+    const uint32_t unit_b = (uint32_t)p.bn * 32u * PIECES;   // filter bytes of one (tap, group)
+    bool ok = true;
+    int issued = 0;                                          // stages the loader has filled
+
+    // ================= filters: the loader's walk over its blocks' taps, resumed where it stopped
+    int lb = b0, lt = -1, lstage = 0;                        // block, next tap within it (-1: the block has not been started), stage
+    uint32_t lphase = 1;
+    auto load_stages = [&](int most) {                       // (one thread) fills up to `most` stages
+        while (lb < b1 && most > 0) {
+            const int plane = lb / p.nchb, chb = lb - plane * p.nchb;
+            const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
+            const int nx = p.plane[plane].nx, ntap = p.plane[plane].ny * nx;
+            const int t_end = p.tsplit > 1 ? (part + 1) * ntap / p.tsplit : ntap;
+            if (lt < 0) lt = p.tsplit > 1 ? part * ntap / p.tsplit : 0;
+            const uint32_t bytes = unit_b * (uint32_t)gn, tap_bytes = (uint32_t)p.groups * unit_b;
+            const int row_taps = XCOL ? 1 : p.kw;            // taps of a filter row
+            const uint32_t step_x = tap_bytes * (uint32_t)p.stride, step_y = tap_bytes * (uint32_t)(row_taps * p.stride) - step_x * (uint32_t)(nx - 1);
+            int jx = lt % nx;
+            const unsigned char* src = p.Wimg + ((size_t)ntile * (row_taps * p.kh) * p.groups + g0) * unit_b +
+                                       (size_t)((p.plane[plane].ky0 + lt / nx * p.stride) * row_taps + p.plane[plane].kx0 + jx * p.stride) * tap_bytes;
+            for (; lt < t_end && most > 0; --most) {
+                if (!mbar_wait(smem_u32(&S->bempty[lstage]), lphase, p.wait_limit) || *(volatile int*)&S->fail) { ok = false; return; }
+                const int tn = min(p.tps, t_end - lt);
+                const uint32_t bar = smem_u32(&S->bfull[lstage]);
+                mbar_arrive_expect_tx(bar, bytes * (uint32_t)tn);
+                uint32_t dst = bstage_u32 + lstage * p.stage_bytes;
+                for (int t = 0; t < tn; ++t) {
+                    bulk_copy_g2s(dst, src, bytes, bar);
+                    dst += bytes;
+                    if (++jx == nx) { jx = 0; src += step_y; } else src += step_x;
+                }
+                lt += tn;
+                ++issued;
+                if (++lstage == p.stages) { lstage = 0; lphase ^= 1; }
+            }
+            if (lt >= t_end) { ++lb; lt = -1; }
+        }
+    };
+
+    pdl_launch_dependents();
+    if (tid == 0) {
+        for (int s = 0; s < p.abuf; ++s) { mbar_init(smem_u32(&S->afull[s]), WN_FILL); mbar_init(smem_u32(&S->aempty[s]), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&S->dfull[s]), 1); mbar_init(smem_u32(&S->dempty[s]), WN_FILL); }
+        mbar_init(smem_u32(&S->done), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&S->tmem_base)), "r"(p.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == WN_FILL + 32) {
+        S->fail = 0;
+        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&S->bfull[s]), 1); mbar_init(smem_u32(&S->bempty[s]), 1); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+        if (p.eager) load_stages(2);                          // (filters are nobody's work: no wait for the predecessors)
+    }
+    // ---- the tile's rows, and the first plane's table
+    int active;
+    {
+        int q = -1;
+        bool bit = false;
+        if (tid < WN_FILL) {
+            pdl_wait();                                      // bitmaps and inputs are the predecessors' work
+            if (tid < p.mt * TC_M) {
+                const int hwq = p.Hq * p.Wq;
+                const int lin = lin0 + tid, img = wn_div(lin, p.div_img), rem = lin - img * hwq, oy = wn_div(rem, p.div_row), ox = rem - oy * p.Wq;
+                if (img < p.n && oy < p.oh && ox < p.ow) q = (img * p.oh + oy) * p.ow + ox;
+                if (!DENSE && q >= 0 && !((oact[q >> 5] >> (q & 31)) & 1u)) q = -1;
+                bit = DENSE ? (p.count_bitmap && q >= 0 && ((p.count_bitmap[q >> 5] >> (q & 31)) & 1u)) : q >= 0;
+                S->q[tid] = q;
+            }
+            wn_table<DENSE, XCOL>(p, in_act, S, lin0, b0 / p.nchb);
+        }
+        tc_fence_before();
+        active = __syncthreads_count(bit);
+        tc_fence_after();
+        if (active && tid == 0 && ntile == 0 && split == 0) atomicAdd(shift_bytes(p.ocount, arena_off), active);
+    }
+    const uint32_t tmem = S->tmem_base;
+    if (!DENSE && active == 0) {                             // nothing to update (every share of the tile sees the same)
+        if (tid == WN_FILL + 32)
+            for (int j = 0; j < issued; ++j) mbar_wait(smem_u32(&S->bfull[j]), 0, WAIT_LIMIT_DEFAULT);
+        if (warp == 8)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
+        return;
+    }
+    // this thread's accumulator rows and columns: with two tiles each warpgroup drains one, else each half of the columns
+    const int wg = warp >> 2, m_own = p.mt > 1 ? wg : 0;
+    const int c_lo = p.mt > 1 ? 0 : wg * 64, c_hi = p.mt > 1 ? p.bn : min(p.bn, c_lo + 64);
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    float facc[DT == T_F32 ? 128 : 1];                       // fp32: the promoted sums of this thread's row
+
+    if (warp < 8) {
+        // ================= windows
+        if (DT == T_F32) {
+            #pragma unroll
+            for (int j = 0; j < 128; ++j) facc[j] = 0.f;
+        }
+        auto promote = [&](int ib) -> bool {                 // adds the leading accumulator of block ib to the registers and gives it back
+            if (DT != T_F32) return true;
+            const int pb = p.mt > 1 ? 0 : (ib & 1);          // (two tiles: one leading accumulator each, else two in turn)
+            const int use = p.mt > 1 ? ib : ib >> 1;
+            bool got = mbar_wait(smem_u32(&S->dfull[pb]), use & 1, p.wait_limit);
+            got = __all_sync(0xffffffffu, got);
+            if (!got) return false;
+            tc_fence_after();
+            #pragma unroll
+            for (int c0 = 0; c0 < 128; c0 += 32) {
+                if (c_lo + c0 < c_hi) {
+                    uint32_t v[32];
+                    wn_ld32(tmem + lane_base + (uint32_t)((p.mt > 1 ? m_own : pb) * p.bn + c_lo + c0), v);
+                    #pragma unroll
+                    for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? c0 + j : 0] += __uint_as_float(v[j]);
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(smem_u32(&S->dempty[pb]));
+            return true;
+        };
+        const bool lag = DT == T_I8 && !XCOL && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
+        int last_plane = b0 / p.nchb, ib = 0;
+        for (int b = b0; b < b1; ++b, ++ib) {
+            const int buf = ib % p.abuf;
+            ok = mbar_wait(smem_u32(&S->aempty[buf]), ((ib / p.abuf) & 1) ^ 1, p.wait_limit) && *(volatile int*)&S->fail == 0;
+            if (!wn_agree(ok)) { ok = false; break; }
+            const int plane = b / p.nchb, chb = b - plane * p.nchb;
+            const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
+            if (plane != last_plane) {
+                last_plane = plane;
+                wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane);
+                wn_meet();
+            }
+            const uint32_t Ab = base_u32 + buf * p.abytes;
+            unsigned char* Ap = base + buf * p.abytes;
+            const int cl = XCOL && DT == T_I8 ? (p.kw + 3) >> 2 : gn * 2;      // 16-byte chunks per pixel
+            const uint32_t piece = (uint32_t)(gn * 2 * p.L) * 16u;              // bytes between the fp32 pieces' windows
+            const unsigned magic = cl > 1 ? (unsigned)(((1ull << 32) + cl - 1) / cl) : 0u;
+            const int items = p.span * cl;
+            if (DT == T_I8 && !XCOL) {
+                const unsigned char* src0 = reinterpret_cast<const unsigned char*>(A) + g0 * 32;
+                #pragma unroll 4
+                for (int idx = tid; idx < items; idx += WN_FILL) {
+                    const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
+                    const int off = S->src[i];
+                    cp_async16(Ab + (uint32_t)(c * p.L + i) * 16u, off >= 0 ? src0 + off + c * 16 : src0, off >= 0 ? 16u : 0u);
+                }
+                cp_async_commit();
+                if (!lag) {
+                    cp_async_wait<0>();
+                    fence_async_smem();
+                    mbar_arrive(smem_u32(&S->afull[buf]));
+                } else if (ib > 0) {
+                    cp_async_wait<1>();
+                    fence_async_smem();
+                    mbar_arrive(smem_u32(&S->afull[(ib - 1) % p.abuf]));
+                }
+            } else if (DT == T_I8) {
+                // first layer, a 4-byte word per pixel: four neighbouring pixels of an image row are one chunk
+                const uint32_t* Aw = reinterpret_cast<const uint32_t*>(A);
+                #pragma unroll 4
+                for (int idx = tid; idx < items; idx += WN_FILL) {
+                    const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
+                    const int row = S->src[i], x = S->x0[i] + 4 * c;
+                    uint32_t v[4] = {0u, 0u, 0u, 0u};
+                    if (row >= 0) {
+                        unsigned bits = 0xfu;                // which of the four pixels count
+                        if (!DENSE) {
+                            const int g = max(row + x, 0), sh = g & 31;
+                            unsigned long long two = in_act[g >> 5];
+                            if (sh > 28 && row + p.w > ((g >> 5) + 1) * 32) two |= (unsigned long long)in_act[(g >> 5) + 1] << 32;
+                            bits = (unsigned)(two >> sh);
+                            if (row + x < 0) bits <<= -(row + x);
+                        }
+                        #pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (x + e >= 0 && x + e < p.w && (bits >> e & 1u)) v[e] = Aw[row + x + e];
+                    }
+                    *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = make_uint4(v[0], v[1], v[2], v[3]);
+                }
+                fence_async_smem();
+                mbar_arrive(smem_u32(&S->afull[buf]));
+            } else if (DT == T_BIN) {
+                // bits -> bytes: +2 / -2 per changed channel (dense: +1 / -1), 0 beyond the channels and outside the image
+                const uint32_t* Cu = reinterpret_cast<const uint32_t*>(A) + g0;
+                const uint32_t* Nu = reinterpret_cast<const uint32_t*>(Anew) + g0;
+                #pragma unroll 4
+                for (int idx = tid; idx < items; idx += WN_FILL) {
+                    const int i = (int)__umulhi((unsigned)idx, magic), c = idx - i * cl;      // (cl >= 2)
+                    const int off = S->src[i];
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (off >= 0) {
+                        const int ch0 = (g0 * 2 + c) * 16;
+                        const uint32_t valid = ch0 >= p.c_in ? 0u : (ch0 + 16 > p.c_in ? (1u << (p.c_in - ch0)) - 1u : 0xffffu);
+                        const int sh = (c & 1) * 16;
+                        const uint32_t nb = Nu[off + (c >> 1)] >> sh;
+                        uint32_t pos, neg;
+                        if (DENSE) { pos = nb & valid; neg = ~nb & valid; }
+                        else { const uint32_t ch = (Cu[off + (c >> 1)] >> sh) & valid; pos = ch & nb; neg = ch & ~nb; }
+                        const uint32_t pm = DENSE ? 0x01u : 0x02u, nm = DENSE ? 0xffu : 0xfeu;
+                        v.x = wn_spread4(pos) * pm + wn_spread4(neg) * nm;
+                        v.y = wn_spread4(pos >> 4) * pm + wn_spread4(neg >> 4) * nm;
+                        v.z = wn_spread4(pos >> 8) * pm + wn_spread4(neg >> 8) * nm;
+                        v.w = wn_spread4(pos >> 12) * pm + wn_spread4(neg >> 12) * nm;
+                    }
+                    *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = v;
+                }
+                fence_async_smem();
+                mbar_arrive(smem_u32(&S->afull[buf]));
+            } else {
+                const float* Af = reinterpret_cast<const float*>(A);
+                const bool vec = (p.row_units & 3) == 0;
+                #pragma unroll 2
+                for (int idx = tid; idx < items; idx += WN_FILL) {
+                    const int i = (int)__umulhi((unsigned)idx, magic), c = idx - i * cl;
+                    const int off = S->src[i];
+                    float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                    if (off >= 0) {
+                        if (XCOL) {
+                            // two neighbouring pixels x 4 channels
+                            const int xx = S->x0[i] + 2 * (g0 * 2 + c);
+                            #pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int pix = off + xx + e;
+                                if (xx + e >= 0 && xx + e < p.w && (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u))) {
+                                    #pragma unroll
+                                    for (int ch = 0; ch < 4; ++ch) if (ch < p.c_in) x[e * 4 + ch] = Af[(size_t)pix * p.row_units + ch];
+                                }
+                            }
+                        } else {
+                            const int ch0 = (g0 * 2 + c) * 8;
+                            if (vec) {
+                                if (ch0 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0); x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w; }
+                                if (ch0 + 4 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0 + 4); x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w; }
+                            } else {
+                                #pragma unroll
+                                for (int j = 0; j < 8; ++j) if (ch0 + j < p.c_in) x[j] = Af[off + ch0 + j];
+                            }
+                        }
+                    }
+                    uint32_t s[3][4];
+                    #pragma unroll
+                    for (int j = 0; j < 4; ++j) wn_split(x[2 * j], x[2 * j + 1], s[0][j], s[1][j], s[2][j]);
+                    unsigned char* dst = Ap + (size_t)(c * p.L + i) * 16;
+                    #pragma unroll
+                    for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + k * piece) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
+                }
+                fence_async_smem();
+                mbar_arrive(smem_u32(&S->afull[buf]));
+                if (ib > 0 && !promote(ib - 1)) { *(volatile int*)&S->fail = 1; ok = false; }
+                // (a warp whose wait ran out says so when the warps meet at the next block)
+            }
+        }
+        if (DT == T_I8 && !XCOL) {
+            cp_async_wait<0>();
+            fence_async_smem();
+            if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[(ib - 1) % p.abuf]));
+        }
+        if (DT == T_F32 && ok && ib > 0 && !promote(ib - 1)) ok = false;
+    } else if (warp == 9) {
+        if (lane == 0) load_stages(1 << 30);
+    } else {
+        // ================= MMAs.  The whole warp walks and one elected lane issues: what the walk costs per stage is what
+        // the MMAs of a stage have to be longer than, and a lone thread's divergent walk is twice as long (a stage of four
+        // 128-column MMAs, 256 clocks of tensor work: 340 clocks, against 870 for a single thread with quotients in the loop)
+        const uint32_t e = wn_elect();
+        const uint32_t idesc = DT == T_F32 ? (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24)
+                                           : tc_instr_desc(p.bn);
+        // (everything below in 16-byte units)
+        const uint32_t a_step = 2u * (uint32_t)p.L, b_unit = unit_b >> 4, b_piece = 2u * (uint32_t)p.bn, bn = (uint32_t)p.bn;
+        const uint32_t stage_step = p.stage_bytes >> 4, b_lo0 = wn_desc_lo(bstage_u32, bn);
+        int ib = 0, stage = 0, buf = 0;
+        uint32_t phase = 0, a_phase = 0, b_stage = b_lo0;
+        uint32_t first = 0;                                  // 0 until the CTA's first MMA has been issued
+        for (int b = b0; b < b1 && ok; ++b, ++ib) {
+            const int plane = b / p.nchb, chb = b - plane * p.nchb;
+            const int gn = min(p.gblk, p.groups - chb * p.gblk);
+            const int nx = p.plane[plane].nx, ntap = p.plane[plane].ny * nx;
+            const int t_lo = p.tsplit > 1 ? part * ntap / p.tsplit : 0, t_hi = p.tsplit > 1 ? (part + 1) * ntap / p.tsplit : ntap;
+            const int jy = t_lo / nx;
+            int j = t_lo - jy * nx;
+            if (!mbar_wait(smem_u32(&S->afull[buf]), a_phase, p.wait_limit)) { ok = false; break; }
+            // fp32: the leading product's accumulator has to be free (two tiles: from the block before, else from two before)
+            const int pb = p.mt > 1 ? 0 : (ib & 1), use = p.mt > 1 ? ib : ib >> 1;
+            const uint32_t a_piece = (uint32_t)gn * a_step;
+            uint32_t a_row = wn_desc_lo(base_u32 + buf * p.abytes, (uint32_t)p.L) + (uint32_t)(p.plane[plane].shift0 - p.min_shift + jy * p.Wq), a_tap = a_row + (uint32_t)j;
+            const uint32_t d0 = tmem + (DT == T_F32 && p.mt == 1 ? (uint32_t)pb * bn : 0u), d1 = tmem + bn, dc = tmem + 2u * bn;   // (dc: fp32, the small products)
+            uint32_t fresh = 0;                              // fp32: 0 until the block's first MMA
+            for (int t0 = t_lo; t0 < t_hi; t0 += p.tps) {
+                if (!mbar_wait(smem_u32(&S->bfull[stage]), phase, p.wait_limit)) { ok = false; break; }
+                tc_fence_after();
+                uint32_t b_lo = b_stage;
+                for (int tn = min(p.tps, t_hi - t0); tn > 0; --tn) {
+                    uint32_t a_lo = a_tap;
+                    if (DT == T_F32) {
+                        for (int g = gn; g > 0; --g) {
+                            const uint32_t a1 = a_lo + a_piece, a2 = a1 + a_piece, b1_ = b_lo + b_piece, b2 = b1_ + b_piece;
+                            // the small products first: they do not wait for the leading accumulator to be drained
+                            wn_mma<true>(dc, a_lo, b1_, idesc, first, e);
+                            wn_mma<true>(dc, a1, b_lo, idesc, 1u, e);
+                            wn_mma<true>(dc, a_lo, b2, idesc, 1u, e);
+                            wn_mma<true>(dc, a1, b1_, idesc, 1u, e);
+                            wn_mma<true>(dc, a2, b_lo, idesc, 1u, e);
+                            if (p.mt > 1) {
+                                const uint32_t e0 = a_lo + TC_M, e1 = a1 + TC_M, e2 = a2 + TC_M, dd = dc + bn;
+                                wn_mma<true>(dd, e0, b1_, idesc, first, e);
+                                wn_mma<true>(dd, e1, b_lo, idesc, 1u, e);
+                                wn_mma<true>(dd, e0, b2, idesc, 1u, e);
+                                wn_mma<true>(dd, e1, b1_, idesc, 1u, e);
+                                wn_mma<true>(dd, e2, b_lo, idesc, 1u, e);
+                            }
+                            if (fresh == 0) {
+                                if (!mbar_wait(smem_u32(&S->dempty[pb]), (use & 1) ^ 1, p.wait_limit)) ok = false;
+                                tc_fence_after();
+                            }
+                            wn_mma<true>(d0, a_lo, b_lo, idesc, fresh, e);
+                            if (p.mt > 1) wn_mma<true>(d1, a_lo + TC_M, b_lo, idesc, fresh, e);
+                            fresh = first = 1;
+                            a_lo += a_step;
+                            b_lo += b_unit;
+                        }
+                    } else {
+                        #pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            if (g >= gn) break;
+                            wn_mma<false>(d0, a_lo, b_lo, idesc, g == 0 ? first : 1u, e);
+                            if (p.mt > 1) wn_mma<false>(d1, a_lo + TC_M, b_lo, idesc, g == 0 ? first : 1u, e);
+                            a_lo += a_step;
+                            b_lo += b_unit;
+                        }
+                        first = 1;
+                    }
+                    if (++j == nx) { j = 0; a_row += (uint32_t)p.Wq; a_tap = a_row; } else ++a_tap;
+                }
+                wn_commit(smem_u32(&S->bempty[stage]), e);
+                b_stage += stage_step;
+                if (++stage == p.stages) { stage = 0; phase ^= 1; b_stage = b_lo0; }
+                if (DT == T_F32 && !ok) break;
+            }
+            if (!ok) break;
+            wn_commit(smem_u32(&S->aempty[buf]), e);
+            if (DT == T_F32) wn_commit(smem_u32(&S->dfull[pb]), e);
+            if (++buf == p.abuf) { buf = 0; a_phase ^= 1; }
+        }
+        if (ok) wn_commit(smem_u32(&S->done), e);
+        else if (first) {
+            // giving up with MMAs issued: they must have completed before the tensor memory is freed
+            *(volatile int*)&S->fail = 1;
+            __threadfence_block();
+            wn_commit(smem_u32(&S->done), e);
+            mbar_wait(smem_u32(&S->done), 0, WAIT_LIMIT_DEFAULT);
+        }
+    }
+    if (!ok) { *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
+
+    // ================= accumulators out: rows of the tile(s) go to shared memory (the windows are done with); there a
+    // projection row is the work of a warp (half a warp where 64 columns are drained at a time): a lane owns 4
+    // neighbouring channels
+    const int n0 = ntile * p.bn, ncols = min(p.bn, p.c_out - n0);
+    const bool halves = p.mt > 1 && p.bn > 64;               // two tiles: 64 columns at a time, so that both fit
+    const int cw = halves ? 64 : p.bn;                       // columns per pass
+    const int ldr = cw + 4;                                  // words per staged row (16-byte aligned, staggered over the banks)
+    const bool vec = (p.c_out & 3) == 0;
+    const bool adds = !DENSE && !p.store;                    // delta: onto the stored projection
+    const bool bulk_add = adds && vec && !p.cluster;         // ... by the copy engine, a row per thread (exact in any order for integers,
+                                                             // one share only for fp32)
+    uint32_t* staged = reinterpret_cast<uint32_t*>(base);
+    if (warp < 8) {
+        if (ok && !mbar_wait(smem_u32(&S->done), 0, p.wait_limit)) { ok = false; *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
+        wn_meet();                                           // the warps agree: nobody stores results of a tile that gave up
+        ok = __all_sync(0xffffffffu, ok && *(volatile int*)&S->fail == 0);
+        tc_fence_after();
+    }
+    #pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass > 0 && !halves) break;
+        const int p0 = pass * 64;                            // first column of the pass (own columns: c_lo + c0)
+        if (warp < 8 && ok) {
+            const int r = m_own * TC_M + (warp & 3) * 32 + lane;
+            uint32_t* row = staged + (size_t)r * ldr;
+            if (pass > 0) { if (bulk_add) __syncwarp(); else wn_meet(); }    // the first pass's rows have left
+            #pragma unroll
+            for (int c0 = 0; c0 < 128; c0 += 32) {
+                if (c_lo + c0 < c_hi && (!halves || (c0 >> 6) == pass)) {
+                    uint32_t v[32];
+                    wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 + m_own : m_own) * p.bn + c_lo + c0), v);
+                    #pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        if (c_lo + c0 + j >= c_hi) break;
+                        uint4 o;
+                        if (DT == T_F32)
+                            o = make_uint4(__float_as_uint(__uint_as_float(v[j]) + facc[DT == T_F32 ? c0 + j : 0]),
+                                           __float_as_uint(__uint_as_float(v[j + 1]) + facc[DT == T_F32 ? c0 + j + 1 : 0]),
+                                           __float_as_uint(__uint_as_float(v[j + 2]) + facc[DT == T_F32 ? c0 + j + 2 : 0]),
+                                           __float_as_uint(__uint_as_float(v[j + 3]) + facc[DT == T_F32 ? c0 + j + 3 : 0]));
+                        else o = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        *reinterpret_cast<uint4*>(row + c_lo + c0 + j - p0) = o;
+                    }
+                }
+            }
+            if (bulk_add) {
+                const int lo = halves ? p0 : c_lo, hi = min(halves ? min(p0 + 64, c_hi) : c_hi, ncols), q = S->q[r];
+                fence_async_smem();                          // this thread's part of the row -> visible to the copy engine
+                if (q >= 0 && hi > lo) {
+                    char* dst = reinterpret_cast<char*>(P) + ((size_t)q * p.c_out + n0 + lo) * 4;
+                    if (DT == T_F32)
+                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
+                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(hi - lo) * 4u) : "memory");
+                    else
+                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;"
+                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(hi - lo) * 4u) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                }
+            }
+        }
+        __syncwarp();
+        if (bulk_add) continue;
+        if (p.cluster) wn_cluster_meet();                    // every share's partial tile is in its shared memory
+        else if (warp < 8) wn_meet();
+        if (warp < 8 && ok) {
+            // rows split, split + ks, ... of the tile (one share: all rows), a few at a time per warp or half warp, all shares'
+            // reads of a turn in flight together (one after the other, eight shares took 6 us)
+            const int shares = p.cluster ? p.ks : 1, mine = p.cluster ? split : 0;
+            const int rows = p.mt * TC_M;
+            const bool wide = cw > 64;
+            const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
+            const int ch = (wide ? lane : lane & 15) * 4;    // first own channel of the pass
+            const bool act_lane = p0 + ch < ncols;
+            auto close = [&](auto nr, auto ns) {
+            constexpr int NR = decltype(nr)::value, NS = decltype(ns)::value;
+            for (int k0 = team * NR; mine + k0 * shares < rows; k0 += teams * NR) {
+                uint32_t o[NR][4];
+                uint4 t[NS][NR];
+                int q[NR];
+                #pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const int r = mine + (k0 + u) * shares;
+                    q[u] = r < rows ? S->q[r] : -1;
+                    o[u][0] = o[u][1] = o[u][2] = o[u][3] = 0;
+                    if (q[u] < 0 || !act_lane) continue;
+                    if (adds || (DENSE && p.bias)) {
+                        const uint32_t* from = (adds ? reinterpret_cast<const uint32_t*>(P) + (size_t)q[u] * p.c_out
+                                                     : reinterpret_cast<const uint32_t*>(p.bias)) + n0 + p0 + ch;
+                        if (vec) { const uint4 w = *reinterpret_cast<const uint4*>(from); o[u][0] = w.x; o[u][1] = w.y; o[u][2] = w.z; o[u][3] = w.w; }
+                        else {
+                            #pragma unroll
+                            for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) o[u][j] = from[j];
+                        }
+                    }
+                }
+                #pragma unroll
+                for (int s = 0; s < NS; ++s)
+                    #pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        t[s][u] = make_uint4(0, 0, 0, 0);
+                        if (s >= shares || q[u] < 0 || !act_lane) continue;
+                        const uint32_t* at = staged + (size_t)(mine + (k0 + u) * shares) * ldr + ch;
+                        t[s][u] = NS > 1 ? wn_ld_remote(smem_u32(at), (uint32_t)s) : *reinterpret_cast<const uint4*>(at);
+                    }
+                #pragma unroll
+                for (int u = 0; u < NR; ++u)
+                    #pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        if (s >= shares) break;
+                        const uint32_t w[4] = {t[s][u].x, t[s][u].y, t[s][u].z, t[s][u].w};
+                        #pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            o[u][j] = DT == T_F32 ? __float_as_uint(__uint_as_float(o[u][j]) + __uint_as_float(w[j])) : o[u][j] + w[j];
+                    }
+                #pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    if (q[u] < 0 || !act_lane) continue;
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)q[u] * p.c_out + n0 + p0 + ch;
+                    if (vec) *reinterpret_cast<uint4*>(dst) = make_uint4(o[u][0], o[u][1], o[u][2], o[u][3]);
+                    else {
+                        #pragma unroll
+                        for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) dst[j] = o[u][j];
+                    }
+                }
+            }
+            };
+            using std::integral_constant;
+            if (shares == 1) close(integral_constant<int, 4>{}, integral_constant<int, 1>{});
+            else if (shares <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+            else close(integral_constant<int, 1>{}, integral_constant<int, 8>{});
+        }
+        __syncwarp();
+        if (p.cluster) wn_cluster_meet();                    // nobody's shared memory goes away while it is read
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (tid == WN_FILL + 32 && S->fail) {
+        // a role gave up: bulk copies still in flight must land before the CTA's shared memory goes away
+        for (int j = max(0, issued - p.stages); j < issued; ++j)
+            mbar_wait(smem_u32(&S->bfull[j % p.stages]), (j / p.stages) & 1, WAIT_LIMIT_DEFAULT);
+    }
+    if (warp == 8)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
+}
+
+// ------------------------------------------------------------------------------------------------
+// Filters as operand tiles: [n tile][tap][group][pieces][2 chunks][bn][16 bytes].  One thread per 16 bytes.
+// K within a tap: channels (int8 and binary: bytes; fp32: bf16 pieces); first layers: tap = filter row, K = kx * 4 + channel.
+// ------------------------------------------------------------------------------------------------
+template <int DT, bool XCOL>
+__global__ void pack_weights_win_kernel(const void* W, unsigned char* img, int c_in, int c_out, int kh, int kw, int taps, int groups,
+                                        int bn, int n_tiles)
+{
+    const size_t total = (size_t)n_tiles * taps * groups * 2 * bn;
+    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= total) return;
+    const int r = (int)(idx % bn), c = (int)(idx / bn % 2), g = (int)(idx / ((size_t)2 * bn) % groups);
+    const int tap = (int)(idx / ((size_t)2 * bn * groups) % taps), nt = (int)(idx / ((size_t)2 * bn * groups * taps));
+    const int co = nt * bn + r;
+    constexpr int E = DT == T_F32 ? 8 : 16, PIECES = DT == T_F32 ? 3 : 1;
+    unsigned char* dst = img + ((((size_t)nt * taps + tap) * groups + g) * PIECES * 2 + c) * bn * 16 + (size_t)r * 16;
+    auto at = [&](int e) -> size_t {                          // element e of this chunk, as an index into W ((size_t)-1: none)
+        const int k = (g * 2 + c) * E + e;
+        int ci, ky, kx;
+        if (XCOL) { ky = tap; kx = k >> 2; ci = k & 3; } else { ky = tap / kw; kx = tap - ky * kw; ci = k; }
+        if (co >= c_out || ci >= c_in || kx >= kw) return (size_t)-1;
+        return (((size_t)co * c_in + ci) * kh + ky) * kw + kx;
+    };
+    if (DT == T_F32) {
+        uint32_t s[3][4];
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const size_t a = at(2 * j), b = at(2 * j + 1);
+            wn_split(a == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[a], b == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[b],
+                     s[0][j], s[1][j], s[2][j]);
+        }
+        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + (size_t)k * 2 * bn * 16) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
+    } else {
+        uint32_t v[4] = {0, 0, 0, 0};
+        #pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const size_t a = at(e);
+            const int x = a == (size_t)-1 ? 0 : reinterpret_cast<const int8_t*>(W)[a];
+            v[e >> 2] |= ((uint32_t)x & 0xffu) << (8 * (e & 3));
+        }
+        *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// host side
+// ------------------------------------------------------------------------------------------------
+static int host_floor_div(int a, int s) { return a >= 0 ? a / s : -((s - 1 - a) / s); }
+
+// The geometry of a layer that does not depend on how it is launched; false: the layer keeps the other kernels.
+static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
+{
+    const rrm_layer_desc& d = L.d;
+    const Tensor& in = net->tensors[d.src];
+    const bool xcol = d.dtype == RRM_F32 ? d.c_in <= 4 : (d.dtype == RRM_I8 && in.cs == 4);
+    if (d.dtype == RRM_I8 && !xcol && in.cs % 32 != 0) return false;
+    p.n = d.n; p.h = d.h; p.w = d.w; p.oh = L.oh; p.ow = L.ow; p.kh = d.kh; p.kw = d.kw; p.stride = d.stride; p.pad = d.pad;
+    p.c_in = d.c_in; p.c_out = d.c_out; p.row_units = in.cs;
+    const int pyn = d.stride < d.kh ? d.stride : d.kh, pxn = xcol ? 1 : (d.stride < d.kw ? d.stride : d.kw);
+    p.planes = pyn * pxn;
+    if (p.planes > WN_MAX_PLANES) return false;
+    const int fy_lo = host_floor_div(-d.pad, d.stride), fy_hi = host_floor_div(d.kh - 1 - d.pad, d.stride);
+    const int fx_lo = xcol ? 0 : fy_lo, fx_hi = xcol ? 0 : host_floor_div(d.kw - 1 - d.pad, d.stride);
+    auto pitch = [&](int o, int size, int lo, int hi) {      // room for the pixels and for the zeros that taps reach beyond them
+        const int last = (size - 1) / d.stride;
+        int v = o;
+        v = v > o + hi ? v : o + hi;
+        v = v > last + 1 - lo ? v : last + 1 - lo;
+        return v;
+    };
+    p.Wq = xcol ? L.ow : pitch(L.ow, d.w, fx_lo, fx_hi);
+    p.Hq = pitch(L.oh, d.h, fy_lo, fy_hi);
+    p.min_shift = fy_lo * p.Wq + fx_lo;
+    const int max_shift = fy_hi * p.Wq + fx_hi;
+    for (int i = 0; i < p.planes; ++i) {
+        WinPlane& a = p.plane[i];
+        a.ky0 = i / pxn; a.kx0 = i % pxn;
+        const int fy = host_floor_div(a.ky0 - d.pad, d.stride), fx = xcol ? 0 : host_floor_div(a.kx0 - d.pad, d.stride);
+        a.ny = ceil_div(d.kh - a.ky0, d.stride); a.nx = xcol ? 1 : ceil_div(d.kw - a.kx0, d.stride);
+        a.ry = a.ky0 - d.pad - fy * d.stride; a.rx = xcol ? 0 : a.kx0 - d.pad - fx * d.stride;
+        a.shift0 = fy * p.Wq + fx;
+    }
+    auto divisor = [](int v) {
+        WinDiv r;
+        unsigned s = 0;
+        while ((1u << s) < (unsigned)v) ++s;
+        r.sh = 31 + s;
+        r.m = (unsigned)(((1ull << r.sh) + v - 1) / v);
+        return r;
+    };
+    p.div_img = divisor(p.Hq * p.Wq); p.div_row = divisor(p.Wq);
+    p.span = TC_M + max_shift - p.min_shift;                 // (one accumulator tile)
+    if (p.span > WN_MAX_SPAN) return false;
+    // (rows of the linear space without a projection pixel are work for nothing: with more than half of them a layer
+    // such as a filter that covers the whole map is better off with its rows compacted)
+    if ((long long)L.oh * L.ow * 2 < (long long)p.Hq * p.Wq) return false;
+    const int e = d.dtype == RRM_F32 ? 16 : 32;              // K elements of a group
+    p.groups = xcol ? ceil_div(d.kw * 4, e) : ceil_div(d.dtype == RRM_I8 ? in.cs : d.c_in, e);
+    const int plane_taps = ceil_div(d.kh, d.stride) * (xcol ? 1 : ceil_div(d.kw, d.stride));
+    if (d.dtype == RRM_F32 && plane_taps * (xcol ? p.groups : 1) > WN_PROMOTE) return false;
+    return true;
+}
+
+static bool win_xcol(const rrm_net* net, const Layer& L)
+{
+    return L.d.dtype == RRM_F32 ? L.d.c_in <= 4 : (L.d.dtype == RRM_I8 && net->tensors[L.d.src].cs == 4);
+}
+
+static int slots(int span) { return round_up(span, 8) + 1; }    // (neighbouring chunks of a pixel fall into different banks)
+
+// How a launch cuts the work: accumulator tiles and shares of K per CTA, window blocks, filter stages.  `wave`: CTAs that
+// are to be kept busy.
+static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool store, int frames, int wave)
+{
+    const bool f32 = L.d.dtype == RRM_F32;
+    const int pieces = f32 ? 3 : 1;
+    p.bn = L.win_bn;
+    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    const long long tiles = (rows + TC_M - 1) / TC_M * L.win_ntiles * frames;
+    const int base_span = p.span, planes = p.planes;
+    const int plane_taps = ceil_div(p.kh, p.stride) * (xcol ? 1 : ceil_div(p.kw, p.stride));
+    const size_t unit = (size_t)p.bn * 32 * pieces, tail = sizeof(WinTail) + 128;
+    const size_t room = f32 ? WN_SMEM_LIMIT - 1024 : WN_SMEM_LIMIT / 2 - 2048;   // (integer kernels: two CTAs per SM)
+    // two accumulator tiles per CTA share every filter stage (what bounds a full machine is the filters' way from L2),
+    // once that leaves a CTA per SM
+    int mt = tiles >= 2ll * 148 && rows > TC_M ? 2 : 1;
+    // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
+    // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
+    const bool clustered = dense || store || f32 || (p.c_out & 3) != 0;
+    int want = 1;
+    while (mt == 1 && want < (clustered ? 8 : 16) && tiles * (want + 1) <= wave) ++want;
+    for (; mt >= 1; mt /= 2) {
+        p.mt = mt;
+        p.span = base_span + (mt - 1) * TC_M;
+        p.L = slots(p.span);
+        const size_t staging = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4;
+        int gblk = xcol ? p.groups : (p.groups < 4 ? p.groups : 4);
+        if (f32 && !xcol) while (gblk > 1 && gblk * plane_taps > 18) gblk = (gblk + 1) / 2;
+        if (!xcol) while (gblk > 1 && planes * ceil_div(p.groups, gblk) < want) gblk = (gblk + 1) / 2;
+        for (;; gblk = (gblk + 1) / 2) {
+            p.gblk = gblk;
+            p.nchb = ceil_div(p.groups, gblk);
+            p.nblk = planes * p.nchb;
+            p.tsplit = 1;
+            p.ks = want < p.nblk ? want : p.nblk;
+            p.per = ceil_div(p.nblk, p.ks);
+            p.ks = ceil_div(p.nblk, p.per);                  // no empty share
+            if (!f32 && p.ks == p.nblk && planes == 1 && want >= 2 * p.nblk && plane_taps >= 2) {
+                p.tsplit = want / p.nblk < plane_taps ? want / p.nblk : plane_taps;
+                p.ks = p.nblk * p.tsplit;
+            }
+            p.cluster = clustered && p.ks > 1;
+            p.abytes = (unsigned)(((size_t)gblk * 2 * pieces * p.L * 16 + 127) & ~(size_t)127);
+            p.tps = 1;
+            while ((size_t)p.tps * 2 * gblk * unit <= (f32 ? 24u : 16u) * 1024 && p.tps < plane_taps) p.tps *= 2;
+            p.stage_bytes = (unsigned)(p.tps * gblk * unit);
+            for (p.abuf = p.per < WN_MAX_ABUF ? p.per : WN_MAX_ABUF; p.abuf >= 1; --p.abuf) {
+                const size_t a = (size_t)p.abuf * p.abytes + tail;
+                if (a + 3 * (size_t)p.stage_bytes > room) continue;
+                const size_t fit = (room - a) / p.stage_bytes;
+                p.stages = (int)(fit < WN_MAX_STAGES ? fit : WN_MAX_STAGES);
+                const size_t used = (size_t)p.abuf * p.abytes + (size_t)p.stages * p.stage_bytes;
+                p.tail_off = (unsigned)((used > staging ? used : staging) + 15) & ~15u;      // (the drained rows go where windows and stages were)
+                if (p.tail_off + tail > room) continue;
+                const unsigned cols = f32 ? (mt > 1 ? 3 : 2) * p.bn + round_up(p.bn, 32) : (mt - 1) * p.bn + round_up(p.bn, 32);
+                p.tmem_cols = 32;
+                while (p.tmem_cols < cols) p.tmem_cols *= 2;
+                p.eager = dense || tiles * p.ks <= 2 * 148;
+                return true;
+            }
+            if (gblk == 1 || xcol) break;
+        }
+    }
+    return false;
+}
+
+// Shared memory of a launch.  At least as large a part of an SM's as the CTA's share of the 512 tensor-memory columns: CTAs
+// that fit an SM together can then always allocate their columns together.  (A CTA that waits for columns while the rest
+// of its cluster waits for it, beside another cluster in the mirrored state, would wait forever.)
+static size_t win_smem(const WinParams& p)
+{
+    const size_t need = p.tail_off + sizeof(WinTail) + 128;
+    const size_t share = (size_t)p.tmem_cols * 228 * 1024 / 512 - 1024;
+    return need > share ? need : share;
+}
+
+template <int DT, bool XCOL>
+static int win_allow()
+{
+    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, false, XCOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    return RRM_OK;
+}
+
+// Packs the filters of a layer the window kernel takes; RRM_ERR_UNSUPPORTED: the layer keeps the other kernels.
+int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
+{
+    const rrm_layer_desc& d = L.d;
+    WinParams p{};
+    if (!win_geometry(net, L, p)) return RRM_ERR_UNSUPPORTED;
+    const bool xcol = win_xcol(net, L), f32 = d.dtype == RRM_F32;
+    L.win_ntiles = ceil_div(d.c_out, 128);
+    L.win_bn = round_up(ceil_div(d.c_out, L.win_ntiles), 16);
+    L.win_ntiles = ceil_div(d.c_out, L.win_bn);
+    if (!win_plan(L, p, xcol, true, false, 1, 148)) return RRM_ERR_UNSUPPORTED;
+    const int taps = xcol ? d.kh : d.kh * d.kw;
+    const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
+    void* img = nullptr;
+    if (cudaMalloc(&img, chunks * 16 * (f32 ? 3 : 1)) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
+    net->allocs.push_back(img);
+    L.win_Wimg = img;
+    const unsigned grid = (unsigned)((chunks + 255) / 256);
+    unsigned char* im = reinterpret_cast<unsigned char*>(img);
+    if (f32 && xcol) pack_weights_win_kernel<T_F32, true><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
+    else if (f32) pack_weights_win_kernel<T_F32, false><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
+    else if (xcol) pack_weights_win_kernel<T_I8, true><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
+    else pack_weights_win_kernel<T_I8, false><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
+    RRM_CUDA_TRY(cudaGetLastError());
+    RRM_TRY((win_allow<T_F32, true>())); RRM_TRY((win_allow<T_F32, false>()));
+    RRM_TRY((win_allow<T_I8, true>())); RRM_TRY((win_allow<T_I8, false>()));
+    RRM_TRY((win_allow<T_BIN, false>()));
+    L.win_ready = true;
+    return RRM_OK;
+}
+
+template <int DT, bool XCOL>
+static cudaError_t win_launch(const WinParams& p, bool dense, dim3 grid, size_t smem, cudaStream_t st)
+{
+    return dense ? launch_seq_cluster(conv_win_kernel<DT, true, XCOL>, grid, dim3(WN_THREADS), smem, st, p.cluster ? p.ks : 1, p)
+                 : launch_seq_cluster(conv_win_kernel<DT, false, XCOL>, grid, dim3(WN_THREADS), smem, st, p.cluster ? p.ks : 1, p);
+}
+
+// F*dI (dense: F*X + b); arguments as for launch_conv_tc.
+int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
+                    const uint32_t* count_bitmap, void* P_dst, int frames, long long arena_stride)
+{
+    const rrm_layer_desc& d = L.d;
+    WinParams p{};
+    if (!win_geometry(net, L, p)) return RRM_ERR_UNSUPPORTED;
+    const bool xcol = win_xcol(net, L), bin = d.dtype == RRM_BIN;
+    const bool batched = P_dst && frames >= 1 && arena_stride != 0;
+    const int nf = batched ? frames : 1;
+    if (!win_plan(L, p, xcol, dense, batched, nf, net->many_in_flight ? 74 : 148)) return RRM_ERR_UNSUPPORTED;
+    const void* X = stateless ? in.X2 : in.X;
+    p.A = bin ? in.D : (dense ? X : in.D);
+    p.Anew = (!dense && !stateless && in.Xn_cur) ? in.Xn_cur : X;    // (chunks of frames: this frame's copy of the new rows)
+    p.in_act = in.act; p.oact = L.oact; p.ocount = L.ocount;
+    p.Wimg = reinterpret_cast<const unsigned char*>(L.win_Wimg); p.bias = L.bias;
+    p.P = P_dst && !dense ? P_dst : (stateless ? L.P2 : L.P);
+    p.errw = net->errw;
+    p.wait_limit = net->opt.wait_limit;
+    p.count_bitmap = count_bitmap;
+    p.frames = nf;
+    p.row_stride = (long long)in.bytes(); p.arena_stride = arena_stride; p.p_stride = (long long)L.opixels() * d.c_out;
+    p.store = batched ? 1 : 0;
+    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)L.win_ntiles, (unsigned)(nf * p.ks));
+    const size_t smem = win_smem(p);
+    cudaError_t e;
+    if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, grid, smem, st) : win_launch<T_F32, false>(p, dense, grid, smem, st);
+    else if (d.dtype == RRM_I8) e = xcol ? win_launch<T_I8, true>(p, dense, grid, smem, st) : win_launch<T_I8, false>(p, dense, grid, smem, st);
+    else e = win_launch<T_BIN, false>(p, dense, grid, smem, st);
+    RRM_CUDA_TRY(e);
+    return RRM_OK;
+}
+
+}  // namespace rrm

@@ -151,6 +151,37 @@ def test_single_layer_shapes(dtype, c_in, c_out, hw, k, s, p):
     _run([sp], video, n=2, stats=True)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "i8", "bin"])
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [
+    (32, 64, (11, 10), 3, 1, 1, 1),          # one accumulator tile, K cut into parts of one block's taps
+    (160, 130, (8, 9), 3, 1, 1, 2),          # ragged blocks of K groups, two column tiles of uneven width
+    (24, 33, (30, 31), 3, 2, 1, 3),          # stride 2: four planes; rows that are no multiple of 16 bytes
+    (20, 16, (25, 23), 5, 3, 2, 1),          # stride 3: nine planes, some with fewer taps
+    (16, 20, (140, 139), 3, 1, 1, 2),        # enough rows for two accumulator tiles per thread block
+    (2, 72, (41, 38), 9, 4, 3, 2),           # few channels: filter rows side by side
+    (12, 24, (3, 1400), 3, 1, 1, 1)])        # a window wider than shared memory takes: the other kernels
+def test_window_convolution_tile_edges(dtype, c_in, c_out, hw, k, s, p, n, monkeypatch):
+    rng = np.random.default_rng(c_in * 1000 + c_out * 10 + k)
+    sp = _spec(dtype, c_in, hw, c_out, k, s, p, rng)
+    video = _video(dtype, c_in, hw, 5, n, rng)
+    _run([sp], video, n=n, stats=True, keyframe_at=(4,))
+    # the same frames as one chunk, every kernel taking all of them
+    monkeypatch.setenv("RRM_CHUNK_BY_LAYER", "1")
+    net = _rrm().net_from_specs([sp], n=n)
+    net.set_options(chunk_dense_activity=2.0, stack_dense_activity=2.0)
+    outs = net.new_output(frames=5)
+    net.step_seq(torch.stack([_frame_to_dev([sp], f) for f in video]), outs, 5)
+    for t in range(5):
+        want = orc.dense_forward([sp], video[t])[0][1]
+        got = outs[t].cpu().numpy()
+        if dtype == "f32":
+            assert float(np.abs(got - want).max()) <= F32_TOL * float(np.abs(want).max()), t
+        else:
+            np.testing.assert_array_equal(got.astype(np.int64), want, err_msg=f"frame {t}")
+    _compare([sp], net, video[4], 4)
+    net.close()
+
+
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [(16, 70, (13, 13), 3, 1, 1), (8, 12, (17, 15), 5, 2, 2), (64, 16, (10, 10), 3, 1, 1),
                                                  (3, 6, (35, 35), 11, 4, 0)])
