@@ -188,7 +188,12 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
     net->cleared_bytes = cleared;
     bind_arena(net, reinterpret_cast<char*>(net->cleared));
     RRM_TRY(dev_alloc(net, (void**)&net->aecs, (size_t)(1 + n_layers) * 8));
-    for (int l = 0; l < n_layers; ++l) RRM_TRY(conv_layer_create(net, net->layers[l], W[l], B ? B[l] : nullptr));
+    for (int l = 0; l < n_layers; ++l) {
+        Layer& L = net->layers[l];
+        const Tensor& out = net->tensors[l + 1];
+        RRM_TRY(conv_layer_create(net, L, W[l], B ? B[l] : nullptr));
+        if (dense_applies_f(net, l) && L.d.pool_k > 0) RRM_TRY(dev_alloc(net, &L.Apre, (size_t)L.opixels() * out.row_bytes()));
+    }
     {
         // dense evaluation of high-activity frames: only where a frame is real work (>= 1 GMAC), so that the
         // per-layer counters stay available on small stacks, and only if no layer pins its variant
@@ -668,9 +673,11 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
     for (int m0 = 0; m0 < T && status == RRM_OK; m0 += per) {
         const int F = T - m0 < per ? T - m0 : per;
         scale(F);
+        net->keep_image = kind == 1 && m0 + F == T ? (F - 1) * n0 : -1;
         fail(launch_import(net, reinterpret_cast<const char*>(net->chunk_in) + (size_t)m0 * bi, false, true, st));
         for (int l = 0; l < L && status == RRM_OK; ++l) fail(launch_layer(net, l, true, true, st));
         fail(launch_export_tensor(net, L, reinterpret_cast<char*>(net->chunk_out) + (size_t)m0 * bo, true, st));
+        net->keep_image = -1;
         unscale();
     }
     if (kind == 1 && status == RRM_OK) {

@@ -199,6 +199,7 @@ struct Layer {
     bool win_ready = false;
     void* win_Wimg = nullptr;               // [n_tiles][tap][K group][pieces][2][bn][16 bytes] operand tiles of the filters
     int win_bn = 0, win_ntiles = 0;
+    void* Apre = nullptr;                   // pooled integer layers: f before the pool window, a row per projection pixel (keyframes)
     bool on_tensor() const { return tc_ready || win_ready; }
     // few-row dense FC on the tensor cores (weights as the M operand, K split over CTAs)
     int32_t* ft_acc = nullptr;              // [rows][tiles * 128] partial sums, zero between launches
@@ -247,6 +248,8 @@ struct rrm_net {
     void* frame_buf = nullptr;        // the step's input frame, boundary layout
     void* out_buf = nullptr;          // the step's last tensor, boundary layout
     bool graph_off = false;           // RRM_NO_GRAPH=1: launch kernel by kernel (debugging)
+    int keep_image = -1;              // stateless dense pass batched over frames, state wanted: first image of the last frame, whose
+                                      // projections the convolution stores as the state (layers whose kernel applies f)
     bool many_in_flight = false;      // set while a chunk graph is captured: its launches share the machine with those of
                                       // neighbouring frames, so grids are sized for throughput instead of latency
     // where a captured sequence reads the frame and writes the output: the nodes (kernel arguments or a copy) that
@@ -355,8 +358,13 @@ int zero_projection(void* P, long long words, cudaStream_t st);
 
 // ---- rrm_conv_win.cu
 int conv_win_create(rrm_net* net, Layer& L, const void* W_dev);
+// f applied by the convolution kernel (dense passes): where its result goes (the output tensor's rows, or for a pooled
+// layer a row per projection pixel), the shortcut, and the projection to keep (nullptr: none) from pixel keep_from on.
+struct WinOutput { void* X; const void* res; int cs, bits; void* P; int keep_from; };
 int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
-                    const uint32_t* count_bitmap = nullptr, void* P_dst = nullptr, int frames = 1, long long arena_stride = 0);
+                    const uint32_t* count_bitmap = nullptr, void* P_dst = nullptr, int frames = 1, long long arena_stride = 0,
+                    const WinOutput* out = nullptr);
+int launch_pool_window(const Layer& L, const Tensor& out, const void* A, void* X, cudaStream_t st);
 
 // ---- rrm_conv.cu
 int conv_layer_create(rrm_net* net, Layer& L, const void* W_dev, const void* bias_dev);
@@ -372,6 +380,7 @@ struct SplitProjection {
 int launch_layer(rrm_net* net, int l, bool dense, bool stateless, cudaStream_t st,
                  const std::function<int(int)>* hook = nullptr, bool dense_in_step = false,
                  const SplitProjection* split = nullptr);
+bool dense_applies_f(const rrm_net* net, int l);
 int launch_export_tensor(rrm_net* net, int t, void* dst_dev, bool stateless, cudaStream_t st);
 int launch_export_projection(rrm_net* net, int l, void* dst_dev, cudaStream_t st);
 int reset_state(rrm_net* net, cudaStream_t st);

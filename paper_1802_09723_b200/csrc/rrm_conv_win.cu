@@ -38,6 +38,7 @@
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
+#include <climits>
 #include <type_traits>
 
 namespace rrm {
@@ -86,12 +87,20 @@ struct WinParams {
     int frames;               // several frames in one launch (delta only; gridDim.z = frames x ks), distances as in TcParams
     long long row_stride, arena_stride, p_stride;
     int store;                // delta: the product is stored, not added
+    // f in the kernel (dense passes): the layer's output, or what its pool window takes the maximum of, pixel by pixel
+    void* X;                  // [opixels][cs] int8, sign words or float
+    const void* res;          // shortcut values, laid out like X, or nullptr
+    const void* bn_scale;
+    const void* bn_shift;
+    int cs, bits, shift, act_fn, theta;      // (bits: signs, 32 channels per word)
+    int keep_from;            // first projection pixel whose projection is stored (at P); INT_MAX: none
 };
 
 struct WinTail {
     unsigned long long afull[WN_MAX_ABUF], aempty[WN_MAX_ABUF], bfull[WN_MAX_STAGES], bempty[WN_MAX_STAGES], dfull[2], dempty[2], done;
     uint32_t tmem_base;
     int fail;
+    int bias[128];                            // of the CTA's columns (f in the kernel)
     int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
     int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
     int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row
@@ -215,8 +224,27 @@ __device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_
     }
 }
 
-// DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.
-template <int DT, bool DENSE, bool XCOL>
+// f without pool window of 4 neighbouring channels (c: channel within the layer; channels beyond the last give zero)
+template <int PT, int OT, typename pt>
+__device__ __forceinline__ void wn_f(const WinParams& p, int c, const pt (&x)[4], const pt (&res)[4], pt (&y)[4])
+{
+    const pt v[1][4] = {{x[0], x[1], x[2], x[3]}};
+    if (p.bn_scale) epi_f<PT, OT, 1, true, pt>(v, 1u, c, res, p.c_out, p.act_fn, p.shift, p.bn_scale, p.bn_shift, y);
+    else epi_f<PT, OT, 1, false, pt>(v, 1u, c, res, p.c_out, p.act_fn, p.shift, nullptr, nullptr, y);
+}
+__device__ __forceinline__ uint32_t wn_pack4(const int (&y)[4])
+{
+    return ((uint32_t)y[0] & 0xffu) | ((uint32_t)y[1] & 0xffu) << 8 | ((uint32_t)y[2] & 0xffu) << 16 | (uint32_t)y[3] << 24;
+}
+__device__ __forceinline__ void wn_unpack4(uint32_t w, int (&y)[4])
+{
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = (int)(int8_t)(w >> (8 * j));
+}
+
+// DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.  ACT (dense passes): f is applied here and the output written,
+// instead of the projection by this kernel and f by another; the projection is stored only where a state needs it.
+template <int DT, bool DENSE, bool XCOL, bool ACT>
 __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kernel(const __grid_constant__ WinParams p)
 {
     constexpr int PIECES = DT == T_F32 ? 3 : 1;
@@ -311,6 +339,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 S->q[tid] = q;
             }
             wn_table<DENSE, XCOL>(p, in_act, S, lin0, b0 / p.nchb);
+            if (ACT && tid < p.bn) S->bias[tid] = p.bias && ntile * p.bn + tid < p.c_out ? reinterpret_cast<const int*>(p.bias)[ntile * p.bn + tid] : 0;
         }
         tc_fence_before();
         active = __syncthreads_count(bit);
@@ -607,13 +636,75 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     uint32_t* staged = reinterpret_cast<uint32_t*>(base);
     if (warp < 8) {
         if (ok && !mbar_wait(smem_u32(&S->done), 0, p.wait_limit)) { ok = false; *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
-        wn_meet();                                           // the warps agree: nobody stores results of a tile that gave up
-        ok = __all_sync(0xffffffffu, ok && *(volatile int*)&S->fail == 0);
+        ok = wn_agree(ok && *(volatile int*)&S->fail == 0);   // nobody stores results of a tile that gave up
         tc_fence_after();
+    }
+    const bool direct = ACT && DT != T_F32 && !p.cluster;    // f straight from the accumulator registers
+    if (ACT && DT != T_F32 && direct && warp < 8 && ok) {
+        const int r = m_own * TC_M + (warp & 3) * 32 + lane;
+        const int q = S->q[r];
+        const bool keep = q >= p.keep_from;                  // (q >= 0 then)
+        uint32_t* row = staged + (size_t)r * ldr;
+        int32_t* dstP = reinterpret_cast<int32_t*>(P) + (size_t)(keep ? q - p.keep_from : 0) * p.c_out + n0;
+        #pragma unroll
+        for (int c0 = 0; c0 < 128; c0 += 32) {
+            if (c_lo + c0 >= c_hi) continue;                 // (uniform; columns come in whole groups of 32)
+            const int cc = c_lo + c0;
+            uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+            if (p.res && q >= 0) {
+                const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const int8_t*>(p.res) + (size_t)q * p.cs + n0 + cc);
+                if (n0 + cc < p.cs) { rw[0] = src[0]; rw[1] = src[1]; }
+            }
+            uint32_t v[32];
+            __syncwarp();
+            wn_ld32(tmem + lane_base + (uint32_t)(m_own * p.bn + cc), v);
+            #pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += (uint32_t)S->bias[cc + j];
+            if (keep) {
+                if (vec) {
+                    const int rc = halves ? cc & 63 : cc;    // (two tiles: the row buffer holds 64 columns at a time)
+                    if (halves && rc == 0 && c0 > 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    #pragma unroll
+                    for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(row + rc + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    const int cols = min(32, ncols - cc);
+                    fence_async_smem();
+                    if (cols > 0) {
+                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                     ::"l"(dstP + cc), "r"(smem_u32(row + rc)), "r"((uint32_t)cols * 4u) : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                } else {
+                    #pragma unroll
+                    for (int j = 0; j < 32; ++j) if (cc + j < ncols) dstP[cc + j] = (int32_t)v[j];
+                }
+            }
+            if (q < 0) continue;
+            if (p.bits) {
+                uint32_t word = 0;
+                #pragma unroll
+                for (int j = 0; j < 32; ++j) if (cc + j < ncols && (int)v[j] >= p.theta) word |= 1u << j;
+                if (((n0 + cc) >> 5) < p.cs) reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + ((n0 + cc) >> 5)] = word;
+            } else if (n0 + cc < p.cs) {
+                const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
+                uint32_t o[8];
+                #pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
+                    int res[4], y[4];
+                    wn_unpack4(rr[j], res);
+                    wn_f<T_I32, T_I8, int>(p, n0 + cc + 4 * j, x, res, y);
+                    o[j] = wn_pack4(y);
+                }
+                uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
+                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+            }
+        }
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the row buffers may be released
     }
     #pragma unroll
     for (int pass = 0; pass < 2; ++pass) {
-        if (pass > 0 && !halves) break;
+        if (direct || (pass > 0 && !halves)) break;
         const int p0 = pass * 64;                            // first column of the pass (own columns: c_lo + c0)
         if (warp < 8 && ok) {
             const int r = m_own * TC_M + (warp & 3) * 32 + lane;
@@ -667,9 +758,10 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
             const int ch = (wide ? lane : lane & 15) * 4;    // first own channel of the pass
             const bool act_lane = p0 + ch < ncols;
+            const bool pad_lane = ACT && DT != T_F32 && p0 + ch < p.bn;      // (channels up to the padded width get a value too)
             auto close = [&](auto nr, auto ns) {
             constexpr int NR = decltype(nr)::value, NS = decltype(ns)::value;
-            for (int k0 = team * NR; mine + k0 * shares < rows; k0 += teams * NR) {
+            for (int k0 = team * NR; mine + (wide ? k0 : k0 & ~(2 * NR - 1)) * shares < rows; k0 += teams * NR) {   // (whole warps stay together)
                 uint32_t o[NR][4];
                 uint4 t[NS][NR];
                 int q[NR];
@@ -708,10 +800,50 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                         for (int j = 0; j < 4; ++j)
                             o[u][j] = DT == T_F32 ? __float_as_uint(__uint_as_float(o[u][j]) + __uint_as_float(w[j])) : o[u][j] + w[j];
                     }
+                if (ACT) {
+                    #pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        const int c = n0 + p0 + ch;
+                        if (DT != T_F32 && p.bits) {
+                            uint32_t word = 0;
+                            #pragma unroll
+                            for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols && (int)o[u][j] >= p.theta) word |= 1u << (4 * (lane & 7) + j);
+                            word |= __shfl_xor_sync(0xffffffffu, word, 1);
+                            word |= __shfl_xor_sync(0xffffffffu, word, 2);
+                            word |= __shfl_xor_sync(0xffffffffu, word, 4);
+                            if (q[u] >= 0 && (lane & 7) == 0 && p0 + ch < p.bn && (c >> 5) < p.cs)
+                                reinterpret_cast<uint32_t*>(p.X)[(size_t)q[u] * p.cs + (c >> 5)] = word;
+                        } else if (DT != T_F32) {
+                            if (q[u] < 0 || !pad_lane || c >= p.cs) continue;
+                            const size_t at = (size_t)q[u] * p.cs + c;
+                            const int x[4] = {(int)o[u][0], (int)o[u][1], (int)o[u][2], (int)o[u][3]};
+                            int res[4] = {0, 0, 0, 0}, y[4];
+                            if (p.res) wn_unpack4(*reinterpret_cast<const uint32_t*>(reinterpret_cast<const int8_t*>(p.res) + at), res);
+                            wn_f<T_I32, T_I8, int>(p, c, x, res, y);
+                            *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(p.X) + at) = wn_pack4(y);
+                        } else {
+                            if (q[u] < 0 || !act_lane) continue;
+                            const size_t at = (size_t)q[u] * p.cs + c;
+                            float x[4], res[4] = {0.f, 0.f, 0.f, 0.f}, y[4];
+                            #pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                x[j] = __uint_as_float(o[u][j]);
+                                if (p.res && p0 + ch + j < ncols) res[j] = reinterpret_cast<const float*>(p.res)[at + j];
+                            }
+                            wn_f<T_F32, T_F32, float>(p, c, x, res, y);
+                            float* dst = reinterpret_cast<float*>(p.X) + at;
+                            if (vec) *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
+                            else {
+                                #pragma unroll
+                                for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) dst[j] = y[j];
+                            }
+                        }
+                    }
+                }
                 #pragma unroll
                 for (int u = 0; u < NR; ++u) {
-                    if (q[u] < 0 || !act_lane) continue;
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)q[u] * p.c_out + n0 + p0 + ch;
+                    if (q[u] < (ACT ? p.keep_from : 0) || !act_lane) continue;
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(q[u] - (ACT ? p.keep_from : 0)) * p.c_out + n0 + p0 + ch;
                     if (vec) *reinterpret_cast<uint4*>(dst) = make_uint4(o[u][0], o[u][1], o[u][2], o[u][3]);
                     else {
                         #pragma unroll
@@ -737,6 +869,60 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     }
     if (warp == 8)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
+}
+
+// Max-pool windows over what the convolution kernel wrote pixel by pixel: bytes (16 channels per thread) or sign words
+// (the sign of a maximum is the OR of the signs).  Bound by its reads; the int32 projections it would otherwise read are
+// four times as many bytes.
+template <int KW, bool BITS>
+__global__ void __launch_bounds__(256) pool_window_kernel(const void* __restrict__ A, void* X, int oh, int ow, int th, int tw, int units, int s,
+                                                          int pad, int total)
+{
+    using T = typename std::conditional<BITS, uint32_t, uint4>::type;
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (i >= total) return;
+    const int u = i % units, r = i / units, tx = r % tw, ty = r / tw % th, ns = r / (tw * th);
+    const T* src = reinterpret_cast<const T*>(A) + (size_t)ns * oh * ow * units + u;
+    T v[KW * KW];
+    bool in[KW * KW];
+    #pragma unroll
+    for (int k = 0; k < KW * KW; ++k) {
+        const int y = ty * s - pad + k / KW, x = tx * s - pad + k % KW;
+        in[k] = y >= 0 && y < oh && x >= 0 && x < ow;
+        if (in[k]) v[k] = src[(size_t)(y * ow + x) * units];
+    }
+    T o{};
+    bool have = false;
+    #pragma unroll
+    for (int k = 0; k < KW * KW; ++k) {
+        if (!in[k]) continue;
+        if constexpr (BITS) o |= v[k];
+        else if (!have) o = v[k];
+        else { o.x = __vmaxs4(o.x, v[k].x); o.y = __vmaxs4(o.y, v[k].y); o.z = __vmaxs4(o.z, v[k].z); o.w = __vmaxs4(o.w, v[k].w); }
+        have = true;
+    }
+    reinterpret_cast<T*>(X)[i] = o;
+}
+
+int launch_pool_window(const Layer& L, const Tensor& out, const void* A, void* X, cudaStream_t st)
+{
+    const rrm_layer_desc& d = L.d;
+    const bool bits = out.dtype == T_BIN;
+    const int units = bits ? out.cs : out.cs / 16;
+    const long long total = (long long)out.pixels() * units;
+    const dim3 grid((unsigned)((total + 255) / 256));
+    cudaError_t e = cudaSuccess;
+    auto go = [&](auto kernel) { e = launch_seq(kernel, dim3(grid), dim3(256), 0, st, A, X, L.oh, L.ow, L.th, L.tw, units, d.pool_s, d.pool_p, (int)total); };
+    switch (d.pool_k) {
+        case 1: if (bits) go(pool_window_kernel<1, true>); else go(pool_window_kernel<1, false>); break;
+        case 2: if (bits) go(pool_window_kernel<2, true>); else go(pool_window_kernel<2, false>); break;
+        case 3: if (bits) go(pool_window_kernel<3, true>); else go(pool_window_kernel<3, false>); break;
+        default: return RRM_ERR_UNSUPPORTED;
+    }
+    RRM_CUDA_TRY(e);
+    return RRM_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -928,8 +1114,9 @@ static size_t win_smem(const WinParams& p)
 template <int DT, bool XCOL>
 static int win_allow()
 {
-    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, false, XCOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
-    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, false, XCOL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
     return RRM_OK;
 }
 
@@ -941,7 +1128,8 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     if (!win_geometry(net, L, p)) return RRM_ERR_UNSUPPORTED;
     const bool xcol = win_xcol(net, L), f32 = d.dtype == RRM_F32;
     L.win_ntiles = ceil_div(d.c_out, 128);
-    L.win_bn = round_up(ceil_div(d.c_out, L.win_ntiles), 16);
+    // (integer layers: whole groups of 32 columns, so that a padded output row is covered by the column tiles)
+    L.win_bn = round_up(ceil_div(d.c_out, L.win_ntiles), f32 ? 16 : 32);
     L.win_ntiles = ceil_div(d.c_out, L.win_bn);
     if (!win_plan(L, p, xcol, true, false, 1, 148)) return RRM_ERR_UNSUPPORTED;
     const int taps = xcol ? d.kh : d.kh * d.kw;
@@ -965,15 +1153,17 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
 }
 
 template <int DT, bool XCOL>
-static cudaError_t win_launch(const WinParams& p, bool dense, dim3 grid, size_t smem, cudaStream_t st)
+static cudaError_t win_launch(const WinParams& p, bool dense, bool act, dim3 grid, size_t smem, cudaStream_t st)
 {
-    return dense ? launch_seq_cluster(conv_win_kernel<DT, true, XCOL>, grid, dim3(WN_THREADS), smem, st, p.cluster ? p.ks : 1, p)
-                 : launch_seq_cluster(conv_win_kernel<DT, false, XCOL>, grid, dim3(WN_THREADS), smem, st, p.cluster ? p.ks : 1, p);
+    const int cl = p.cluster ? p.ks : 1;
+    if (act) return launch_seq_cluster(conv_win_kernel<DT, true, XCOL, true>, grid, dim3(WN_THREADS), smem, st, cl, p);
+    return dense ? launch_seq_cluster(conv_win_kernel<DT, true, XCOL, false>, grid, dim3(WN_THREADS), smem, st, cl, p)
+                 : launch_seq_cluster(conv_win_kernel<DT, false, XCOL, false>, grid, dim3(WN_THREADS), smem, st, cl, p);
 }
 
 // F*dI (dense: F*X + b); arguments as for launch_conv_tc.
 int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
-                    const uint32_t* count_bitmap, void* P_dst, int frames, long long arena_stride)
+                    const uint32_t* count_bitmap, void* P_dst, int frames, long long arena_stride, const WinOutput* out)
 {
     const rrm_layer_desc& d = L.d;
     WinParams p{};
@@ -994,13 +1184,18 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     p.frames = nf;
     p.row_stride = (long long)in.bytes(); p.arena_stride = arena_stride; p.p_stride = (long long)L.opixels() * d.c_out;
     p.store = batched ? 1 : 0;
+    if (out) {
+        p.X = out->X; p.res = out->res; p.cs = out->cs; p.bits = out->bits;
+        p.bn_scale = L.bn_scale; p.bn_shift = L.bn_shift; p.shift = d.shift; p.act_fn = d.act; p.theta = d.theta;
+        p.P = out->P; p.keep_from = out->P ? out->keep_from : INT_MAX;
+    }
     const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
     const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)L.win_ntiles, (unsigned)(nf * p.ks));
     const size_t smem = win_smem(p);
     cudaError_t e;
-    if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, grid, smem, st) : win_launch<T_F32, false>(p, dense, grid, smem, st);
-    else if (d.dtype == RRM_I8) e = xcol ? win_launch<T_I8, true>(p, dense, grid, smem, st) : win_launch<T_I8, false>(p, dense, grid, smem, st);
-    else e = win_launch<T_BIN, false>(p, dense, grid, smem, st);
+    if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, out, grid, smem, st) : win_launch<T_F32, false>(p, dense, out, grid, smem, st);
+    else if (d.dtype == RRM_I8) e = xcol ? win_launch<T_I8, true>(p, dense, out, grid, smem, st) : win_launch<T_I8, false>(p, dense, out, grid, smem, st);
+    else e = win_launch<T_BIN, false>(p, dense, out, grid, smem, st);
     RRM_CUDA_TRY(e);
     return RRM_OK;
 }
