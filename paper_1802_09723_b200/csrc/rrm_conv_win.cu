@@ -100,7 +100,7 @@ struct WinTail {
     unsigned long long afull[WN_MAX_ABUF], aempty[WN_MAX_ABUF], bfull[WN_MAX_STAGES], bempty[WN_MAX_STAGES], dfull[2], dempty[2], done;
     uint32_t tmem_base;
     int fail;
-    int bias[128];                            // of the CTA's columns (f in the kernel)
+    alignas(16) int bias[128];                // of the CTA's columns (f in the kernel)
     int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
     int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
     int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row
@@ -232,14 +232,44 @@ __device__ __forceinline__ void wn_f(const WinParams& p, int c, const pt (&x)[4]
     if (p.bn_scale) epi_f<PT, OT, 1, true, pt>(v, 1u, c, res, p.c_out, p.act_fn, p.shift, p.bn_scale, p.bn_shift, y);
     else epi_f<PT, OT, 1, false, pt>(v, 1u, c, res, p.c_out, p.act_fn, p.shift, nullptr, nullptr, y);
 }
-__device__ __forceinline__ uint32_t wn_pack4(const int (&y)[4])
+// four integers, saturated to int8 each, as one word
+__device__ __forceinline__ uint32_t wn_pack4(int y0, int y1, int y2, int y3)
 {
-    return ((uint32_t)y[0] & 0xffu) | ((uint32_t)y[1] & 0xffu) << 8 | ((uint32_t)y[2] & 0xffu) << 16 | (uint32_t)y[3] << 24;
+    uint32_t hi, w;
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(y3), "r"(y2), "r"(0));
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(y1), "r"(y0), "r"(hi));
+    return w;
 }
 __device__ __forceinline__ void wn_unpack4(uint32_t w, int (&y)[4])
 {
     #pragma unroll
     for (int j = 0; j < 4; ++j) y[j] = (int)(int8_t)(w >> (8 * j));
+}
+// the same with the explicit affine (kept out of line: few layers have one, and the drain's code is fetched once per CTA)
+__device__ __noinline__ uint32_t wn_f8_bn(const WinParams& p, int c, int x0, int x1, int x2, int x3, uint32_t res)
+{
+    const int x[4] = {x0, x1, x2, x3};
+    int r[4], y[4];
+    wn_unpack4(res, r);
+    wn_f<T_I32, T_I8, int>(p, c, x, r, y);
+    return wn_pack4(y[0], y[1], y[2], y[3]);
+}
+// int8 f of 4 neighbouring channels: requantisation (round half up), [+ shortcut], activation; the saturation at 127 is the
+// packing's.  Channels beyond the layer's last have zero filters, bias and shortcut.
+__device__ __forceinline__ uint32_t wn_f8(const WinParams& p, int c, const int (&x)[4], uint32_t res)
+{
+    if (p.bn_scale) return wn_f8_bn(p, c, x[0], x[1], x[2], x[3], res);
+    const int rnd = p.shift > 0 ? 1 << (p.shift - 1) : 0, lo = p.act_fn == RRM_ACT_RELU ? 0 : -127;
+    int y[4];
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = (x[j] + rnd) >> p.shift;
+    if (p.res) {
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = max(-127, min(127, y[j])) + (int)(int8_t)(res >> (8 * j));
+    }
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = max(y[j], lo);
+    return wn_pack4(y[0], y[1], y[2], y[3]);
 }
 
 // DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.  ACT (dense passes): f is applied here and the output written,
@@ -646,63 +676,70 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         const bool keep = q >= p.keep_from;                  // (q >= 0 then)
         uint32_t* row = staged + (size_t)r * ldr;
         int32_t* dstP = reinterpret_cast<int32_t*>(P) + (size_t)(keep ? q - p.keep_from : 0) * p.c_out + n0;
-        #pragma unroll
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-            if (c_lo + c0 >= c_hi) continue;                 // (uniform; columns come in whole groups of 32)
-            const int cc = c_lo + c0;
-            uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-            if (p.res && q >= 0) {
-                const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const int8_t*>(p.res) + (size_t)q * p.cs + n0 + cc);
-                if (n0 + cc < p.cs) { rw[0] = src[0]; rw[1] = src[1]; }
-            }
-            uint32_t v[32];
-            __syncwarp();
-            wn_ld32(tmem + lane_base + (uint32_t)(m_own * p.bn + cc), v);
-            #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += (uint32_t)S->bias[cc + j];
-            if (keep) {
-                if (vec) {
-                    const int rc = halves ? cc & 63 : cc;    // (two tiles: the row buffer holds 64 columns at a time)
-                    if (halves && rc == 0 && c0 > 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                    #pragma unroll
-                    for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(row + rc + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                    const int cols = min(32, ncols - cc);
-                    fence_async_smem();
-                    if (cols > 0) {
-                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                                     ::"l"(dstP + cc), "r"(smem_u32(row + rc)), "r"((uint32_t)cols * 4u) : "memory");
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        // (a loop, not unrolled: every CTA runs this code once, so its length is instruction fetches.  64 columns per turn of the
+        // row buffer, 32 per turn of the accumulator)
+        #pragma unroll 1
+        for (int cb = c_lo; cb < c_hi; cb += 64) {
+            if (keep && cb > c_lo) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            #pragma unroll 1
+            for (int cc = cb; cc < min(cb + 64, c_hi); cc += 32) {
+                const bool inside = q >= 0 && n0 + cc < (p.bits ? p.cs * 32 : p.cs);
+                uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+                if (p.res && inside) {
+                    const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const int8_t*>(p.res) + (size_t)q * p.cs + n0 + cc);
+                    rw[0] = src[0]; rw[1] = src[1];
+                }
+                uint32_t v[32];
+                __syncwarp();
+                wn_ld32(tmem + lane_base + (uint32_t)(m_own * p.bn + cc), v);
+                #pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const int4 b = *reinterpret_cast<const int4*>(S->bias + cc + j);
+                    v[j] += (uint32_t)b.x; v[j + 1] += (uint32_t)b.y; v[j + 2] += (uint32_t)b.z; v[j + 3] += (uint32_t)b.w;
+                }
+                if (keep) {
+                    if (vec) {
+                        uint32_t* at = row + (cc - cb) + (halves ? 0 : cb);
+                        #pragma unroll
+                        for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(at + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    } else {
+                        #pragma unroll
+                        for (int j = 0; j < 32; ++j) if (cc + j < ncols) dstP[cc + j] = (int32_t)v[j];
                     }
-                } else {
+                }
+                if (!inside) continue;
+                if (p.bits) {
+                    uint32_t word = 0;
                     #pragma unroll
-                    for (int j = 0; j < 32; ++j) if (cc + j < ncols) dstP[cc + j] = (int32_t)v[j];
+                    for (int j = 0; j < 32; ++j) word |= (uint32_t)((int)v[j] >= p.theta) << j;
+                    if (ncols - cc < 32) word &= (1u << max(ncols - cc, 0)) - 1u;
+                    reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + ((n0 + cc) >> 5)] = word;
+                } else {
+                    const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
+                    uint32_t o[8];
+                    #pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
+                        o[j] = wn_f8(p, n0 + cc + 4 * j, x, rr[j]);
+                    }
+                    uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
+                    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
                 }
             }
-            if (q < 0) continue;
-            if (p.bits) {
-                uint32_t word = 0;
-                #pragma unroll
-                for (int j = 0; j < 32; ++j) if (cc + j < ncols && (int)v[j] >= p.theta) word |= 1u << j;
-                if (((n0 + cc) >> 5) < p.cs) reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + ((n0 + cc) >> 5)] = word;
-            } else if (n0 + cc < p.cs) {
-                const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
-                uint32_t o[8];
-                #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
-                    int res[4], y[4];
-                    wn_unpack4(rr[j], res);
-                    wn_f<T_I32, T_I8, int>(p, n0 + cc + 4 * j, x, res, y);
-                    o[j] = wn_pack4(y);
+            if (keep && vec) {
+                const int cols = min(min(64, c_hi - cb), ncols - cb);
+                fence_async_smem();
+                if (cols > 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                 ::"l"(dstP + cb), "r"(smem_u32(row + (halves ? 0 : cb))), "r"((uint32_t)cols * 4u) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
-                uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
-                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
         }
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the row buffers may be released
     }
-    #pragma unroll
+    #pragma unroll (DT == T_F32 ? 2 : 1)
     for (int pass = 0; pass < 2; ++pass) {
         if (direct || (pass > 0 && !halves)) break;
         const int p0 = pass * 64;                            // first column of the pass (own columns: c_lo + c0)
@@ -710,7 +747,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const int r = m_own * TC_M + (warp & 3) * 32 + lane;
             uint32_t* row = staged + (size_t)r * ldr;
             if (pass > 0) { if (bulk_add) __syncwarp(); else wn_meet(); }    // the first pass's rows have left
-            #pragma unroll
+            #pragma unroll (DT == T_F32 ? 4 : 1)
             for (int c0 = 0; c0 < 128; c0 += 32) {
                 if (c_lo + c0 < c_hi && (!halves || (c0 >> 6) == pass)) {
                     uint32_t v[32];
@@ -817,10 +854,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                             if (q[u] < 0 || !pad_lane || c >= p.cs) continue;
                             const size_t at = (size_t)q[u] * p.cs + c;
                             const int x[4] = {(int)o[u][0], (int)o[u][1], (int)o[u][2], (int)o[u][3]};
-                            int res[4] = {0, 0, 0, 0}, y[4];
-                            if (p.res) wn_unpack4(*reinterpret_cast<const uint32_t*>(reinterpret_cast<const int8_t*>(p.res) + at), res);
-                            wn_f<T_I32, T_I8, int>(p, c, x, res, y);
-                            *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(p.X) + at) = wn_pack4(y);
+                            const uint32_t res = p.res ? *reinterpret_cast<const uint32_t*>(reinterpret_cast<const int8_t*>(p.res) + at) : 0u;
+                            *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(p.X) + at) = wn_f8(p, c, x, res);
                         } else {
                             if (q[u] < 0 || !act_lane) continue;
                             const size_t at = (size_t)q[u] * p.cs + c;
