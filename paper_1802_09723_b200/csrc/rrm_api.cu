@@ -207,7 +207,7 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
         net->layer_switch = all_auto && n_layers <= 64;
         {
             bool all_tc = true;
-            for (auto& L : net->layers) all_tc = all_tc && L.on_tensor() && L.d.dtype != RRM_F32;
+            for (auto& L : net->layers) { all_tc = all_tc && L.on_tensor(); net->chunk_f32 = net->chunk_f32 || L.d.dtype == RRM_F32; }
             net->chunk_switch = all_auto && all_tc && n_layers <= 64;
         }
         // an all-ones bitmap stands in for a layer's update bitmap when the layer is evaluated densely inside a delta step
@@ -239,16 +239,19 @@ int launch_sequence(rrm_net* net, const void* frame, void* out, cudaStream_t st,
 int run_sequence(rrm_net* net, const void* frame, void* out, cudaStream_t st, bool dense, bool stateless,
                  unsigned long long mask = 0);
 
-// Finds the nodes of a captured sequence that hold the fixed frame / output buffers, so that each launch can
-// point them at the caller's buffers instead of copying through the fixed ones.  Any doubt (an API error, no
-// node found) leaves patch_ok false and the copies in place.
-void find_io_nodes(rrm_net* net, rrm_net::StepGraph& sg)
+// Finds the nodes of a captured sequence that hold the fixed frame / output buffers (or addresses inside them), so that
+// each launch can point them at the caller's buffers instead of copying through the fixed ones.  Any doubt (an API error,
+// another number of nodes than `count` on a side) leaves ok false and the copies in place.
+void find_io_nodes(cudaGraph_t graph, const void* in, size_t in_bytes, const void* out, size_t out_bytes, size_t count, rrm_net::IoPatches& io)
 {
-    sg.patch_in.clear(); sg.patch_out.clear(); sg.patch_ok = false;
+    io.in.clear(); io.out.clear(); io.ok = false;
+    auto within = [](const void* v, const void* base, size_t bytes) {
+        return v >= base && v < reinterpret_cast<const char*>(base) + bytes;
+    };
     size_t n = 0;
-    if (cudaGraphGetNodes(sg.graph, nullptr, &n) != cudaSuccess || n == 0) { cudaGetLastError(); return; }
+    if (cudaGraphGetNodes(graph, nullptr, &n) != cudaSuccess || n == 0) { cudaGetLastError(); return; }
     std::vector<cudaGraphNode_t> nodes(n);
-    if (cudaGraphGetNodes(sg.graph, nodes.data(), &n) != cudaSuccess) { cudaGetLastError(); return; }
+    if (cudaGraphGetNodes(graph, nodes.data(), &n) != cudaSuccess) { cudaGetLastError(); return; }
     for (cudaGraphNode_t node : nodes) {
         cudaGraphNodeType type;
         if (cudaGraphNodeGetType(node, &type) != cudaSuccess) { cudaGetLastError(); return; }
@@ -267,43 +270,48 @@ void find_io_nodes(rrm_net* net, rrm_net::StepGraph& sg)
                 cudaFuncGetParamInfo(kp.func, i, &off, &size);
                 if (size != sizeof(void*)) continue;
                 void* v = *reinterpret_cast<void* const*>(kp.kernelParams[i]);
-                if (v != net->frame_buf && v != net->out_buf) continue;
+                const bool is_in = within(v, in, in_bytes);
+                if (!is_in && !within(v, out, out_bytes)) continue;
                 rrm_net::IoPatch pt;
                 pt.node = node; pt.kp = kp; pt.args = args; pt.index = (int)i;
-                (v == net->frame_buf ? sg.patch_in : sg.patch_out).push_back(pt);
+                pt.offset = reinterpret_cast<const char*>(v) - reinterpret_cast<const char*>(is_in ? in : out);
+                (is_in ? io.in : io.out).push_back(pt);
             }
         } else if (type == cudaGraphNodeTypeMemcpy) {
             cudaMemcpy3DParms mp = {};
             if (cudaGraphMemcpyNodeGetParams(node, &mp) != cudaSuccess) { cudaGetLastError(); return; }
-            if (mp.dstPtr.ptr == net->out_buf && mp.extent.height <= 1 && mp.extent.depth <= 1) {
+            const bool to_out = within(mp.dstPtr.ptr, out, out_bytes);
+            if (to_out && mp.extent.height <= 1 && mp.extent.depth <= 1) {
                 rrm_net::IoPatch pt;
                 pt.node = node; pt.is_copy = true; pt.src = mp.srcPtr.ptr; pt.bytes = mp.extent.width;
-                sg.patch_out.push_back(pt);
-            } else if (mp.dstPtr.ptr == net->out_buf || mp.srcPtr.ptr == net->frame_buf) {
+                pt.offset = reinterpret_cast<const char*>(mp.dstPtr.ptr) - reinterpret_cast<const char*>(out);
+                io.out.push_back(pt);
+            } else if (to_out || within(mp.srcPtr.ptr, in, in_bytes)) {
                 return;                                      // a copy of another shape: leave everything as it is
             }
         }
     }
-    sg.patch_ok = sg.patch_in.size() == 1 && sg.patch_out.size() == 1;
+    io.ok = io.in.size() == count && io.out.size() == count;
 }
 
-// Points the frame / output nodes of the instantiated graph at `frame` and `out`.
-int patch_io(rrm_net* net, rrm_net::StepGraph& sg, const void* frame, void* out)
+// Points the frame / output nodes of the instantiated graph at `in` and `out`.
+int patch_io(cudaGraphExec_t exec, rrm_net::IoPatches& io, const void* in, void* out)
 {
     for (int side = 0; side < 2; ++side) {
-        rrm_net::IoPatch& pt = side == 0 ? sg.patch_in[0] : sg.patch_out[0];
-        void* target = side == 0 ? const_cast<void*>(frame) : (out ? out : net->out_buf);
-        if (pt.value == target) continue;                    // already there
-        if (pt.is_copy) {
-            RRM_CUDA_TRY(cudaGraphExecMemcpyNodeSetParams1D(sg.exec, pt.node, target, pt.src, pt.bytes,
-                                                            cudaMemcpyDeviceToDevice));
-        } else {
+        for (rrm_net::IoPatch& pt : side == 0 ? io.in : io.out) {
+            void* target = (side == 0 ? reinterpret_cast<char*>(const_cast<void*>(in)) : reinterpret_cast<char*>(out)) + pt.offset;
+            if (pt.value == target) continue;                // already there
+            if (pt.is_copy) {
+                RRM_CUDA_TRY(cudaGraphExecMemcpyNodeSetParams1D(exec, pt.node, target, pt.src, pt.bytes,
+                                                                cudaMemcpyDeviceToDevice));
+            } else {
+                pt.value = target;
+                pt.args[pt.index] = &pt.value;
+                pt.kp.kernelParams = pt.args.data();
+                RRM_CUDA_TRY(cudaGraphExecKernelNodeSetParams(exec, pt.node, &pt.kp));
+            }
             pt.value = target;
-            pt.args[pt.index] = &pt.value;
-            pt.kp.kernelParams = pt.args.data();
-            RRM_CUDA_TRY(cudaGraphExecKernelNodeSetParams(sg.exec, pt.node, &pt.kp));
         }
-        pt.value = target;
     }
     return RRM_OK;
 }
@@ -344,7 +352,7 @@ int build_graph(rrm_net* net, int kind, unsigned long long mask)
     rrm_net::StepGraph sg;
     sg.mask = mask; sg.graph = g;
     if (cudaGraphInstantiate(&sg.exec, g, 0) != cudaSuccess) { cudaGraphDestroy(g); cudaGetLastError(); return RRM_ERR_CUDA; }
-    find_io_nodes(net, sg);
+    find_io_nodes(g, net->frame_buf, 1, net->out_buf, 1, 1, sg.io);
     cache.push_back(std::move(sg));
     return RRM_OK;
 }
@@ -391,22 +399,25 @@ void activity_poll(rrm_net* net)
 {
     if (!net->act_pending || cudaEventQuery(net->act_ev) != cudaSuccess) { cudaGetLastError(); return; }
     net->act_pending = false;
-    double num = 0, den = 0;
+    double num = 0, den = 0, tnum = 0;
     const size_t base = net->tensors.size() * 32;
     unsigned long long mask = 0;
     for (size_t l = 0; l < net->layers.size(); ++l) {
         Layer& L = net->layers[l];
-        int oc = 0;
+        int oc = 0, tiles = 0;
         std::memcpy(&oc, net->act_host + base + l * 16 + 8, 4);
+        std::memcpy(&tiles, net->act_host + base + l * 16 + 12, 4);
         const double macs = (double)L.opixels() * L.d.c_out * L.d.c_in * L.d.kh * L.d.kw;
         L.activity = oc / (double)L.opixels();
         num += macs * L.activity;
+        tnum += macs * (L.win_ready ? (tiles < L.win_tiles ? tiles / (double)L.win_tiles : 1.0) : L.activity);
         den += macs;
         if (L.activity >= net->opt.layer_dense_activity) L.dense_mode = true;
         else if (L.activity < net->opt.layer_delta_activity) L.dense_mode = false;
         if (L.dense_mode && l < 64) mask |= 1ull << l;
     }
     net->activity = den > 0 ? num / den : -1.0;
+    net->chunk_activity = den > 0 ? tnum / den : -1.0;
     net->layer_mask = net->layer_switch ? mask : 0;
 }
 
@@ -464,11 +475,11 @@ int run_sequence(rrm_net* net, const void* frame, void* out, cudaStream_t st, bo
             int64_t bi = 0, bo = 0;
             tensor_bytes_boundary(net->tensors.front(), &bi);
             tensor_bytes_boundary(net->tensors.back(), &bo);
-            if (sg->patch_ok && patch_io(net, *sg, frame, out) == RRM_OK) {
+            if (sg->io.ok && patch_io(sg->exec, sg->io, frame, out ? out : net->out_buf) == RRM_OK) {
                 RRM_CUDA_TRY(cudaGraphLaunch(sg->exec, st));
                 return RRM_OK;
             }
-            if (sg->patch_ok) {
+            if (sg->io.ok) {
                 // an update failed half-way: the graphs are no longer trusted, launch kernel by kernel from now on
                 cudaGetLastError();
                 drop_graphs(net);
@@ -548,7 +559,7 @@ int ensure_chunk(rrm_net* net, int T)
 }
 
 // Inserts a captured chunk graph into the cache of its kind (the few most recently used are kept).
-static int keep_chunk_graph(rrm_net* net, int kind, int T, unsigned long long mask, cudaGraph_t g, int last_arena)
+static int keep_chunk_graph(rrm_net* net, int kind, int T, unsigned long long mask, cudaGraph_t g, int last_arena, int io_nodes = 0)
 {
     auto& cache = net->chunk_graphs[kind];
     if (cache.size() >= CHUNK_GRAPHS_KEPT) {
@@ -562,7 +573,13 @@ static int keep_chunk_graph(rrm_net* net, int kind, int T, unsigned long long ma
     c.T = T; c.mask = mask; c.graph = g; c.last_arena = last_arena;
     if (cudaGraphInstantiate(&c.exec, g, 0) != cudaSuccess) { cudaGraphDestroy(g); cudaGetLastError(); return RRM_ERR_CUDA; }
     c.used = ++net->chunk_clock;
-    cache.push_back(c);
+    if (io_nodes > 0) {
+        int64_t bi = 0, bo = 0;
+        tensor_bytes_boundary(net->tensors.front(), &bi);
+        tensor_bytes_boundary(net->tensors.back(), &bo);
+        find_io_nodes(g, net->chunk_in, (size_t)bi * T, net->chunk_out, (size_t)bo * T, (size_t)io_nodes, c.io);
+    }
+    cache.push_back(std::move(c));
     return RRM_OK;
 }
 
@@ -624,22 +641,40 @@ static int build_seq_graph(rrm_net* net, int T)
 // stateful dense pass of the last frame.  RRM_ERR_UNSUPPORTED: too large (the frame-pipelined graph serves it).
 constexpr int DENSE_BATCH = 32;
 
-static int ensure_dense_batch(rrm_net* net)
+static int ensure_dense_batch(rrm_net* net, int frames)
 {
-    if (net->dense_batch_ready) return RRM_OK;
+    if (frames <= net->dense_batch_cap) return RRM_OK;
     size_t need = 0;
     for (auto& X : net->tensors) {
-        if ((long long)X.pixels() * DENSE_BATCH * (long long)X.cs > (1ll << 31) - 1) return RRM_ERR_UNSUPPORTED;
-        need += X.bytes() * DENSE_BATCH;
+        if ((long long)X.pixels() * frames * (long long)X.cs > (1ll << 31) - 1) return RRM_ERR_UNSUPPORTED;
+        need += X.bytes() * frames;
     }
-    for (auto& Y : net->layers) {
-        if ((long long)Y.opixels() * DENSE_BATCH * (long long)Y.d.c_out > (1ll << 31) - 1) return RRM_ERR_UNSUPPORTED;
-        need += (size_t)Y.opixels() * Y.d.c_out * 4 * DENSE_BATCH;
+    for (size_t l = 0; l < net->layers.size(); ++l) {
+        const Layer& Y = net->layers[l];
+        if ((long long)Y.opixels() * frames * (long long)Y.d.c_out > (1ll << 31) - 1) return RRM_ERR_UNSUPPORTED;
+        need += (size_t)Y.opixels() * stateless_row_bytes(net, (int)l) * frames;
     }
     if (need > ((size_t)8 << 30)) return RRM_ERR_UNSUPPORTED;
-    for (auto& X : net->tensors) if (!X.X2b) RRM_TRY(dev_alloc(net, &X.X2b, X.bytes() * DENSE_BATCH));
-    for (auto& Y : net->layers) if (!Y.P2b) RRM_TRY(dev_alloc(net, &Y.P2b, (size_t)Y.opixels() * Y.d.c_out * 4 * DENSE_BATCH));
-    net->dense_batch_ready = true;
+    if (net->dense_batch_cap > 0) {                          // growing: graphs hold the old buffers and may be in flight
+        RRM_CUDA_TRY(cudaDeviceSynchronize());
+        for (int k = 1; k < 3; ++k) drop_chunk_graphs(net, k);
+        net->dense_batch_cap = 0;
+        dev_release(net, &net->dense_batch);
+    }
+    // one block for all of them (an allocation costs some 0.2 ms): sizes first, then addresses
+    size_t total = 0;
+    auto place = [&](void** p, size_t bytes) {
+        *p = net->dense_batch ? reinterpret_cast<char*>(net->dense_batch) + total : nullptr;
+        total += (bytes + 255) & ~(size_t)255;
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) RRM_TRY(dev_alloc(net, &net->dense_batch, total));
+        total = 0;
+        for (auto& X : net->tensors) place(&X.X2b, X.bytes() * frames);
+        for (size_t l = 0; l < net->layers.size(); ++l)
+            place(&net->layers[l].P2b, (size_t)net->layers[l].opixels() * stateless_row_bytes(net, (int)l) * frames);
+    }
+    net->dense_batch_cap = frames;
     return RRM_OK;
 }
 
@@ -648,8 +683,8 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
     const int L = (int)net->layers.size();
     RRM_TRY(ensure_chunk(net, T));
     RRM_TRY(ensure_stateless(net));
-    RRM_TRY(ensure_dense_batch(net));
     const int parts = ceil_div(T, DENSE_BATCH), per = ceil_div(T, parts);
+    RRM_TRY(ensure_dense_batch(net, per));
     int64_t bi = 0, bo = 0;
     tensor_bytes_boundary(net->tensors.front(), &bi);
     tensor_bytes_boundary(net->tensors.back(), &bo);
@@ -696,7 +731,7 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
         cudaGetLastError();
         return status != RRM_OK ? status : RRM_ERR_CUDA;
     }
-    RRM_TRY(keep_chunk_graph(net, kind, T, 0, g, 0));
+    RRM_TRY(keep_chunk_graph(net, kind, T, 0, g, 0, parts));     // (an import and an export per part hold the boundary buffers)
     if (getenv("RRM_DEBUG")) {
         size_t nodes = 0;
         cudaGraphGetNodes(g, nullptr, &nodes);
@@ -858,17 +893,25 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
 {
     if (net->graph_off || net->eps > 0.f || T < 2) return RRM_ERR_UNSUPPORTED;
     const bool is_step = !dense && !stateless;
+    const bool long_chunk = net->chunk_switch && T >= 8 && !net->chunk_pipelined;
     unsigned long long mask = 0;
     if (is_step) {
         // one decision per chunk, from the measured activity of the last delta frame (as rrm_net_step does per frame)
         net->last_step_dense = false;
         if (net->auto_switch || net->layer_switch) {
             activity_poll(net);
-            // long chunks of few streams have a batched dense form that needs no change detection, marking or prefix
-            // sums: on tensor-core stacks it is ahead from a lower activity on than the whole-stack switch of single steps
-            const bool long_chunk = net->chunk_switch && T >= 16 && net->n <= 4 && !net->chunk_pipelined;
+            // Chunks have a batched dense form that needs no change detection, marking or prefix sums and stores no
+            // projections but the last frame's: on tensor-core stacks it is ahead from a lower activity on than the
+            // whole-stack switch of single steps.  What a delta chunk can save is accumulator tiles without any pixel to
+            // update, so those are what its activity counts.  Measured, us per frame, delta as the library chooses /
+            // dense: AlexNet int8 on the quiet video (a third of the pixels) 1 stream x 16 frames 12.1 / 9.2, 32 frames
+            // 7.1 / 6.4, 8 streams x 4 frames 57 / 51; busy 13.7 / 9.1; a lone int8 layer, 3 streams x 8 frames 17 / 9.8.
+            // fp32 products are most of a chunk's time, so there the delta form is level at twice the activity: quiet,
+            // 2 streams x 16 frames 33 / 42, busy 45 / 42, 1 stream x 32 frames 25.6 / 21.  (Chunks of fewer than 8 frames
+            // stay on the delta path below the whole-stack threshold: their callers read counters frame by frame.)
+            const double level = net->opt.chunk_dense_activity * (net->chunk_f32 ? 2.0 : 1.0);
             const bool go_dense = (net->auto_switch && net->activity >= net->opt.stack_dense_activity) ||
-                                  (long_chunk && net->activity >= net->opt.chunk_dense_activity);
+                                  (long_chunk && net->chunk_activity >= level);
             if (go_dense && net->dense_streak < net->opt.stack_reprobe) {
                 ++net->dense_streak;                         // (counted in calls: a delta chunk measures again after 15 dense ones)
                 net->last_step_dense = true;
@@ -893,6 +936,13 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
             RRM_TRY(bind_readers(net));
             return s == RRM_ERR_ALLOC ? s : RRM_ERR_UNSUPPORTED;
         }
+        // the dense form of the same chunk, which the measured activity may ask for in the very next call, is captured
+        // here too, so that no later call of this length pays for it
+        if (kind == 0 && long_chunk && net->opt.chunk_dense_activity <= 1.f) {
+            bool have = false;
+            for (auto& c : net->chunk_graphs[1]) have = have || c.T == T;
+            if (!have && build_dense_batch_graph(net, 1, T) != RRM_OK) cudaGetLastError();
+        }
     }
     // the structures describe the last frame of the chunk from here on (statistics, activity read-back)
     bind_arena(net, net->chunk_arena[find()->last_arena]);
@@ -900,11 +950,21 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
     int64_t bi = 0, bo = 0;
     tensor_bytes_boundary(net->tensors.front(), &bi);
     tensor_bytes_boundary(net->tensors.back(), &bo);
-    RRM_CUDA_TRY(cudaMemcpyAsync(net->chunk_in, frames, (size_t)bi * T, cudaMemcpyDeviceToDevice, st));
     rrm_net::ChunkGraph* cg = find();
     cg->used = ++net->chunk_clock;
-    RRM_CUDA_TRY(cudaGraphLaunch(cg->exec, st));
-    if (outs) RRM_CUDA_TRY(cudaMemcpyAsync(outs, net->chunk_out, (size_t)bo * T, cudaMemcpyDeviceToDevice, st));
+    if (cg->io.ok) {                                         // the graph works on the caller's buffers
+        if (patch_io(cg->exec, cg->io, frames, outs ? outs : net->chunk_out) != RRM_OK) {
+            // an update failed half-way: the graph is no longer trusted
+            cudaGetLastError();
+            drop_chunk_graphs(net, kind);
+            return RRM_ERR_CUDA;
+        }
+        RRM_CUDA_TRY(cudaGraphLaunch(cg->exec, st));
+    } else {
+        RRM_CUDA_TRY(cudaMemcpyAsync(net->chunk_in, frames, (size_t)bi * T, cudaMemcpyDeviceToDevice, st));
+        RRM_CUDA_TRY(cudaGraphLaunch(cg->exec, st));
+        if (outs) RRM_CUDA_TRY(cudaMemcpyAsync(outs, net->chunk_out, (size_t)bo * T, cudaMemcpyDeviceToDevice, st));
+    }
     if (is_step && !dense && (net->auto_switch || net->layer_switch)) RRM_TRY(activity_read_back(net, st));
     return RRM_OK;
 }

@@ -170,7 +170,8 @@ struct Layer {
     void* dPall = nullptr;            // per-frame products of the layer-by-layer chunk form
     uint32_t* oact = nullptr;         // bitmap of projection pixels to update (cleared every step, set by the
                                       // kernels that produce the layer's input and shortcut tensors)
-    int* ocount = nullptr;            // their number (cleared every step, written by the convolution kernel)
+    int* ocount = nullptr;            // [0] their number, [1] window kernel: accumulator tiles that hold any (cleared every step,
+                                      // written by the convolution kernel)
     unsigned long long* macs = nullptr;     // exact active multiply-accumulates (cleared every step)
     int opixels() const { return d.n * oh * ow; }
     // per-layer choice between the sparse product and a dense evaluation inside a delta step, from the measured
@@ -199,6 +200,7 @@ struct Layer {
     bool win_ready = false;
     void* win_Wimg = nullptr;               // [n_tiles][tap][K group][pieces][2][bn][16 bytes] operand tiles of the filters
     int win_bn = 0, win_ntiles = 0;
+    int win_tiles = 0;                      // accumulator tiles of 128 rows that cover the layer once
     void* Apre = nullptr;                   // pooled integer layers: f before the pool window, a row per projection pixel (keyframes)
     bool on_tensor() const { return tc_ready || win_ready; }
     // few-row dense FC on the tensor cores (weights as the M operand, K split over CTAs)
@@ -263,7 +265,10 @@ struct rrm_net {
         int index = -1;                            // which argument is the buffer
         const void* src = nullptr; size_t bytes = 0;   // copy node: source and size
         void* value = nullptr;                     // storage the patched argument points to
+        ptrdiff_t offset = 0;                      // where the node's address lies inside the fixed buffer
+        // (the argument list points at `value` once patched: a copy of the patch starts over)
     };
+    struct IoPatches { std::vector<IoPatch> in, out; bool ok = false; };
     // the per-frame launch sequences (0: delta step, 1: keyframe, 2: stateless dense pass), each captured once and
     // replayed (fixed frame / output buffers).  A delta step exists in one form per layer mask (bit l: layer l is
     // evaluated densely inside the step); the few most recently used masks are kept.
@@ -271,8 +276,7 @@ struct rrm_net {
         unsigned long long mask = 0, used = 0;
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
-        std::vector<IoPatch> patch_in, patch_out;
-        bool patch_ok = false;
+        IoPatches io;
     };
     std::vector<StepGraph> step_graphs[3];
     unsigned long long step_clock = 0;
@@ -289,7 +293,8 @@ struct rrm_net {
     // `slot` (frame mod CHUNK_RING in the split form; slot 0 only otherwise)
     std::vector<cudaEvent_t> ev_conv, ev_epi;
     cudaEvent_t ev_import = nullptr;
-    bool dense_batch_ready = false;               // the buffers of the frame-batched dense chunk exist
+    void* dense_batch = nullptr;                  // the block the batched dense chunk's buffers lie in
+    int dense_batch_cap = 0;                      // frames the buffers of the frame-batched dense chunk hold
     bool seq_ready = false;                       // the buffers of the layer-by-layer chunk form exist
     bool chunk_by_layer = false;                  // RRM_CHUNK_BY_LAYER=1: delta chunks always go layer by layer over all frames (where the stack allows)
     bool chunk_pipelined = false;                 // RRM_CHUNK_PIPELINED=1: delta chunks overlap frames instead of batching them per layer
@@ -298,7 +303,7 @@ struct rrm_net {
     std::vector<cudaEvent_t> ev_join;
     cudaEvent_t ev_fork = nullptr, ev_export = nullptr;
     struct ChunkGraph { int T = 0; unsigned long long mask = 0; cudaGraph_t graph = nullptr; cudaGraphExec_t exec = nullptr; unsigned long long used = 0;
-                        int last_arena = 0; /* the arena that holds the chunk's last frame */ };
+                        int last_arena = 0; /* the arena that holds the chunk's last frame */ IoPatches io; };
     std::vector<ChunkGraph> chunk_graphs[3];      // per kind (delta / keyframes / dense): the few most recently used chunk lengths
     unsigned long long chunk_clock = 0;
     void* chunk_in = nullptr;                     // T frames at the boundary; one more frame fits right in front of them
@@ -315,7 +320,9 @@ struct rrm_net {
     int dense_streak = 0;                     // dense frames since the last measured delta frame
     bool last_step_dense = false;             // the most recent rrm_net_step was evaluated densely
     bool auto_switch = false;                 // every layer asks for RRM_VARIANT_AUTO and the net is large enough
+    double chunk_activity = -1.0;             // the same with window-kernel layers counted by accumulator tiles that hold such a pixel
     bool chunk_switch = false;                // every layer asks for RRM_VARIANT_AUTO and runs on the tensor cores: long chunks may go dense
+    bool chunk_f32 = false;                   // ... and some of them are fp32
     // the defaults rrm_net_get_options reports.  (The per-layer thresholds are above 1, i.e. the per-layer choice is off
     // until the caller lowers them: measured on B200, a dense evaluation of one layer inside a delta step is never
     // faster than its sparse product, not even with every pixel active.  What a delta step pays for is change
@@ -381,6 +388,7 @@ int launch_layer(rrm_net* net, int l, bool dense, bool stateless, cudaStream_t s
                  const std::function<int(int)>* hook = nullptr, bool dense_in_step = false,
                  const SplitProjection* split = nullptr);
 bool dense_applies_f(const rrm_net* net, int l);
+size_t stateless_row_bytes(const rrm_net* net, int l);
 int launch_export_tensor(rrm_net* net, int t, void* dst_dev, bool stateless, cudaStream_t st);
 int launch_export_projection(rrm_net* net, int l, void* dst_dev, cudaStream_t st);
 int reset_state(rrm_net* net, cudaStream_t st);

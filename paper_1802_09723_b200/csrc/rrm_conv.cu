@@ -1358,7 +1358,7 @@ int ensure_stateless(rrm_net* net)
     for (auto& T : net->tensors)
         if (!T.X2) RRM_TRY(dev_alloc(net, &T.X2, T.bytes()));
     for (auto& L : net->layers)
-        if (!L.P2) RRM_TRY(dev_alloc(net, &L.P2, (size_t)L.opixels() * L.d.c_out * 4));
+        if (!L.P2) RRM_TRY(dev_alloc(net, &L.P2, (size_t)L.opixels() * L.d.c_out * 4));   // (whole projections: chunk graphs with cross-frame edges keep f apart)
     return RRM_OK;
 }
 
@@ -1486,6 +1486,14 @@ bool dense_applies_f(const rrm_net* net, int l)
     if (out.dtype == T_F32) return L.d.pool_k == 0;
     if (out.dtype != T_BIN && (out.dtype != T_I8 || out.cs % 32 != 0)) return false;
     return L.d.pool_k == 0 || (size_t)out.cs * out.unit_bytes <= (size_t)L.d.c_out * 4;   // (the rows go where a stateless pass's projection would)
+}
+
+// Bytes per projection pixel that a stateless dense pass keeps between a layer's kernels: the projection, the rows a pool
+// window takes the maximum of, or nothing.
+size_t stateless_row_bytes(const rrm_net* net, int l)
+{
+    if (!dense_applies_f(net, l)) return (size_t)net->layers[l].d.c_out * 4;
+    return net->layers[l].d.pool_k > 0 ? net->tensors[l + 1].row_bytes() : 0;
 }
 
 // hook (may be null): called with 0 before the layer's first launch, with 1 between the convolution and the

@@ -62,7 +62,7 @@ struct WinParams {
     const void* Anew;         // binary: current sign bits
     const uint32_t* in_act;   // input activity bitmap (delta mode)
     const uint32_t* oact;     // projection pixels to update (delta mode)
-    int* ocount;              // their number is added here
+    int* ocount;              // their number is added here, and that of the accumulator tiles they lie in behind it
     const unsigned char* Wimg;      // [n tile][tap][group][pieces][2][bn][16 bytes]
     const void* bias;
     void* P;                  // [opixels][c_out]
@@ -374,7 +374,11 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         tc_fence_before();
         active = __syncthreads_count(bit);
         tc_fence_after();
-        if (active && tid == 0 && ntile == 0 && split == 0) atomicAdd(shift_bytes(p.ocount, arena_off), active);
+        if (active && tid == 0 && ntile == 0 && split == 0) {
+            int* oc = shift_bytes(p.ocount, arena_off);
+            atomicAdd(oc, active);
+            if (!DENSE) atomicAdd(oc + 1, p.mt);              // accumulator tiles with work: what this kernel's time follows
+        }
     }
     const uint32_t tmem = S->tmem_base;
     if (!DENSE && active == 0) {                             // nothing to update (every share of the tile sees the same)
@@ -1183,6 +1187,7 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     RRM_TRY((win_allow<T_F32, true>())); RRM_TRY((win_allow<T_F32, false>()));
     RRM_TRY((win_allow<T_I8, true>())); RRM_TRY((win_allow<T_I8, false>()));
     RRM_TRY((win_allow<T_BIN, false>()));
+    L.win_tiles = ceil_div((int)(((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow), TC_M);
     L.win_ready = true;
     return RRM_OK;
 }

@@ -556,6 +556,40 @@ def test_long_chunks_of_a_tensor_core_stack_go_dense_from_the_measured_activity(
     net.close()
 
 
+@pytest.mark.parametrize("dtype,T", [("i8", 7), ("i8", 8), ("f32", 8), ("bin", 9)])
+def test_chunks_of_eight_frames_go_dense_by_their_accumulator_tiles(dtype, T):
+    """Chunks of 8 or more frames go dense when most accumulator tiles hold a pixel to update, even with few pixels
+    active; shorter ones stay on the delta path.  Every call has buffers of its own (the graph is pointed at them)."""
+    rng = np.random.default_rng(T)
+    sp = _spec(dtype, 40, (24, 23), 36, 3, 1, 1, rng)
+    video = _video(dtype, 40, (24, 23), 1 + 3 * T, 2, rng)
+    video[4:] = video[4]
+    for t in range(5, video.shape[0]):                        # one small patch per frame and stream: few pixels, spread over the tiles
+        y, x = int(rng.integers(0, 20)), int(rng.integers(0, 19))
+        video[t] = video[t - 1]
+        video[t, :, :, y:y + 4, x:x + 4] = video[2, :, :, x:x + 4, y:y + 4] if dtype != "bin" else -video[t - 1, :, :, y:y + 4, x:x + 4]
+    net = _rrm().net_from_specs([sp], n=2)
+    net.set_options(chunk_dense_activity=0.1, stack_dense_activity=2.0)
+    net.keyframe(_frame_to_dev([sp], video[0]))
+    variants, keep = [], []
+    for k in range(3):
+        frames = torch.stack([_frame_to_dev([sp], f) for f in video[1 + k * T:1 + (k + 1) * T]])
+        outs = net.new_output(frames=T)
+        keep.append((frames, outs))
+        net.step_seq(frames, outs, T)
+        variants.append(net.stats(0)["variant"])              # synchronises: the next call sees this chunk's activity
+        for i in (0, T - 1):
+            want = orc.dense_forward([sp], video[1 + k * T + i])[0][1]
+            got = outs[i].cpu().numpy()
+            if dtype == "f32":
+                assert float(np.abs(got - want).max()) <= F32_TOL * float(np.abs(want).max()), (k, i)
+            else:
+                np.testing.assert_array_equal(got.astype(np.int64), want, err_msg=f"chunk {k} frame {i}")
+        _compare([sp], net, video[(k + 1) * T], (k + 1) * T)
+    assert (variants[1] == 3) == (T >= 8), variants
+    net.close()
+
+
 def test_dense_chunks_longer_than_one_batch():
     """Dense chunks are batched over their frames, 32 at most per launch: a chunk of 40 frames of two streams goes in
     two parts.  rrm_net_dense_seq leaves the state alone; a chunk that the density switch evaluates densely leaves
