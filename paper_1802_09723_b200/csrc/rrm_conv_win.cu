@@ -13,7 +13,9 @@
 //   - a stride s splits the input into s * s planes (pixels of equal remainders), each with taps of its own that are
 //     again shifts within the plane; a block of the K loop is one plane and some channels;
 //   - first layers (at most 4 channels) have too few K bytes per pixel: their windows hold, per output column, the kw
-//     pixels of a filter row side by side (a copy per column instead of one per tap), and the taps are the filter rows.
+//     pixels of a filter row side by side, and the taps are the filter rows.  Where the stride is one or two 16-byte chunks
+//     of pixels, neighbouring columns' chunks are the same pixels: the window then is the row itself in one or two arrays,
+//     a chunk further right in the filter row being the next slot, instead of a copy of kw pixels per column.
 // Pixels that did not change (delta) or lie outside the image are zero in the window.  A tile none of whose projection
 // pixels has to be updated leaves at once; there is no compaction of rows below that (a tile's MMAs cost less than
 // finding its rows did).
@@ -82,6 +84,8 @@ struct WinParams {
     int eager;                // filter copies start before it is known whether the tile has anything to update
     int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
     int tps, stages, abuf;    // taps per filter stage, stages, window buffers
+    int xarr;                 // first layers: arrays of an image row's chunks (0: the chunks of every column side by side)
+    unsigned a_step, a_lbo;   // 16-byte slots between a pixel's K groups, and between the two chunks of a group
     unsigned stage_bytes, abytes, tail_off, tmem_cols;    // (tail_off: barriers and tables, behind windows, stages and drained rows)
     unsigned wait_limit;
     int frames;               // several frames in one launch (delta only; gridDim.z = frames x ks), distances as in TcParams
@@ -436,8 +440,9 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             }
             const uint32_t Ab = base_u32 + buf * p.abytes;
             unsigned char* Ap = base + buf * p.abytes;
-            const int cl = XCOL && DT == T_I8 ? (p.kw + 3) >> 2 : gn * 2;      // 16-byte chunks per pixel
-            const uint32_t piece = (uint32_t)(gn * 2 * p.L) * 16u;              // bytes between the fp32 pieces' windows
+            const int arrays = XCOL && p.xarr ? p.xarr : gn * 2;               // of p.L slots each
+            const int cl = XCOL && DT == T_I8 && !p.xarr ? (p.kw + 3) >> 2 : arrays;      // 16-byte chunks to copy per pixel
+            const uint32_t piece = (uint32_t)(arrays * p.L) * 16u;              // bytes between the fp32 pieces' windows
             const unsigned magic = cl > 1 ? (unsigned)(((1ull << 32) + cl - 1) / cl) : 0u;
             const int items = p.span * cl;
             if (DT == T_I8 && !XCOL) {
@@ -515,7 +520,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 const bool vec = (p.row_units & 3) == 0;
                 #pragma unroll 2
                 for (int idx = tid; idx < items; idx += WN_FILL) {
-                    const int i = (int)__umulhi((unsigned)idx, magic), c = idx - i * cl;
+                    const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
                     const int off = S->src[i];
                     float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                     if (off >= 0) {
@@ -570,7 +575,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         const uint32_t idesc = DT == T_F32 ? (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24)
                                            : tc_instr_desc(p.bn);
         // (everything below in 16-byte units)
-        const uint32_t a_step = 2u * (uint32_t)p.L, b_unit = unit_b >> 4, b_piece = 2u * (uint32_t)p.bn, bn = (uint32_t)p.bn;
+        const uint32_t a_step = p.a_step, b_unit = unit_b >> 4, b_piece = 2u * (uint32_t)p.bn, bn = (uint32_t)p.bn;
         const uint32_t stage_step = p.stage_bytes >> 4, b_lo0 = wn_desc_lo(bstage_u32, bn);
         int ib = 0, stage = 0, buf = 0;
         uint32_t phase = 0, a_phase = 0, b_stage = b_lo0;
@@ -585,8 +590,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             if (!mbar_wait(smem_u32(&S->afull[buf]), a_phase, p.wait_limit)) { ok = false; break; }
             // fp32: the leading product's accumulator has to be free (two tiles: from the block before, else from two before)
             const int pb = p.mt > 1 ? 0 : (ib & 1), use = p.mt > 1 ? ib : ib >> 1;
-            const uint32_t a_piece = (uint32_t)gn * a_step;
-            uint32_t a_row = wn_desc_lo(base_u32 + buf * p.abytes, (uint32_t)p.L) + (uint32_t)(p.plane[plane].shift0 - p.min_shift + jy * p.Wq), a_tap = a_row + (uint32_t)j;
+            const uint32_t a_piece = (uint32_t)((XCOL && p.xarr ? p.xarr : gn * 2) * p.L);
+            uint32_t a_row = wn_desc_lo(base_u32 + buf * p.abytes, p.a_lbo) + (uint32_t)(p.plane[plane].shift0 - p.min_shift + jy * p.Wq), a_tap = a_row + (uint32_t)j;
             const uint32_t d0 = tmem + (DT == T_F32 && p.mt == 1 ? (uint32_t)pb * bn : 0u), d1 = tmem + bn, dc = tmem + 2u * bn;   // (dc: fp32, the small products)
             uint32_t fresh = 0;                              // fp32: 0 until the block's first MMA
             for (int t0 = t_lo; t0 < t_hi; t0 += p.tps) {
@@ -1034,7 +1039,13 @@ static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
         v = v > last + 1 - lo ? v : last + 1 - lo;
         return v;
     };
-    p.Wq = xcol ? L.ow : pitch(L.ow, d.w, fx_lo, fx_hi);
+    const int e = d.dtype == RRM_F32 ? 16 : 32;              // K elements of a group
+    p.groups = xcol ? ceil_div(d.kw * 4, e) : ceil_div(d.dtype == RRM_I8 ? in.cs : d.c_in, e);
+    // first layers: pixels of a 16-byte chunk; a row in one or two arrays where the stride is as many chunks
+    const int px = d.dtype == RRM_F32 ? 2 : 4;
+    p.xarr = xcol && d.stride % px == 0 && d.stride / px <= 2 ? d.stride / px : 0;
+    const int reach = p.xarr ? (2 * p.groups - 1) / p.xarr : 0;      // slots from a column's first chunk to its last
+    p.Wq = xcol ? L.ow + reach : pitch(L.ow, d.w, fx_lo, fx_hi);
     p.Hq = pitch(L.oh, d.h, fy_lo, fy_hi);
     p.min_shift = fy_lo * p.Wq + fx_lo;
     const int max_shift = fy_hi * p.Wq + fx_hi;
@@ -1055,13 +1066,11 @@ static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
         return r;
     };
     p.div_img = divisor(p.Hq * p.Wq); p.div_row = divisor(p.Wq);
-    p.span = TC_M + max_shift - p.min_shift;                 // (one accumulator tile)
+    p.span = TC_M + max_shift - p.min_shift + reach;         // (one accumulator tile)
     if (p.span > WN_MAX_SPAN) return false;
     // (rows of the linear space without a projection pixel are work for nothing: with more than half of them a layer
     // such as a filter that covers the whole map is better off with its rows compacted)
     if ((long long)L.oh * L.ow * 2 < (long long)p.Hq * p.Wq) return false;
-    const int e = d.dtype == RRM_F32 ? 16 : 32;              // K elements of a group
-    p.groups = xcol ? ceil_div(d.kw * 4, e) : ceil_div(d.dtype == RRM_I8 ? in.cs : d.c_in, e);
     const int plane_taps = ceil_div(d.kh, d.stride) * (xcol ? 1 : ceil_div(d.kw, d.stride));
     if (d.dtype == RRM_F32 && plane_taps * (xcol ? p.groups : 1) > WN_PROMOTE) return false;
     return true;
@@ -1116,7 +1125,9 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
                 p.ks = p.nblk * p.tsplit;
             }
             p.cluster = clustered && p.ks > 1;
-            p.abytes = (unsigned)(((size_t)gblk * 2 * pieces * p.L * 16 + 127) & ~(size_t)127);
+            p.abytes = (unsigned)(((size_t)(p.xarr ? p.xarr : gblk * 2) * pieces * p.L * 16 + 127) & ~(size_t)127);
+            p.a_lbo = p.xarr == 1 ? 1u : (unsigned)p.L;
+            p.a_step = p.xarr ? 2u / (unsigned)p.xarr : 2u * (unsigned)p.L;
             p.tps = 1;
             while ((size_t)p.tps * 2 * gblk * unit <= (f32 ? 24u : 16u) * 1024 && p.tps < plane_taps) p.tps *= 2;
             p.stage_bytes = (unsigned)(p.tps * gblk * unit);

@@ -158,7 +158,8 @@ def test_single_layer_shapes(dtype, c_in, c_out, hw, k, s, p):
     (24, 33, (30, 31), 3, 2, 1, 3),          # stride 2: four planes; rows that are no multiple of 16 bytes
     (20, 16, (25, 23), 5, 3, 2, 1),          # stride 3: nine planes, some with fewer taps
     (16, 20, (140, 139), 3, 1, 1, 2),        # enough rows for two accumulator tiles per thread block
-    (2, 72, (41, 38), 9, 4, 3, 2),           # few channels: filter rows side by side
+    (2, 72, (41, 38), 9, 4, 3, 2),           # few channels, stride 4: the windows are image rows in one (int8) or two (fp32) arrays
+    (3, 16, (45, 52), 9, 8, 2, 1),           # ... stride 8: in two (int8), or column by column (fp32)
     (12, 24, (3, 1400), 3, 1, 1, 1)])        # a window wider than shared memory takes: the other kernels
 def test_window_convolution_tile_edges(dtype, c_in, c_out, hw, k, s, p, n, monkeypatch):
     rng = np.random.default_rng(c_in * 1000 + c_out * 10 + k)
