@@ -175,7 +175,6 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
     for (auto& T : net->tensors) {
         RRM_TRY(dev_alloc(net, &T.X, T.bytes()));
         RRM_TRY(dev_alloc(net, &T.D, T.bytes()));
-        RRM_TRY(dev_alloc(net, (void**)&T.pnnz, (size_t)T.pixels() * 4));
         cleared += (size_t)T.act_words() * 4;
     }
     for (auto& L : net->layers) cleared += (size_t)ceil_div(L.opixels(), 32) * 4;

@@ -117,7 +117,6 @@ struct Tensor {
     void* X = nullptr;                // current value (= snapshot of the previous frame before a step)
     void* D = nullptr;                // delta rows, valid only for pixels whose `act` bit is set
     uint32_t* act = nullptr;          // bitmap over n*h*w pixels (cleared every step)
-    int* pnnz = nullptr;              // per-pixel count of non-zero delta elements (valid where act is set)
     unsigned long long* nnz = nullptr;      // total non-zero delta elements (cleared every step)
     unsigned long long* npix = nullptr;     // active pixels (cleared every step)
     double* trunc = nullptr;                // fp32: sum of squares of the truncated delta entries (cleared every step)

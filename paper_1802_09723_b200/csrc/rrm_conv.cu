@@ -541,7 +541,7 @@ constexpr int IMP_TP = 32;                  // pixels per tile = lanes of the wa
 
 template <typename T, bool DELTA>
 __global__ void __launch_bounds__(256) import_nchw_kernel(const T* __restrict__ src, T* X, T* D, uint32_t* act,
-                                                          int* pnnz, unsigned long long* nnz,
+                                                          unsigned long long* nnz,
                                                           unsigned long long* npix, int* errw,
                                                           int c, int cs, int hw, int w, Readers readers,
                                                           float eps, double* trunc, SeqFrames sf)
@@ -618,7 +618,6 @@ __global__ void __launch_bounds__(256) import_nchw_kernel(const T* __restrict__ 
         if (cnt > 0) {
             const size_t gp = gp0 + tid;
             atomicOr(&act[gp >> 5], 1u << (gp & 31));
-            pnnz[gp] = cnt;
         }
         int tot = cnt;
         #pragma unroll
@@ -654,9 +653,8 @@ __global__ void __launch_bounds__(256) import_nchw_kernel(const T* __restrict__ 
 
 // int8 frames with up to 4 channels (one 4-byte word per pixel): one thread per pixel, plane reads coalesced
 // across the warp, the activity word of 32 consecutive pixels written by one lane from a ballot.
-template <bool DELTA>
 __global__ void __launch_bounds__(256) import_i8_word_kernel(const int8_t* __restrict__ src, uint32_t* X, uint32_t* D,
-                                                            uint32_t* act, int* pnnz, unsigned long long* nnz,
+                                                            uint32_t* act, unsigned long long* nnz,
                                                             unsigned long long* npix, int* errw, int c, int h, int w,
                                                             int pixels, Readers readers)
 {
@@ -669,26 +667,20 @@ __global__ void __launch_bounds__(256) import_i8_word_kernel(const int8_t* __res
         const int ns = gp / hw, pix = gp - ns * hw;
         uint32_t nw = 0;
         for (int ch = 0; ch < c; ++ch) nw |= ((uint32_t)(uint8_t)src[((size_t)ns * c + ch) * hw + pix]) << (8 * ch);
-        if (DELTA) {
-            const uint32_t ow = X[gp];
-            if (nw != ow) {
-                uint32_t dw = 0;
-                #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int d = (int)(int8_t)(nw >> (8 * j)) - (int)(int8_t)(ow >> (8 * j));
-                    if (d < -128 || d > 127) atomicOr(errw, ERRW_BOUNDS);
-                    dw |= ((uint32_t)d & 0xffu) << (8 * j);
-                    cnt += d != 0;
-                }
-                D[gp] = dw;
-                X[gp] = nw;
-                pnnz[gp] = cnt;
+        const uint32_t ow = X[gp];
+        if (nw != ow) {
+            uint32_t dw = 0;
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int d = (int)(int8_t)(nw >> (8 * j)) - (int)(int8_t)(ow >> (8 * j));
+                if (d < -128 || d > 127) atomicOr(errw, ERRW_BOUNDS);
+                dw |= ((uint32_t)d & 0xffu) << (8 * j);
+                cnt += d != 0;
             }
-        } else {
+            D[gp] = dw;
             X[gp] = nw;
         }
     }
-    if (!DELTA) return;
     const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
     if (m == 0) return;                                      // uniform inside the warp
     if (lane == 0) act[gp >> 5] = m;                         // gp of lane 0 is a multiple of 32: the word is this warp's alone
@@ -786,58 +778,68 @@ __global__ void __launch_bounds__(256, 4) import_i8_word_frames_kernel(const int
     }
 }
 
-// fp32 frames of at most 4 channels, several frames per launch, no truncation (Sec. 3.4 off): the same walk as
-// import_i8_word_frames_kernel - a thread per pixel reads its channel planes of frame g and g - 1 (coalesced along the
-// pixels), writes the delta row of a changed pixel and, in the last frame, the snapshot.
-__global__ void __launch_bounds__(256, 4) import_f32_px_frames_kernel(const float* __restrict__ src, float* X, float* D, uint32_t* act,
-                                                                     unsigned long long* nnz, unsigned long long* npix,
-                                                                     int c, int h, int w, int pixels, Readers readers, SeqFrames sf)
+// fp32 frames of at most 4 channels, no truncation (Sec. 3.4 off), a thread per pixel and group: reads its channel planes
+// (coalesced along the pixels), writes the delta row of a changed pixel.  IMP_STEP compares with the snapshot and moves it
+// on, IMP_FRAMES takes several frames (frame = blockIdx.z) and compares with the frame before at the boundary (the last
+// frame writes the snapshot), IMP_DENSE writes the rows.  A warp takes 32 * G consecutive pixels, all reads of a thread in
+// flight together; each group of 32 owns its activity word.  Against the tiled kernel (32 pixels x 3 channels per CTA), 8
+// frames of 227 x 227: step 44 -> 13 us.
+enum { IMP_DENSE, IMP_STEP, IMP_FRAMES };
+template <int MODE, int G>
+__global__ void __launch_bounds__(256, 4) import_f32_px_kernel(const float* __restrict__ src, float* X, float* D, uint32_t* act,
+                                                              unsigned long long* nnz, unsigned long long* npix,
+                                                              int c, int h, int w, int pixels, Readers readers, SeqFrames sf)
 {
     const int lane = threadIdx.x & 31;
-    const int base = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 128;
+    const int base = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 32 * G;
     const int hw = h * w;
-    {
+    long long arena_off = 0;
+    if (MODE == IMP_FRAMES) {
         const long long g = blockIdx.z;
         src += g * sf.in_stride;
         D = shift_bytes(D, g * sf.row_stride);
-        act = shift_bytes(act, g * sf.arena_stride); nnz = shift_bytes(nnz, g * sf.arena_stride);
-        npix = shift_bytes(npix, g * sf.arena_stride);
+        arena_off = g * sf.arena_stride;
+        act = shift_bytes(act, arena_off); nnz = shift_bytes(nnz, arena_off); npix = shift_bytes(npix, arena_off);
     }
-    const long long arena_off = (long long)blockIdx.z * sf.arena_stride;
-    const bool write_x = (int)blockIdx.z == sf.frames - 1;
+    const bool write_x = MODE != IMP_FRAMES || (int)blockIdx.z == sf.frames - 1;
     pdl_launch_dependents();
     pdl_wait();
-    float nv[4][4], pv[4][4];
+    float nv[G][4], pv[G][4];
     #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < G; ++k) {
         const int gp = base + 32 * k + lane;
+        const int ns = gp / hw, pix = gp - ns * hw;
         #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
             nv[k][ch] = pv[k][ch] = 0.f;
             if (gp >= pixels || ch >= c) continue;
-            const int ns = gp / hw, pix = gp - ns * hw;
             const size_t o = ((size_t)ns * c + ch) * hw + pix;
             nv[k][ch] = src[o];
-            pv[k][ch] = (src - sf.in_stride)[o];
+            if (MODE == IMP_FRAMES) pv[k][ch] = (src - sf.in_stride)[o];
+            if (MODE == IMP_STEP) pv[k][ch] = X[(size_t)gp * c + ch];
         }
     }
-    #pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
+    unsigned cnts = 0;                                       // this thread's changed channels, 4 bits per group
+    #pragma unroll
+    for (int k = 0; k < G; ++k) {
         const int gp = base + 32 * k + lane;
-        if (base + 32 * k >= pixels) break;                  // uniform inside the warp
-        int cnt = 0;
-        if (gp < pixels) {
-            #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
-                if (ch >= c) break;
-                if (write_x) X[(size_t)gp * c + ch] = nv[k][ch];
-                cnt += nv[k][ch] != pv[k][ch];
-            }
-            if (cnt) {
-                #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) if (ch < c) D[(size_t)gp * c + ch] = nv[k][ch] - pv[k][ch];
-            }
+        if (gp >= pixels) continue;
+        unsigned cnt = 0;
+        #pragma unroll
+        for (int ch = 0; ch < 4; ++ch) if (ch < c) cnt += nv[k][ch] != pv[k][ch];
+        #pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+            if (ch >= c) break;
+            if (write_x && (MODE != IMP_STEP || cnt)) X[(size_t)gp * c + ch] = nv[k][ch];
+            if (MODE != IMP_DENSE && cnt) D[(size_t)gp * c + ch] = nv[k][ch] - pv[k][ch];
         }
+        cnts |= cnt << (4 * k);
+    }
+    if (MODE == IMP_DENSE) return;
+    #pragma unroll 1
+    for (int k = 0; k < G; ++k) {
+        const int gp = base + 32 * k + lane;
+        const int cnt = (int)(cnts >> (4 * k) & 15u);
         const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
         if (m == 0) continue;                                // uniform inside the warp
         if (lane == 0) act[gp >> 5] = m;                     // gp of lane 0 is a multiple of 32: the word is this group's alone
@@ -859,10 +861,154 @@ __global__ void __launch_bounds__(256, 4) import_f32_px_frames_kernel(const floa
     }
 }
 
+// Dense int8 frames of at most 4 channels: four pixels of a thread's reads in flight together.
+__global__ void __launch_bounds__(256) import_i8_word_dense_kernel(const int8_t* __restrict__ src, uint32_t* X, int c, int hw, int pixels)
+{
+    const int base = blockIdx.x * 1024 + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    uint32_t v[4] = {0, 0, 0, 0};
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int gp = base + 256 * k;
+        if (gp >= pixels) continue;
+        const int ns = gp / hw, pix = gp - ns * hw;
+        #pragma unroll
+        for (int ch = 0; ch < 4; ++ch) if (ch < c) v[k] |= ((uint32_t)(uint8_t)src[((size_t)ns * c + ch) * hw + pix]) << (8 * ch);
+    }
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) if (base + 256 * k < pixels) X[base + 256 * k] = v[k];
+}
+
+// int8 between the boundary layout and whole 32-byte pixel rows, a 128-pixel x 32-channel tile at a time through shared
+// memory: rows as 16-byte groups, planes along the pixels (as words where a plane's address allows).  EXPORT: rows -> planes.
+// grid = (pixel tiles, channel tiles x n, frames).  30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread
+// per element, import of 48 channels 10.8 -> 7.0 against the 32-pixel tiles.
+template <bool EXPORT>
+__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, int ctiles,
+                                                          long long src_stride, long long dst_stride)
+{
+    __shared__ __align__(16) int8_t tile[32][132];
+    const int p0 = blockIdx.x * 128, c0 = (int)(blockIdx.y % ctiles) * 32;
+    const long long ns = blockIdx.y / ctiles;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, px = threadIdx.x >> 1, half = (threadIdx.x & 1) * 16;
+    src += blockIdx.z * src_stride;
+    dst += blockIdx.z * dst_stride;
+    pdl_launch_dependents();
+    pdl_wait();
+    const long long row = ((ns * hw + p0 + px) * cs) + c0 + half;
+    if (EXPORT && p0 + px < hw) {
+        const uint4 v = *reinterpret_cast<const uint4*>(src + row);
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        #pragma unroll
+        for (int j = 0; j < 16; ++j) tile[half + j][px] = (int8_t)(u[j >> 2] >> (8 * (j & 3)));
+    }
+    if (EXPORT) __syncthreads();
+    #pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int ch = warp * 4 + k;
+        const long long o = (ns * c + c0 + ch) * hw + p0;
+        const bool live = c0 + ch < c, words = live && p0 + 128 <= hw && ((uintptr_t)((EXPORT ? dst : src) + o) & 3) == 0;
+        uint32_t* const t = reinterpret_cast<uint32_t*>(&tile[ch][lane * 4]);
+        if (words) {
+            if (EXPORT) *reinterpret_cast<uint32_t*>(dst + o + lane * 4) = *t;
+            else *t = *reinterpret_cast<const uint32_t*>(src + o + lane * 4);
+        } else {
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int q = j * 32 + lane;
+                const bool in = live && p0 + q < hw;
+                if (EXPORT) { if (in) dst[o + q] = tile[ch][q]; }
+                else tile[ch][q] = in ? src[o + q] : (int8_t)0;
+            }
+        }
+    }
+    if (EXPORT) return;
+    __syncthreads();
+    if (p0 + px >= hw) return;
+    uint32_t u[4] = {0, 0, 0, 0};
+    #pragma unroll
+    for (int j = 0; j < 16; ++j) u[j >> 2] |= (uint32_t)(uint8_t)tile[half + j][px] << (8 * (j & 3));
+    *reinterpret_cast<uint4*>(dst + row) = make_uint4(u[0], u[1], u[2], u[3]);
+}
+
+// One frame of a tensor of 4-channel groups (fp32, or int8 rows of whole 32-byte groups), up to 64 channels, against the
+// snapshot: a CTA takes 32 pixels, 16 lanes a pixel.  A lone frame's import is a chain of round trips, so plane and
+// snapshot reads are issued together and a pixel's 16 lanes agree on its activity with a ballot (the tiled kernel reads
+// the snapshot after the turn-around and counts through shared-memory atomics: 64 x 56 x 56 fp32 8.8 -> 4.5 us).
+template <typename T>
+__global__ void __launch_bounds__(256) import_step_kernel(const T* __restrict__ src, T* X, T* D, uint32_t* act, unsigned long long* nnz,
+                                                         unsigned long long* npix, int* errw, int c, int cs, int hw, int w, Readers readers)
+{
+    using V = typename std::conditional<sizeof(T) == 4, float4, char4>::type;
+    __shared__ T s_x[IMP_TP][64 + (sizeof(T) == 4 ? 1 : 4)];
+    __shared__ int s_cnt[IMP_TP];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ns = blockIdx.y, pix0 = blockIdx.x * IMP_TP;
+    const int quad = tid & 15;                               // this lane's 4 channels
+    const bool mine = quad * 4 < cs;
+    pdl_launch_dependents();
+    pdl_wait();
+    T v[8];
+    V old[2];
+    const size_t gp0 = (size_t)ns * hw + pix0;
+    #pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int ch = warp + 8 * k;
+        v[k] = ch < c && pix0 + lane < hw ? src[((size_t)ns * c + ch) * hw + pix0 + lane] : (T)0;
+    }
+    #pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int pl = (tid >> 4) + 16 * k;
+        if (mine && pix0 + pl < hw) old[k] = *reinterpret_cast<const V*>(X + (gp0 + pl) * cs + quad * 4);
+    }
+    #pragma unroll
+    for (int k = 0; k < 8; ++k) s_x[lane][warp + 8 * k] = v[k];
+    __syncthreads();
+    #pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int pl = (tid >> 4) + 16 * k;
+        int cnt = 0;
+        V nv{}, dv{};
+        if (mine && pix0 + pl < hw) {
+            const T* at = &s_x[pl][quad * 4];
+            nv.x = at[0]; nv.y = at[1]; nv.z = at[2]; nv.w = at[3];
+            dv.x = nv.x - old[k].x; dv.y = nv.y - old[k].y; dv.z = nv.z - old[k].z; dv.w = nv.w - old[k].w;
+            cnt = (nv.x != old[k].x) + (nv.y != old[k].y) + (nv.z != old[k].z) + (nv.w != old[k].w);
+            if (sizeof(T) == 1 && cnt) {
+                auto far = [](int a, int b) { return a - b < -128 || a - b > 127; };
+                if (far((int)nv.x, (int)old[k].x) || far((int)nv.y, (int)old[k].y) || far((int)nv.z, (int)old[k].z) || far((int)nv.w, (int)old[k].w))
+                    atomicOr(errw, ERRW_BOUNDS);
+            }
+            if (cnt) *reinterpret_cast<V*>(X + (gp0 + pl) * cs + quad * 4) = nv;
+        }
+        #pragma unroll
+        for (int o = 8; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+        if (cnt && mine && pix0 + pl < hw) *reinterpret_cast<V*>(D + (gp0 + pl) * cs + quad * 4) = dv;
+        if (quad == 0) s_cnt[pl] = cnt;
+    }
+    __syncthreads();
+    if (warp > 0) return;
+    const int pix = pix0 + lane;
+    const int cnt = pix < hw ? s_cnt[lane] : 0;
+    const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
+    if (m == 0) return;
+    if (cnt > 0) atomicOr(&act[(gp0 + lane) >> 5], 1u << ((gp0 + lane) & 31));
+    const int tot = __reduce_add_sync(0xffffffffu, cnt);
+    unsigned long long macs[MAX_READERS];
+    scatter_changed_warp(readers, ns, pix / w, pix % w, cnt, lane, macs);
+    if (lane == 0) {
+        atomicAdd(nnz, (unsigned long long)tot);
+        atomicAdd(npix, (unsigned long long)__popc(m));
+        #pragma unroll
+        for (int i = 0; i < MAX_READERS; ++i) if (i < readers.n && readers.r[i].macs && macs[i]) atomicAdd(readers.r[i].macs, macs[i]);
+    }
+}
+
 // Binary frames arrive already pixel-major and bit-packed: one thread per pixel.
 template <bool DELTA>
 __global__ void import_bin_kernel(const uint32_t* __restrict__ src, uint32_t* X, uint32_t* D, uint32_t* act,
-                                  int* pnnz, unsigned long long* nnz, unsigned long long* npix, int cw, int pixels,
+                                  unsigned long long* nnz, unsigned long long* npix, int cw, int pixels,
                                   int h, int w, Readers readers, uint32_t* Xn, SeqFrames sf)
 {
     const int gp = blockIdx.x * blockDim.x + threadIdx.x;
@@ -893,7 +1039,6 @@ __global__ void import_bin_kernel(const uint32_t* __restrict__ src, uint32_t* X,
         }
         if (DELTA && cnt) {
             atomicOr(&act[gp >> 5], 1u << (gp & 31));
-            pnnz[gp] = cnt;
         }
     }
     if (!DELTA) return;
@@ -932,7 +1077,6 @@ struct EpiParams {
     void* X;                  // output tensor values
     void* D;                  // output tensor delta rows
     uint32_t* act;
-    int* pnnz;
     unsigned long long* nnz;
     unsigned long long* npix;
     int* errw;
@@ -1161,7 +1305,6 @@ __global__ void __launch_bounds__(256) epilogue_kernel(EpiParams p)
     __syncthreads();
     if (sub == 0 && lane == 0 && r < tpix && s_cnt[slot]) {
         atomicOr(&p.act[r >> 5], 1u << (r & 31));
-        p.pnnz[r] = s_cnt[slot];
         atomicAdd(&s_nnz, (unsigned)s_cnt[slot]);
         atomicAdd(&s_npix, 1u);
     }
@@ -1381,28 +1524,45 @@ int launch_import(rrm_net* net, const void* frame, bool delta, bool stateless, c
     if (T.dtype == T_BIN) {
         const int blocks = ceil_div(T.pixels(), 256);
         if (delta) launch_seq(import_bin_kernel<true>, dim3(blocks, 1, gz), dim3(256), 0, st, (const uint32_t*)frame, (uint32_t*)X, (uint32_t*)T.D,
-                                                                  T.act, T.pnnz, T.nnz, T.npix, T.cs, T.pixels(),
+                                                                  T.act, T.nnz, T.npix, T.cs, T.pixels(),
                                                                   T.h, T.w, T.readers, (uint32_t*)(stateless ? nullptr : T.Xn_cur), sf);
         else launch_seq(import_bin_kernel<false>, dim3(blocks), dim3(256), 0, st, (const uint32_t*)frame, (uint32_t*)X, nullptr, nullptr,
-                                                              nullptr, nullptr, nullptr, T.cs, T.pixels(), T.h, T.w,
+                                                              nullptr, nullptr, T.cs, T.pixels(), T.h, T.w,
                                                               Readers{}, (uint32_t*)nullptr, sf);
     } else if (T.dtype == T_I8 && T.cs == 4) {
         const int blocks = ceil_div(T.pixels(), 256);
         if (seq) launch_seq(import_i8_word_frames_kernel, dim3(ceil_div(T.pixels(), 1024), 1, gz), dim3(256), 0, st, (const int8_t*)frame, (uint32_t*)X,
                             (uint32_t*)T.D, T.act, T.nnz, T.npix, net->errw, T.c, T.h, T.w, T.pixels(), T.readers, sf);
-        else if (delta) launch_seq(import_i8_word_kernel<true>, dim3(blocks), dim3(256), 0, st, (const int8_t*)frame, (uint32_t*)X, (uint32_t*)T.D, T.act,
-                                                                      T.pnnz, T.nnz, T.npix, net->errw, T.c, T.h, T.w,
+        else if (delta) launch_seq(import_i8_word_kernel, dim3(blocks), dim3(256), 0, st, (const int8_t*)frame, (uint32_t*)X, (uint32_t*)T.D, T.act,
+                                                                      T.nnz, T.npix, net->errw, T.c, T.h, T.w,
                                                                       T.pixels(), T.readers);
-        else launch_seq(import_i8_word_kernel<false>, dim3(blocks), dim3(256), 0, st, (const int8_t*)frame, (uint32_t*)X, nullptr, nullptr, nullptr,
-                                                                  nullptr, nullptr, net->errw, T.c, T.h, T.w, T.pixels(),
-                                                                  Readers{});
+        else launch_seq(import_i8_word_dense_kernel, dim3(ceil_div(T.pixels(), 1024)), dim3(256), 0, st, (const int8_t*)frame, (uint32_t*)X, T.c, hw, T.pixels());
     } else {
         dim3 grid(ceil_div(hw, IMP_TP), T.n, gz);
         const size_t smem = (size_t)IMP_TP * (T.cs + 1) * T.unit_bytes * (seq ? 2 : 1);
         if (smem > 200 * 1024) return RRM_ERR_UNSUPPORTED;
-        if (T.dtype == T_F32 && seq && T.c <= 4 && !(net->eps > 0.f)) {
-            launch_seq(import_f32_px_frames_kernel, dim3(ceil_div(T.pixels(), 1024), 1, gz), dim3(256), 0, st, (const float*)frame, (float*)X,
-                       (float*)T.D, T.act, T.nnz, T.npix, T.c, T.h, T.w, T.pixels(), T.readers, sf);
+        const bool exact = !(net->eps > 0.f);
+        if (T.dtype == T_F32 && T.c <= 4 && (exact || !delta)) {
+            // (four groups of pixels per thread once that still leaves a CTA per SM; a lone frame's chain is shorter with one)
+            const bool wide = seq || T.pixels() >= 148 * 1024;
+            const dim3 g(ceil_div(T.pixels(), wide ? 1024 : 256), 1, gz);
+            auto go = [&](auto kernel) {
+                launch_seq(kernel, dim3(g), dim3(256), 0, st, (const float*)frame, (float*)X, (float*)T.D, T.act, T.nnz, T.npix, T.c, T.h, T.w,
+                           T.pixels(), T.readers, sf);
+            };
+            if (seq) go(import_f32_px_kernel<IMP_FRAMES, 4>);
+            else if (delta) { if (wide) go(import_f32_px_kernel<IMP_STEP, 4>); else go(import_f32_px_kernel<IMP_STEP, 1>); }
+            else { if (wide) go(import_f32_px_kernel<IMP_DENSE, 4>); else go(import_f32_px_kernel<IMP_DENSE, 1>); }
+        } else if (T.dtype == T_F32 && delta && !seq && exact && T.cs % 4 == 0 && T.cs <= 64) {
+            launch_seq(import_step_kernel<float>, dim3(grid), dim3(256), 0, st, (const float*)frame, (float*)X, (float*)T.D, T.act, T.nnz, T.npix,
+                       net->errw, T.c, T.cs, hw, T.w, T.readers);
+        } else if (T.dtype == T_I8 && delta && !seq && T.cs <= 64) {
+            launch_seq(import_step_kernel<int8_t>, dim3(grid), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, (int8_t*)T.D, T.act, T.nnz, T.npix,
+                       net->errw, T.c, T.cs, hw, T.w, T.readers);
+        } else if (T.dtype == T_I8 && !delta) {
+            const int ctiles = T.cs / 32;
+            launch_seq(transpose_i8_kernel<false>, dim3(ceil_div(hw, 128), ctiles * T.n), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, T.c, T.cs, hw,
+                       ctiles, 0ll, 0ll);
         } else if (T.dtype == T_F32) {
             auto kd = import_nchw_kernel<float, true>;
             auto kn = import_nchw_kernel<float, false>;
@@ -1410,21 +1570,15 @@ int launch_import(rrm_net* net, const void* frame, bool delta, bool stateless, c
                 cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 cudaFuncSetAttribute(kn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             }
-            if (delta) launch_seq(kd, dim3(grid), dim3(256), smem, st, (const float*)frame, (float*)X, (float*)T.D, T.act, T.pnnz, T.nnz,
+            if (delta) launch_seq(kd, dim3(grid), dim3(256), smem, st, (const float*)frame, (float*)X, (float*)T.D, T.act, T.nnz,
                                                    T.npix, net->errw, T.c, T.cs, hw, T.w, T.readers, net->eps, T.trunc, sf);
             else launch_seq(kn, dim3(grid), dim3(256), smem, st, (const float*)frame, (float*)X, nullptr, nullptr, nullptr, nullptr,
-                                             nullptr, net->errw, T.c, T.cs, hw, T.w, Readers{}, 0.f, nullptr, sf);
+                                             net->errw, T.c, T.cs, hw, T.w, Readers{}, 0.f, nullptr, sf);
         } else {
             auto kd = import_nchw_kernel<int8_t, true>;
-            auto kn = import_nchw_kernel<int8_t, false>;
-            if (smem > 48 * 1024) {
-                cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                cudaFuncSetAttribute(kn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            }
-            if (delta) launch_seq(kd, dim3(grid), dim3(256), smem, st, (const int8_t*)frame, (int8_t*)X, (int8_t*)T.D, T.act, T.pnnz,
+            if (smem > 48 * 1024) cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            launch_seq(kd, dim3(grid), dim3(256), smem, st, (const int8_t*)frame, (int8_t*)X, (int8_t*)T.D, T.act,
                                                    T.nnz, T.npix, net->errw, T.c, T.cs, hw, T.w, T.readers, 0.f, nullptr, sf);
-            else launch_seq(kn, dim3(grid), dim3(256), smem, st, (const int8_t*)frame, (int8_t*)X, nullptr, nullptr, nullptr, nullptr,
-                                             nullptr, net->errw, T.c, T.cs, hw, T.w, Readers{}, 0.f, nullptr, sf);
         }
     }
     RRM_CUDA_TRY(cudaGetLastError());
@@ -1559,7 +1713,7 @@ int launch_layer(rrm_net* net, int l, bool dense, bool stateless, cudaStream_t s
     e.dP = split ? split->dP : nullptr; e.Q = split ? split->Q : nullptr; e.Z = split ? split->Z : nullptr;
     e.oact_prev = split ? split->prev_oact : nullptr; e.opix = L.opixels(); e.Xn = split ? out.Xn_cur : nullptr;
     e.resX = res ? (stateless ? res->X2 : res->X) : nullptr;
-    e.X = stateless ? out.X2 : out.X; e.D = out.D; e.act = out.act; e.pnnz = out.pnnz; e.nnz = out.nnz;
+    e.X = stateless ? out.X2 : out.X; e.D = out.D; e.act = out.act; e.nnz = out.nnz;
     e.npix = out.npix; e.errw = out.has_consumer ? net->errw : nullptr;
     e.n = d.n; e.oh = L.oh; e.ow = L.ow; e.th = L.th; e.tw = L.tw; e.c_out = d.c_out; e.cs = out.cs;
     e.pool_k = d.pool_k; e.pool_s = d.pool_s; e.pool_p = d.pool_p; e.act_fn = d.act; e.shift = d.shift; e.theta = d.theta;
@@ -1719,7 +1873,10 @@ int launch_export_tensor(rrm_net* net, int t, void* dst, bool stateless, cudaStr
     const int hw = T.h * T.w;
     const long long total = (long long)T.n * T.c * hw;
     const int blocks = (int)((total + 255) / 256);
-    if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, dim3(blocks), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, total, 0ll, 0ll);
+    if (T.dtype == T_I8 && T.cs % 32 == 0) {
+        const int ctiles = T.cs / 32;
+        launch_seq(transpose_i8_kernel<true>, dim3(ceil_div(hw, 128), ctiles * T.n, 1), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, ctiles, 0ll, 0ll);
+    } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, dim3(blocks), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, total, 0ll, 0ll);
     else {
         const int ctiles = ceil_div(T.c, 32);
         launch_seq(export_nchw_tiled_kernel, dim3(ceil_div(hw, 32), ctiles * T.n, 1), dim3(32, 8), 0, st, (const uint32_t*)X, (uint32_t*)dst,
@@ -1741,7 +1898,11 @@ int launch_export_seq(rrm_net* net, int frames, void* dst, cudaStream_t st)
     const int hw = T.h * T.w;
     const long long total = (long long)T.n * T.c * hw;
     const dim3 grid((unsigned)((total + 255) / 256), (unsigned)frames);
-    if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, grid, dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, total,
+    if (T.dtype == T_I8 && T.cs % 32 == 0) {
+        const int ctiles = T.cs / 32;
+        launch_seq(transpose_i8_kernel<true>, dim3(ceil_div(hw, 128), ctiles * T.n, frames), dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, ctiles,
+                   (long long)T.bytes(), total);
+    } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, grid, dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, total,
                                     (long long)T.bytes(), total);
     else {
         const int ctiles = ceil_div(T.c, 32);

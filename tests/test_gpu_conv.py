@@ -183,6 +183,32 @@ def test_window_convolution_tile_edges(dtype, c_in, c_out, hw, k, s, p, n, monke
     net.close()
 
 
+@pytest.mark.parametrize("dtype,c_in,c_out,hw,n", [
+    ("f32", 3, 40, (9, 15), 2), ("f32", 4, 8, (320, 300), 2),         # a thread per pixel; four pixel groups per thread
+    ("f32", 64, 36, (13, 9), 2), ("f32", 8, 5, (6, 6), 3),            # 16 lanes per pixel: full, and few of them at work
+    ("i8", 64, 33, (16, 16), 2), ("i8", 33, 70, (11, 13), 3),         # planes aligned to words, and not; ragged channel tiles
+    ("i8", 96, 16, (17, 8), 1), ("i8", 3, 130, (33, 31), 2)])
+def test_boundary_layouts(dtype, c_in, c_out, hw, n):
+    """The kernels between the boundary layout and pixel rows: frames in, outputs out, frame by frame and in a dense
+    chunk, at the edges of their tiles."""
+    rng = np.random.default_rng(c_in * 100 + c_out)
+    kw = dict(act="relu", shift=11) if dtype == "i8" else {}
+    sp = _spec(dtype, c_in, hw, c_out, 1, 1, 0, rng, **kw)
+    video = _video(dtype, c_in, hw, 5, n, rng)
+    _run([sp], video, n=n, stats=True, keyframe_at=(4,))
+    net = _rrm().net_from_specs([sp], n=n)
+    outs = net.new_output(frames=3)
+    net.dense_seq(dev(video[1:4]), outs, 3)
+    for t in range(3):
+        want = orc.dense_forward([sp], video[1 + t])[0][1]
+        got = outs[t].cpu().numpy()
+        if dtype == "f32":
+            assert float(np.abs(got - want).max()) <= F32_TOL * float(np.abs(want).max()), t
+        else:
+            np.testing.assert_array_equal(got.astype(np.int64), want, err_msg=f"frame {t}")
+    net.close()
+
+
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [(16, 70, (13, 13), 3, 1, 1), (8, 12, (17, 15), 5, 2, 2), (64, 16, (10, 10), 3, 1, 1),
                                                  (3, 6, (35, 35), 11, 4, 0)])
