@@ -24,7 +24,7 @@
 // of the nine products of pieces are formed; what the other three would add is below 2^-25 of a product, less than the
 // rounding of one fp32 multiplication.  The tensor core adds in fp32 but truncates, so the leading product has an
 // accumulator that is added to registers (round to nearest) after at most WN_PROMOTE K steps of 16, and the five
-// small ones have one of their own.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
+// small ones have two of their own.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
 // a chain of fmaf 6e-7; without the promotion 1.7e-6, with everything in one accumulator 1.5e-5.
 //
 // Roles: warps 0-7 fill windows and drain accumulators, warp 8 issues the MMAs, warp 9 the bulk copies of the filters
@@ -33,10 +33,12 @@
 // and a dense pass needs no zeroed projection).  Every wait on an mbarrier is bounded; one that runs out sets
 // ERRW_TIMEOUT and the CTA leaves through the common exit.
 //
-// Measured, AlexNet-shaped stack at 227 x 227, against the kernels that gathered rows tap by tap (fp32: on the CUDA cores):
-// fp32, 32 frames of one stream 1700 -> 818 us (conv2: 351 -> 195, conv4: 412 -> 167), 8 streams 546 -> 269; int8, one
-// frame 84 -> 70, 32 dense frames 266 -> 212 (conv1: 62 -> 44, conv2: 43 -> 28); ResNet-18 shape, 4 streams 344 -> 278.
-// A launch of a few tiles is a chain of ~7 us: rows and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7.
+// What bounds it: in a long K loop the MMAs' operand reads from shared memory (an MMA of 128 columns reads 8 KB, the 64
+// clocks it takes), beside which the filter copies write another quarter (fp32 step of 768 MMA clocks: 1064 measured, 1180
+// with six separate MMAs and the barrier looked at only when it is needed); in a launch of a few tiles a chain of ~7 us (rows
+// and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  Against kernels that gathered rows tap by tap (fp32: on the
+// CUDA cores), AlexNet-shaped stack at 227 x 227: fp32 32 dense frames conv2 / conv4 192 / 86 -> 175 / 62 us since the MMAs
+// of a step are issued together (delta, gathered: 351 / 412), 8 streams 546 -> 206 for the whole stack; int8 frame 84 -> 70.
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
@@ -65,7 +67,7 @@ struct WinParams {
     const uint32_t* in_act;   // input activity bitmap (delta mode)
     const uint32_t* oact;     // projection pixels to update (delta mode)
     int* ocount;              // their number is added here, and that of the accumulator tiles they lie in behind it
-    const unsigned char* Wimg;      // [n tile][tap][group][pieces][2][bn][16 bytes]
+    const unsigned char* Wimg;      // [n tile][tap][group][2][pieces][bn][16 bytes]
     const void* bias;
     void* P;                  // [opixels][c_out]
     int* errw;
@@ -115,25 +117,42 @@ struct WinTail {
 // units of 16 bytes; the high half is the same for all (row groups 128 bytes apart, no swizzle).
 __device__ __forceinline__ uint32_t wn_desc_lo(uint32_t addr, uint32_t k_slots) { return ((addr & 0x3ffffu) >> 4) | k_slots << 16; }
 constexpr uint32_t WN_DESC_HI = (128u >> 4) | 1u << 14;
-// One MMA (kind::i8 or kind::f16) of the lane with e != 0, in code the whole warp runs.  The descriptors come as 32-bit
-// halves of which only the low one changes from MMA to MMA.
-template <bool F16>
-__device__ __forceinline__ void wn_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate, uint32_t e)
+// The MMAs of one K step, issued by the lane with e != 0 in code the whole warp runs.  The descriptors come as 32-bit halves
+// of which only the low one changes.
+__device__ __forceinline__ void wn_step_i8(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate, uint32_t e)
 {
-    if (F16)
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
-            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
-    else
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
-            "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
-            "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
-            "@q tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
+        ::"r"(d), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
+}
+// fp32: six products of pieces in four MMAs.  A filter tile's pieces lie side by side along the columns, so an MMA of twice
+// the width adds one input piece times two filter pieces to the two accumulators of small products at d1:
+// a0 * (b1, b2), a1 * (b0, b1), a2 * b0; the leading a0 * b0 goes to d0.
+__device__ __forceinline__ void wn_step_f32(uint32_t d0, uint32_t d1, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t b0, uint32_t b1, uint32_t idesc,
+                                            uint32_t idesc2, uint32_t acc0, uint32_t acc1, uint32_t e)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, r, q, t;\n\t.reg .b64 x, y, z, u, v;\n\t"
+        "mov.b64 x, {%2, %7};\n\tmov.b64 y, {%3, %7};\n\tmov.b64 z, {%4, %7};\n\tmov.b64 u, {%5, %7};\n\tmov.b64 v, {%6, %7};\n\t"
+        "setp.ne.b32 p, %10, 0;\n\tsetp.ne.b32 r, %11, 0;\n\tsetp.ne.b32 q, %12, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], x, v, %9, r;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], y, u, %9, t;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], z, u, %8, t;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], x, u, %8, p;\n\t}"
+        ::"r"(d0), "r"(d1), "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(WN_DESC_HI), "r"(idesc), "r"(idesc2), "r"(acc0), "r"(acc1), "r"(e) : "memory");
+}
+// one look at a barrier
+__device__ __forceinline__ uint32_t mbar_poll(uint32_t bar, uint32_t parity)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"(bar), "r"(parity) : "memory");
+    return r;
 }
 __device__ __forceinline__ void wn_commit(uint32_t bar, uint32_t e)
 {
@@ -283,7 +302,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
 {
     constexpr int PIECES = DT == T_F32 ? 3 : 1;
     extern __shared__ unsigned char wn_smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (the same in all lanes, and known to the compiler to be)
     const int tile = blockIdx.x, ntile = blockIdx.y;
     const int frame = (!DENSE && p.frames > 1) ? blockIdx.z / p.ks : 0, split = blockIdx.z - frame * p.ks;
     // (the frame's data; the parameters themselves stay in constant memory)
@@ -396,27 +416,26 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     const int wg = warp >> 2, m_own = p.mt > 1 ? wg : 0;
     const int c_lo = p.mt > 1 ? 0 : wg * 64, c_hi = p.mt > 1 ? p.bn : min(p.bn, c_lo + 64);
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    float facc[DT == T_F32 ? 128 : 1];                       // fp32: the promoted sums of this thread's row
+    float facc[DT == T_F32 ? 64 : 1];                        // fp32 (one tile per CTA): the promoted sums of this thread's half row
 
     if (warp < 8) {
         // ================= windows
         if (DT == T_F32) {
             #pragma unroll
-            for (int j = 0; j < 128; ++j) facc[j] = 0.f;
+            for (int j = 0; j < 64; ++j) facc[j] = 0.f;
         }
         auto promote = [&](int ib) -> bool {                 // adds the leading accumulator of block ib to the registers and gives it back
             if (DT != T_F32) return true;
-            const int pb = p.mt > 1 ? 0 : (ib & 1);          // (two tiles: one leading accumulator each, else two in turn)
-            const int use = p.mt > 1 ? ib : ib >> 1;
-            bool got = mbar_wait(smem_u32(&S->dfull[pb]), use & 1, p.wait_limit);
+            const int pb = ib & 1;
+            bool got = mbar_wait(smem_u32(&S->dfull[pb]), (ib >> 1) & 1, p.wait_limit);
             got = __all_sync(0xffffffffu, got);
             if (!got) return false;
             tc_fence_after();
             #pragma unroll
-            for (int c0 = 0; c0 < 128; c0 += 32) {
+            for (int c0 = 0; c0 < 64; c0 += 32) {
                 if (c_lo + c0 < c_hi) {
                     uint32_t v[32];
-                    wn_ld32(tmem + lane_base + (uint32_t)((p.mt > 1 ? m_own : pb) * p.bn + c_lo + c0), v);
+                    wn_ld32(tmem + lane_base + (uint32_t)(pb * p.bn + c_lo + c0), v);
                     #pragma unroll
                     for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? c0 + j : 0] += __uint_as_float(v[j]);
                 }
@@ -568,18 +587,23 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     } else if (warp == 9) {
         if (lane == 0) load_stages(1 << 30);
     } else {
-        // ================= MMAs.  The whole warp walks and one elected lane issues: what the walk costs per stage is what
-        // the MMAs of a stage have to be longer than, and a lone thread's divergent walk is twice as long (a stage of four
-        // 128-column MMAs, 256 clocks of tensor work: 340 clocks, against 870 for a single thread with quotients in the loop)
+        // ================= MMAs.  The whole warp walks and one elected lane issues.  What the walk costs is what the MMAs of
+        // a stage have to be longer than: a step's MMAs are one block of instructions, and the next stage's barrier is polled
+        // before this stage's MMAs are issued.
         const uint32_t e = wn_elect();
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        auto wait = [&](unsigned long long* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, p.wait_limit)); };
         const uint32_t idesc = DT == T_F32 ? (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.bn >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24)
                                            : tc_instr_desc(p.bn);
+        const uint32_t idesc2 = (idesc & ~(0x3fu << 17)) | ((uint32_t)(2 * p.bn >> 3) << 17);     // twice the columns
         // (everything below in 16-byte units)
-        const uint32_t a_step = p.a_step, b_unit = unit_b >> 4, b_piece = 2u * (uint32_t)p.bn, bn = (uint32_t)p.bn;
-        const uint32_t stage_step = p.stage_bytes >> 4, b_lo0 = wn_desc_lo(bstage_u32, bn);
+        const uint32_t a_step = p.a_step, b_unit = unit_b >> 4, bn = (uint32_t)p.bn;
+        const uint32_t stage_step = p.stage_bytes >> 4, b_lo0 = wn_desc_lo(bstage_u32, PIECES * bn);
+        const uint32_t full0 = smem_u32(&S->bfull[0]), empty0 = smem_u32(&S->bempty[0]);
         int ib = 0, stage = 0, buf = 0;
         uint32_t phase = 0, a_phase = 0, b_stage = b_lo0;
         uint32_t first = 0;                                  // 0 until the CTA's first MMA has been issued
+        bool ready = false;                                  // the coming stage has been seen full
         for (int b = b0; b < b1 && ok; ++b, ++ib) {
             const int plane = b / p.nchb, chb = b - plane * p.nchb;
             const int gn = min(p.gblk, p.groups - chb * p.gblk);
@@ -587,67 +611,46 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const int t_lo = p.tsplit > 1 ? part * ntap / p.tsplit : 0, t_hi = p.tsplit > 1 ? (part + 1) * ntap / p.tsplit : ntap;
             const int jy = t_lo / nx;
             int j = t_lo - jy * nx;
-            if (!mbar_wait(smem_u32(&S->afull[buf]), a_phase, p.wait_limit)) { ok = false; break; }
-            // fp32: the leading product's accumulator has to be free (two tiles: from the block before, else from two before)
-            const int pb = p.mt > 1 ? 0 : (ib & 1), use = p.mt > 1 ? ib : ib >> 1;
+            if (!wait(&S->afull[buf], a_phase)) { ok = false; break; }
+            // fp32: two leading accumulators in turn; this one has to have been drained of the block before the last
+            if (DT == T_F32 && !wait(&S->dempty[ib & 1], ((ib >> 1) & 1) ^ 1)) { ok = false; break; }
             const uint32_t a_piece = (uint32_t)((XCOL && p.xarr ? p.xarr : gn * 2) * p.L);
-            uint32_t a_row = wn_desc_lo(base_u32 + buf * p.abytes, p.a_lbo) + (uint32_t)(p.plane[plane].shift0 - p.min_shift + jy * p.Wq), a_tap = a_row + (uint32_t)j;
-            const uint32_t d0 = tmem + (DT == T_F32 && p.mt == 1 ? (uint32_t)pb * bn : 0u), d1 = tmem + bn, dc = tmem + 2u * bn;   // (dc: fp32, the small products)
+            const uint32_t row_jump = (uint32_t)(p.Wq - nx + 1);
+            uint32_t a_tap = wn_desc_lo(base_u32 + buf * p.abytes, p.a_lbo) + (uint32_t)(p.plane[plane].shift0 - p.min_shift + jy * p.Wq + j);
+            const uint32_t d0 = tm + (DT == T_F32 ? (uint32_t)(ib & 1) * bn : 0u), d1 = tm + (DT == T_F32 ? 2u * bn : bn);   // (fp32: d1 the small products)
             uint32_t fresh = 0;                              // fp32: 0 until the block's first MMA
             for (int t0 = t_lo; t0 < t_hi; t0 += p.tps) {
-                if (!mbar_wait(smem_u32(&S->bfull[stage]), phase, p.wait_limit)) { ok = false; break; }
+                if (!ready && !__all_sync(0xffffffffu, mbar_wait(full0 + 8u * stage, phase, p.wait_limit))) { ok = false; break; }
                 tc_fence_after();
+                const uint32_t done_bar = empty0 + 8u * stage;
                 uint32_t b_lo = b_stage;
-                for (int tn = min(p.tps, t_hi - t0); tn > 0; --tn) {
-                    uint32_t a_lo = a_tap;
-                    if (DT == T_F32) {
-                        for (int g = gn; g > 0; --g) {
-                            const uint32_t a1 = a_lo + a_piece, a2 = a1 + a_piece, b1_ = b_lo + b_piece, b2 = b1_ + b_piece;
-                            // the small products first: they do not wait for the leading accumulator to be drained
-                            wn_mma<true>(dc, a_lo, b1_, idesc, first, e);
-                            wn_mma<true>(dc, a1, b_lo, idesc, 1u, e);
-                            wn_mma<true>(dc, a_lo, b2, idesc, 1u, e);
-                            wn_mma<true>(dc, a1, b1_, idesc, 1u, e);
-                            wn_mma<true>(dc, a2, b_lo, idesc, 1u, e);
-                            if (p.mt > 1) {
-                                const uint32_t e0 = a_lo + TC_M, e1 = a1 + TC_M, e2 = a2 + TC_M, dd = dc + bn;
-                                wn_mma<true>(dd, e0, b1_, idesc, first, e);
-                                wn_mma<true>(dd, e1, b_lo, idesc, 1u, e);
-                                wn_mma<true>(dd, e0, b2, idesc, 1u, e);
-                                wn_mma<true>(dd, e1, b1_, idesc, 1u, e);
-                                wn_mma<true>(dd, e2, b_lo, idesc, 1u, e);
-                            }
-                            if (fresh == 0) {
-                                if (!mbar_wait(smem_u32(&S->dempty[pb]), (use & 1) ^ 1, p.wait_limit)) ok = false;
-                                tc_fence_after();
-                            }
-                            wn_mma<true>(d0, a_lo, b_lo, idesc, fresh, e);
-                            if (p.mt > 1) wn_mma<true>(d1, a_lo + TC_M, b_lo, idesc, fresh, e);
-                            fresh = first = 1;
-                            a_lo += a_step;
-                            b_lo += b_unit;
-                        }
-                    } else {
-                        #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            if (g >= gn) break;
-                            wn_mma<false>(d0, a_lo, b_lo, idesc, g == 0 ? first : 1u, e);
-                            if (p.mt > 1) wn_mma<false>(d1, a_lo + TC_M, b_lo, idesc, g == 0 ? first : 1u, e);
-                            a_lo += a_step;
-                            b_lo += b_unit;
-                        }
-                        first = 1;
-                    }
-                    if (++j == nx) { j = 0; a_row += (uint32_t)p.Wq; a_tap = a_row; } else ++a_tap;
-                }
-                wn_commit(smem_u32(&S->bempty[stage]), e);
                 b_stage += stage_step;
                 if (++stage == p.stages) { stage = 0; phase ^= 1; b_stage = b_lo0; }
-                if (DT == T_F32 && !ok) break;
+                const uint32_t poll = DT == T_F32 ? mbar_poll(full0 + 8u * stage, phase) : 0u;
+                for (int tn = min(p.tps, t_hi - t0); tn > 0; --tn) {
+                    uint32_t a_lo = a_tap;
+                    #pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g >= gn) break;
+                        if (DT == T_F32) wn_step_f32(d0, d1, a_lo, a_lo + a_piece, a_lo + 2 * a_piece, b_lo, b_lo + bn, idesc, idesc2, fresh, first, e);
+                        else {
+                            wn_step_i8(d0, a_lo, b_lo, idesc, g == 0 ? first : 1u, e);
+                            if (p.mt > 1) wn_step_i8(d1, a_lo + TC_M, b_lo, idesc, g == 0 ? first : 1u, e);
+                        }
+                        fresh = 1;
+                        if (DT == T_F32) first = 1;
+                        a_lo += a_step;
+                        b_lo += b_unit;
+                    }
+                    first = 1;
+                    if (++j == nx) { j = 0; a_tap += row_jump; } else ++a_tap;
+                }
+                wn_commit(done_bar, e);
+                ready = DT == T_F32 && __all_sync(0xffffffffu, poll != 0);
             }
             if (!ok) break;
             wn_commit(smem_u32(&S->aempty[buf]), e);
-            if (DT == T_F32) wn_commit(smem_u32(&S->dfull[pb]), e);
+            if (DT == T_F32) wn_commit(smem_u32(&S->dfull[ib & 1]), e);
             if (++buf == p.abuf) { buf = 0; a_phase ^= 1; }
         }
         if (ok) wn_commit(smem_u32(&S->done), e);
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         }
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the row buffers may be released
     }
-    #pragma unroll (DT == T_F32 ? 2 : 1)
+    #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
         if (direct || (pass > 0 && !halves)) break;
         const int p0 = pass * 64;                            // first column of the pass (own columns: c_lo + c0)
@@ -756,11 +759,16 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const int r = m_own * TC_M + (warp & 3) * 32 + lane;
             uint32_t* row = staged + (size_t)r * ldr;
             if (pass > 0) { if (bulk_add) __syncwarp(); else wn_meet(); }    // the first pass's rows have left
-            #pragma unroll (DT == T_F32 ? 4 : 1)
-            for (int c0 = 0; c0 < 128; c0 += 32) {
+            #pragma unroll (DT == T_F32 ? 2 : 1)
+            for (int c0 = 0; c0 < (DT == T_F32 ? 64 : 128); c0 += 32) {
                 if (c_lo + c0 < c_hi && (!halves || (c0 >> 6) == pass)) {
                     uint32_t v[32];
-                    wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 + m_own : m_own) * p.bn + c_lo + c0), v);
+                    if (DT == T_F32) {                       // (the second accumulator of small products)
+                        wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + c_lo + c0), v);
+                        #pragma unroll
+                        for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? c0 + j : 0] += __uint_as_float(v[j]);
+                    }
+                    wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + c_lo + c0), v);
                     #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
                         if (c_lo + c0 + j >= c_hi) break;
@@ -970,7 +978,7 @@ int launch_pool_window(const Layer& L, const Tensor& out, const void* A, void* X
 }
 
 // ------------------------------------------------------------------------------------------------
-// Filters as operand tiles: [n tile][tap][group][pieces][2 chunks][bn][16 bytes].  One thread per 16 bytes.
+// Filters as operand tiles: [n tile][tap][group][2 chunks][pieces][bn][16 bytes].  One thread per 16 bytes.
 // K within a tap: channels (int8 and binary: bytes; fp32: bf16 pieces); first layers: tap = filter row, K = kx * 4 + channel.
 // ------------------------------------------------------------------------------------------------
 template <int DT, bool XCOL>
@@ -984,7 +992,7 @@ __global__ void pack_weights_win_kernel(const void* W, unsigned char* img, int c
     const int tap = (int)(idx / ((size_t)2 * bn * groups) % taps), nt = (int)(idx / ((size_t)2 * bn * groups * taps));
     const int co = nt * bn + r;
     constexpr int E = DT == T_F32 ? 8 : 16, PIECES = DT == T_F32 ? 3 : 1;
-    unsigned char* dst = img + ((((size_t)nt * taps + tap) * groups + g) * PIECES * 2 + c) * bn * 16 + (size_t)r * 16;
+    unsigned char* dst = img + ((((size_t)nt * taps + tap) * groups + g) * 2 + c) * PIECES * bn * 16 + (size_t)r * 16;
     auto at = [&](int e) -> size_t {                          // element e of this chunk, as an index into W ((size_t)-1: none)
         const int k = (g * 2 + c) * E + e;
         int ci, ky, kx;
@@ -1000,7 +1008,7 @@ __global__ void pack_weights_win_kernel(const void* W, unsigned char* img, int c
             wn_split(a == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[a], b == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[b],
                      s[0][j], s[1][j], s[2][j]);
         }
-        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + (size_t)k * 2 * bn * 16) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
+        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + (size_t)k * bn * 16) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
     } else {
         uint32_t v[4] = {0, 0, 0, 0};
         #pragma unroll
@@ -1041,6 +1049,7 @@ static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
     };
     const int e = d.dtype == RRM_F32 ? 16 : 32;              // K elements of a group
     p.groups = xcol ? ceil_div(d.kw * 4, e) : ceil_div(d.dtype == RRM_I8 ? in.cs : d.c_in, e);
+    if (xcol && p.groups > 4) return false;                  // (a block holds up to four K groups, a first layer's block all of them)
     // first layers: pixels of a 16-byte chunk; a row in one or two arrays where the stride is as many chunks
     const int px = d.dtype == RRM_F32 ? 2 : 4;
     p.xarr = xcol && d.stride % px == 0 && d.stride / px <= 2 ? d.stride / px : 0;
@@ -1098,7 +1107,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     const size_t room = f32 ? WN_SMEM_LIMIT - 1024 : WN_SMEM_LIMIT / 2 - 2048;   // (integer kernels: two CTAs per SM)
     // two accumulator tiles per CTA share every filter stage (what bounds a full machine is the filters' way from L2),
     // once that leaves a CTA per SM
-    int mt = tiles >= 2ll * 148 && rows > TC_M ? 2 : 1;
+    int mt = !f32 && tiles >= 2ll * 148 && rows > TC_M ? 2 : 1;
     // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
     // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
     const bool clustered = dense || store || f32 || (p.c_out & 3) != 0;
@@ -1139,7 +1148,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
                 const size_t used = (size_t)p.abuf * p.abytes + (size_t)p.stages * p.stage_bytes;
                 p.tail_off = (unsigned)((used > staging ? used : staging) + 15) & ~15u;      // (the drained rows go where windows and stages were)
                 if (p.tail_off + tail > room) continue;
-                const unsigned cols = f32 ? (mt > 1 ? 3 : 2) * p.bn + round_up(p.bn, 32) : (mt - 1) * p.bn + round_up(p.bn, 32);
+                const unsigned cols = f32 ? 3 * p.bn + round_up(p.bn, 32) : (mt - 1) * p.bn + round_up(p.bn, 32);
                 p.tmem_cols = 32;
                 while (p.tmem_cols < cols) p.tmem_cols *= 2;
                 p.eager = dense || tiles * p.ks <= 2 * 148;
