@@ -1073,7 +1073,6 @@ int rrm_net_destroy(rrm_net* net)
     if (!net) return RRM_ERR_INVALID_ARG;
     cudaDeviceSynchronize();
     for (auto& L : net->layers) {
-        if (L.seq_ev) cudaEventDestroy(L.seq_ev);
         if (L.seq_stat_host) cudaFreeHost(L.seq_stat_host);
     }
     drop_graphs(net);

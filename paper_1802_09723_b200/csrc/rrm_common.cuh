@@ -76,6 +76,24 @@ inline cudaError_t launch_seq(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return launch_seq_cluster(kernel, grid, block, smem, st, 1, static_cast<A&&>(args)...);
 }
 
+// A launch outside graphs that may start while its predecessor on the stream drains (the FC entry points are one launch
+// per call, and their launch latency, set-up and first weight copies are a third of a call).  The kernel calls pdl_wait
+// before it touches anything but its own constants, and reads what a predecessor may have written past the L1 cache.
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_y, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1; at[1].val.clusterDim.y = (unsigned)cluster_y; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // storage type of a tensor inside the library (always pixel-major: [n][h][w][cs])
 enum { T_F32 = 0, T_I8 = 1, T_BIN = 2, T_I32 = 3 };
 
@@ -215,11 +233,11 @@ struct Layer {
     int seq_last_T = 0;                     // frames of the most recent chunk (0: last call was a single-frame step)
     // measured density of the previous chunk, read back without stalling the stream: chooses between the
     // column gather and the dense tensor-core evaluation of the next chunk
-    unsigned* seq_stat_host = nullptr;      // pinned copy of seq_stat
-    int seq_stat_host_cap = 0;              // frames it holds
-    cudaEvent_t seq_ev = nullptr;           // the copy into seq_stat_host has landed
-    bool seq_ev_pending = false;
-    int seq_pending_rows = 0;               // frame x stream rows of the pending copy
+    unsigned long long* seq_stat_host = nullptr;   // pinned, one word per frame x stream row: chunk number << 32 | non-zeros,
+                                                   // written by the kernels
+    int seq_stat_host_cap = 0;              // rows it holds
+    unsigned seq_epoch = 0;                 // number of the last chunk whose counters were asked for
+    int seq_pending_rows = 0;               // rows of that chunk, while they have not all been seen; 0: none asked for
     double seq_density = -1.0;              // non-zero fraction of the last chunk whose counters were read; < 0: unknown
     int seq_last_variant = RRM_VARIANT_GATHER;
 };
@@ -353,7 +371,8 @@ int fc_dense_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int 
 int fc_tc_create(rrm_net* net, Layer& L);
 bool fc_tc_usable(const Layer& L, int rows);
 int fc_tc_launches(int rows);
-int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, bool stateless, unsigned* stat, cudaStream_t st);
+int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, bool stateless, unsigned* stat, cudaStream_t st,
+              unsigned long long* host = nullptr);
 
 // ---- rrm_conv_tc.cu
 bool conv_tc_eligible(const rrm_net* net, const Layer& L);

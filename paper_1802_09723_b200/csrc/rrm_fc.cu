@@ -69,9 +69,11 @@ __global__ void __cluster_dims__(FC_CL, 1, 1) __launch_bounds__(FC_THREADS) fc_d
     const int width = min(FC_OW, K - slice * FC_OW);
 
     cluster_arrive_relaxed();                        // waited for just before the first remote store
+    pdl_launch_dependents();
+    pdl_wait();
     // stored projection of this slice: fetched now, needed at the very end
     int p_old = 0;
-    if (kg == 0 && tid < width) p_old = Ps[tid];
+    if (kg == 0 && tid < width) p_old = __ldcg(Ps + tid);
 
     // ---- 1. non-zero delta bytes per 16-byte chunk; each thread owns FC_PT consecutive chunks
     const int c_begin = tid * FC_PT;
@@ -81,8 +83,8 @@ __global__ void __cluster_dims__(FC_CL, 1, 1) __launch_bounds__(FC_THREADS) fc_d
         xa[i] = make_uint4(0, 0, 0, 0);
         xb[i] = xa[i];
         if (c_begin + i < nchunks) {
-            xa[i] = __ldg(xt4 + c_begin + i);
-            if (xp4) xb[i] = __ldg(xp4 + c_begin + i);
+            xa[i] = __ldcg(xt4 + c_begin + i);
+            if (xp4) xb[i] = __ldcg(xp4 + c_begin + i);
         }
     }
     // raw bytes to shared memory (the gather looks the delta of an entry up there) and a 64-bit mask
@@ -249,11 +251,13 @@ __global__ void __launch_bounds__(FC_THREADS) fc_scan_kernel(FcParams p, void* s
     const uint4* xp4 = p.xprev ? reinterpret_cast<const uint4*>(p.xprev + (size_t)s * C) : nullptr;
     const int c_begin = tid * FC_PT;
     unsigned long long m = 0;
+    pdl_launch_dependents();
+    pdl_wait();
     #pragma unroll
     for (int i = 0; i < FC_PT; ++i) {
         if (c_begin + i < nchunks) {
-            const uint4 a = __ldg(xt4 + c_begin + i);
-            const uint4 b = xp4 ? xp4[c_begin + i] : make_uint4(0, 0, 0, 0);
+            const uint4 a = __ldcg(xt4 + c_begin + i);
+            const uint4 b = xp4 ? __ldcg(xp4 + c_begin + i) : make_uint4(0, 0, 0, 0);
             reinterpret_cast<uint4*>(s_xt)[c_begin + i] = a;
             reinterpret_cast<uint4*>(s_xp)[c_begin + i] = b;
             // the thread that read a chunk of the snapshot is the one that overwrites it: in place is safe
@@ -319,12 +323,14 @@ __global__ void __launch_bounds__(FC_THREADS) fc_gather_kernel(FcParams p, const
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slice = blockIdx.x, s = blockIdx.y;
     const int C = p.c_in, K = p.c_out;
-    const int total = reinterpret_cast<const int*>(scratch)[s];
+    pdl_launch_dependents();
+    pdl_wait();
+    const int total = __ldcg(reinterpret_cast<const int*>(scratch) + s);
     const uint32_t* entries = fc_scratch_entries(const_cast<void*>(scratch), n) + (size_t)s * C;
     int32_t* Ps = p.P + (size_t)s * K + slice * FC_OW;
     const int width = min(FC_OW, K - slice * FC_OW);
     int p_old = 0;
-    if (tid < width) p_old = Ps[tid];
+    if (tid < width) p_old = __ldcg(Ps + tid);
     const int sub = tid & 7, grp = tid >> 3;
     const int o0 = slice * FC_OW + sub * 16;
     int acc[16];
@@ -339,7 +345,7 @@ __global__ void __launch_bounds__(FC_THREADS) fc_gather_kernel(FcParams p, const
             #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int eu = e + u * FC_GROUPS;
-                ent[u] = eu < total ? __ldg(entries + eu) : 0xffffffffu;
+                ent[u] = eu < total ? __ldcg(entries + eu) : 0xffffffffu;
             }
             #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -469,10 +475,10 @@ int fc_fused_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, bool de
     }
     if (n < FC_TWO_KERNEL_MIN_STREAMS) {
         dim3 grid(FC_CL, slices, n);
-        fc_delta_i8_kernel<<<grid, FC_THREADS, 0, st>>>(p);
+        RRM_CUDA_TRY(launch_overlapped(fc_delta_i8_kernel, grid, dim3(FC_THREADS), 0, st, 1, p));
     } else {
-        fc_scan_kernel<<<n, FC_THREADS, 0, st>>>(p, L.fc_scratch, n);
-        fc_gather_kernel<<<dim3(slices, n), FC_THREADS, 0, st>>>(p, L.fc_scratch, n);
+        RRM_CUDA_TRY(launch_overlapped(fc_scan_kernel, dim3(n), dim3(FC_THREADS), 0, st, 1, p, L.fc_scratch, n));
+        RRM_CUDA_TRY(launch_overlapped(fc_gather_kernel, dim3(slices, n), dim3(FC_THREADS), 0, st, 1, p, L.fc_scratch, n));
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
@@ -544,8 +550,8 @@ extern "C" int rrm_fc_step_noalloc(const int8_t* Wt_dev, const int8_t* Xt_dev, i
     p.Wt = Wt_dev; p.P = P_dev; p.Y = Y_dev; p.stat = nullptr;
     p.c_in = c_in; p.c_out = c_out; p.shift = shift; p.act = act;
     cudaStream_t st = (cudaStream_t)stream;
-    fc_scan_kernel<<<n, FC_THREADS, 0, st>>>(p, scratch, n);
-    fc_gather_kernel<<<dim3(ceil_div(c_out, FC_OW), n), FC_THREADS, 0, st>>>(p, scratch, n);
+    RRM_CUDA_TRY(launch_overlapped(fc_scan_kernel, dim3(n), dim3(FC_THREADS), 0, st, 1, p, scratch, n));
+    RRM_CUDA_TRY(launch_overlapped(fc_gather_kernel, dim3(ceil_div(c_out, FC_OW), n), dim3(FC_THREADS), 0, st, 1, p, scratch, n));
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
 }

@@ -42,6 +42,8 @@ struct FcSeqParams {
     void* Y;                 // [T][n][c_out] int32 (shift < 0) or int8, or nullptr
     unsigned* counters;      // [n][slices], zero on entry, zero again on exit
     unsigned* stat;          // [T*n][2]: non-zero entries / active groups of 32 inputs per frame, or nullptr
+    unsigned long long* host;       // pinned host words, one per row: epoch << 32 | non-zero entries; or nullptr
+    unsigned epoch;
     int T, n, c_in, c_out, shift, act;
     const uint32_t* Wsp;     // weight-sparse form: [c_in][slices] records of sp_stride words (map, then packed groups)
     int sp_stride;
@@ -80,6 +82,16 @@ __global__ void __launch_bounds__(SQ_THREADS, DEEP ? 2 : 3) fc_seq_kernel(FcSeqP
     const int width = min(OW, K - slice * OW);
 
     if (tid == 0) { s_count = 0; s_groups = 0; }
+    pdl_launch_dependents();
+    // before anything of the predecessors': touch one line in every 2 MiB of the weights, so that the address translations
+    // the gather will need are fetched now instead of on its first loads
+    {
+        const size_t wbytes = SW ? (size_t)C * slices * p.sp_stride * 4 : (size_t)C * K;
+        const size_t off = (size_t)tid << 21;
+        const char* wptr = SW ? reinterpret_cast<const char*>(p.Wsp) : reinterpret_cast<const char*>(p.Wt);
+        if (off < wbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(wptr + off));
+    }
+    pdl_wait();
     // ---- 1. scan: chunk i*256 + tid for i < SQ_PT, all loads first
     const uint4* xt4 = reinterpret_cast<const uint4*>(p.x + ((size_t)t * p.n + s) * C);
     const uint4* xp4 = nullptr;
@@ -91,18 +103,12 @@ __global__ void __launch_bounds__(SQ_THREADS, DEEP ? 2 : 3) fc_seq_kernel(FcSeqP
         a[i] = make_uint4(0, 0, 0, 0);
         b[i] = a[i];
         if (chunk < nchunks) {
-            a[i] = __ldg(xt4 + chunk);
-            if (xp4) b[i] = __ldg(xp4 + chunk);
+            a[i] = __ldcg(xt4 + chunk);
+            if (xp4) b[i] = __ldcg(xp4 + chunk);
         }
     }
-    // while the frame is on its way: touch one line in every 2 MiB of the weights, so that the
-    // address translations the gather will need are fetched now instead of on its first loads
+    // while the frame is on its way: likewise the stored projection (or the bias), which only the closing sum reads
     {
-        const size_t wbytes = SW ? (size_t)C * slices * p.sp_stride * 4 : (size_t)C * K;
-        const size_t off = (size_t)tid << 21;
-        const char* wptr = SW ? reinterpret_cast<const char*>(p.Wsp) : reinterpret_cast<const char*>(p.Wt);
-        if (off < wbytes) asm volatile("prefetch.global.L2 [%0];" ::"l"(wptr + off));
-        // likewise the stored projection (or the bias), which only the closing sum reads
         const int32_t* pp = p.bias ? p.bias + slice * OW : p.P + (size_t)s * K + slice * OW;
         if (t == 0 && tid * 32 < width) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp + tid * 32));
     }
@@ -161,6 +167,7 @@ __global__ void __launch_bounds__(SQ_THREADS, DEEP ? 2 : 3) fc_seq_kernel(FcSeqP
     if (p.stat && slice == 0 && tid == 0) {
         p.stat[blockIdx.y * 2 + 0] = (unsigned)total;
         p.stat[blockIdx.y * 2 + 1] = (unsigned)s_groups;
+        if (p.host) *(volatile unsigned long long*)(p.host + blockIdx.y) = (unsigned long long)p.epoch << 32 | (unsigned)total;
     }
 
     // ---- 2. gather: LANES lanes x 16 bytes span the slice; SQ_U rounds of CPR columns in flight
@@ -329,7 +336,7 @@ __global__ void __launch_bounds__(SQ_THREADS, DEEP ? 2 : 3) fc_seq_kernel(FcSeqP
     if (p.bias) {
         v = *reinterpret_cast<const int4*>(p.bias + o);
     } else {
-        v = *reinterpret_cast<const int4*>(p.P + (size_t)s * K + o);
+        v = __ldcg(reinterpret_cast<const int4*>(p.P + (size_t)s * K + o));
         for (int f = 0; f < fs; ++f) {
             const int4 q = s_share[f * OG + og];
             v.x += q.x; v.y += q.y; v.z += q.z; v.w += q.w;
@@ -362,7 +369,7 @@ __global__ void __launch_bounds__(SQ_THREADS, DEEP ? 2 : 3) fc_seq_kernel(FcSeqP
 // Non-zero delta entries and active groups of 32 inputs of every (frame, stream) of a chunk: the
 // delta + scan step alone, for chunks that are then evaluated densely.
 __global__ void __launch_bounds__(SQ_THREADS) fc_count_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ xprev,
-                                                            unsigned* stat, int n, int C)
+                                                            unsigned* stat, int n, int C, unsigned long long* host, unsigned epoch)
 {
     __shared__ int s_nnz, s_grp;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -387,7 +394,10 @@ __global__ void __launch_bounds__(SQ_THREADS) fc_count_kernel(const int8_t* __re
     for (int o = 16; o > 0; o >>= 1) { nnz += __shfl_down_sync(0xffffffffu, nnz, o); grp += __shfl_down_sync(0xffffffffu, grp, o); }
     if (lane == 0) { atomicAdd(&s_nnz, nnz); atomicAdd(&s_grp, grp); }
     __syncthreads();
-    if (tid == 0) { stat[blockIdx.x * 2] = (unsigned)s_nnz; stat[blockIdx.x * 2 + 1] = (unsigned)s_grp; }
+    if (tid == 0) {
+        stat[blockIdx.x * 2] = (unsigned)s_nnz; stat[blockIdx.x * 2 + 1] = (unsigned)s_grp;
+        if (host) *(volatile unsigned long long*)(host + blockIdx.x) = (unsigned long long)epoch << 32 | (unsigned)s_nnz;
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -398,22 +408,35 @@ __global__ void __launch_bounds__(SQ_THREADS) fc_count_kernel(const int8_t* __re
 // and, for chunks of few rows (one launch that reads W once), rrm_options.fc_dense_rows (rows x non-zero fraction;
 // measured break-even on fc6, 32 rows: 2.2 % non-zeros).
 
-// Copies the chunk's counters to pinned host memory behind the work already on the stream.
-static int seq_read_back(Layer& L, int rows, cudaStream_t st)
+// The words in pinned memory that a chunk's kernels write its counters to, stamped with the chunk's number (a copy behind
+// the kernel and its event would keep the next chunk's launch from overlapping this one); nullptr while an older chunk's
+// are still awaited.
+static unsigned long long* seq_ask_counters(Layer& L, int rows)
 {
-    if (L.seq_ev_pending) return RRM_OK;                     // an older copy is still in flight: keep it
+    if (L.seq_pending_rows > 0) return nullptr;
     if (rows > L.seq_stat_host_cap) {
         if (L.seq_stat_host) cudaFreeHost(L.seq_stat_host);
         L.seq_stat_host = nullptr; L.seq_stat_host_cap = 0;
-        if (cudaMallocHost(reinterpret_cast<void**>(&L.seq_stat_host), (size_t)rows * 2 * 4) != cudaSuccess) { cudaGetLastError(); return RRM_OK; }
+        if (cudaMallocHost(reinterpret_cast<void**>(&L.seq_stat_host), (size_t)rows * 8) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+        for (int i = 0; i < rows; ++i) L.seq_stat_host[i] = 0;
         L.seq_stat_host_cap = rows;
     }
-    if (!L.seq_ev && cudaEventCreateWithFlags(&L.seq_ev, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); return RRM_OK; }
-    RRM_CUDA_TRY(cudaMemcpyAsync(L.seq_stat_host, L.seq_stat, (size_t)rows * 2 * 4, cudaMemcpyDeviceToHost, st));
-    RRM_CUDA_TRY(cudaEventRecord(L.seq_ev, st));
-    L.seq_ev_pending = true;
+    if (++L.seq_epoch == 0) L.seq_epoch = 1;
     L.seq_pending_rows = rows;
-    return RRM_OK;
+    return L.seq_stat_host;
+}
+
+// Takes the awaited chunk's density in once all its rows have arrived; never waits.
+static void seq_poll_counters(Layer& L)
+{
+    unsigned long long nz = 0;
+    for (int i = 0; i < L.seq_pending_rows; ++i) {
+        const unsigned long long v = *(volatile unsigned long long*)(L.seq_stat_host + i);
+        if ((unsigned)(v >> 32) != L.seq_epoch) return;
+        nz += (unsigned)v;
+    }
+    if (L.seq_pending_rows > 0) L.seq_density = (double)nz / ((double)L.seq_pending_rows * L.d.c_in);
+    L.seq_pending_rows = 0;
 }
 
 int fc_dense_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bool stateless, cudaStream_t st);
@@ -493,6 +516,7 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
     p.counters = L.seq_counters;
     p.T = T; p.n = n; p.c_in = C; p.c_out = K; p.shift = L.d.shift; p.act = L.d.act;
     p.Wsp = L.Wsp; p.sp_stride = L.sp_stride;
+    p.host = nullptr; p.epoch = 0;
     if (dense) {
         p.xprev = nullptr;
         p.bias = reinterpret_cast<const int32_t*>(L.bias);
@@ -501,15 +525,9 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
         else { p.xnext = L.xs[L.xs_cur ^ 1]; L.xs_cur ^= 1; p.P = reinterpret_cast<int32_t*>(L.P); }
     } else {
         // ---- which evaluation: the previous chunk's measured density decides (temporal coherence is the
-        // method's premise).  Its counters were copied to pinned memory behind the chunk; they are used
-        // once that copy has landed, and never waited for.
-        if (L.seq_ev_pending && cudaEventQuery(L.seq_ev) == cudaSuccess) {
-            unsigned long long nz = 0;
-            for (int i = 0; i < L.seq_pending_rows; ++i) nz += L.seq_stat_host[2 * i];
-            L.seq_density = (double)nz / ((double)L.seq_pending_rows * C);
-            L.seq_ev_pending = false;
-        }
-        cudaGetLastError();                                  // cudaErrorNotReady from the query is not an error
+        // method's premise).  Its kernels write the counters to pinned memory; they are used once all have arrived, and
+        // never waited for.
+        seq_poll_counters(L);
         // (up to 1024 rows go through the streaming form, 256 rows per launch, each launch at the cost of reading W
         // once: it wins as soon as the rows' gathered columns add up to about that many bytes)
         const bool use_dense = L.tc_ready && L.d.variant == RRM_VARIANT_AUTO && (long long)T * n >= 8 &&
@@ -517,16 +535,18 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
                                                        : L.seq_density >= (double)net->opt.fc_dense_density);
         L.seq_last_T = T;
         L.seq_last_variant = use_dense ? RRM_VARIANT_DENSE : (L.Wsp ? RRM_VARIANT_SPARSE_W : RRM_VARIANT_GATHER);
+        unsigned long long* const host = seq_ask_counters(L, T * n);
+        p.host = host; p.epoch = L.seq_epoch;
         if (use_dense) {
             // the results are the same integers: P_t = b + W X_t for every frame, state := last frame
             if (fc_tc_usable(L, T * n)) {
                 // few rows: one launch streams W once, and its idle warps count the delta entries meanwhile
-                RRM_TRY(fc_tc_run(net, L, X_dev, Y_dev, T * n, false, L.seq_stat, st));
+                RRM_TRY(fc_tc_run(net, L, X_dev, Y_dev, T * n, false, L.seq_stat, st, host));
             } else {
-                fc_count_kernel<<<T * n, SQ_THREADS, 0, st>>>(reinterpret_cast<const int8_t*>(X_dev), L.xs[L.xs_cur], L.seq_stat, n, C);
+                fc_count_kernel<<<T * n, SQ_THREADS, 0, st>>>(reinterpret_cast<const int8_t*>(X_dev), L.xs[L.xs_cur], L.seq_stat, n, C, host, L.seq_epoch);
                 RRM_TRY(fc_dense_tc_run(net, L, X_dev, Y_dev, T, false, st));
             }
-            return seq_read_back(L, T * n, st);
+            return RRM_OK;
         }
         p.xprev = L.xs[L.xs_cur];
         p.xnext = L.xs[L.xs_cur ^ 1];
@@ -546,6 +566,7 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
     // taking the frame before it (still in X) as its "previous" frame
     const int piece_max = SQ_TAIL * (SQ_THREADS / (4 * lanes));
     const int8_t* snapshot = p.xprev;
+    unsigned long long* const host0 = dense ? nullptr : p.host;
     int8_t* const xnext = p.xnext;
     const size_t ybytes = (size_t)n * K * (L.d.shift < 0 ? 4 : 1);
     for (int t0 = 0; t0 < T; t0 += piece_max) {
@@ -555,18 +576,17 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
         p.xnext = t0 + piece == T ? xnext : nullptr;
         p.Y = Y_dev ? reinterpret_cast<char*>(Y_dev) + (size_t)t0 * ybytes : nullptr;
         p.stat = dense ? nullptr : L.seq_stat + (size_t)t0 * n * 2;
+        p.host = dense || !host0 ? nullptr : host0 + (size_t)t0 * n;
         p.T = piece;
         dim3 grid(ceil_div(K, 16 * lanes), piece * n);
         const size_t dyn = seq_dyn_smem(C, lanes, L.Wsp ? L.sp_stride : 0);
-        if (L.Wsp && grid.x * grid.y <= 2 * 148) fc_seq_kernel<32, true, true><<<grid, SQ_THREADS, dyn, st>>>(p);
-        else if (L.Wsp) fc_seq_kernel<32, false, true><<<grid, SQ_THREADS, dyn, st>>>(p);
-        else if (lanes == 32 && grid.x * grid.y <= 2 * 148) fc_seq_kernel<32, true, false><<<grid, SQ_THREADS, dyn, st>>>(p);
-        else if (lanes == 32) fc_seq_kernel<32, false, false><<<grid, SQ_THREADS, dyn, st>>>(p);
-        else if (lanes == 16) fc_seq_kernel<16, false, false><<<grid, SQ_THREADS, dyn, st>>>(p);
-        else fc_seq_kernel<8, false, false><<<grid, SQ_THREADS, dyn, st>>>(p);
+        auto go = [&](auto kernel) { return launch_overlapped(kernel, grid, dim3(SQ_THREADS), dyn, st, 1, p); };
+        const bool deep = grid.x * grid.y <= 2 * 148;
+        RRM_CUDA_TRY(L.Wsp ? (deep ? go(fc_seq_kernel<32, true, true>) : go(fc_seq_kernel<32, false, true>))
+                     : lanes == 32 ? (deep ? go(fc_seq_kernel<32, true, false>) : go(fc_seq_kernel<32, false, false>))
+                     : lanes == 16 ? go(fc_seq_kernel<16, false, false>) : go(fc_seq_kernel<8, false, false>));
     }
     RRM_CUDA_TRY(cudaGetLastError());
-    if (!dense) RRM_TRY(seq_read_back(L, T * n, st));
     return RRM_OK;
 }
 

@@ -46,6 +46,8 @@ struct FtParams {
     int32_t* Pstate;          // receives the rows from state_from on; may be null
     int8_t* snap;             // receives X of the rows from state_from on; may be null
     unsigned* stat;           // [rows][2]: non-zero delta entries and active groups of 32 inputs per row; may be null
+    unsigned long long* host; // pinned host words, one per row: epoch << 32 | non-zero entries; may be null
+    unsigned epoch;
     const int8_t* xprev;      // the n rows before this launch's first row (the delta of row r is against row r - n)
     int n;                    // streams
     int* errw;
@@ -96,6 +98,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
     const uint32_t stage_bytes = FT_A_BYTES + b_bytes;
     FtSmemTail* S = reinterpret_cast<FtSmemTail*>(base + (size_t)p.stages * stage_bytes);
 
+    pdl_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&S->full[s]), 1);            // the loader's expect_tx
@@ -117,6 +120,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
     bool ok = true;
     int n_loaded = 0;                                        // loader: stages issued
 
+    if (warp != 5) pdl_wait();                               // rows, snapshot and state are the predecessors'; the loader starts on W
     if (warp < 4) {
         // ================= the CTAs of the first output block refresh the input snapshot (their K share of the state rows)
         if (p.snap && mtile == 0) {
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
             for (int i = tid; i < (p.rows - p.state_from) * w16; i += 128) {
                 const int r = i / w16, k = k_lo + (i - r * w16) * 16;
                 *reinterpret_cast<int4*>(p.snap + (size_t)r * p.c_in + k) =
-                    *reinterpret_cast<const int4*>(p.X + (size_t)(p.state_from + r) * p.c_in + k);
+                    __ldcg(reinterpret_cast<const int4*>(p.X + (size_t)(p.state_from + r) * p.c_in + k));
             }
         }
         // ================= while W streams: the delta scan's counters (Alg. 1: dI = I_t - I_{t-1}), one row per CTA and turn
@@ -141,7 +145,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
                     const int chunk = b0 + tid;
                     unsigned m = 0;
                     if (chunk < c16) {
-                        const uint4 a = __ldg(xt4 + chunk), b = __ldg(xp4 + chunk);
+                        const uint4 a = __ldcg(xt4 + chunk), b = __ldcg(xp4 + chunk);
                         m = differing_bytes(a, b);
                     }
                     nnz += __popc(m);
@@ -152,7 +156,10 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
                 for (int o = 16; o > 0; o >>= 1) { nnz += __shfl_down_sync(0xffffffffu, nnz, o); grp += __shfl_down_sync(0xffffffffu, grp, o); }
                 if (lane == 0) { atomicAdd(&S->cnt_nnz, nnz); atomicAdd(&S->cnt_grp, grp); }
                 asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (tid == 0) { p.stat[row * 2] = (unsigned)S->cnt_nnz; p.stat[row * 2 + 1] = (unsigned)S->cnt_grp; }
+                if (tid == 0) {
+                    p.stat[row * 2] = (unsigned)S->cnt_nnz; p.stat[row * 2 + 1] = (unsigned)S->cnt_grp;
+                    if (p.host) *(volatile unsigned long long*)(p.host + row) = (unsigned long long)p.epoch << 32 | (unsigned)S->cnt_nnz;
+                }
                 asm volatile("bar.sync 1, 128;" ::: "memory");
             }
         }
@@ -160,18 +167,30 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
         // ================= loader: per slab one 16 KB bulk copy of W and one tensor copy of the input rows
         if (lane == 0) {
             const int8_t* src = p.Wimg + ((size_t)mtile * p.slabs + s_begin) * FT_A_BYTES;
-            for (int it = 0; it < mine; ++it) {
+            auto copy_w = [&](int it, int stage) {
+                const uint32_t bar = smem_u32(&S->full[stage]);
+                mbar_arrive_expect_tx(bar, stage_bytes);
+                bulk_copy_g2s(base_u32 + (uint32_t)stage * stage_bytes, src + (size_t)it * FT_A_BYTES, FT_A_BYTES, bar);
+            };
+            auto copy_x = [&](int it, int stage) {
+                asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                             ::"r"(base_u32 + (uint32_t)stage * stage_bytes + FT_A_BYTES), "l"(&tmapX), "r"((s_begin + it) * FT_SLAB), "r"(0),
+                               "r"(smem_u32(&S->full[stage])) : "memory");
+            };
+            // the ring's first filling: the weights do not wait for the predecessor on the stream, the rows do
+            const int head = p.wait_limit > 0 ? min(mine, p.stages) : 0;
+            for (int it = 0; it < head; ++it) copy_w(it, it);
+            pdl_wait();
+            for (int it = 0; it < head; ++it) copy_x(it, it);
+            n_loaded = head;
+            for (int it = head; it < mine; ++it) {
                 const int stage = it % p.stages;
                 if (!mbar_wait(smem_u32(&S->empty[stage]), ((it / p.stages) & 1) ^ 1, p.wait_limit)) { ok = false; break; }
-                const uint32_t bar = smem_u32(&S->full[stage]);
-                const uint32_t dst = base_u32 + (uint32_t)stage * stage_bytes;
-                mbar_arrive_expect_tx(bar, stage_bytes);
-                asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                             ::"r"(dst + FT_A_BYTES), "l"(&tmapX), "r"((s_begin + it) * FT_SLAB), "r"(0), "r"(bar) : "memory");
-                bulk_copy_g2s(dst, src + (size_t)it * FT_A_BYTES, FT_A_BYTES, bar);
+                copy_w(it, stage);
+                copy_x(it, stage);
                 n_loaded = it + 1;
             }
-        }
+        } else pdl_wait();
     } else {
         // ================= MMA issuer
         if (lane == 0) {
@@ -258,14 +277,19 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
         const uint32_t red_u32 = smem_u32(red);
         for (int i = tid; i < my_rows * (TC_M / 4); i += FT_THREADS) {
             const int row = (int)rank + (i / (TC_M / 4)) * p.ksplit, o4 = (i % (TC_M / 4)) * 4;
-            int4 w = make_int4(0, 0, 0, 0);
-            for (int c = 0; c < p.ksplit; ++c) {
+            // (all shares' reads in flight together)
+            int4 t[8];
+            #pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                t[c] = make_int4(0, 0, 0, 0);
+                if (c >= p.ksplit) continue;
                 uint32_t remote;
-                int4 t;
                 asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(red_u32 + (uint32_t)(row * TC_M + o4) * 4u), "r"(c));
-                asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(t.x), "=r"(t.y), "=r"(t.z), "=r"(t.w) : "r"(remote) : "memory");
-                w.x += t.x; w.y += t.y; w.z += t.z; w.w += t.w;
+                asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(t[c].x), "=r"(t[c].y), "=r"(t[c].z), "=r"(t[c].w) : "r"(remote) : "memory");
             }
+            int4 w = t[0];
+            #pragma unroll
+            for (int c = 1; c < 8; ++c) { w.x += t[c].x; w.y += t[c].y; w.z += t[c].z; w.w += t[c].w; }
             const int oo = mtile * TC_M + o4;
             if (oo < p.c_out) ft_finish4(p, row, oo, w);
         }
@@ -314,6 +338,9 @@ static FtPlan ft_plan(const Layer& L)
     FtPlan f;
     int ks = 148 / L.tc_ntiles;
     ks = ks < 1 ? 1 : (ks > L.tc_slabs ? L.tc_slabs : ks);
+    // narrow layers: no more shares than a cluster closes, where a share's slabs are in the ring at once anyway (beyond that
+    // the shares meet in global memory; 4096 -> 1008, 55 rows: 9.2 -> 8.2 us per call with 8 shares instead of 16)
+    if (ks > 8 && ceil_div(L.tc_slabs, 8) <= 8) ks = 8;
     f.per = ceil_div(L.tc_slabs, ks);
     f.ksplit = ceil_div(L.tc_slabs, f.per);
     return f;
@@ -386,7 +413,8 @@ int fc_tc_create(rrm_net* net, Layer& L)
 // rows = frames x streams, frame-major.  stateless: Y only.  Otherwise the stored projection and the
 // input snapshot become those of the last frame (the last n rows).  stat (may be null, not with stateless)
 // receives per row the counters of the delta against the row n before it (the snapshot for the first n).
-int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, bool stateless, unsigned* stat, cudaStream_t st)
+int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, bool stateless, unsigned* stat, cudaStream_t st,
+              unsigned long long* host)
 {
     const int C = L.d.c_in, K = L.d.c_out, n = L.d.n;
     if (reinterpret_cast<uintptr_t>(X_dev) & 15) return RRM_ERR_INVALID_ARG;    // the copy engine wants 16-byte aligned rows
@@ -424,6 +452,7 @@ int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, 
         p.Pstate = has_state ? reinterpret_cast<int32_t*>(L.P) + (size_t)state_off * K : nullptr;
         p.snap = has_state ? L.xs[L.xs_cur] + (size_t)state_off * C : nullptr;
         p.stat = stat && !stateless ? stat + (size_t)r0 * 2 : nullptr;
+        p.host = host ? host + r0 : nullptr; p.epoch = L.seq_epoch;
         p.xprev = r0 == 0 ? old_snap : reinterpret_cast<const int8_t*>(X_dev) + (size_t)(r0 - n) * C;
         // the piece's rows as a 2-D byte tensor [rows][c_in]; a box is one slab of all rows, swizzled on the way in
         CUtensorMap tm;
@@ -435,14 +464,9 @@ int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, 
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return RRM_ERR_CUDA;
         const size_t dyn = 1024 + (size_t)p.stages * stage_bytes + sizeof(FtSmemTail);
-        if (L.ft_cluster) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at[1];
-            ft_cluster_config(cfg, at, L.tc_ntiles, f.ksplit, dyn, st);
-            RRM_CUDA_TRY(cudaLaunchKernelEx(&cfg, fc_tc_kernel<true>, p, tm));
-        } else {
-            fc_tc_kernel<false><<<dim3(L.tc_ntiles, f.ksplit), FT_THREADS, dyn, st>>>(p, tm);
-        }
+        const dim3 grid(L.tc_ntiles, f.ksplit);
+        if (L.ft_cluster) RRM_CUDA_TRY(launch_overlapped(fc_tc_kernel<true>, grid, dim3(FT_THREADS), dyn, st, f.ksplit, p, tm));
+        else RRM_CUDA_TRY(launch_overlapped(fc_tc_kernel<false>, grid, dim3(FT_THREADS), dyn, st, 1, p, tm));
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
