@@ -119,22 +119,30 @@ def lib():
 
 
 def _check(status, what):
-    if status != 0:
+    if status:
         raise RRMError(f"{what}: {lib().rrm_strerror(status).decode()} ({status})")
 
 
 def _ptr(t):
-    if t is None:
-        return None
     if isinstance(t, torch.Tensor):
         return t.data_ptr()
+    if t is None:
+        return None
     if isinstance(t, np.ndarray):
         return t.ctypes.data
     return int(t)
 
 
+# The current stream's handle without a torch.cuda.Stream object around it: a frame of a small layer takes a few
+# microseconds on the GPU, and so did making that object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
