@@ -83,7 +83,6 @@ struct WinParams {
     int ks, per;              // CTAs that share a tile's blocks, blocks of each
     int tsplit;               // > 1: a share is one block's taps, cut into so many parts (ks = nblk * tsplit)
     int cluster;              // the shares of a tile form a cluster that adds them up (0: each adds onto the projection by itself)
-    int eager;                // filter copies start before it is known whether the tile has anything to update
     int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
     int tps, stages, abuf;    // taps per filter stage, stages, window buffers
     int xarr;                 // first layers: arrays of an image row's chunks (0: the chunks of every column side by side)
@@ -319,44 +318,10 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     const int lin0 = tile * p.mt * TC_M;
     const int b0 = p.tsplit > 1 ? split / p.tsplit : split * p.per, b1 = min(p.nblk, b0 + p.per);
     const int part = p.tsplit > 1 ? split - b0 * p.tsplit : 0;
+    const int plane0 = b0 / p.nchb;
     const uint32_t unit_b = (uint32_t)p.bn * 32u * PIECES;   // filter bytes of one (tap, group)
     bool ok = true;
     int issued = 0;                                          // stages the loader has filled
-
-    // ================= filters: the loader's walk over its blocks' taps, resumed where it stopped
-    int lb = b0, lt = -1, lstage = 0;                        // block, next tap within it (-1: the block has not been started), stage
-    uint32_t lphase = 1;
-    auto load_stages = [&](int most) {                       // (one thread) fills up to `most` stages
-        while (lb < b1 && most > 0) {
-            const int plane = lb / p.nchb, chb = lb - plane * p.nchb;
-            const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
-            const int nx = p.plane[plane].nx, ntap = p.plane[plane].ny * nx;
-            const int t_end = p.tsplit > 1 ? (part + 1) * ntap / p.tsplit : ntap;
-            if (lt < 0) lt = p.tsplit > 1 ? part * ntap / p.tsplit : 0;
-            const uint32_t bytes = unit_b * (uint32_t)gn, tap_bytes = (uint32_t)p.groups * unit_b;
-            const int row_taps = XCOL ? 1 : p.kw;            // taps of a filter row
-            const uint32_t step_x = tap_bytes * (uint32_t)p.stride, step_y = tap_bytes * (uint32_t)(row_taps * p.stride) - step_x * (uint32_t)(nx - 1);
-            int jx = lt % nx;
-            const unsigned char* src = p.Wimg + ((size_t)ntile * (row_taps * p.kh) * p.groups + g0) * unit_b +
-                                       (size_t)((p.plane[plane].ky0 + lt / nx * p.stride) * row_taps + p.plane[plane].kx0 + jx * p.stride) * tap_bytes;
-            for (; lt < t_end && most > 0; --most) {
-                if (!mbar_wait(smem_u32(&S->bempty[lstage]), lphase, p.wait_limit) || *(volatile int*)&S->fail) { ok = false; return; }
-                const int tn = min(p.tps, t_end - lt);
-                const uint32_t bar = smem_u32(&S->bfull[lstage]);
-                mbar_arrive_expect_tx(bar, bytes * (uint32_t)tn);
-                uint32_t dst = bstage_u32 + lstage * p.stage_bytes;
-                for (int t = 0; t < tn; ++t) {
-                    bulk_copy_g2s(dst, src, bytes, bar);
-                    dst += bytes;
-                    if (++jx == nx) { jx = 0; src += step_y; } else src += step_x;
-                }
-                lt += tn;
-                ++issued;
-                if (++lstage == p.stages) { lstage = 0; lphase ^= 1; }
-            }
-            if (lt >= t_end) { ++lb; lt = -1; }
-        }
-    };
 
     pdl_launch_dependents();
     if (tid == 0) {
@@ -374,8 +339,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         S->fail = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&S->bfull[s]), 1); mbar_init(smem_u32(&S->bempty[s]), 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
-        if (p.eager) load_stages(2);                          // (filters are nobody's work: no wait for the predecessors)
     }
     // ---- the tile's rows, and the first plane's table
     int active;
@@ -392,7 +355,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 bit = DENSE ? (p.count_bitmap && q >= 0 && ((p.count_bitmap[q >> 5] >> (q & 31)) & 1u)) : q >= 0;
                 S->q[tid] = q;
             }
-            wn_table<DENSE, XCOL>(p, in_act, S, lin0, b0 / p.nchb);
+            wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane0);
             if (ACT && tid < p.bn) S->bias[tid] = p.bias && ntile * p.bn + tid < p.c_out ? reinterpret_cast<const int*>(p.bias)[ntile * p.bn + tid] : 0;
         }
         tc_fence_before();
@@ -406,8 +369,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     }
     const uint32_t tmem = S->tmem_base;
     if (!DENSE && active == 0) {                             // nothing to update (every share of the tile sees the same)
-        if (tid == WN_FILL + 32)
-            for (int j = 0; j < issued; ++j) mbar_wait(smem_u32(&S->bfull[j]), 0, WAIT_LIMIT_DEFAULT);
         if (warp == 8)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
         return;
@@ -445,18 +406,23 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             return true;
         };
         const bool lag = DT == T_I8 && !XCOL && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
-        int last_plane = b0 / p.nchb, ib = 0;
+        int plane = plane0, chb = b0 - plane0 * p.nchb, ib = 0, buf = -1;
+        uint32_t phase = 0;                                  // of aempty: the ring's first filling waits for nobody
         for (int b = b0; b < b1; ++b, ++ib) {
-            const int buf = ib % p.abuf;
-            ok = mbar_wait(smem_u32(&S->aempty[buf]), ((ib / p.abuf) & 1) ^ 1, p.wait_limit) && *(volatile int*)&S->fail == 0;
-            if (!wn_agree(ok)) { ok = false; break; }
-            const int plane = b / p.nchb, chb = b - plane * p.nchb;
+            if (++buf == p.abuf) { buf = 0; phase ^= 1; }
+            if (ib >= p.abuf || p.wait_limit == 0) {
+                ok = mbar_wait(smem_u32(&S->aempty[buf]), phase ^ 1, p.wait_limit) && *(volatile int*)&S->fail == 0;
+                if (!wn_agree(ok)) { ok = false; break; }
+            }
+            const bool new_plane = ib > 0 && chb == p.nchb;
+            if (chb == p.nchb) { chb = 0; ++plane; }
             const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
-            if (plane != last_plane) {
-                last_plane = plane;
+            if (new_plane) {
+                wn_meet();                                   // (everyone is done with the last plane's)
                 wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane);
                 wn_meet();
             }
+            ++chb;
             const uint32_t Ab = base_u32 + buf * p.abytes;
             unsigned char* Ap = base + buf * p.abytes;
             const int arrays = XCOL && p.xarr ? p.xarr : gn * 2;               // of p.L slots each
@@ -480,7 +446,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 } else if (ib > 0) {
                     cp_async_wait<1>();
                     fence_async_smem();
-                    mbar_arrive(smem_u32(&S->afull[(ib - 1) % p.abuf]));
+                    mbar_arrive(smem_u32(&S->afull[buf > 0 ? buf - 1 : p.abuf - 1]));
                 }
             } else if (DT == T_I8) {
                 // first layer, a 4-byte word per pixel: four neighbouring pixels of an image row are one chunk
@@ -581,11 +547,44 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         if (DT == T_I8 && !XCOL) {
             cp_async_wait<0>();
             fence_async_smem();
-            if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[(ib - 1) % p.abuf]));
+            if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[buf]));
         }
         if (DT == T_F32 && ok && ib > 0 && !promote(ib - 1)) ok = false;
     } else if (warp == 9) {
-        if (lane == 0) load_stages(1 << 30);
+        // ================= filters: a stage's taps, one bulk copy each (one thread)
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 1;
+            for (int b = b0; b < b1 && ok; ++b) {
+                const int plane = b / p.nchb, chb = b - plane * p.nchb;
+                const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
+                const int nx = p.plane[plane].nx, ntap = p.plane[plane].ny * nx;
+                const int t_end = p.tsplit > 1 ? (part + 1) * ntap / p.tsplit : ntap;
+                int lt = p.tsplit > 1 ? part * ntap / p.tsplit : 0;
+                const uint32_t bytes = unit_b * (uint32_t)gn, tap_bytes = (uint32_t)p.groups * unit_b;
+                const int row_taps = XCOL ? 1 : p.kw;        // taps of a filter row
+                const uint32_t step_x = tap_bytes * (uint32_t)p.stride, step_y = tap_bytes * (uint32_t)(row_taps * p.stride) - step_x * (uint32_t)(nx - 1);
+                const int jy = lt / nx;
+                int jx = lt - jy * nx;
+                const unsigned char* src = p.Wimg + ((size_t)ntile * (row_taps * p.kh) * p.groups + g0) * unit_b +
+                                           (size_t)((p.plane[plane].ky0 + jy * p.stride) * row_taps + p.plane[plane].kx0 + jx * p.stride) * tap_bytes;
+                while (lt < t_end) {
+                    if (!mbar_wait(smem_u32(&S->bempty[stage]), phase, p.wait_limit) || *(volatile int*)&S->fail) { ok = false; break; }
+                    const int tn = min(p.tps, t_end - lt);
+                    const uint32_t bar = smem_u32(&S->bfull[stage]);
+                    mbar_arrive_expect_tx(bar, bytes * (uint32_t)tn);
+                    uint32_t dst = bstage_u32 + stage * p.stage_bytes;
+                    for (int t = 0; t < tn; ++t) {
+                        bulk_copy_g2s(dst, src, bytes, bar);
+                        dst += bytes;
+                        if (++jx == nx) { jx = 0; src += step_y; } else src += step_x;
+                    }
+                    lt += tn;
+                    ++issued;
+                    if (++stage == p.stages) { stage = 0; phase ^= 1; }
+                }
+            }
+        }
     } else {
         // ================= MMAs.  The whole warp walks and one elected lane issues.  What the walk costs is what the MMAs of
         // a stage have to be longer than: a step's MMAs are one block of instructions, and the next stage's barrier is polled
@@ -709,11 +708,17 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     const int4 b = *reinterpret_cast<const int4*>(S->bias + cc + j);
                     v[j] += (uint32_t)b.x; v[j + 1] += (uint32_t)b.y; v[j + 2] += (uint32_t)b.z; v[j + 3] += (uint32_t)b.w;
                 }
-                if (keep) {
+                if (keep) {                                  // (before f: the fence waits for this thread's stores, the output's too)
                     if (vec) {
                         uint32_t* at = row + (cc - cb) + (halves ? 0 : cb);
                         #pragma unroll
                         for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(at + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        const int cols = min(32, ncols - cc);
+                        fence_async_smem();
+                        if (cols > 0)
+                            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                         ::"l"(dstP + cc), "r"(smem_u32(at)), "r"((uint32_t)cols * 4u) : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     } else {
                         #pragma unroll
                         for (int j = 0; j < 32; ++j) if (cc + j < ncols) dstP[cc + j] = (int32_t)v[j];
@@ -737,15 +742,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
                     dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
                     dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
-                }
-            }
-            if (keep && vec) {
-                const int cols = min(min(64, c_hi - cb), ncols - cb);
-                fence_async_smem();
-                if (cols > 0) {
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                                 ::"l"(dstP + cb), "r"(smem_u32(row + (halves ? 0 : cb))), "r"((uint32_t)cols * 4u) : "memory");
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
             }
         }
@@ -907,7 +903,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             using std::integral_constant;
             if (shares == 1) close(integral_constant<int, 4>{}, integral_constant<int, 1>{});
             else if (shares <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
-            else close(integral_constant<int, 1>{}, integral_constant<int, 8>{});
+            else close(integral_constant<int, 2>{}, integral_constant<int, 8>{});
         }
         __syncwarp();
         if (p.cluster) wn_cluster_meet();                    // nobody's shared memory goes away while it is read
@@ -1151,7 +1147,6 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
                 const unsigned cols = f32 ? 3 * p.bn + round_up(p.bn, 32) : (mt - 1) * p.bn + round_up(p.bn, 32);
                 p.tmem_cols = 32;
                 while (p.tmem_cols < cols) p.tmem_cols *= 2;
-                p.eager = dense || tiles * p.ks <= 2 * 148;
                 return true;
             }
             if (gblk == 1 || xcol) break;
