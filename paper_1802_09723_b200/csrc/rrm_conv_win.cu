@@ -51,6 +51,7 @@ constexpr int WN_FILL = 256;                  // threads that fill windows and d
 constexpr int WN_THREADS = WN_FILL + 64;
 constexpr int WN_MAX_STAGES = 8, WN_MAX_ABUF = 4, WN_MAX_MT = 2;
 constexpr int WN_MAX_SPAN = 1152;             // pixels of one plane of a window
+constexpr int WN_TURN = 36;                  // words per row where a warp turns 32 rows x 32 columns around (16-byte aligned, staggered over the banks)
 constexpr int WN_PROMOTE = 32;                // fp32: K steps the leading product accumulates before it is promoted
 constexpr size_t WN_SMEM_LIMIT = 227 * 1024;
 
@@ -278,20 +279,23 @@ __device__ __noinline__ uint32_t wn_f8_bn(const WinParams& p, int c, int x0, int
 }
 // int8 f of 4 neighbouring channels: requantisation (round half up), [+ shortcut], activation; the saturation at 127 is the
 // packing's.  Channels beyond the layer's last have zero filters, bias and shortcut.
-__device__ __forceinline__ uint32_t wn_f8(const WinParams& p, int c, const int (&x)[4], uint32_t res)
+__device__ __forceinline__ uint32_t wn_f8_plain(const int (&x)[4], uint32_t res, int rnd, int sh, int lo, bool with_res)
 {
-    if (p.bn_scale) return wn_f8_bn(p, c, x[0], x[1], x[2], x[3], res);
-    const int rnd = p.shift > 0 ? 1 << (p.shift - 1) : 0, lo = p.act_fn == RRM_ACT_RELU ? 0 : -127;
     int y[4];
     #pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = (x[j] + rnd) >> p.shift;
-    if (p.res) {
+    for (int j = 0; j < 4; ++j) y[j] = (x[j] + rnd) >> sh;
+    if (with_res) {
         #pragma unroll
         for (int j = 0; j < 4; ++j) y[j] = max(-127, min(127, y[j])) + (int)(int8_t)(res >> (8 * j));
     }
     #pragma unroll
     for (int j = 0; j < 4; ++j) y[j] = max(y[j], lo);
     return wn_pack4(y[0], y[1], y[2], y[3]);
+}
+__device__ __forceinline__ uint32_t wn_f8(const WinParams& p, int c, const int (&x)[4], uint32_t res)
+{
+    if (p.bn_scale) return wn_f8_bn(p, c, x[0], x[1], x[2], x[3], res);
+    return wn_f8_plain(x, res, p.shift > 0 ? 1 << (p.shift - 1) : 0, p.shift, p.act_fn == RRM_ACT_RELU ? 0 : -127, p.res != nullptr);
 }
 
 // DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.  ACT (dense passes): f is applied here and the output written,
@@ -663,17 +667,14 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     }
     if (!ok) { *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
 
-    // ================= accumulators out: rows of the tile(s) go to shared memory (the windows are done with); there a
-    // projection row is the work of a warp (half a warp where 64 columns are drained at a time): a lane owns 4
-    // neighbouring channels
+    // ================= accumulators out, through shared memory where rows have to be turned around (the windows are done with)
     const int n0 = ntile * p.bn, ncols = min(p.bn, p.c_out - n0);
     const bool halves = p.mt > 1 && p.bn > 64;               // two tiles: 64 columns at a time, so that both fit
     const int cw = halves ? 64 : p.bn;                       // columns per pass
     const int ldr = cw + 4;                                  // words per staged row (16-byte aligned, staggered over the banks)
     const bool vec = (p.c_out & 3) == 0;
     const bool adds = !DENSE && !p.store;                    // delta: onto the stored projection
-    const bool bulk_add = adds && vec && !p.cluster;         // ... by the copy engine, a row per thread (exact in any order for integers,
-                                                             // one share only for fp32)
+    const bool bulk_add = DT != T_F32 && adds && vec && !p.cluster;   // ... integers by the copy engine, a row per thread (exact in any order)
     uint32_t* staged = reinterpret_cast<uint32_t*>(base);
     if (warp < 8) {
         if (ok && !mbar_wait(smem_u32(&S->done), 0, p.wait_limit)) { ok = false; *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
@@ -734,10 +735,23 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 } else {
                     const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
                     uint32_t o[8];
-                    #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
-                        o[j] = wn_f8(p, n0 + cc + 4 * j, x, rr[j]);
+                    if (!p.bn_scale) {
+                        const int rnd = p.shift > 0 ? 1 << (p.shift - 1) : 0, sh = p.shift, lo = p.act_fn == RRM_ACT_RELU ? 0 : -127;
+                        if (!p.res) {
+                            #pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                o[j] = wn_pack4(max(((int)v[4 * j] + rnd) >> sh, lo), max(((int)v[4 * j + 1] + rnd) >> sh, lo),
+                                                max(((int)v[4 * j + 2] + rnd) >> sh, lo), max(((int)v[4 * j + 3] + rnd) >> sh, lo));
+                        } else {
+                            #pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
+                                o[j] = wn_f8_plain(x, rr[j], rnd, sh, lo, true);
+                            }
+                        }
+                    } else {
+                        #pragma unroll
+                        for (int j = 0; j < 8; ++j) o[j] = wn_f8_bn(p, n0 + cc + 4 * j, (int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3], rr[j]);
                     }
                     uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
                     dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -747,166 +761,212 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         }
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the row buffers may be released
     }
-    #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-        if (direct || (pass > 0 && !halves)) break;
-        const int p0 = pass * 64;                            // first column of the pass (own columns: c_lo + c0)
-        if (warp < 8 && ok) {
-            const int r = m_own * TC_M + (warp & 3) * 32 + lane;
-            uint32_t* row = staged + (size_t)r * ldr;
-            if (pass > 0) { if (bulk_add) __syncwarp(); else wn_meet(); }    // the first pass's rows have left
-            #pragma unroll (DT == T_F32 ? 2 : 1)
-            for (int c0 = 0; c0 < (DT == T_F32 ? 64 : 128); c0 += 32) {
-                if (c_lo + c0 < c_hi && (!halves || (c0 >> 6) == pass)) {
-                    uint32_t v[32];
-                    if (DT == T_F32) {                       // (the second accumulator of small products)
-                        wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + c_lo + c0), v);
-                        #pragma unroll
-                        for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? c0 + j : 0] += __uint_as_float(v[j]);
-                    }
-                    wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + c_lo + c0), v);
+    // one value group of 4 neighbouring channels (c: column of the tile) of projection pixel q leaves: f and the output row
+    // (ACT), the projection where it is kept.  Every lane of a warp comes here (signs are put together by shuffles).
+    auto emit = [&](int q, int c, const uint32_t (&o)[4]) {
+        const int ch = n0 + c;
+        if (ACT && DT != T_F32 && p.bits) {
+            uint32_t word = 0;
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) if (c + j < ncols && (int)o[j] >= p.theta) word |= 1u << (4 * (lane & 7) + j);
+            word |= __shfl_xor_sync(0xffffffffu, word, 1);
+            word |= __shfl_xor_sync(0xffffffffu, word, 2);
+            word |= __shfl_xor_sync(0xffffffffu, word, 4);
+            if (q >= 0 && (lane & 7) == 0 && c < p.bn && (ch >> 5) < p.cs) reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + (ch >> 5)] = word;
+        } else if (ACT && DT != T_F32) {
+            if (q >= 0 && c < p.bn && ch < p.cs) {           // (channels up to the padded width get a value too)
+                const size_t at = (size_t)q * p.cs + ch;
+                const int x[4] = {(int)o[0], (int)o[1], (int)o[2], (int)o[3]};
+                const uint32_t res = p.res ? *reinterpret_cast<const uint32_t*>(reinterpret_cast<const int8_t*>(p.res) + at) : 0u;
+                *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(p.X) + at) = wn_f8(p, ch, x, res);
+            }
+        } else if (ACT) {
+            if (q >= 0 && c < ncols) {
+                const size_t at = (size_t)q * p.cs + ch;
+                float x[4], res[4] = {0.f, 0.f, 0.f, 0.f}, y[4];
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    x[j] = __uint_as_float(o[j]);
+                    if (p.res && c + j < ncols) res[j] = reinterpret_cast<const float*>(p.res)[at + j];
+                }
+                if (p.bn_scale) wn_f<T_F32, T_F32, float>(p, ch, x, res, y);
+                else {
                     #pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        if (c_lo + c0 + j >= c_hi) break;
-                        uint4 o;
-                        if (DT == T_F32)
-                            o = make_uint4(__float_as_uint(__uint_as_float(v[j]) + facc[DT == T_F32 ? c0 + j : 0]),
-                                           __float_as_uint(__uint_as_float(v[j + 1]) + facc[DT == T_F32 ? c0 + j + 1 : 0]),
-                                           __float_as_uint(__uint_as_float(v[j + 2]) + facc[DT == T_F32 ? c0 + j + 2 : 0]),
-                                           __float_as_uint(__uint_as_float(v[j + 3]) + facc[DT == T_F32 ? c0 + j + 3 : 0]));
-                        else o = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                        *reinterpret_cast<uint4*>(row + c_lo + c0 + j - p0) = o;
+                    for (int j = 0; j < 4; ++j) {
+                        y[j] = x[j] + res[j];
+                        if (p.act_fn == RRM_ACT_RELU) y[j] = y[j] > 0 ? y[j] : 0;
+                        else if (p.act_fn == RRM_ACT_LEAKY) y[j] = y[j] > 0 ? y[j] : 0.1f * y[j];
                     }
                 }
+                float* dst = reinterpret_cast<float*>(p.X) + at;
+                if (vec) *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
+                else {
+                    #pragma unroll
+                    for (int j = 0; j < 4; ++j) if (c + j < ncols) dst[j] = y[j];
+                }
             }
-            if (bulk_add) {
-                const int lo = halves ? p0 : c_lo, hi = min(halves ? min(p0 + 64, c_hi) : c_hi, ncols), q = S->q[r];
+        }
+        if (q < (ACT ? p.keep_from : 0) || c >= ncols) return;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(q - (ACT ? p.keep_from : 0)) * p.c_out + ch;
+        if (vec) *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+        else {
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) if (c + j < ncols) dst[j] = o[j];
+        }
+    };
+    auto plus = [](uint32_t a, uint32_t b) -> uint32_t { return DT == T_F32 ? __float_as_uint(__uint_as_float(a) + __uint_as_float(b)) : a + b; };
+    // what the sums are added to: the bias (dense), the stored projection (delta)
+    auto base_of = [&](int q, int c, uint32_t (&o)[4]) {
+        o[0] = o[1] = o[2] = o[3] = 0;
+        if (q < 0 || c >= ncols || !(adds || (DENSE && p.bias))) return;
+        const uint32_t* from = (adds ? reinterpret_cast<const uint32_t*>(P) + (size_t)q * p.c_out : reinterpret_cast<const uint32_t*>(p.bias)) + n0 + c;
+        if (vec) { const uint4 w = *reinterpret_cast<const uint4*>(from); o[0] = w.x; o[1] = w.y; o[2] = w.z; o[3] = w.w; }
+        else {
+            #pragma unroll
+            for (int j = 0; j < 4; ++j) if (c + j < ncols) o[j] = from[j];
+        }
+    };
+    // 32 columns of this thread's accumulator row, from column cc of the tile on (k: index into the promoted sums)
+    auto take32 = [&](int cc, int k, uint32_t (&v)[32]) {
+        __syncwarp();
+        if (DT == T_F32) {
+            wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + cc), v);
+            #pragma unroll
+            for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? k + j : 0] += __uint_as_float(v[j]);
+        }
+        wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + cc), v);
+        if (DT == T_F32) {
+            #pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + facc[DT == T_F32 ? k + j : 0]);
+        }
+    };
+    if (!direct && !p.cluster && !bulk_add) {
+        // one share: a warp turns its 32 rows x 32 columns around in shared memory of its own (eight lanes a row, whole
+        // lines), without a barrier of the CTA
+        if (warp < 8 && ok) {
+            uint32_t* mine = staged + (size_t)warp * 32 * WN_TURN;
+            const int q_own = S->q[m_own * TC_M + (warp & 3) * 32 + lane];
+            const int sub = lane >> 3, c4 = (lane & 7) * 4;
+            #pragma unroll (DT == T_F32 ? 2 : 1)
+            for (int k = 0; k < (DT == T_F32 ? 64 : 128); k += 32) {
+                const int cc = c_lo + k;
+                if (cc >= c_hi) continue;                    // (the same in all lanes)
+                uint32_t v[32];
+                take32(cc, k, v);
+                #pragma unroll
+                for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(mine + lane * WN_TURN + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                __syncwarp();
+                uint32_t base4[4];
+                if (!adds) base_of(0, cc + c4, base4);       // (the bias: the same for every row)
+                #pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t o[4][4];
+                    int q[4];
+                    #pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        q[i] = __shfl_sync(0xffffffffu, q_own, (half * 4 + i) * 4 + sub);
+                        if (adds) base_of(q[i], cc + c4, o[i]);
+                        else { o[i][0] = base4[0]; o[i][1] = base4[1]; o[i][2] = base4[2]; o[i][3] = base4[3]; }
+                    }
+                    #pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint4 t = *reinterpret_cast<const uint4*>(mine + ((half * 4 + i) * 4 + sub) * WN_TURN + c4);
+                        o[i][0] = plus(o[i][0], t.x); o[i][1] = plus(o[i][1], t.y); o[i][2] = plus(o[i][2], t.z); o[i][3] = plus(o[i][3], t.w);
+                        emit(q[i], cc + c4, o[i]);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    } else if (!direct && !p.cluster) {
+        // integer shares: every share adds its rows onto the projection by itself, through the copy engine
+        #pragma unroll 1
+        for (int pass = 0; pass < (halves ? 2 : 1); ++pass) {
+            const int p0 = pass * 64;                        // first column of the pass
+            if (warp < 8 && ok) {
+                const int r = m_own * TC_M + (warp & 3) * 32 + lane;
+                uint32_t* row = staged + (size_t)r * ldr;
+                const int lo = halves ? p0 : c_lo, hi = halves ? min(p0 + 64, c_hi) : c_hi;
+                #pragma unroll 1
+                for (int cc = lo; cc < hi; cc += 32) {
+                    uint32_t v[32];
+                    take32(cc, 0, v);
+                    #pragma unroll
+                    for (int j = 0; j < 32; j += 4) if (cc + j < hi) *reinterpret_cast<uint4*>(row + cc + j - p0) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                }
+                const int q = S->q[r], end = min(hi, ncols);
                 fence_async_smem();                          // this thread's part of the row -> visible to the copy engine
-                if (q >= 0 && hi > lo) {
-                    char* dst = reinterpret_cast<char*>(P) + ((size_t)q * p.c_out + n0 + lo) * 4;
-                    if (DT == T_F32)
-                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
-                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(hi - lo) * 4u) : "memory");
-                    else
-                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;"
-                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(hi - lo) * 4u) : "memory");
+                if (q >= 0 && end > lo) {
+                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;"
+                                 ::"l"(reinterpret_cast<char*>(P) + ((size_t)q * p.c_out + n0 + lo) * 4), "r"(smem_u32(row + lo - p0)),
+                                   "r"((uint32_t)(end - lo) * 4u) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 }
             }
         }
-        __syncwarp();
-        if (bulk_add) continue;
-        if (p.cluster) wn_cluster_meet();                    // every share's partial tile is in its shared memory
-        else if (warp < 8) wn_meet();
+    } else if (p.cluster) {
         if (warp < 8 && ok) {
-            // rows split, split + ks, ... of the tile (one share: all rows), a few at a time per warp or half warp, all shares'
-            // reads of a turn in flight together (one after the other, eight shares took 6 us)
-            const int shares = p.cluster ? p.ks : 1, mine = p.cluster ? split : 0;
-            const int rows = p.mt * TC_M;
-            const bool wide = cw > 64;
-            const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
-            const int ch = (wide ? lane : lane & 15) * 4;    // first own channel of the pass
-            const bool act_lane = p0 + ch < ncols;
-            const bool pad_lane = ACT && DT != T_F32 && p0 + ch < p.bn;      // (channels up to the padded width get a value too)
-            auto close = [&](auto nr, auto ns) {
-            constexpr int NR = decltype(nr)::value, NS = decltype(ns)::value;
-            for (int k0 = team * NR; mine + (wide ? k0 : k0 & ~(2 * NR - 1)) * shares < rows; k0 += teams * NR) {   // (whole warps stay together)
-                uint32_t o[NR][4];
-                uint4 t[NS][NR];
-                int q[NR];
+            uint32_t* row = staged + (size_t)((warp & 3) * 32 + lane) * ldr;
+            #pragma unroll (DT == T_F32 ? 2 : 1)
+            for (int k = 0; k < 64; k += 32) {
+                const int cc = c_lo + k;
+                if (cc >= c_hi) continue;
+                uint32_t v[32];
+                take32(cc, k, v);
                 #pragma unroll
-                for (int u = 0; u < NR; ++u) {
-                    const int r = mine + (k0 + u) * shares;
-                    q[u] = r < rows ? S->q[r] : -1;
-                    o[u][0] = o[u][1] = o[u][2] = o[u][3] = 0;
-                    if (q[u] < 0 || !act_lane) continue;
-                    if (adds || (DENSE && p.bias)) {
-                        const uint32_t* from = (adds ? reinterpret_cast<const uint32_t*>(P) + (size_t)q[u] * p.c_out
-                                                     : reinterpret_cast<const uint32_t*>(p.bias)) + n0 + p0 + ch;
-                        if (vec) { const uint4 w = *reinterpret_cast<const uint4*>(from); o[u][0] = w.x; o[u][1] = w.y; o[u][2] = w.z; o[u][3] = w.w; }
-                        else {
-                            #pragma unroll
-                            for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) o[u][j] = from[j];
-                        }
-                    }
-                }
-                #pragma unroll
-                for (int s = 0; s < NS; ++s)
-                    #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
-                        t[s][u] = make_uint4(0, 0, 0, 0);
-                        if (s >= shares || q[u] < 0 || !act_lane) continue;
-                        const uint32_t* at = staged + (size_t)(mine + (k0 + u) * shares) * ldr + ch;
-                        t[s][u] = NS > 1 ? wn_ld_remote(smem_u32(at), (uint32_t)s) : *reinterpret_cast<const uint4*>(at);
-                    }
-                #pragma unroll
-                for (int u = 0; u < NR; ++u)
-                    #pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        if (s >= shares) break;
-                        const uint32_t w[4] = {t[s][u].x, t[s][u].y, t[s][u].z, t[s][u].w};
-                        #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            o[u][j] = DT == T_F32 ? __float_as_uint(__uint_as_float(o[u][j]) + __uint_as_float(w[j])) : o[u][j] + w[j];
-                    }
-                if (ACT) {
-                    #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
-                        const int c = n0 + p0 + ch;
-                        if (DT != T_F32 && p.bits) {
-                            uint32_t word = 0;
-                            #pragma unroll
-                            for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols && (int)o[u][j] >= p.theta) word |= 1u << (4 * (lane & 7) + j);
-                            word |= __shfl_xor_sync(0xffffffffu, word, 1);
-                            word |= __shfl_xor_sync(0xffffffffu, word, 2);
-                            word |= __shfl_xor_sync(0xffffffffu, word, 4);
-                            if (q[u] >= 0 && (lane & 7) == 0 && p0 + ch < p.bn && (c >> 5) < p.cs)
-                                reinterpret_cast<uint32_t*>(p.X)[(size_t)q[u] * p.cs + (c >> 5)] = word;
-                        } else if (DT != T_F32) {
-                            if (q[u] < 0 || !pad_lane || c >= p.cs) continue;
-                            const size_t at = (size_t)q[u] * p.cs + c;
-                            const int x[4] = {(int)o[u][0], (int)o[u][1], (int)o[u][2], (int)o[u][3]};
-                            const uint32_t res = p.res ? *reinterpret_cast<const uint32_t*>(reinterpret_cast<const int8_t*>(p.res) + at) : 0u;
-                            *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(p.X) + at) = wn_f8(p, c, x, res);
-                        } else {
-                            if (q[u] < 0 || !act_lane) continue;
-                            const size_t at = (size_t)q[u] * p.cs + c;
-                            float x[4], res[4] = {0.f, 0.f, 0.f, 0.f}, y[4];
-                            #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                x[j] = __uint_as_float(o[u][j]);
-                                if (p.res && p0 + ch + j < ncols) res[j] = reinterpret_cast<const float*>(p.res)[at + j];
-                            }
-                            wn_f<T_F32, T_F32, float>(p, c, x, res, y);
-                            float* dst = reinterpret_cast<float*>(p.X) + at;
-                            if (vec) *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
-                            else {
-                                #pragma unroll
-                                for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) dst[j] = y[j];
-                            }
-                        }
-                    }
-                }
-                #pragma unroll
-                for (int u = 0; u < NR; ++u) {
-                    if (q[u] < (ACT ? p.keep_from : 0) || !act_lane) continue;
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(q[u] - (ACT ? p.keep_from : 0)) * p.c_out + n0 + p0 + ch;
-                    if (vec) *reinterpret_cast<uint4*>(dst) = make_uint4(o[u][0], o[u][1], o[u][2], o[u][3]);
-                    else {
-                        #pragma unroll
-                        for (int j = 0; j < 4; ++j) if (p0 + ch + j < ncols) dst[j] = o[u][j];
-                    }
-                }
+                for (int j = 0; j < 32; j += 4) if (cc + j < c_hi) *reinterpret_cast<uint4*>(row + cc + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
             }
+            // rows split, split + ks, ... of the tile, a few at a time per warp (half a warp where the tile has up to 64
+            // columns), all shares' reads of a turn in flight together; what they are added to is on its way before the
+            // shares meet
+            const bool wide = p.bn > 64;
+            const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
+            const int c = (wide ? lane : lane & 15) * 4;
+            auto close = [&](auto nr, auto ns) {
+                constexpr int NR = decltype(nr)::value, NS = decltype(ns)::value;
+                uint32_t o[NR][4];
+                int q[NR];
+                auto begin = [&](int k0) {
+                    #pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        const int r = split + (k0 + u) * p.ks;
+                        q[u] = r < TC_M ? S->q[r] : -1;
+                        base_of(q[u], c, o[u]);
+                    }
+                };
+                begin(team * NR);
+                __syncwarp();
+                wn_cluster_meet();                           // every share's partial tile is in its shared memory
+                for (int k0 = team * NR; split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M;) {      // (whole warps stay together)
+                    uint4 t[NS][NR];
+                    #pragma unroll
+                    for (int s = 0; s < NS; ++s)
+                        #pragma unroll
+                        for (int u = 0; u < NR; ++u) {
+                            t[s][u] = make_uint4(0, 0, 0, 0);
+                            if (s < p.ks && q[u] >= 0 && c < p.bn) t[s][u] = wn_ld_remote(smem_u32(staged + (size_t)(split + (k0 + u) * p.ks) * ldr + c), (uint32_t)s);
+                        }
+                    #pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        #pragma unroll
+                        for (int s = 0; s < NS; ++s) {
+                            if (s >= p.ks) break;
+                            o[u][0] = plus(o[u][0], t[s][u].x); o[u][1] = plus(o[u][1], t[s][u].y);
+                            o[u][2] = plus(o[u][2], t[s][u].z); o[u][3] = plus(o[u][3], t[s][u].w);
+                        }
+                        emit(q[u], c, o[u]);
+                    }
+                    k0 += teams * NR;
+                    if (split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M) begin(k0);
+                }
             };
             using std::integral_constant;
-            if (shares == 1) close(integral_constant<int, 4>{}, integral_constant<int, 1>{});
-            else if (shares <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+            if (p.ks <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
             else close(integral_constant<int, 2>{}, integral_constant<int, 8>{});
-        }
+        } else wn_cluster_meet();
         __syncwarp();
-        if (p.cluster) wn_cluster_meet();                    // nobody's shared memory goes away while it is read
+        wn_cluster_meet();                                   // nobody's shared memory goes away while it is read
     }
     tc_fence_before();
     __syncthreads();
@@ -1113,7 +1173,9 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
         p.mt = mt;
         p.span = base_span + (mt - 1) * TC_M;
         p.L = slots(p.span);
-        const size_t staging = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4;
+        // drained rows: a tile's (64 columns of it where there are two), or 32 rows x 32 columns per warp
+        const size_t whole = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4, turned = (size_t)8 * 32 * WN_TURN * 4;
+        const size_t staging = whole > turned ? whole : turned;
         int gblk = xcol ? p.groups : (p.groups < 4 ? p.groups : 4);
         if (f32 && !xcol) while (gblk > 1 && gblk * plane_taps > 18) gblk = (gblk + 1) / 2;
         if (!xcol) while (gblk > 1 && planes * ceil_div(p.groups, gblk) < want) gblk = (gblk + 1) / 2;
