@@ -37,8 +37,10 @@
 // clocks it takes), beside which the filter copies write another quarter (fp32 step of 768 MMA clocks: 1064 measured, 1180
 // with six separate MMAs and the barrier looked at only when it is needed); in a launch of a few tiles a chain of ~7 us (rows
 // and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  Against kernels that gathered rows tap by tap (fp32: on the
-// CUDA cores), AlexNet-shaped stack at 227 x 227: fp32 32 dense frames conv2 / conv4 192 / 86 -> 175 / 62 us since the MMAs
-// of a step are issued together (delta, gathered: 351 / 412), 8 streams 546 -> 206 for the whole stack; int8 frame 84 -> 70.
+// CUDA cores), AlexNet-shaped stack at 227 x 227: fp32 32 frames conv2 / conv4 351 / 412 (delta) -> 152 / 53 us (dense), 8
+// streams 546 -> 188 for the whole stack; int8 frame 84 -> 64.  fp32 tiles of 64 columns, two CTAs per SM, were slower
+// than 128 and one (conv2 152 -> 179, conv4 53 -> 83, 11x11 first layer 107 -> 111: every window is then filled twice as
+// often, and an MMA of 128 columns has no smem bandwidth to spare for it).
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
@@ -674,7 +676,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     const int ldr = cw + 4;                                  // words per staged row (16-byte aligned, staggered over the banks)
     const bool vec = (p.c_out & 3) == 0;
     const bool adds = !DENSE && !p.store;                    // delta: onto the stored projection
-    const bool bulk_add = DT != T_F32 && adds && vec && !p.cluster;   // ... integers by the copy engine, a row per thread (exact in any order)
+    const bool bulk_add = adds && vec && !p.cluster;         // ... by the copy engine, a row per thread (exact in any order for integers,
+                                                             // one share only for fp32)
     uint32_t* staged = reinterpret_cast<uint32_t*>(base);
     if (warp < 8) {
         if (ok && !mbar_wait(smem_u32(&S->done), 0, p.wait_limit)) { ok = false; *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
@@ -879,7 +882,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             }
         }
     } else if (!direct && !p.cluster) {
-        // integer shares: every share adds its rows onto the projection by itself, through the copy engine
+        // every share adds its rows onto the projection by itself, through the copy engine
         #pragma unroll 1
         for (int pass = 0; pass < (halves ? 2 : 1); ++pass) {
             const int p0 = pass * 64;                        // first column of the pass
@@ -887,19 +890,25 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 const int r = m_own * TC_M + (warp & 3) * 32 + lane;
                 uint32_t* row = staged + (size_t)r * ldr;
                 const int lo = halves ? p0 : c_lo, hi = halves ? min(p0 + 64, c_hi) : c_hi;
-                #pragma unroll 1
-                for (int cc = lo; cc < hi; cc += 32) {
+                #pragma unroll (DT == T_F32 ? 2 : 1)
+                for (int k = 0; k < 64; k += 32) {
+                    const int cc = lo + k;
+                    if (cc >= hi) continue;
                     uint32_t v[32];
-                    take32(cc, 0, v);
+                    take32(cc, k, v);
                     #pragma unroll
                     for (int j = 0; j < 32; j += 4) if (cc + j < hi) *reinterpret_cast<uint4*>(row + cc + j - p0) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
                 }
                 const int q = S->q[r], end = min(hi, ncols);
                 fence_async_smem();                          // this thread's part of the row -> visible to the copy engine
                 if (q >= 0 && end > lo) {
-                    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;"
-                                 ::"l"(reinterpret_cast<char*>(P) + ((size_t)q * p.c_out + n0 + lo) * 4), "r"(smem_u32(row + lo - p0)),
-                                   "r"((uint32_t)(end - lo) * 4u) : "memory");
+                    char* dst = reinterpret_cast<char*>(P) + ((size_t)q * p.c_out + n0 + lo) * 4;
+                    if (DT == T_F32)
+                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
+                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(end - lo) * 4u) : "memory");
+                    else
+                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.s32 [%0], [%1], %2;"
+                                     ::"l"(dst), "r"(smem_u32(row + lo - p0)), "r"((uint32_t)(end - lo) * 4u) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 }
