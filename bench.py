@@ -362,8 +362,9 @@ def conv_measure(name, variant="auto", steps=60, warmup=5, frames=None, streams=
         macs = st["dense_macs"] if dense_step else st["active_macs"]
         fin = 1.0 if dense_step else st["active_in_pixels"] / max(1, st["in_pixels"])
         fout = 1.0 if dense_step else st["active_out_pixels"] / max(1, st["out_pixels"])
-        on_tensor = sp.dtype != "f32" and st["variant"] in (2, 3)
-        peak_l = tens if on_tensor else {"f32": alu["ffma"], "i8": alu["dp4a"], "bin": alu["popc"]}[sp.dtype]
+        on_tensor = st["variant"] in (2, 3)
+        # (fp32 on the tensor cores: six bf16 products per multiply-add, bf16 at half the int8 rate)
+        peak_l = (tens / 12 if sp.dtype == "f32" else tens) if on_tensor else {"f32": alu["ffma"], "i8": alu["dp4a"], "bin": alu["popc"]}[sp.dtype]
         t_mac = macs / (peak_l * 1e12) * 1e6
         nbytes = st["in_pixels"] * fin * sp.c_in * unit_bytes[sp.dtype] + st["out_pixels"] * fout * sp.c_out * 4 * (2 if dense_step else 3)
         t_byte = nbytes / (hbm * 1e9) * 1e6
@@ -379,8 +380,9 @@ def conv_measure(name, variant="auto", steps=60, warmup=5, frames=None, streams=
           "note": "Eq. 9: MAC-weighted sparsity of the layer inputs (S0) and of their deltas (S); Eq. 10: eta = sum(rho MACs) / "
                   "sum(rho_hat MACs); dense_over_active_macs uses the exact MAC count instead of Table 1's rho x dense MACs"}
     mac_bound = byte_us < mac_us
-    peak = (alu["ffma"] if dtype == "f32" else tens) if mac_bound else hbm
-    roofline = {"bound": ("alu" if dtype == "f32" else "tensor") if mac_bound else "hbm",
+    f32_tensor = dtype == "f32" and any(e["variant"] in ("tensor", "dense") for e in per_layer)
+    peak = ((tens / 12 if f32_tensor else alu["ffma"]) if dtype == "f32" else tens) if mac_bound else hbm
+    roofline = {"bound": ("alu" if dtype == "f32" and not f32_tensor else "tensor") if mac_bound else "hbm",
                 "achieved": roof_us * 1e-3 / ms * peak, "peak": peak, "unit": "TMAC/s" if mac_bound else "GB/s",
                 "frac": roof_us * 1e-3 / ms, "traffic": None,
                 "peak_kind": f"of {('measured by rrm_measure_alu_peak' if dtype == 'f32' else tens_kind) if mac_bound else hbm_kind}",

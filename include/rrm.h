@@ -28,7 +28,8 @@
  *     kernel of a stack step on its own instead of replaying a captured CUDA graph; RRM_DEBUG=1 names a failing
  *     CUDA call (file, line, error string) on stderr and prints the shape of captured chunk graphs; RRM_PDL=1
  *     launches the kernels of a stack step with programmatic dependent launch (each kernel's set-up overlaps its
- *     predecessor's tail; off by default: measured, it does not pay inside replayed graphs); RRM_CHUNK_INPLACE=1
+ *     predecessor's tail; off by default: measured, it does not pay inside replayed graphs; the kernels of a lone FC
+ *     layer, which are plain launches, always use it); RRM_CHUNK_INPLACE=1
  *     makes the delta chunks of a stack (rrm_net_step_seq) add each frame's product straight onto the stored
  *     projection, as single steps do, instead of keeping it in a per-frame buffer that the epilogue merges (the
  *     default, which lets the convolution of frame t+1 run beside the epilogue of frame t; same results).
@@ -65,7 +66,8 @@ enum { RRM_F32 = 0, RRM_I8 = 1, RRM_BIN = 2 };
 enum { RRM_ACT_NONE = 0, RRM_ACT_RELU = 1, RRM_ACT_SIGN = 2,
        RRM_ACT_LEAKY = 3 /* fp32 only: x > 0 ? x : 0.1 x, the leaky ReLU of the YOLOv2-style stacks of Sec. 4.4 */ };
 /* How F*dI is evaluated.  As a request in rrm_layer_desc.variant: AUTO lets the library pick per layer: the kernel
- * (tensor cores for int8 and binary layers, CUDA cores for fp32) and, from the measured density, whether the layer
+ * (tensor cores; fp32 as three bf16 pieces per value, six products, at fp32 accuracy; the CUDA cores for the shapes
+ * those kernels do not take) and, from the measured density, whether the layer
  * runs the sparse product at all.  In a stack whose layers all ask for AUTO every layer's share of projection
  * pixels to update is read back after each delta step (asynchronously); a layer whose share reached
  * rrm_options.layer_dense_activity is evaluated densely inside the following delta steps (P = F*X + b from the
