@@ -38,7 +38,8 @@
 // with six separate MMAs and the barrier looked at only when it is needed); in a launch of a few tiles a chain of ~7 us (rows
 // and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  Against kernels that gathered rows tap by tap (fp32: on the
 // CUDA cores), AlexNet-shaped stack at 227 x 227: fp32 32 frames conv2 / conv4 351 / 412 (delta) -> 152 / 53 us (dense), 8
-// streams 546 -> 188 for the whole stack; int8 frame 84 -> 64.  fp32 tiles of 64 columns, two CTAs per SM, were slower
+// streams 546 -> 189 for the whole stack; int8 frame 84 -> 63.  Filling with a turn's loads ahead of its stores, and first
+// layers with one table for all planes: 8 fp32 streams 194 -> 189, 50 binary frames 167 -> 163, 32 int8 frames 147 -> 144.  fp32 tiles of 64 columns, two CTAs per SM, were slower
 // than 128 and one (conv2 152 -> 179, conv4 53 -> 83, 11x11 first layer 107 -> 111: every window is then filled twice as
 // often, and an MMA of 128 columns has no smem bandwidth to spare for it).
 #include "rrm_common.cuh"
@@ -111,7 +112,7 @@ struct WinTail {
     alignas(16) int bias[128];                // of the CTA's columns (f in the kernel)
     int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
     int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
-    int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row
+    int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row * 256 + input rows from the tap's first on (at most 255)
 };
 
 // ---- small device helpers
@@ -234,8 +235,10 @@ __device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_
             const int img = wn_div(lin, p.div_img), rem = lin - img * hwq, Y = wn_div(rem, p.div_row), X = rem - Y * p.Wq;
             const int iy = Y * p.stride + ry;
             if (XCOL) {
-                x0 = X * p.stride - p.pad;
-                if (img < p.n && iy < p.h) off = (img * p.h + iy) * p.w;
+                // (one table for all planes, which are rows further down: the first one's row, and how many rows are left)
+                const int y0 = Y * p.stride, left = min(p.h - y0, 255);
+                if (img < p.n && left > 0) off = (img * p.h + y0) * p.w;
+                x0 = (X * p.stride - p.pad) * 256 + max(left, 0);
             } else {
                 const int ix = X * p.stride + rx;
                 if (img < p.n && iy < p.h && ix < p.w) {
@@ -422,8 +425,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             }
             const bool new_plane = ib > 0 && chb == p.nchb;
             if (chb == p.nchb) { chb = 0; ++plane; }
-            const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0);
-            if (new_plane) {
+            const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0), ry = XCOL ? p.plane[plane].ry : 0;
+            if (new_plane && !XCOL) {
                 wn_meet();                                   // (everyone is done with the last plane's)
                 wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane);
                 wn_meet();
@@ -457,25 +460,35 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             } else if (DT == T_I8) {
                 // first layer, a 4-byte word per pixel: four neighbouring pixels of an image row are one chunk
                 const uint32_t* Aw = reinterpret_cast<const uint32_t*>(A);
-                #pragma unroll 4
-                for (int idx = tid; idx < items; idx += WN_FILL) {
+                auto fetch = [&](int idx, uint32_t (&v)[4]) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
-                    const int row = S->src[i], x = S->x0[i] + 4 * c;
-                    uint32_t v[4] = {0u, 0u, 0u, 0u};
-                    if (row >= 0) {
-                        unsigned bits = 0xfu;                // which of the four pixels count
-                        if (!DENSE) {
-                            const int g = max(row + x, 0), sh = g & 31;
-                            unsigned long long two = in_act[g >> 5];
-                            if (sh > 28 && row + p.w > ((g >> 5) + 1) * 32) two |= (unsigned long long)in_act[(g >> 5) + 1] << 32;
-                            bits = (unsigned)(two >> sh);
-                            if (row + x < 0) bits <<= -(row + x);
-                        }
-                        #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (x + e >= 0 && x + e < p.w && (bits >> e & 1u)) v[e] = Aw[row + x + e];
+                    const int row0 = S->src[i], xl = S->x0[i], row = row0 + ry * p.w, x = (xl >> 8) + 4 * c;
+                    v[0] = v[1] = v[2] = v[3] = 0u;
+                    if (row0 < 0 || ry >= (xl & 255)) return;
+                    unsigned bits = 0xfu;                    // which of the four pixels count
+                    if (!DENSE) {
+                        const int g = max(row + x, 0), sh = g & 31;
+                        unsigned long long two = in_act[g >> 5];
+                        if (sh > 28 && row + p.w > ((g >> 5) + 1) * 32) two |= (unsigned long long)in_act[(g >> 5) + 1] << 32;
+                        bits = (unsigned)(two >> sh);
+                        if (row + x < 0) bits <<= -(row + x);
                     }
-                    *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = make_uint4(v[0], v[1], v[2], v[3]);
+                    #pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (x + e >= 0 && x + e < p.w && (bits >> e & 1u)) v[e] = Aw[row + x + e];
+                };
+                // (a turn's loads are all on their way before its first store: the compiler does not move them across)
+                for (int idx = tid; idx < items; idx += 2 * WN_FILL) {
+                    uint32_t v[2][4];
+                    fetch(idx, v[0]);
+                    const bool two = idx + WN_FILL < items;
+                    if (two) fetch(idx + WN_FILL, v[1]);
+                    #pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (u > 0 && !two) break;
+                        const int id = idx + u * WN_FILL, i = magic ? (int)__umulhi((unsigned)id, magic) : id, c = id - i * cl;
+                        *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = make_uint4(v[u][0], v[u][1], v[u][2], v[u][3]);
+                    }
                 }
                 fence_async_smem();
                 mbar_arrive(smem_u32(&S->afull[buf]));
@@ -483,66 +496,91 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 // bits -> bytes: +2 / -2 per changed channel (dense: +1 / -1), 0 beyond the channels and outside the image
                 const uint32_t* Cu = reinterpret_cast<const uint32_t*>(A) + g0;
                 const uint32_t* Nu = reinterpret_cast<const uint32_t*>(Anew) + g0;
-                #pragma unroll 4
-                for (int idx = tid; idx < items; idx += WN_FILL) {
-                    const int i = (int)__umulhi((unsigned)idx, magic), c = idx - i * cl;      // (cl >= 2)
-                    const int off = S->src[i];
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (off >= 0) {
-                        const int ch0 = (g0 * 2 + c) * 16;
-                        const uint32_t valid = ch0 >= p.c_in ? 0u : (ch0 + 16 > p.c_in ? (1u << (p.c_in - ch0)) - 1u : 0xffffu);
-                        const int sh = (c & 1) * 16;
-                        const uint32_t nb = Nu[off + (c >> 1)] >> sh;
-                        uint32_t pos, neg;
-                        if (DENSE) { pos = nb & valid; neg = ~nb & valid; }
-                        else { const uint32_t ch = (Cu[off + (c >> 1)] >> sh) & valid; pos = ch & nb; neg = ch & ~nb; }
-                        const uint32_t pm = DENSE ? 0x01u : 0x02u, nm = DENSE ? 0xffu : 0xfeu;
-                        v.x = wn_spread4(pos) * pm + wn_spread4(neg) * nm;
-                        v.y = wn_spread4(pos >> 4) * pm + wn_spread4(neg >> 4) * nm;
-                        v.z = wn_spread4(pos >> 8) * pm + wn_spread4(neg >> 8) * nm;
-                        v.w = wn_spread4(pos >> 12) * pm + wn_spread4(neg >> 12) * nm;
+                // (a turn's loads are all on their way before its first store: the compiler does not move them across)
+                for (int idx = tid; idx < items; idx += 4 * WN_FILL) {
+                    uint32_t nw[4], cw4[4];
+                    int off[4];
+                    #pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int id = idx + u * WN_FILL, i = (int)__umulhi((unsigned)id, magic), c = id - i * cl;      // (cl >= 2)
+                        off[u] = id < items ? S->src[i] : -1;
+                        if (off[u] >= 0) {
+                            nw[u] = Nu[off[u] + (c >> 1)];
+                            if (!DENSE) cw4[u] = Cu[off[u] + (c >> 1)];
+                        }
                     }
-                    *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = v;
+                    #pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int id = idx + u * WN_FILL, i = (int)__umulhi((unsigned)id, magic), c = id - i * cl;
+                        if (id >= items) break;
+                        uint4 v = make_uint4(0, 0, 0, 0);
+                        if (off[u] >= 0) {
+                            const int ch0 = (g0 * 2 + c) * 16;
+                            const uint32_t valid = ch0 >= p.c_in ? 0u : (ch0 + 16 > p.c_in ? (1u << (p.c_in - ch0)) - 1u : 0xffffu);
+                            const int sh = (c & 1) * 16;
+                            const uint32_t nb = nw[u] >> sh;
+                            uint32_t pos, neg;
+                            if (DENSE) { pos = nb & valid; neg = ~nb & valid; }
+                            else { const uint32_t ch = (cw4[u] >> sh) & valid; pos = ch & nb; neg = ch & ~nb; }
+                            const uint32_t pm = DENSE ? 0x01u : 0x02u, nm = DENSE ? 0xffu : 0xfeu;
+                            v.x = wn_spread4(pos) * pm + wn_spread4(neg) * nm;
+                            v.y = wn_spread4(pos >> 4) * pm + wn_spread4(neg >> 4) * nm;
+                            v.z = wn_spread4(pos >> 8) * pm + wn_spread4(neg >> 8) * nm;
+                            v.w = wn_spread4(pos >> 12) * pm + wn_spread4(neg >> 12) * nm;
+                        }
+                        *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = v;
+                    }
                 }
                 fence_async_smem();
                 mbar_arrive(smem_u32(&S->afull[buf]));
             } else {
                 const float* Af = reinterpret_cast<const float*>(A);
                 const bool vec = (p.row_units & 3) == 0;
-                #pragma unroll 2
-                for (int idx = tid; idx < items; idx += WN_FILL) {
+                auto fetch = [&](int idx, float (&x)[8]) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
                     const int off = S->src[i];
-                    float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    if (off >= 0) {
-                        if (XCOL) {
-                            // two neighbouring pixels x 4 channels
-                            const int xx = S->x0[i] + 2 * (g0 * 2 + c);
-                            #pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int pix = off + xx + e;
-                                if (xx + e >= 0 && xx + e < p.w && (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u))) {
-                                    #pragma unroll
-                                    for (int ch = 0; ch < 4; ++ch) if (ch < p.c_in) x[e * 4 + ch] = Af[(size_t)pix * p.row_units + ch];
-                                }
-                            }
-                        } else {
-                            const int ch0 = (g0 * 2 + c) * 8;
-                            if (vec) {
-                                if (ch0 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0); x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w; }
-                                if (ch0 + 4 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0 + 4); x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w; }
-                            } else {
+                    #pragma unroll
+                    for (int j = 0; j < 8; ++j) x[j] = 0.f;
+                    if (XCOL) {
+                        // two neighbouring pixels x 4 channels
+                        const int xl = S->x0[i], xx = (xl >> 8) + 2 * (g0 * 2 + c);
+                        if (off < 0 || ry >= (xl & 255)) return;
+                        #pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int pix = off + ry * p.w + xx + e;
+                            if (xx + e >= 0 && xx + e < p.w && (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u))) {
                                 #pragma unroll
-                                for (int j = 0; j < 8; ++j) if (ch0 + j < p.c_in) x[j] = Af[off + ch0 + j];
+                                for (int ch = 0; ch < 4; ++ch) if (ch < p.c_in) x[e * 4 + ch] = Af[(size_t)pix * p.row_units + ch];
                             }
                         }
+                    } else if (off >= 0) {
+                        const int ch0 = (g0 * 2 + c) * 8;
+                        if (vec) {
+                            if (ch0 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0); x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w; }
+                            if (ch0 + 4 < p.c_in) { const float4 t = *reinterpret_cast<const float4*>(Af + off + ch0 + 4); x[4] = t.x; x[5] = t.y; x[6] = t.z; x[7] = t.w; }
+                        } else {
+                            #pragma unroll
+                            for (int j = 0; j < 8; ++j) if (ch0 + j < p.c_in) x[j] = Af[off + ch0 + j];
+                        }
                     }
+                };
+                auto put = [&](int idx, const float (&x)[8]) {
+                    const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
                     uint32_t s[3][4];
                     #pragma unroll
                     for (int j = 0; j < 4; ++j) wn_split(x[2 * j], x[2 * j + 1], s[0][j], s[1][j], s[2][j]);
                     unsigned char* dst = Ap + (size_t)(c * p.L + i) * 16;
                     #pragma unroll
                     for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + k * piece) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
+                };
+                // (a turn's loads are all on their way before its first store: the compiler does not move them across)
+                constexpr int TURN = 3;
+                for (int idx = tid; idx < items; idx += TURN * WN_FILL) {
+                    float x[TURN][8];
+                    #pragma unroll
+                    for (int u = 0; u < TURN; ++u) if (idx + u * WN_FILL < items) fetch(idx + u * WN_FILL, x[u]);
+                    #pragma unroll
+                    for (int u = 0; u < TURN; ++u) if (idx + u * WN_FILL < items) put(idx + u * WN_FILL, x[u]);
                 }
                 fence_async_smem();
                 mbar_arrive(smem_u32(&S->afull[buf]));
@@ -1114,7 +1152,7 @@ static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
     };
     const int e = d.dtype == RRM_F32 ? 16 : 32;              // K elements of a group
     p.groups = xcol ? ceil_div(d.kw * 4, e) : ceil_div(d.dtype == RRM_I8 ? in.cs : d.c_in, e);
-    if (xcol && p.groups > 4) return false;                  // (a block holds up to four K groups, a first layer's block all of them)
+    if (xcol && (p.groups > 4 || d.stride > 128)) return false;                  // (a block holds up to four K groups, a first layer's block all of them)
     // first layers: pixels of a 16-byte chunk; a row in one or two arrays where the stride is as many chunks
     const int px = d.dtype == RRM_F32 ? 2 : 4;
     p.xarr = xcol && d.stride % px == 0 && d.stride / px <= 2 ? d.stride / px : 0;
