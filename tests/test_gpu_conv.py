@@ -183,6 +183,16 @@ def test_window_convolution_tile_edges(dtype, c_in, c_out, hw, k, s, p, n, monke
     net.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "i8"])
+@pytest.mark.parametrize("hw,k,s,p,n", [
+    ((601, 18), 5, 4, 2, 1),                 # planes as rows further down: more rows left than the table counts, the last plane one row short
+    ((256, 17), 7, 2, 3, 2)])                # ... and exactly one more than it counts
+def test_first_layer_tables_of_tall_images(dtype, hw, k, s, p, n):
+    rng = np.random.default_rng(hw[0] + k)
+    sp = _spec(dtype, 3, hw, 20, k, s, p, rng)
+    _run([sp], _video(dtype, 3, hw, 4, n, rng), n=n, stats=True, keyframe_at=(3,))
+
+
 @pytest.mark.parametrize("dtype,c_in,c_out,hw,n", [
     ("f32", 3, 40, (9, 15), 2), ("f32", 4, 8, (320, 300), 2),         # a thread per pixel; four pixel groups per thread
     ("f32", 64, 36, (13, 9), 2), ("f32", 8, 5, (6, 6), 3),            # 16 lanes per pixel: full, and few of them at work
