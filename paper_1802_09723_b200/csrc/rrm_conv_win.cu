@@ -1180,6 +1180,7 @@ static bool win_geometry(const rrm_net* net, const Layer& L, WinParams& p)
     p.div_img = divisor(p.Hq * p.Wq); p.div_row = divisor(p.Wq);
     p.span = TC_M + max_shift - p.min_shift + reach;         // (one accumulator tile)
     if (p.span > WN_MAX_SPAN) return false;
+    if (((long long)d.n + 1) * p.Hq * p.Wq + 2 * p.span > INT_MAX) return false;      // (positions are int)
     // (rows of the linear space without a projection pixel are work for nothing: with more than half of them a layer
     // such as a filter that covers the whole map is better off with its rows compacted)
     if ((long long)L.oh * L.ow * 2 < (long long)p.Hq * p.Wq) return false;
@@ -1219,6 +1220,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     for (; mt >= 1; mt /= 2) {
         p.mt = mt;
         p.span = base_span + (mt - 1) * TC_M;
+        if (p.span > WN_MAX_SPAN) continue;                  // (the tables hold no wider window: one tile, which win_geometry has checked)
         p.L = slots(p.span);
         // drained rows: a tile's (64 columns of it where there are two), or 32 rows x 32 columns per warp
         const size_t whole = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4, turned = (size_t)8 * 32 * WN_TURN * 4;
@@ -1336,6 +1338,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     const bool batched = P_dst && frames >= 1 && arena_stride != 0;
     const int nf = batched ? frames : 1;
     if (!win_plan(L, p, xcol, dense, batched, nf, net->many_in_flight ? 74 : 148)) return RRM_ERR_UNSUPPORTED;
+    if (p.span > WN_MAX_SPAN) return RRM_ERR_CAPACITY;       // (never: win_plan takes no such window)
     const void* X = stateless ? in.X2 : in.X;
     p.A = bin ? in.D : (dense ? X : in.D);
     p.Anew = (!dense && !stateless && in.Xn_cur) ? in.Xn_cur : X;    // (chunks of frames: this frame's copy of the new rows)

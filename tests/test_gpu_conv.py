@@ -193,6 +193,30 @@ def test_first_layer_tables_of_tall_images(dtype, hw, k, s, p, n):
     _run([sp], _video(dtype, 3, hw, 4, n, rng), n=n, stats=True, keyframe_at=(3,))
 
 
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [
+    (3, 8, (480, 640), 7, 2, 3), (3, 8, (300, 512), 3, 1, 1), (2, 4, (1080, 1920), 11, 4, 0),      # first layers
+    (16, 8, (240, 470), 3, 1, 1)])                                                                 # ... and one of more channels
+def test_windows_of_wide_images_fit_their_tables(c_in, c_out, hw, k, s, p):
+    """int8 layers large enough for two accumulator tiles per thread block whose window fits the kernel's per-pixel tables
+    with one tile only (a span of 1025 to 1152 pixels): frame by frame, as a keyframe and in a dense chunk."""
+    rng = np.random.default_rng(hw[1] + k)
+    sp = _spec("i8", c_in, hw, c_out, k, s, p, rng)
+    video = _video("i8", c_in, hw, 4, 1, rng)
+    video[2:] = video[1]                                      # a patch at the image's far corner, one in its middle
+    video[2, :, :, -9:, -9:] ^= 1
+    video[3, :, :, hw[0] // 2:hw[0] // 2 + 9, hw[1] // 2:hw[1] // 2 + 9] ^= 3
+    net = _rrm().net_from_specs([sp])
+    out, outs = net.new_output(), net.new_output(frames=2)
+    want = [orc.dense_forward([sp], f)[0][1] for f in video[1:]]
+    for t, call in ((1, net.keyframe), (2, net.step), (3, net.step)):
+        call(dev(video[t]), out)
+        np.testing.assert_array_equal(out.cpu().numpy(), want[t - 1], err_msg=f"frame {t}")
+    net.dense_seq(dev(video[2:4]), outs, 2)
+    np.testing.assert_array_equal(outs.cpu().numpy(), np.stack(want[1:3]), err_msg="dense chunk")
+    assert net.stats(0)["error_word"] == 0
+    net.close()
+
+
 @pytest.mark.parametrize("dtype,c_in,c_out,hw,n", [
     ("f32", 3, 40, (9, 15), 2), ("f32", 4, 8, (320, 300), 2),         # a thread per pixel; four pixel groups per thread
     ("f32", 64, 36, (13, 9), 2), ("f32", 8, 5, (6, 6), 3),            # 16 lanes per pixel: full, and few of them at work
