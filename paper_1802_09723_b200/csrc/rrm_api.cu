@@ -682,7 +682,9 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
     const int L = (int)net->layers.size();
     RRM_TRY(ensure_chunk(net, T));
     RRM_TRY(ensure_stateless(net));
-    const int parts = ceil_div(T, DENSE_BATCH), per = ceil_div(T, parts);
+    // (images of a launch are at most 65535: the imports have them on grid.y)
+    const int most = net->n < 65535 / DENSE_BATCH ? DENSE_BATCH : (net->n < 65535 ? 65535 / net->n : 1);
+    const int parts = ceil_div(T, most), per = ceil_div(T, parts);
     RRM_TRY(ensure_dense_batch(net, per));
     int64_t bi = 0, bo = 0;
     tensor_bytes_boundary(net->tensors.front(), &bi);

@@ -882,15 +882,16 @@ __global__ void __launch_bounds__(256) import_i8_word_dense_kernel(const int8_t*
 
 // int8 between the boundary layout and whole 32-byte pixel rows, a 128-pixel x 32-channel tile at a time through shared
 // memory: rows as 16-byte groups, planes along the pixels (as words where a plane's address allows).  EXPORT: rows -> planes.
-// grid = (pixel tiles, channel tiles x n, frames).  30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread
+// grid = (pixel tiles x channel tiles x n, 1, frames): x alone has room for the product.  30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread
 // per element, import of 48 channels 10.8 -> 7.0 against the 32-pixel tiles.
 template <bool EXPORT>
-__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, int ctiles,
+__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, unsigned ptiles, unsigned ctiles,
                                                           long long src_stride, long long dst_stride)
 {
     __shared__ __align__(16) int8_t tile[32][132];
-    const int p0 = blockIdx.x * 128, c0 = (int)(blockIdx.y % ctiles) * 32;
-    const long long ns = blockIdx.y / ctiles;
+    const unsigned slab = blockIdx.x / ptiles, image = slab / ctiles;
+    const int p0 = (int)(blockIdx.x - slab * ptiles) * 128, c0 = (int)(slab - image * ctiles) * 32;
+    const long long ns = image;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, px = threadIdx.x >> 1, half = (threadIdx.x & 1) * 16;
     src += blockIdx.z * src_stride;
     dst += blockIdx.z * dst_stride;
@@ -1349,13 +1350,14 @@ __global__ void export_nchw_kernel(const T* __restrict__ src, T* dst, int c, int
 }
 
 // The same through a 32 x 32 tile in shared memory (4-byte elements): rows read along the channels, planes written
-// along the pixels, both coalesced.  grid = (pixel tiles, channel tiles x n, frames), block = (32, 8).
+// along the pixels, both coalesced.  grid = (pixel tiles x channel tiles x n, 1, frames), block = (32, 8).
 __global__ void __launch_bounds__(256) export_nchw_tiled_kernel(const uint32_t* __restrict__ src, uint32_t* dst, int c, int cs, int hw,
-                                                                int ctiles, long long src_stride, long long dst_stride)
+                                                                unsigned ptiles, unsigned ctiles, long long src_stride, long long dst_stride)
 {
     __shared__ uint32_t tile[32][33];
-    const int p0 = blockIdx.x * 32, c0 = (int)(blockIdx.y % ctiles) * 32;
-    const long long ns = blockIdx.y / ctiles;
+    const unsigned slab = blockIdx.x / ptiles, image = slab / ctiles;
+    const int p0 = (int)(blockIdx.x - slab * ptiles) * 32, c0 = (int)(slab - image * ctiles) * 32;
+    const long long ns = image;
     src += blockIdx.z * src_stride;
     dst += blockIdx.z * dst_stride;
     pdl_launch_dependents();
@@ -1560,9 +1562,9 @@ int launch_import(rrm_net* net, const void* frame, bool delta, bool stateless, c
             launch_seq(import_step_kernel<int8_t>, dim3(grid), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, (int8_t*)T.D, T.act, T.nnz, T.npix,
                        net->errw, T.c, T.cs, hw, T.w, T.readers);
         } else if (T.dtype == T_I8 && !delta) {
-            const int ctiles = T.cs / 32;
-            launch_seq(transpose_i8_kernel<false>, dim3(ceil_div(hw, 128), ctiles * T.n), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, T.c, T.cs, hw,
-                       ctiles, 0ll, 0ll);
+            const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
+            launch_seq(transpose_i8_kernel<false>, dim3(ptiles * ctiles * T.n), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, T.c, T.cs, hw,
+                       ptiles, ctiles, 0ll, 0ll);
         } else if (T.dtype == T_F32) {
             auto kd = import_nchw_kernel<float, true>;
             auto kn = import_nchw_kernel<float, false>;
@@ -1874,13 +1876,13 @@ int launch_export_tensor(rrm_net* net, int t, void* dst, bool stateless, cudaStr
     const long long total = (long long)T.n * T.c * hw;
     const int blocks = (int)((total + 255) / 256);
     if (T.dtype == T_I8 && T.cs % 32 == 0) {
-        const int ctiles = T.cs / 32;
-        launch_seq(transpose_i8_kernel<true>, dim3(ceil_div(hw, 128), ctiles * T.n, 1), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, ctiles, 0ll, 0ll);
+        const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
+        launch_seq(transpose_i8_kernel<true>, dim3(ptiles * ctiles * T.n), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, ptiles, ctiles, 0ll, 0ll);
     } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, dim3(blocks), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, total, 0ll, 0ll);
     else {
-        const int ctiles = ceil_div(T.c, 32);
-        launch_seq(export_nchw_tiled_kernel, dim3(ceil_div(hw, 32), ctiles * T.n, 1), dim3(32, 8), 0, st, (const uint32_t*)X, (uint32_t*)dst,
-                   T.c, T.cs, hw, ctiles, 0ll, 0ll);
+        const unsigned ptiles = ceil_div(hw, 32), ctiles = ceil_div(T.c, 32);
+        launch_seq(export_nchw_tiled_kernel, dim3(ptiles * ctiles * T.n), dim3(32, 8), 0, st, (const uint32_t*)X, (uint32_t*)dst,
+                   T.c, T.cs, hw, ptiles, ctiles, 0ll, 0ll);
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
@@ -1899,15 +1901,15 @@ int launch_export_seq(rrm_net* net, int frames, void* dst, cudaStream_t st)
     const long long total = (long long)T.n * T.c * hw;
     const dim3 grid((unsigned)((total + 255) / 256), (unsigned)frames);
     if (T.dtype == T_I8 && T.cs % 32 == 0) {
-        const int ctiles = T.cs / 32;
-        launch_seq(transpose_i8_kernel<true>, dim3(ceil_div(hw, 128), ctiles * T.n, frames), dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, ctiles,
+        const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
+        launch_seq(transpose_i8_kernel<true>, dim3(ptiles * ctiles * T.n, 1, frames), dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, ptiles, ctiles,
                    (long long)T.bytes(), total);
     } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, grid, dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, total,
                                     (long long)T.bytes(), total);
     else {
-        const int ctiles = ceil_div(T.c, 32);
-        launch_seq(export_nchw_tiled_kernel, dim3(ceil_div(hw, 32), ctiles * T.n, frames), dim3(32, 8), 0, st, (const uint32_t*)T.Xfull, (uint32_t*)dst,
-                   T.c, T.cs, hw, ctiles, (long long)T.bytes() / 4, total);
+        const unsigned ptiles = ceil_div(hw, 32), ctiles = ceil_div(T.c, 32);
+        launch_seq(export_nchw_tiled_kernel, dim3(ptiles * ctiles * T.n, 1, frames), dim3(32, 8), 0, st, (const uint32_t*)T.Xfull, (uint32_t*)dst,
+                   T.c, T.cs, hw, ptiles, ctiles, (long long)T.bytes() / 4, total);
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;

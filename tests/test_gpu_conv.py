@@ -243,6 +243,37 @@ def test_boundary_layouts(dtype, c_in, c_out, hw, n):
     net.close()
 
 
+@pytest.mark.parametrize("dtype,n,T", [("i8", 512, 1), ("i8", 16, 32), ("f32", 512, 1), ("f32", 16, 32)])
+def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
+    """Channel tiles x streams x frames of a launch at 65536, one more than a grid has along y: 4096 channels in (int8) and out."""
+    rng = np.random.default_rng(n + T)
+    dims = [(4096, 32), (32, 4096)] if dtype == "i8" else [(16, 4096)]
+    specs = []
+    for l, (a, b) in enumerate(dims):
+        kw = dict(act="relu", shift=12) if dtype == "i8" else {}
+        sp = _spec(dtype, a, (1, 1), b, 1, 1, 0, rng, **kw)
+        sp.src = l
+        specs.append(sp)
+    shape = (T, n, dims[0][0], 1, 1)
+    frames = rng.integers(0, 128, size=shape).astype(np.int8) if dtype == "i8" else rng.standard_normal(shape).astype(np.float32)
+    net = _rrm().net_from_specs(specs, n=n)
+    if T == 1:
+        outs = net.new_output()
+        net.keyframe(dev(frames[0]), outs)
+        got = [outs.cpu().numpy()]
+    else:
+        outs = net.new_output(frames=T)
+        net.dense_seq(dev(frames), outs, T)
+        got = outs.cpu().numpy()
+    for t in range(0, T, 31):
+        want = orc.dense_forward(specs, frames[t])[0][-1]
+        if dtype == "f32":
+            assert float(np.abs(got[t] - want).max()) <= F32_TOL * float(np.abs(want).max()), t
+        else:
+            np.testing.assert_array_equal(got[t].astype(np.int64), want, err_msg=f"frame {t}")
+    net.close()
+
+
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [(16, 70, (13, 13), 3, 1, 1), (8, 12, (17, 15), 5, 2, 2), (64, 16, (10, 10), 3, 1, 1),
                                                  (3, 6, (35, 35), 11, 4, 0)])
