@@ -193,7 +193,8 @@ int rrm_step_host(rrm_layer* layer, const void* Xt_host, void* Yt_host, void* st
  * next chunk densely on the tensor cores instead when that density was high: outputs, state and
  * counters are the same integers either way.  The first call with a larger T than any before
  * allocates scratch memory (T * N * c_out * 4 bytes); later calls do not.
- * T * N must not exceed 65535.  Asynchronous on `stream`.  After the call rrm_get_stats reports the
+ * T * N must not exceed 65535.  For a lone int8 FC layer X_dev (here and in the calls of one frame) must be 16-byte
+ * aligned, and Y_dev here as well (int8 outputs: 4-byte): RRM_ERR_INVALID_ARG otherwise.  Asynchronous on `stream`.  After the call rrm_get_stats reports the
  * counters summed over the chunk's frames (lone int8 FC layer) or those of the chunk's last frame (other layers). */
 int rrm_step_seq(rrm_layer* layer, const void* X_dev, void* Y_dev, int T, void* stream);
 /* T frames through the dense path, each on its own (Y_t = f(F*X_t + b)); RRM state untouched. */

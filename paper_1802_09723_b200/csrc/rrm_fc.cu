@@ -449,6 +449,7 @@ int fc_fused_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, bool de
 {
     const int C = L.d.c_in, K = L.d.c_out, n = L.d.n;
     const int slices = ceil_div(K, FC_OW);
+    if (reinterpret_cast<uintptr_t>(X_dev) & 15) return RRM_ERR_INVALID_ARG;    // every kernel reads the rows in 16-byte pieces
     // (without the few-row tensor-core form a handful of rows is served faster by the gather kernel with every entry active)
     if (dense && L.tc_ready && (n >= 4 || fc_tc_usable(L, n))) return fc_dense_tc_run(net, L, X_dev, Y_dev, 1, stateless, st);
     FcParams p;

@@ -415,7 +415,10 @@ static unsigned long long* seq_ask_counters(Layer& L, int rows)
 {
     if (L.seq_pending_rows > 0) return nullptr;
     if (rows > L.seq_stat_host_cap) {
-        if (L.seq_stat_host) cudaFreeHost(L.seq_stat_host);
+        if (L.seq_stat_host) {
+            cudaDeviceSynchronize();                         // (a chunk given up half-way may still write to the old words)
+            cudaFreeHost(L.seq_stat_host);
+        }
         L.seq_stat_host = nullptr; L.seq_stat_host_cap = 0;
         if (cudaMallocHost(reinterpret_cast<void**>(&L.seq_stat_host), (size_t)rows * 8) != cudaSuccess) { cudaGetLastError(); return nullptr; }
         for (int i = 0; i < rows; ++i) L.seq_stat_host[i] = 0;
@@ -501,11 +504,12 @@ bool fc_seq_supported(const Layer& L) { return L.fc_fused && L.d.c_in <= SQ_MAX_
 
 // T frames of every stream in one launch.  dense: every entry is visited and frames are independent
 // (P_t = b + W X_t); stateless: the RRM state (snapshot, stored projection) is left untouched.
-int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bool dense, bool stateless, cudaStream_t st)
+static int fc_seq_launch(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bool dense, bool stateless, cudaStream_t st)
 {
     const int C = L.d.c_in, K = L.d.c_out, n = L.d.n;
     if (T < 1) return RRM_ERR_INVALID_ARG;
     if ((long long)T * n > 65535) return RRM_ERR_CAPACITY;
+    if (reinterpret_cast<uintptr_t>(X_dev) & 15) return RRM_ERR_INVALID_ARG;    // every kernel reads the rows in 16-byte pieces
     if (dense && stateless && L.tc_ready) return fc_dense_tc_run(net, L, X_dev, Y_dev, T, true, st);
     RRM_TRY(seq_ensure(net, L, T));
     FcSeqParams p;
@@ -535,6 +539,7 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
                                                        : L.seq_density >= (double)net->opt.fc_dense_density);
         L.seq_last_T = T;
         L.seq_last_variant = use_dense ? RRM_VARIANT_DENSE : (L.Wsp ? RRM_VARIANT_SPARSE_W : RRM_VARIANT_GATHER);
+        if (!use_dense && (reinterpret_cast<uintptr_t>(Y_dev) & (L.d.shift < 0 ? 15 : 3))) return RRM_ERR_INVALID_ARG;
         unsigned long long* const host = seq_ask_counters(L, T * n);
         p.host = host; p.epoch = L.seq_epoch;
         if (use_dense) {
@@ -588,6 +593,14 @@ int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bo
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
+}
+
+int fc_seq_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int T, bool dense, bool stateless, cudaStream_t st)
+{
+    const unsigned asked = L.seq_epoch;
+    const int status = fc_seq_launch(net, L, X_dev, Y_dev, T, dense, stateless, st);
+    if (status != RRM_OK && L.seq_epoch != asked) L.seq_pending_rows = 0;    // counters of a chunk that was not launched never arrive
+    return status;
 }
 
 // ------------------------------------------------------------------------------------------------

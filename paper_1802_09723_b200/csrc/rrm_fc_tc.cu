@@ -418,6 +418,7 @@ int fc_tc_run(rrm_net* net, Layer& L, const void* X_dev, void* Y_dev, int rows, 
 {
     const int C = L.d.c_in, K = L.d.c_out, n = L.d.n;
     if (reinterpret_cast<uintptr_t>(X_dev) & 15) return RRM_ERR_INVALID_ARG;    // the copy engine wants 16-byte aligned rows
+    if (L.ft_cluster && (reinterpret_cast<uintptr_t>(Y_dev) & (L.d.shift < 0 ? 15 : 3))) return RRM_ERR_INVALID_ARG;   // (outputs in fours)
     const FtPlan f = ft_plan(L);
     FtParams p;
     p.Wimg = L.tc_Wimg;

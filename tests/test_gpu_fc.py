@@ -273,6 +273,36 @@ def test_fc6_dense_chunks_take_over_at_high_measured_density():
     layer.close()
 
 
+def test_refused_chunk_does_not_stop_the_density_measurement():
+    """A chunk of misaligned frames is refused; the chunks after it are measured as before: dense while the input is busy,
+    back to the column gather once it is still."""
+    rrm = _rrm()
+    c_in, T = 1024, 8
+    spec = wl.fc6_i8(c_in=c_in, c_out=512)[0]
+    seq = wl.fc_run_sequence(frames=2 * T + 1, c_in=c_in, rho=0.5, seed=31)
+    layer = rrm.layer_from_spec(spec)
+    frames, Y = dev(seq), layer.new_output(frames=T)
+    layer.keyframe(frames[0], None)
+    odd = torch.empty(T * c_in + 1, dtype=torch.int8, device="cuda")[1:]
+    variants = []
+    for first in (1, 1 + T):
+        with pytest.raises(rrm.RRMError):
+            layer.step_seq(odd, Y, T)
+        layer.step_seq(frames[first:first + T], Y, T)
+        variants.append(layer.stats(0)["variant"])            # synchronises: the counters have arrived at the next call
+    with pytest.raises(rrm.RRMError):
+        layer.step_seq(odd, Y, T)
+    still = frames[2 * T].expand(T, *frames.shape[1:]).contiguous()
+    for _ in range(3):
+        layer.step_seq(still, Y, T)
+        variants.append(layer.stats(0)["variant"])
+    want = orc.dense_forward([spec], seq[2 * T])[0][1]
+    for i in (0, T - 1):
+        np.testing.assert_array_equal(Y[i].cpu().numpy().astype(np.int64), want)
+    assert variants[1] == 3 and variants[-1] == 1, variants
+    layer.close()
+
+
 # ------------------------------------------------------------------ few-row dense FC on the tensor cores
 @pytest.mark.parametrize("c_in,c_out,shift,act,n,T", [
     (9216, 4096, -1, "none", 1, 1),       # one row: the keyframe / rrm_dense of the fc6 shape
