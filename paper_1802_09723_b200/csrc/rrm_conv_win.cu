@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         if (active && tid == 0 && ntile == 0 && split == 0) {
             int* oc = shift_bytes(p.ocount, arena_off);
             atomicAdd(oc, active);
-            if (!DENSE) atomicAdd(oc + 1, p.mt);              // accumulator tiles with work: what this kernel's time follows
+            atomicAdd(oc + 1, p.mt);                         // accumulator tiles with work (dense inside a delta step: that a delta would have)
         }
     }
     const uint32_t tmem = S->tmem_base;

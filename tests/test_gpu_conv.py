@@ -682,6 +682,34 @@ def test_chunks_of_eight_frames_go_dense_by_their_accumulator_tiles(dtype, T):
     net.close()
 
 
+def test_layers_dense_inside_delta_chunks_count_their_accumulator_tiles():
+    """A layer that the per-layer choice evaluates densely inside delta chunks still reports how many accumulator tiles its
+    update would touch, so that a chunk in which everything changes lets the next one go dense as a whole."""
+    rng = np.random.default_rng(77)
+    T, sp = 8, _spec("i8", 40, (64, 64), 36, 3, 1, 1, rng)
+    video = np.empty((1 + 3 * T, 1, 40, 64, 64), np.int8)
+    video[0] = rng.integers(0, 128, size=video[0].shape)
+    for t in range(1, 1 + T):                                 # an eighth of the rows changes: enough for the layer, too little for the chunk
+        video[t] = video[t - 1]
+        video[t, :, :, :8] = 127 - video[t - 1, :, :, :8]
+    for t in range(1 + T, 1 + 3 * T):
+        video[t] = 127 - video[t - 1]
+    net = _rrm().net_from_specs([sp])
+    net.set_options(layer_dense_activity=0.1, layer_delta_activity=0.05, chunk_dense_activity=0.5, stack_dense_activity=2.0)
+    net.keyframe(dev(video[0]))
+    outs, seen = net.new_output(frames=T), []
+    for k in range(3):
+        net.step_seq(dev(video[1 + k * T:1 + (k + 1) * T]), outs, T)
+        st = net.stats(0)                                     # synchronises: the next call sees this chunk's counters
+        seen.append((st["variant"], st["nnz_elems"] >= 0))
+        for i in (0, T - 1):
+            want = orc.dense_forward([sp], video[1 + k * T + i])[0][1]
+            np.testing.assert_array_equal(outs[i].cpu().numpy().astype(np.int64), want, err_msg=f"chunk {k} frame {i}")
+    # sparse; dense inside the delta step, counted; dense as a whole, nothing counted
+    assert seen == [(2, True), (3, True), (3, False)], seen
+    net.close()
+
+
 def test_dense_chunks_longer_than_one_batch():
     """Dense chunks are batched over their frames, 32 at most per launch: a chunk of 40 frames of two streams goes in
     two parts.  rrm_net_dense_seq leaves the state alone; a chunk that the density switch evaluates densely leaves
