@@ -937,13 +937,6 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
             RRM_TRY(bind_readers(net));
             return s == RRM_ERR_ALLOC ? s : RRM_ERR_UNSUPPORTED;
         }
-        // the dense form of the same chunk, which the measured activity may ask for in the very next call, is captured
-        // here too, so that no later call of this length pays for it
-        if (kind == 0 && long_chunk && net->opt.chunk_dense_activity <= 1.f) {
-            bool have = false;
-            for (auto& c : net->chunk_graphs[1]) have = have || c.T == T;
-            if (!have && build_dense_batch_graph(net, 1, T) != RRM_OK) cudaGetLastError();
-        }
     }
     // the structures describe the last frame of the chunk from here on (statistics, activity read-back)
     bind_arena(net, net->chunk_arena[find()->last_arena]);

@@ -710,6 +710,39 @@ def test_layers_dense_inside_delta_chunks_count_their_accumulator_tiles():
     net.close()
 
 
+def test_chunks_that_never_go_dense_take_no_memory_for_it():
+    """The frame-batched dense form of long chunks is set up once the measured activity asks for it, not with the first
+    delta chunk."""
+    rng = np.random.default_rng(78)
+    T, sp = 16, _spec("i8", 64, (120, 120), 64, 3, 1, 1, rng)
+    still = rng.integers(0, 128, size=(1, 1, 64, 120, 120)).astype(np.int8).repeat(1 + T, 0)
+    frames = dev(still)
+    busy = frames.clone()
+    busy[1::2] = 127 - busy[1::2]
+
+    def taken(threshold, *chunks):
+        net = _rrm().net_from_specs([sp])
+        net.set_options(chunk_dense_activity=threshold, stack_dense_activity=2.0)
+        outs = net.new_output(frames=T)
+        net.keyframe(frames[0])
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        for c in chunks:
+            net.step_seq(c[1:], outs, T)
+            torch.cuda.synchronize()
+        after = torch.cuda.mem_get_info()[0]
+        variant = net.stats(0)["variant"]
+        net.close()
+        return before - after, variant
+
+    batch = T * 120 * 120 * 64 * 2                            # the batched input and output tensors, at least
+    never, v0 = taken(2.0, frames, frames)
+    quiet, v1 = taken(0.4, frames, frames)
+    dense, v2 = taken(0.4, busy, busy)
+    assert (v0, v1, v2) == (2, 2, 3)
+    assert abs(quiet - never) < batch // 4 and dense - never >= batch // 2, (never, quiet, dense, batch)
+
+
 def test_dense_chunks_longer_than_one_batch():
     """Dense chunks are batched over their frames, 32 at most per launch: a chunk of 40 frames of two streams goes in
     two parts.  rrm_net_dense_seq leaves the state alone; a chunk that the density switch evaluates densely leaves
