@@ -947,6 +947,12 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
     rrm_net::ChunkGraph* cg = find();
     cg->used = ++net->chunk_clock;
     if (cg->io.ok) {                                         // the graph works on the caller's buffers
+        // (a chunk in several parts writes outputs before it reads its last frames: overlapping ones are read from a copy)
+        const char *in0 = reinterpret_cast<const char*>(frames), *out0 = reinterpret_cast<const char*>(outs);
+        if (outs && out0 < in0 + (size_t)bi * T && in0 < out0 + (size_t)bo * T) {
+            RRM_CUDA_TRY(cudaMemcpyAsync(net->chunk_in, frames, (size_t)bi * T, cudaMemcpyDeviceToDevice, st));
+            frames = net->chunk_in;
+        }
         if (patch_io(cg->exec, cg->io, frames, outs ? outs : net->chunk_out) != RRM_OK) {
             // an update failed half-way: the graph is no longer trusted
             cudaGetLastError();

@@ -743,6 +743,23 @@ def test_chunks_that_never_go_dense_take_no_memory_for_it():
     assert abs(quiet - never) < batch // 4 and dense - never >= batch // 2, (never, quiet, dense, batch)
 
 
+@pytest.mark.parametrize("shift", [0, 7])
+def test_dense_chunks_whose_outputs_overlap_their_frames(shift):
+    """40 frames go in two parts; the first part's outputs lie on frames of the second."""
+    rng = np.random.default_rng(79)
+    T, sp = 40, _spec("i8", 64, (9, 10), 64, 3, 1, 1, rng, act="relu", shift=9)
+    video = rng.integers(0, 128, size=(T, 1, 64, 9, 10)).astype(np.int8)
+    net = _rrm().net_from_specs([sp])
+    both = torch.zeros((T + shift, 1, 64, 9, 10), dtype=torch.int8, device="cuda")
+    for _ in range(2):
+        both[:T] = dev(video)
+        net.dense_seq(both[:T], both[shift:], T)
+        got = both[shift:].cpu().numpy()
+        for t in range(T):
+            np.testing.assert_array_equal(got[t].astype(np.int64), orc.dense_forward([sp], video[t])[0][1], err_msg=f"frame {t}")
+    net.close()
+
+
 def test_dense_chunks_longer_than_one_batch():
     """Dense chunks are batched over their frames, 32 at most per launch: a chunk of 40 frames of two streams goes in
     two parts.  rrm_net_dense_seq leaves the state alone; a chunk that the density switch evaluates densely leaves
