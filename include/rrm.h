@@ -66,8 +66,10 @@ enum { RRM_F32 = 0, RRM_I8 = 1, RRM_BIN = 2 };
 enum { RRM_ACT_NONE = 0, RRM_ACT_RELU = 1, RRM_ACT_SIGN = 2,
        RRM_ACT_LEAKY = 3 /* fp32 only: x > 0 ? x : 0.1 x, the leaky ReLU of the YOLOv2-style stacks of Sec. 4.4 */ };
 /* How F*dI is evaluated.  As a request in rrm_layer_desc.variant: AUTO lets the library pick per layer: the kernel
- * (tensor cores; fp32 as three bf16 pieces per value, six products, at fp32 accuracy; the CUDA cores for the shapes
- * those kernels do not take) and, from the measured density, whether the layer
+ * (tensor cores; fp32 as three bf16 pieces per value, six products, at fp32 accuracy for normal numbers of any size;
+ * infinities, NaNs and values beyond bf16's largest, 3.39e38, act as in fp32 arithmetic, but the 128 output pixels around
+ * one are then summed without the tensor cores, slowly; the CUDA cores for the shapes those kernels do not take and for
+ * fp32 layers with such a filter value) and, from the measured density, whether the layer
  * runs the sparse product at all.  In a stack whose layers all ask for AUTO every layer's share of projection
  * pixels to update is read back after each delta step (asynchronously); a layer whose share reached
  * rrm_options.layer_dense_activity is evaluated densely inside the following delta steps (P = F*X + b from the

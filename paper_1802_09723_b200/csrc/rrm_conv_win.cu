@@ -22,9 +22,13 @@
 //
 // fp32 layers: every operand is split into three bf16 pieces (8 + 8 + 8 bits: all 24 bits of the significand), and six
 // of the nine products of pieces are formed; what the other three would add is below 2^-25 of a product, less than the
-// rounding of one fp32 multiplication.  The tensor core adds in fp32 but truncates, so the leading product has an
-// accumulator that is added to registers (round to nearest) after at most WN_PROMOTE K steps of 16, and the five
-// small ones have two of their own.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
+// rounding of one fp32 multiplication.  The second and third piece are kept 2^9 and 2^18 times as large, so that the pieces
+// of small values do not fall below bf16's exponents; the products of equal scale share an accumulator.  The tensor core
+// adds in fp32 but truncates, so the leading product has an accumulator that is added to registers (round to nearest)
+// after at most WN_PROMOTE K steps of 16, and the five small ones have two of their own.  A value whose first piece is no
+// finite number (an infinity, a NaN, or a float above bf16's largest) makes its third piece a NaN, by which a CTA notices
+// it: such a CTA forms its sums one by one from the operands instead (wn_exact_row), and a layer with such a filter
+// keeps the CUDA cores.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
 // a chain of fmaf 6e-7; without the promotion 1.7e-6, with everything in one accumulator 1.5e-5.
 //
 // Roles: warps 0-7 fill windows and drain accumulators, warp 8 issues the MMAs, warp 9 the bulk copies of the filters
@@ -109,6 +113,7 @@ struct WinTail {
     unsigned long long afull[WN_MAX_ABUF], aempty[WN_MAX_ABUF], bfull[WN_MAX_STAGES], bempty[WN_MAX_STAGES], dfull[2], dempty[2], done;
     uint32_t tmem_base;
     int fail;
+    int exact;                                // fp32: a window holds a value whose pieces are no finite numbers
     alignas(16) int bias[128];                // of the CTA's columns (f in the kernel)
     int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
     int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
@@ -132,9 +137,9 @@ __device__ __forceinline__ void wn_step_i8(uint32_t d, uint32_t a_lo, uint32_t b
         ::"r"(d), "r"(a_lo), "r"(b_lo), "r"(WN_DESC_HI), "r"(idesc), "r"(accumulate), "r"(e) : "memory");
 }
 // fp32: six products of pieces in four MMAs.  A filter tile's pieces lie side by side along the columns, so an MMA of twice
-// the width adds one input piece times two filter pieces to the two accumulators of small products at d1:
-// a0 * (b1, b2), a1 * (b0, b1), a2 * b0; the leading a0 * b0 goes to d0.
-__device__ __forceinline__ void wn_step_f32(uint32_t d0, uint32_t d1, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t b0, uint32_t b1, uint32_t idesc,
+// the width adds one input piece times two filter pieces to the two accumulators of small products, d1 (scale 2^9) and d2
+// (2^18) right behind it: a0 * (b1, b2), a1 * (b0, b1), and a2 * b0 to d2; the leading a0 * b0 goes to d0.
+__device__ __forceinline__ void wn_step_f32(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t b0, uint32_t b1, uint32_t idesc,
                                             uint32_t idesc2, uint32_t acc0, uint32_t acc1, uint32_t e)
 {
     asm volatile(
@@ -143,9 +148,9 @@ __device__ __forceinline__ void wn_step_f32(uint32_t d0, uint32_t d1, uint32_t a
         "setp.ne.b32 p, %10, 0;\n\tsetp.ne.b32 r, %11, 0;\n\tsetp.ne.b32 q, %12, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%1], x, v, %9, r;\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%1], y, u, %9, t;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%1], z, u, %8, t;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%13], z, u, %8, t;\n\t"
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], x, u, %8, p;\n\t}"
-        ::"r"(d0), "r"(d1), "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(WN_DESC_HI), "r"(idesc), "r"(idesc2), "r"(acc0), "r"(acc1), "r"(e) : "memory");
+        ::"r"(d0), "r"(d1), "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(WN_DESC_HI), "r"(idesc), "r"(idesc2), "r"(acc0), "r"(acc1), "r"(e), "r"(d2) : "memory");
 }
 // one look at a barrier
 __device__ __forceinline__ uint32_t mbar_poll(uint32_t bar, uint32_t parity)
@@ -182,6 +187,14 @@ __device__ __forceinline__ void wn_ld32(uint32_t taddr, uint32_t (&v)[32])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void wn_zero32(uint32_t taddr)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+        "%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr), "r"(0u) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 // the filling warps agree (and meet): true only if all of them say so
 __device__ __forceinline__ bool wn_agree(bool ok)
 {
@@ -209,15 +222,23 @@ __device__ __forceinline__ uint4 wn_ld_remote(uint32_t addr, uint32_t rank)
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr), "r"(rank) : "memory");
     return v;
 }
-// two floats -> their three bf16 pieces, packed (low half: the first float)
+// two floats -> their three bf16 pieces, packed (low half: the first float); the second 2^9, the third 2^18 times as large
+constexpr float WN_SCALE = 512.f;
 __device__ __forceinline__ void wn_split(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2)
 {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(b), "f"(a));
-    a -= __uint_as_float(p0 << 16); b -= __uint_as_float(p0 & 0xffff0000u);
+    a = (a - __uint_as_float(p0 << 16)) * WN_SCALE; b = (b - __uint_as_float(p0 & 0xffff0000u)) * WN_SCALE;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(b), "f"(a));
-    a -= __uint_as_float(p1 << 16); b -= __uint_as_float(p1 & 0xffff0000u);
+    a = (a - __uint_as_float(p1 << 16)) * WN_SCALE; b = (b - __uint_as_float(p1 & 0xffff0000u)) * WN_SCALE;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(b), "f"(a));
 }
+// a pair of bf16 sums that a NaN among the addends has made one
+__device__ __forceinline__ uint32_t wn_bf16_add(uint32_t a, uint32_t b)
+{
+    asm("add.rn.bf16x2 %0, %0, %1;" : "+r"(a) : "r"(b));
+    return a;
+}
+__device__ __forceinline__ bool wn_bf16_nan(uint32_t a) { return (a & 0x7fffu) > 0x7f80u || (a >> 16 & 0x7fffu) > 0x7f80u; }
 __device__ __forceinline__ uint32_t wn_spread4(uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; }
 __device__ __forceinline__ int wn_div(int x, const WinDiv& d) { return (int)((unsigned long long)(unsigned)x * d.m >> d.sh); }
 
@@ -303,6 +324,45 @@ __device__ __forceinline__ uint32_t wn_f8(const WinParams& p, int c, const int (
     return wn_f8_plain(x, res, p.shift > 0 ? 1 << (p.shift - 1) : 0, p.shift, p.act_fn == RRM_ACT_RELU ? 0 : -127, p.res != nullptr);
 }
 
+// fp32, the way out of windows with infinities, NaNs or values beyond bf16: one row's share of the sums, columns c_lo to
+// c_hi of the tile, from the operands themselves (blocks b0 to b1; a filter value is the sum of its pieces).  lin: the
+// row's position, or -1.  Out of line: ordinary data never come here.
+template <bool DENSE, bool XCOL>
+__device__ __noinline__ void wn_exact_row(const WinParams& p, const float* A, const uint32_t* in_act, int lin, int ntile, int b0, int b1,
+                                          int c_lo, int c_hi, float* sums)
+{
+    for (int c = c_lo; c < c_hi; ++c) sums[c] = 0.f;
+    if (lin < 0) return;
+    const int hwq = p.Hq * p.Wq;
+    const int img = wn_div(lin, p.div_img), rem = lin - img * hwq, oy = wn_div(rem, p.div_row), ox = rem - oy * p.Wq;
+    const int row_taps = XCOL ? 1 : p.kw;
+    for (int b = b0; b < b1; ++b) {
+        const WinPlane& a = p.plane[b / p.nchb];
+        const int k_lo = (b % p.nchb) * p.gblk * 16, k_hi = min(k_lo + p.gblk * 16, XCOL ? p.kw * 4 : p.c_in);
+        for (int t = 0; t < a.ny * a.nx; ++t) {
+            const int ky = a.ky0 + t / a.nx * p.stride, kx0 = a.kx0 + t % a.nx * p.stride;
+            const int iy = oy * p.stride - p.pad + ky;
+            if (iy < 0 || iy >= p.h) continue;
+            const unsigned char* W = p.Wimg + ((size_t)ntile * row_taps * p.kh + (XCOL ? ky : ky * p.kw + kx0)) * p.groups * p.bn * 96;
+            for (int k = k_lo; k < k_hi; ++k) {
+                const int ix = ox * p.stride - p.pad + (XCOL ? k >> 2 : kx0), ci = XCOL ? k & 3 : k;
+                if (ix < 0 || ix >= p.w || ci >= p.c_in) continue;
+                const int pix = (img * p.h + iy) * p.w + ix;
+                if (!DENSE && !((in_act[pix >> 5] >> (pix & 31)) & 1u)) continue;
+                const float x = A[(size_t)pix * p.row_units + ci];
+                if (x == 0.f) continue;                      // (the filters are finite)
+                for (int c = c_lo; c < c_hi; ++c) {
+                    const unsigned short* w = reinterpret_cast<const unsigned short*>(W + (size_t)(k >> 3) * p.bn * 48 + (size_t)c * 16) + (k & 7);
+                    float v = __uint_as_float((uint32_t)w[0] << 16);
+                    v = fmaf(__uint_as_float((uint32_t)w[p.bn * 8] << 16), 1.f / WN_SCALE, v);
+                    v = fmaf(__uint_as_float((uint32_t)w[p.bn * 16] << 16), 1.f / (WN_SCALE * WN_SCALE), v);
+                    sums[c] = fmaf(x, v, sums[c]);
+                }
+            }
+        }
+    }
+}
+
 // DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.  ACT (dense passes): f is applied here and the output written,
 // instead of the projection by this kernel and f by another; the projection is stored only where a state needs it.
 template <int DT, bool DENSE, bool XCOL, bool ACT>
@@ -345,7 +405,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == WN_FILL + 32) {
-        S->fail = 0;
+        S->fail = 0; S->exact = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&S->bfull[s]), 1); mbar_init(smem_u32(&S->bempty[s]), 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -536,6 +596,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             } else {
                 const float* Af = reinterpret_cast<const float*>(A);
                 const bool vec = (p.row_units & 3) == 0;
+                uint32_t thirds = 0;                         // sums of the third pieces
                 auto fetch = [&](int idx, float (&x)[8]) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
                     const int off = S->src[i];
@@ -569,6 +630,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     uint32_t s[3][4];
                     #pragma unroll
                     for (int j = 0; j < 4; ++j) wn_split(x[2 * j], x[2 * j + 1], s[0][j], s[1][j], s[2][j]);
+                    #pragma unroll
+                    for (int j = 0; j < 4; ++j) thirds = wn_bf16_add(thirds, s[2][j]);
                     unsigned char* dst = Ap + (size_t)(c * p.L + i) * 16;
                     #pragma unroll
                     for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + k * piece) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
@@ -584,6 +647,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 }
                 fence_async_smem();
                 mbar_arrive(smem_u32(&S->afull[buf]));
+                if (wn_bf16_nan(thirds)) *(volatile int*)&S->exact = 1;
                 if (ib > 0 && !promote(ib - 1)) { *(volatile int*)&S->fail = 1; ok = false; }
                 // (a warp whose wait ran out says so when the warps meet at the next block)
             }
@@ -675,7 +739,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     #pragma unroll
                     for (int g = 0; g < 4; ++g) {
                         if (g >= gn) break;
-                        if (DT == T_F32) wn_step_f32(d0, d1, a_lo, a_lo + a_piece, a_lo + 2 * a_piece, b_lo, b_lo + bn, idesc, idesc2, fresh, first, e);
+                        if (DT == T_F32) wn_step_f32(d0, d1, d1 + bn, a_lo, a_lo + a_piece, a_lo + 2 * a_piece, b_lo, b_lo + bn, idesc, idesc2, fresh, first, e);
                         else {
                             wn_step_i8(d0, a_lo, b_lo, idesc, g == 0 ? first : 1u, e);
                             if (p.mt > 1) wn_step_i8(d1, a_lo + TC_M, b_lo, idesc, g == 0 ? first : 1u, e);
@@ -721,6 +785,20 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         if (ok && !mbar_wait(smem_u32(&S->done), 0, p.wait_limit)) { ok = false; *(volatile int*)&S->fail = 1; atomicOr(p.errw, ERRW_TIMEOUT); }
         ok = wn_agree(ok && *(volatile int*)&S->fail == 0);   // nobody stores results of a tile that gave up
         tc_fence_after();
+    }
+    if (DT == T_F32 && warp < 8 && ok && *(volatile int*)&S->exact) {         // (the same for all of them)
+        const int r = (warp & 3) * 32 + lane;
+        float* sums = reinterpret_cast<float*>(base) + (size_t)r * (p.bn + 1);   // (odd rows; fewer words than the drained rows')
+        wn_exact_row<DENSE, XCOL>(p, reinterpret_cast<const float*>(A), in_act, S->q[r] >= 0 ? lin0 + r : -1, ntile, b0, b1, c_lo, c_hi, sums);
+        #pragma unroll
+        for (int j = 0; j < 64; ++j) facc[DT == T_F32 ? j : 0] = c_lo + j < c_hi ? sums[c_lo + j] : 0.f;
+        __syncwarp();
+        #pragma unroll 1
+        for (int k = 0; k < 64 && c_lo + k < c_hi; k += 32) {                  // nothing is added to them
+            wn_zero32(tmem + lane_base + (uint32_t)(2 * p.bn + c_lo + k));
+            wn_zero32(tmem + lane_base + (uint32_t)(3 * p.bn + c_lo + k));
+        }
+        wn_meet();                                           // everyone has read its sums: the rows may be written over
     }
     const bool direct = ACT && DT != T_F32 && !p.cluster;    // f straight from the accumulator registers
     if (ACT && DT != T_F32 && direct && warp < 8 && ok) {
@@ -873,12 +951,12 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         if (DT == T_F32) {
             wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + cc), v);
             #pragma unroll
-            for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? k + j : 0] += __uint_as_float(v[j]);
+            for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? k + j : 0] = fmaf(__uint_as_float(v[j]), 1.f / (WN_SCALE * WN_SCALE), facc[DT == T_F32 ? k + j : 0]);
         }
         wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + cc), v);
         if (DT == T_F32) {
             #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + facc[DT == T_F32 ? k + j : 0]);
+            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaf(__uint_as_float(v[j]), 1.f / WN_SCALE, facc[DT == T_F32 ? k + j : 0]));
         }
     };
     if (!direct && !p.cluster && !bulk_add) {
@@ -1084,9 +1162,10 @@ int launch_pool_window(const Layer& L, const Tensor& out, const void* A, void* X
 // Filters as operand tiles: [n tile][tap][group][2 chunks][pieces][bn][16 bytes].  One thread per 16 bytes.
 // K within a tap: channels (int8 and binary: bytes; fp32: bf16 pieces); first layers: tap = filter row, K = kx * 4 + channel.
 // ------------------------------------------------------------------------------------------------
+// fp32: *beyond becomes 1 if a filter value's pieces are no finite numbers.
 template <int DT, bool XCOL>
 __global__ void pack_weights_win_kernel(const void* W, unsigned char* img, int c_in, int c_out, int kh, int kw, int taps, int groups,
-                                        int bn, int n_tiles)
+                                        int bn, int n_tiles, int* beyond)
 {
     const size_t total = (size_t)n_tiles * taps * groups * 2 * bn;
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1110,6 +1189,7 @@ __global__ void pack_weights_win_kernel(const void* W, unsigned char* img, int c
             const size_t a = at(2 * j), b = at(2 * j + 1);
             wn_split(a == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[a], b == (size_t)-1 ? 0.f : reinterpret_cast<const float*>(W)[b],
                      s[0][j], s[1][j], s[2][j]);
+            if (wn_bf16_nan(s[2][j])) *beyond = 1;
         }
         for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(dst + (size_t)k * bn * 16) = make_uint4(s[k][0], s[k][1], s[k][2], s[k][3]);
     } else {
@@ -1299,17 +1379,29 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     if (!win_plan(L, p, xcol, true, false, 1, 148)) return RRM_ERR_UNSUPPORTED;
     const int taps = xcol ? d.kh : d.kh * d.kw;
     const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
+    const size_t bytes = chunks * 16 * (f32 ? 3 : 1);
     void* img = nullptr;
-    if (cudaMalloc(&img, chunks * 16 * (f32 ? 3 : 1)) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
+    if (cudaMalloc(&img, bytes + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
     net->allocs.push_back(img);
-    L.win_Wimg = img;
     const unsigned grid = (unsigned)((chunks + 255) / 256);
     unsigned char* im = reinterpret_cast<unsigned char*>(img);
-    if (f32 && xcol) pack_weights_win_kernel<T_F32, true><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
-    else if (f32) pack_weights_win_kernel<T_F32, false><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
-    else if (xcol) pack_weights_win_kernel<T_I8, true><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
-    else pack_weights_win_kernel<T_I8, false><<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles);
+    int* beyond = reinterpret_cast<int*>(im + bytes);
+    RRM_CUDA_TRY(cudaMemset(beyond, 0, 4));
+    auto pack = [&](auto kernel) { kernel<<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles, beyond); };
+    if (f32) { if (xcol) pack(pack_weights_win_kernel<T_F32, true>); else pack(pack_weights_win_kernel<T_F32, false>); }
+    else if (xcol) pack(pack_weights_win_kernel<T_I8, true>);
+    else pack(pack_weights_win_kernel<T_I8, false>);
     RRM_CUDA_TRY(cudaGetLastError());
+    if (f32) {
+        int has = 0;
+        RRM_CUDA_TRY(cudaMemcpy(&has, beyond, 4, cudaMemcpyDeviceToHost));
+        if (has) {
+            net->allocs.pop_back();
+            cudaFree(img);
+            return RRM_ERR_UNSUPPORTED;
+        }
+    }
+    L.win_Wimg = img;
     RRM_TRY((win_allow<T_F32, true>())); RRM_TRY((win_allow<T_F32, false>()));
     RRM_TRY((win_allow<T_I8, true>())); RRM_TRY((win_allow<T_I8, false>()));
     RRM_TRY((win_allow<T_BIN, false>()));

@@ -274,6 +274,79 @@ def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
     net.close()
 
 
+# fp32 sums against fp64, 2-norm: measured up to 4.0e-7 on the layers below (chains of fused multiply-adds on the CUDA cores:
+# 4.2e-7), twice that here.  Without the third bf16 piece of the operands the tensor-core kernels would be at 3.4e-6, without the
+# promoted sums at 1.7e-6.
+F32_REL = 8e-7
+
+
+@pytest.mark.parametrize("exp_x,exp_w", [(0, 0), (-110, 100), (100, -110)])
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [
+    (3, 40, (47, 51), 11, 4, 0, 1), (4, 16, (200, 180), 3, 1, 1, 1),          # first layers
+    (64, 48, (20, 21), 3, 1, 1, 1), (256, 130, (13, 13), 3, 1, 1, 1), (512, 64, (30, 30), 3, 2, 1, 2),
+    (1500, 32, (1, 1), 1, 1, 0, 40)])
+def test_fp32_layers_keep_fp32_accuracy(c_in, c_out, hw, k, s, p, n, exp_x, exp_w):
+    """Values over twenty powers of two, near one and near the ends of the exponent range, dense and as deltas."""
+    rng = np.random.default_rng(c_in + k)
+    sp = _spec("f32", c_in, hw, c_out, k, s, p, rng)
+    sp.weight = np.ldexp(sp.weight, exp_w).astype(np.float32)
+    sp.bias = np.ldexp(sp.bias, exp_x + exp_w).astype(np.float32)
+    shape = (3, n, c_in) + hw
+    video = np.ldexp(rng.standard_normal(shape) * np.exp2(rng.uniform(-10, 10, size=shape)), exp_x).astype(np.float32)
+    video[1:] = np.where(rng.random((2, n, 1) + hw) < 0.3, video[1:], video[0])
+    net = _rrm().net_from_specs([sp], n=n)
+    for t, call in enumerate((net.keyframe, net.step, net.step)):
+        call(dev(video[t]))
+        want = orc.dense_forward([sp], video[t])[1][0]
+        err = np.linalg.norm(net.projection(0).cpu().numpy().astype(np.float64) - want) / np.linalg.norm(want)
+        assert err <= F32_REL, (t, err)
+    net.close()
+
+
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [
+    (3, 16, (60, 61), 7, 2, 3), (3, 20, (40, 44), 5, 4, 2),                   # first layers: windows of more columns than the filter has
+    (20, 24, (12, 11), 3, 1, 1), (64, 70, (90, 91), 3, 1, 1)])                # a cluster of shares; shares of their own
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan, 3.4e38, -3.399e38])
+def test_fp32_values_without_bf16_pieces(c_in, c_out, hw, k, s, p, value):
+    """Infinities, NaNs and floats above bf16's largest reach the outputs that see them, as in fp32 arithmetic, and no others."""
+    rng = np.random.default_rng(c_in + k)
+    sp = _spec("f32", c_in, hw, c_out, k, s, p, rng)
+    video = rng.standard_normal((2, 1, c_in) + hw).astype(np.float32)
+    video[1] = video[0]
+    video[1, 0, 1, hw[0] // 2, hw[1] // 2] = value
+    video[1, 0, 0, 0, hw[1] - 1] = value
+    net = _rrm().net_from_specs([sp])
+    with np.errstate(all="ignore"):
+        plain = orc.dense_forward([sp], video[0])[1][0]
+        want = orc.dense_forward([sp], video[1])[1][0]
+        want = np.where(np.abs(want) > np.finfo(np.float32).max, np.copysign(np.inf, want), want)
+
+    def check(got, what):
+        np.testing.assert_array_equal(np.isnan(got), np.isnan(want), err_msg=what)
+        np.testing.assert_array_equal(np.isinf(got) * np.sign(got), np.isinf(want) * np.sign(want), err_msg=what)
+        fin = np.isfinite(want)
+        assert np.all(np.abs(got[fin] - want[fin]) <= F32_TOL * np.maximum(np.abs(plain).max(), np.abs(want[fin]))), what
+
+    out, outs = net.new_output(), net.new_output(frames=2)
+    net.keyframe(dev(video[1]), out)
+    check(out.cpu().numpy().astype(np.float64), "keyframe")
+    net.dense_seq(dev(video), outs, 2)
+    check(outs[1].cpu().numpy().astype(np.float64), "dense chunk")
+    net.keyframe(dev(video[0]), out)
+    net.step(dev(video[1]), out)
+    check(out.cpu().numpy().astype(np.float64), "step")
+    # ... and a filter value of that kind (the middle one: it meets no padding)
+    sp.weight[1, 1, k // 2, k // 2] = value
+    net2 = _rrm().net_from_specs([sp])
+    with np.errstate(all="ignore"):
+        want = orc.dense_forward([sp], video[0])[1][0]
+        want = np.where(np.abs(want) > np.finfo(np.float32).max, np.copysign(np.inf, want), want)
+    net2.keyframe(dev(video[0]), out)
+    check(out.cpu().numpy().astype(np.float64), "filter")
+    net.close()
+    net2.close()
+
+
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p", [(16, 70, (13, 13), 3, 1, 1), (8, 12, (17, 15), 5, 2, 2), (64, 16, (10, 10), 3, 1, 1),
                                                  (3, 6, (35, 35), 11, 4, 0)])
