@@ -429,6 +429,7 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_gemm_kernel(ConvParams p)
             }
         }
         // nobody leaves while its tile may still be read
+        __syncwarp();                                        // (the aligned forms want whole warps)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         return;

@@ -210,6 +210,7 @@ __device__ __forceinline__ bool wn_agree(bool ok)
 __device__ __forceinline__ void wn_meet() { asm volatile("barrier.cta.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void wn_cluster_meet()
 {
+    __syncwarp();                                            // (the aligned forms want whole warps)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint4 wn_ld_remote(uint32_t addr, uint32_t rank)
@@ -1061,7 +1062,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     }
                 };
                 begin(team * NR);
-                __syncwarp();
                 wn_cluster_meet();                           // every share's partial tile is in its shared memory
                 for (int k0 = team * NR; split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M;) {      // (whole warps stay together)
                     uint4 t[NS][NR];
@@ -1090,7 +1090,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             if (p.ks <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
             else close(integral_constant<int, 2>{}, integral_constant<int, 8>{});
         } else wn_cluster_meet();
-        __syncwarp();
         wn_cluster_meet();                                   // nobody's shared memory goes away while it is read
     }
     tc_fence_before();

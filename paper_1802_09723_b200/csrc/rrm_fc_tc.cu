@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
 
     if (CLUSTER) {
         // ================= every CTA of the cluster closes its share of the rows: row r belongs to rank r mod ksplit
+        __syncwarp();                                        // (the aligned forms want whole warps)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         uint32_t rank;
@@ -294,6 +295,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) fc_tc_kernel(FtParams p, const 
             if (oo < p.c_out) ft_finish4(p, row, oo, w);
         }
         // nobody leaves while its shared memory may still be read
+        __syncwarp();                                        // (the aligned forms want whole warps)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         return;
