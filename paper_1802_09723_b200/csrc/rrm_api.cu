@@ -910,7 +910,8 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
             // fp32 products are most of a chunk's time, so there the delta form is level at twice the activity: quiet,
             // 2 streams x 16 frames 33 / 42, busy 45 / 42, 1 stream x 32 frames 25.6 / 21.  (Chunks of fewer than 8 frames
             // stay on the delta path below the whole-stack threshold: their callers read counters frame by frame.)
-            const double level = net->opt.chunk_dense_activity * (net->chunk_f32 ? 2.0 : 1.0);
+            // (a value up to 1 stays one that full activity reaches; above 1: never)
+            const double asked = net->opt.chunk_dense_activity, level = net->chunk_f32 && asked <= 1.0 ? (asked < 0.5 ? 2.0 * asked : 1.0) : asked;
             const bool go_dense = (net->auto_switch && net->activity >= net->opt.stack_dense_activity) ||
                                   (long_chunk && net->chunk_activity >= level);
             if (go_dense && net->dense_streak < net->opt.stack_reprobe) {

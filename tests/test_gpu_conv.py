@@ -833,6 +833,22 @@ def test_dense_chunks_whose_outputs_overlap_their_frames(shift):
     net.close()
 
 
+@pytest.mark.parametrize("threshold,goes", [(0.3, True), (0.8, True), (1.0, True), (1.01, False)])
+def test_fp32_chunks_with_everything_changing_go_dense_up_to_a_threshold_of_one(threshold, goes):
+    rng = np.random.default_rng(80)
+    T, sp = 8, _spec("f32", 20, (24, 23), 24, 3, 1, 1, rng)
+    video = rng.standard_normal((2 * T, 1, 20, 24, 23)).astype(np.float32)
+    net = _rrm().net_from_specs([sp])
+    net.set_options(chunk_dense_activity=threshold, stack_dense_activity=2.0)
+    outs = net.new_output(frames=T)
+    for k in range(2):
+        net.step_seq(dev(video[k * T:(k + 1) * T]), outs, T)
+        variant = net.stats(0)["variant"]                     # synchronises: the next call sees this chunk's counters
+        _compare([sp], net, video[(k + 1) * T - 1], k)
+    assert (variant == 3) == goes, variant
+    net.close()
+
+
 def test_dense_chunks_longer_than_one_batch():
     """Dense chunks are batched over their frames, 32 at most per launch: a chunk of 40 frames of two streams goes in
     two parts.  rrm_net_dense_seq leaves the state alone; a chunk that the density switch evaluates densely leaves
