@@ -681,7 +681,6 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
 {
     const int L = (int)net->layers.size();
     RRM_TRY(ensure_chunk(net, T));
-    RRM_TRY(ensure_stateless(net));
     // (images of a launch are at most 65535: the imports have them on grid.y)
     const int most = net->n < 65535 / DENSE_BATCH ? DENSE_BATCH : (net->n < 65535 ? 65535 / net->n : 1);
     const int parts = ceil_div(T, most), per = ceil_div(T, parts);
@@ -691,7 +690,7 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
     tensor_bytes_boundary(net->tensors.back(), &bo);
     cudaStream_t st = net->cap_stream;
     const int n0 = net->n;
-    // the stack with F times as many streams, on the large buffers (restored below)
+    // the stack with F times as many streams, on the large buffers (restored below), which stand in for the stateless pass's own
     auto scale = [&](int F) {
         net->n = n0 * F;
         for (auto& X : net->tensors) { X.n = n0 * F; std::swap(X.X2, X.X2b); }
