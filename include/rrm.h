@@ -255,7 +255,11 @@ int rrm_net_step(rrm_net* net, const void* frame_dev, void* out_dev, void* strea
 int rrm_net_dense(rrm_net* net, const void* frame_dev, void* out_dev, void* stream);
 int rrm_net_step_host(rrm_net* net, const void* frame_host, void* out_host, void* stream);
 /* Chunks of T frames, as rrm_step_seq / rrm_dense_seq / rrm_step_seq_host; outs = [T] last tensors.  After the call
- * rrm_net_get_stats reports the counters of the chunk's last frame. */
+ * rrm_net_get_stats reports the counters of the chunk's last frame.
+ * Reproducibility of fp32 stacks: each form of a step or chunk gives the same bits every time, but a delta and a dense
+ * evaluation round differently, and with RRM_VARIANT_AUTO which of them runs depends on whether the counters of the
+ * call before had arrived.  The bits are those of the last run if the caller waits for each call before the next, asks for
+ * RRM_VARIANT_TENSOR or RRM_VARIANT_GATHER, or sets stack_dense_activity and chunk_dense_activity above 1. */
 int rrm_net_step_seq(rrm_net* net, const void* frames_dev, void* outs_dev, int T, void* stream);
 int rrm_net_dense_seq(rrm_net* net, const void* frames_dev, void* outs_dev, int T, void* stream);
 int rrm_net_step_seq_host(rrm_net* net, const void* frames_host, void* outs_host, int T, void* stream);

@@ -274,6 +274,42 @@ def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
     net.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "i8", "bin"])
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,pool", [
+    (24, 20, (5, 700), 3, 1, 1, (3, 2, 0)),  # wider than 510 pixels
+    (16, 33, (4, 2300), 3, 2, 1, None),      # ... than 2040 at stride 2
+    (40, 70, (7, 7), 7, 1, 0, None),         # a filter that covers the map: more zeros than pixels in a window
+    (3, 12, (6, 300), 5, 1, 2, (2, 2, 0))])  # a first layer, 5x5, wider than 250
+def test_layers_beyond_the_window_kernel(dtype, c_in, c_out, hw, k, s, p, pool, monkeypatch):
+    """What the window convolution does not take runs in the kernel that gathers compacted rows (int8, binary) or on the
+    CUDA cores (fp32): frame by frame, as keyframes, and as chunks of both forms."""
+    rng = np.random.default_rng(hw[1] + k)
+    kw = dict(pool=pool) if dtype == "f32" else dict(act="sign", theta=2, pool=pool) if dtype == "bin" else dict(act="relu", shift=9, pool=pool)
+    sp = _spec(dtype, c_in, hw, c_out, k, s, p, rng, **kw)
+    video = _video(dtype, c_in, hw, 6, 2, rng)
+    _run([sp], video, n=2, stats=True, keyframe_at=(4,))
+    for form in ("RRM_CHUNK_BY_LAYER", "RRM_CHUNK_PIPELINED"):
+        monkeypatch.delenv("RRM_CHUNK_BY_LAYER", raising=False)
+        monkeypatch.setenv(form, "1")
+        net = _rrm().net_from_specs([sp], n=2)
+        net.keyframe(_frame_to_dev([sp], video[0]))
+        net.step_seq(torch.stack([_frame_to_dev([sp], f) for f in video[1:]]), net.new_output(frames=5), 5)
+        _compare([sp], net, video[5], 5)
+        net.close()
+    monkeypatch.delenv("RRM_CHUNK_PIPELINED")
+    net = _rrm().net_from_specs([sp], n=2)
+    dense, one = net.new_output(frames=6), net.new_output()
+    net.dense_seq(torch.stack([_frame_to_dev([sp], f) for f in video]), dense, 6)
+    for t in range(6):
+        net.keyframe(_frame_to_dev([sp], video[t]), one)
+        _compare([sp], net, video[t], t)
+        if dtype == "f32":
+            assert float((dense[t] - one).abs().max()) <= F32_TOL * float(one.abs().max())
+        else:
+            assert torch.equal(dense[t], one), t
+    net.close()
+
+
 # fp32 sums against fp64, 2-norm: measured up to 4.0e-7 on the layers below (chains of fused multiply-adds on the CUDA cores:
 # 4.2e-7), twice that here.  Without the third bf16 piece of the operands the tensor-core kernels would be at 3.4e-6, without the
 # promoted sums at 1.7e-6.
@@ -1032,6 +1068,35 @@ def test_fp32_projections_are_bitwise_reproducible(name):
             net.step(dev(video[t]), out)
         runs.append([net.projection(l).clone() for l in range(len(specs))] + [out.clone()])
         net.close()
+    for other in runs[1:]:
+        for a, b in zip(runs[0], other):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("how", ["variant", "options", "waits"])
+def test_fp32_chunks_are_bitwise_reproducible(how):
+    """Delta and dense forms of an fp32 chunk round differently, and which one runs depends on whether the counters of the
+    chunk before have arrived.  With the variant pinned, with the thresholds out of reach, or with a wait for each chunk
+    before the next, the same video gives the same bits."""
+    rrm = _rrm()
+    specs, T = wl.alexnet_convs("f32", hw=131, scale=4), 8
+    video = dev(np.ascontiguousarray(wl.moving_rect_video(frames=1 + 4 * T, hw=131, dtype="f32", seed=3, side=(12, 24), bg_redraw=0.10)))
+    runs, forms = [], []
+    for rep in range(3):
+        net = rrm.net_from_specs(specs, variant="tensor" if how == "variant" else "auto")
+        if how == "options":
+            net.set_options(chunk_dense_activity=2.0, stack_dense_activity=2.0)
+        net.keyframe(video[0])
+        outs, seen = net.new_output(frames=4 * T), []
+        for k in range(4):
+            net.step_seq(video[1 + k * T:1 + (k + 1) * T], outs[k * T:(k + 1) * T], T)
+            if how == "waits":
+                torch.cuda.synchronize()
+                seen.append(net.stats(1)["variant"])
+        runs.append([outs] + [net.projection(l) for l in range(len(specs))])
+        forms.append(seen)
+        net.close()
+    assert forms[0] == forms[1] == forms[2] and (how != "waits" or 3 in forms[0]), forms
     for other in runs[1:]:
         for a, b in zip(runs[0], other):
             assert torch.equal(a, b)

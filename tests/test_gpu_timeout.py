@@ -1,6 +1,6 @@
 """A bounded device-side wait that runs out is reported, not hung on, and leaves the context usable.
 
-The only form in which this is run on a GPU: rrm_options.wait_limit = 0 on the two tensor-core kernels.  There
+The only form in which this is run on a GPU: rrm_options.wait_limit = 0 on the three tensor-core kernels.  There
 every role of a thread block (copy producers, filter loader, MMA issuer, epilogue) meets its first wait BEFORE it
 has issued any asynchronous copy or MMA, so a wait that gives up at once lets the block leave with nothing in
 flight: it frees its tensor memory and returns.  The host then reads bit 1 of rrm_stats.error_word and gets
@@ -11,8 +11,9 @@ import pytest
 import torch
 
 import workloads as wl
+from workloads.nets import LayerSpec
 from oracle import rrm_oracle as orc
-from helpers import dev
+from helpers import dev, pack_bits_nhwc
 
 pytestmark = pytest.mark.gpu
 
@@ -65,25 +66,48 @@ def test_few_row_fc_kernel_reports_a_wait_that_ran_out_and_recovers():
     layer.close()
 
 
-def test_tensor_core_conv_reports_a_wait_that_ran_out_and_recovers():
+def _lone_layer(dtype, hw):
+    rng = np.random.default_rng(hw[1])
+    sp = LayerSpec("conv", dtype, 40, hw[0], hw[1], 36, 3, 3, 1, 1, src=0, act="sign" if dtype == "bin" else "none", theta=1)
+    sp.weight = ((rng.integers(0, 2, size=(36, 40, 3, 3)) * 2 - 1).astype(np.int8) if dtype == "bin" else
+                 rng.integers(-127, 128, size=(36, 40, 3, 3)).astype(np.int8))
+    sp.bias = rng.integers(-500, 501, size=36).astype(np.int32)
+    video = rng.integers(0, 2, size=(4, 1, 40) + hw) * 2 - 1 if dtype == "bin" else rng.integers(0, 128, size=(4, 1, 40) + hw)
+    return [sp], video.astype(np.int8)
+
+
+@pytest.mark.parametrize("dtype,kernel", [("i8", "windows"), ("f32", "windows"), ("bin", "windows"), ("i8", "rows"), ("bin", "rows")])
+def test_tensor_core_conv_reports_a_wait_that_ran_out_and_recovers(dtype, kernel):
+    """windows: the kernel that keeps windows of the input in shared memory; rows: the one that gathers compacted rows, which
+    takes what is too wide for such a window."""
     import paper_1802_09723_b200 as rrm
-    specs = wl.alexnet_convs("i8", hw=99, scale=8)
-    video = wl.moving_rect_video(frames=4, hw=99, dtype="i8", seed=9, side=(12, 24))
+    if kernel == "rows":
+        specs, video = _lone_layer(dtype, (3, 900))
+    elif dtype == "bin":
+        specs, video = _lone_layer(dtype, (20, 21))
+    else:
+        specs = wl.alexnet_convs(dtype, hw=99, scale=8)
+        video = wl.moving_rect_video(frames=4, hw=99, dtype=dtype, seed=9, side=(12, 24))
+    frames = [dev(pack_bits_nhwc(f).view(np.int32)) if dtype == "bin" else dev(f) for f in video]
     net = rrm.net_from_specs(specs, variant="tensor")
     out = net.new_output()
-    net.step(dev(video[0]), out)
-    assert net.stats(0)["error_word"] == 0 and net.stats(0)["variant"] == 2       # the tensor-core kernel runs these layers
+    net.step(frames[0], out)
+    assert net.stats(0)["error_word"] == 0 and net.stats(0)["variant"] == 2       # a tensor-core kernel runs these layers
     net.set_options(wait_limit=0)
-    net.step(dev(video[1]), out)                               # the first layer's thread blocks give up at their first wait
+    net.step(frames[1], out)                                   # the first layer's thread blocks give up at their first wait
     st = net.stats(0, check=False)
     assert st["status"] == TIMEOUT_STATUS and st["error_word"] & TIMEOUT_BIT, st
     net.set_options(wait_limit=1 << 20)
     net.clear_errors()
-    net.keyframe(dev(video[1]), out)                           # a precise inference replaces the inconsistent state
+    net.keyframe(frames[1], out)                               # a precise inference replaces the inconsistent state
     for t in (2, 3):
-        net.step(dev(video[t]), out)
+        net.step(frames[t], out)
         _, P = orc.dense_forward(specs, video[t])
         for l in range(len(specs)):
-            np.testing.assert_array_equal(net.projection(l).cpu().numpy().astype(np.int64), P[l])
+            got = net.projection(l).cpu().numpy()
+            if dtype == "f32":
+                assert float(np.abs(got - P[l]).max()) <= 1e-4 * float(np.abs(P[l]).max())
+            else:
+                np.testing.assert_array_equal(got.astype(np.int64), P[l])
     assert net.stats(0)["error_word"] == 0
     net.close()
