@@ -28,8 +28,8 @@
 // after at most WN_PROMOTE K steps of 16, and the five small ones have two of their own.  A value whose first piece is no
 // finite number (an infinity, a NaN, or a float above bf16's largest) makes its third piece a NaN, by which a CTA notices
 // it: such a CTA forms its sums one by one from the operands instead (wn_exact_row), and a layer with such a filter
-// keeps the CUDA cores.  Measured against fp64 at K = 2304, normal operands: relative error (2-norm) 1.8e-7,
-// a chain of fmaf 6e-7; without the promotion 1.7e-6, with everything in one accumulator 1.5e-5.
+// keeps the CUDA cores.  Error against fp64 (2-norm, dense, normal operands; a chain of fmaf): 3x3 of 256 channels 2.5e-7
+// (4.1e-7), 5x5 of 96 3.4e-7 (8.3e-7), 11x11 first layer 1.0e-7 (1.6e-7); without the promotion 1.7e-6.
 //
 // Roles: warps 0-7 fill windows and drain accumulators, warp 8 issues the MMAs, warp 9 the bulk copies of the filters
 // (packed at create time as the operand tiles they are).  K can be split over the CTAs of a cluster by blocks: the
@@ -38,14 +38,10 @@
 // ERRW_TIMEOUT and the CTA leaves through the common exit.
 //
 // What bounds it: in a long K loop the MMAs' operand reads from shared memory (an MMA of 128 columns reads 8 KB, the 64
-// clocks it takes), beside which the filter copies write another quarter (fp32 step of 768 MMA clocks: 1064 measured, 1180
-// with six separate MMAs and the barrier looked at only when it is needed); in a launch of a few tiles a chain of ~7 us (rows
-// and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  Against kernels that gathered rows tap by tap (fp32: on the
-// CUDA cores), AlexNet-shaped stack at 227 x 227: fp32 32 frames conv2 / conv4 351 / 412 (delta) -> 152 / 53 us (dense), 8
-// streams 546 -> 189 for the whole stack; int8 frame 84 -> 63.  Filling with a turn's loads ahead of its stores, and first
-// layers with one table for all planes: 8 fp32 streams 194 -> 189, 50 binary frames 167 -> 163, 32 int8 frames 147 -> 144.  fp32 tiles of 64 columns, two CTAs per SM, were slower
-// than 128 and one (conv2 152 -> 179, conv4 53 -> 83, 11x11 first layer 107 -> 111: every window is then filled twice as
-// often, and an MMA of 128 columns has no smem bandwidth to spare for it).
+// clocks it takes), beside which the filter copies write another quarter (fp32 step of 768 MMA clocks: 1064 measured); in a
+// launch of a few tiles a chain of ~7 us (rows and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  AlexNet-shaped
+// stack at 227 x 227 against kernels that gather rows tap by tap (fp32: on the CUDA cores): 8 fp32 streams 546 -> 191 us, 32
+// fp32 frames 1630 -> 469, one int8 frame 83 -> 64, 32 int8 frames 266 -> 144.
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"

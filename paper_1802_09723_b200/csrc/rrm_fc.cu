@@ -11,7 +11,8 @@
 //      memory; CTA 0 of the cluster adds them onto the stored projection P (owner computes, no
 //      atomics), applies f and writes Y_t;
 //   4. one CTA per stream writes the new snapshot into the other half of a ping-pong pair.
-// Cost is HBM-bound: nnz * C_out weight bytes per frame.
+// A launch is a chain of round trips (frame in, list, columns, sums across the cluster): 7.7 us for the 1.9 MB of columns
+// that 5 % of 9216 inputs and 4096 outputs gather.
 #include "rrm_common.cuh"
 #include "rrm_dev.cuh"
 #include <cooperative_groups.h>
