@@ -501,6 +501,31 @@ def compact_conv(r):
     return out
 
 
+def contract_line(line):
+    """What bench.py prints: the contract's keys and a few figures of the secondary measurements, numbers to six digits.
+    Readers of the output keep its last 3000 characters, so the line stays below that; everything else goes to --details."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "ms_per_step_stats", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "dense_equiv_gmacs", "clocks", "e2e", "gpu_launches", "roofline", "cpu_baseline")
+    out = {k: line[k] for k in keys}
+    out["roofline"] = {k: v for k, v in out["roofline"].items() if k != "note"}
+    if line.get("conv"):
+        # us per step: delta or as chosen / own dense path; us per frame of a 32-frame chunk: as chosen / delta forced / dense
+        out["conv_us"] = {}
+        for k, r in line["conv"].items():
+            if isinstance(r, dict) and "ms_per_step" in r:
+                c = r.get("chunk")
+                out["conv_us"][k] = [r["ms_per_step"] * 1e3, r["ms_per_step_dense_path"] * 1e3] + (
+                    [c[f] * 1e3 for f in ("ms_per_frame", "delta_forced_ms_per_frame", "dense_ms_per_frame")] if c else [])
+
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, (list, tuple)) else v
+    return short(out)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -519,6 +544,7 @@ def main():
     ap.add_argument("--frames", type=int, default=None, help="frames of the synthetic video (convolution workloads)")
     ap.add_argument("--streams", type=int, default=None, help="independent videos per call (convolution workloads)")
     ap.add_argument("--opt", action="append", help="rrm_options field=value (convolution workloads), e.g. --opt layer_dense_activity=0.9")
+    ap.add_argument("--details", default=None, help="file that receives every figure of the run as JSON (the printed line holds the contract's)")
     ap.add_argument("--seq", type=int, default=None, help="also time rrm_net_step_seq with this many frames per call (convolution workloads)")
     args = ap.parse_args()
     if args.workload != "cfg2":
@@ -921,8 +947,7 @@ def main():
             "clocks": clocks,
             "e2e": {"value": world * T * 1e3 / e2e_ms, "unit": "frames/s", "h2d_bytes_per_step": T * C_IN,
                     "d2h_bytes_per_step": T * 4 * C_OUT,
-                    "call": "rrm_step_seq_host_async per step, one rrm_host_sync after the last step; steps back to back "
-                            "(no L2 flush between them, unlike `value`: W stays L2-resident), timed on the host clock",
+                    "call": "rrm_step_seq_host_async per step, one rrm_host_sync at the end; back to back, no L2 flush, host clock",
                     "value_waiting_every_call": world * T * 1e3 / e2e_sync_ms},
             "gpu_launches": args.steps,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
@@ -939,7 +964,10 @@ def main():
             "last_step_stats": st,
         }
         line.update(extra)
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(contract_line(line)))
     if world > 1:
         dist.destroy_process_group()
 

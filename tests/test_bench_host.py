@@ -39,6 +39,24 @@ def test_two_ranks_report_the_slowest_rank_and_the_whole_job():
             assert rate == 2 * 32 * 1e3 / 5.0
 
 
+def test_printed_line_holds_the_contract_and_stays_short():
+    text, num = "x" * 160, 12345.678901234567
+    stats = dict.fromkeys(("median", "mean", "min", "max"), num) | {"n": 310}
+    chunk = dict.fromkeys(("ms_per_frame", "delta_forced_ms_per_frame", "dense_ms_per_frame"), num)
+    row = {"ms_per_step": num, "ms_per_step_dense_path": num, "rho_per_layer": [num] * 20, "chunk": chunk}
+    line = dict(metric="frames_per_sec", value=num, unit="frames/s", n_gpus=1, steps=310, warmup=31, ms_per_step=num, ms_per_step_stats=stats,
+                higher_is_better=True, scaling="weak", vs_baseline=None, dtype="i8", data="synthetic", dense_equiv_gmacs=num, gpu_launches=310,
+                config={k: text for k in ("workload", "l2")} | {"measured_density": num}, clocks={"sm_mhz": num, "sm_max_mhz": num, "reasons": []},
+                e2e={"value": num, "unit": "frames/s", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 1, "call": text},
+                roofline={"bound": "hbm", "frac": num, "note": text * 4}, cpu_baseline={"value": num, "sample": text, "dense_sample": text},
+                conv={f"cfg{i}_delta_forced": row for i in range(7)} | {"note": text * 4}, by_rho={str(i): row for i in range(50)})
+    out = json.dumps(bench.contract_line(line))
+    got = json.loads(out)
+    assert len(out) < 2900, len(out)
+    assert got["value"] == 12345.7 and got["e2e"]["h2d_bytes_per_step"] == 1 and got["clocks"]["reasons"] == []
+    assert len(got["conv_us"]["cfg3_delta_forced"]) == 5 and "by_rho" not in got
+
+
 def test_reference_arm_prints_the_contract_line():
     p = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--steps", "3", "--warmup", "1"],
                        capture_output=True, text=True, check=True)
