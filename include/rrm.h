@@ -149,10 +149,9 @@ typedef struct {
                                     pixel to update (accumulator tiles of 128 pixels, or pixels, whichever a layer's
                                     kernel can skip) from which on the next chunks are evaluated densely, batched over
                                     their frames (same results; a delta chunk measures again after stack_reprobe dense
-                                    ones); stacks with fp32 layers: from twice the value on, at most 1.  Above 1: never.
-                                    Default 0.40.  The first dense chunk of a length captures its graph, and one of
-                                    more frames (32 at most per launch) than any before allocates their tensors, up to
-                                    8 GiB; larger chunks go through buffers of one frame */
+                                    ones).  Above 1: never.  Default 0.40.  The first dense chunk of a length captures
+                                    its graph, and one of more frames (32 at most per launch) than any before allocates
+                                    their tensors, up to 8 GiB; larger chunks go through buffers of one frame */
 } rrm_options;
 
 /* ---- single layer (Eq. 2-5) ------------------------------------------------------- */

@@ -206,7 +206,7 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
         net->layer_switch = all_auto && n_layers <= 64;
         {
             bool all_tc = true;
-            for (auto& L : net->layers) { all_tc = all_tc && L.on_tensor(); net->chunk_f32 = net->chunk_f32 || L.d.dtype == RRM_F32; }
+            for (auto& L : net->layers) all_tc = all_tc && L.on_tensor();
             net->chunk_switch = all_auto && all_tc && n_layers <= 64;
         }
         // an all-ones bitmap stands in for a layer's update bitmap when the layer is evaluated densely inside a delta step
@@ -906,13 +906,12 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
             // update, so those are what its activity counts.  Measured, us per frame, delta as the library chooses /
             // dense: AlexNet int8 on the quiet video (a third of the pixels) 1 stream x 16 frames 12.1 / 9.2, 32 frames
             // 7.1 / 6.4, 8 streams x 4 frames 57 / 51; busy 13.7 / 9.1; a lone int8 layer, 3 streams x 8 frames 17 / 9.8.
-            // fp32 products are most of a chunk's time, so there the delta form is level at twice the activity: quiet,
-            // 2 streams x 16 frames 33 / 42, busy 45 / 42, 1 stream x 32 frames 25.6 / 21.  (Chunks of fewer than 8 frames
-            // stay on the delta path below the whole-stack threshold: their callers read counters frame by frame.)
-            // (a value up to 1 stays one that full activity reaches; above 1: never)
-            const double asked = net->opt.chunk_dense_activity, level = net->chunk_f32 && asked <= 1.0 ? (asked < 0.5 ? 2.0 * asked : 1.0) : asked;
+            // fp32, delta / dense: AlexNet busy 18.5 / 14.1, quiet 16.4 / 14.1 (1 stream x 32), 13.8 / 14.2 (2 x 16); lone 3x3
+            // layers, us per chunk: 2 x 16 frames of 64 x 112 x 112 with 0.05 and 0.2 % of the pixels, or 5 % of the 8 x 8 patches, changing
+            // 495, 586, 652 / 512; 4 x 16 of 256 x 28 x 28 460-522 / 361.  (Chunks of fewer than 8 frames stay on the delta path below the whole-stack threshold: their callers
+            // read counters frame by frame.)
             const bool go_dense = (net->auto_switch && net->activity >= net->opt.stack_dense_activity) ||
-                                  (long_chunk && net->chunk_activity >= level);
+                                  (long_chunk && net->chunk_activity >= net->opt.chunk_dense_activity);
             if (go_dense && net->dense_streak < net->opt.stack_reprobe) {
                 ++net->dense_streak;                         // (counted in calls: a delta chunk measures again after 15 dense ones)
                 net->last_step_dense = true;

@@ -339,7 +339,6 @@ struct rrm_net {
     bool auto_switch = false;                 // every layer asks for RRM_VARIANT_AUTO and the net is large enough
     double chunk_activity = -1.0;             // the same with window-kernel layers counted by accumulator tiles that hold such a pixel
     bool chunk_switch = false;                // every layer asks for RRM_VARIANT_AUTO and runs on the tensor cores: long chunks may go dense
-    bool chunk_f32 = false;                   // ... and some of them are fp32
     // the defaults rrm_net_get_options reports.  (The per-layer thresholds are above 1, i.e. the per-layer choice is off
     // until the caller lowers them: measured on B200, a dense evaluation of one layer inside a delta step is never
     // faster than its sparse product, not even with every pixel active.  What a delta step pays for is change
