@@ -881,21 +881,38 @@ __global__ void __launch_bounds__(256) import_i8_word_dense_kernel(const int8_t*
     for (int k = 0; k < 4; ++k) if (base + 256 * k < pixels) X[base + 256 * k] = v[k];
 }
 
+// Tiles of `ptiles` pixel tiles x (channel tiles x images) x frames as a grid: y holds at most 65535 of the middle product,
+// what is more continues in z.  (All of it along x cost a tile's chain another division: 30 frames of 74 x 74, in and out, +1.3 us.)
+struct TileGrid {
+    unsigned ctiles, slabs, frames;
+    TileGrid(unsigned ctiles_, unsigned images, unsigned frames_) : ctiles(ctiles_), slabs(ctiles_ * images), frames(frames_) {}
+    dim3 grid(unsigned ptiles) const { return dim3(ptiles, slabs < 65535u ? slabs : 65535u, frames * ((slabs + 65534u) / 65535u)); }
+    // this CTA's image, channel tile and frame; false: none
+    __device__ __forceinline__ bool mine(long long& image, int& ctile, long long& frame) const
+    {
+        unsigned s = blockIdx.y, f = blockIdx.z;
+        if (f >= frames) { s += f / frames * 65535u; f %= frames; }
+        image = s / ctiles; ctile = (int)(s % ctiles); frame = f;
+        return s < slabs;
+    }
+};
+
 // int8 between the boundary layout and whole 32-byte pixel rows, a 128-pixel x 32-channel tile at a time through shared
 // memory: rows as 16-byte groups, planes along the pixels (as words where a plane's address allows).  EXPORT: rows -> planes.
-// grid = (pixel tiles x channel tiles x n, 1, frames): x alone has room for the product.  30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread
-// per element, import of 48 channels 10.8 -> 7.0 against the 32-pixel tiles.
+// 30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread per element, import of 48 channels 10.8 -> 7.0
+// against the 32-pixel tiles.
 template <bool EXPORT>
-__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, unsigned ptiles, unsigned ctiles,
+__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, TileGrid tg,
                                                           long long src_stride, long long dst_stride)
 {
     __shared__ __align__(16) int8_t tile[32][132];
-    const unsigned slab = blockIdx.x / ptiles, image = slab / ctiles;
-    const int p0 = (int)(blockIdx.x - slab * ptiles) * 128, c0 = (int)(slab - image * ctiles) * 32;
-    const long long ns = image;
+    long long ns, frame;
+    int ctile;
+    if (!tg.mine(ns, ctile, frame)) return;
+    const int p0 = blockIdx.x * 128, c0 = ctile * 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, px = threadIdx.x >> 1, half = (threadIdx.x & 1) * 16;
-    src += blockIdx.z * src_stride;
-    dst += blockIdx.z * dst_stride;
+    src += frame * src_stride;
+    dst += frame * dst_stride;
     pdl_launch_dependents();
     pdl_wait();
     const long long row = ((ns * hw + p0 + px) * cs) + c0 + half;
@@ -1351,16 +1368,17 @@ __global__ void export_nchw_kernel(const T* __restrict__ src, T* dst, int c, int
 }
 
 // The same through a 32 x 32 tile in shared memory (4-byte elements): rows read along the channels, planes written
-// along the pixels, both coalesced.  grid = (pixel tiles x channel tiles x n, 1, frames), block = (32, 8).
+// along the pixels, both coalesced.  block = (32, 8).
 __global__ void __launch_bounds__(256) export_nchw_tiled_kernel(const uint32_t* __restrict__ src, uint32_t* dst, int c, int cs, int hw,
-                                                                unsigned ptiles, unsigned ctiles, long long src_stride, long long dst_stride)
+                                                                TileGrid tg, long long src_stride, long long dst_stride)
 {
     __shared__ uint32_t tile[32][33];
-    const unsigned slab = blockIdx.x / ptiles, image = slab / ctiles;
-    const int p0 = (int)(blockIdx.x - slab * ptiles) * 32, c0 = (int)(slab - image * ctiles) * 32;
-    const long long ns = image;
-    src += blockIdx.z * src_stride;
-    dst += blockIdx.z * dst_stride;
+    long long ns, frame;
+    int ctile;
+    if (!tg.mine(ns, ctile, frame)) return;
+    const int p0 = blockIdx.x * 32, c0 = ctile * 32;
+    src += frame * src_stride;
+    dst += frame * dst_stride;
     pdl_launch_dependents();
     pdl_wait();
     for (int k = threadIdx.y; k < 32; k += 8) {
@@ -1563,9 +1581,8 @@ int launch_import(rrm_net* net, const void* frame, bool delta, bool stateless, c
             launch_seq(import_step_kernel<int8_t>, dim3(grid), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, (int8_t*)T.D, T.act, T.nnz, T.npix,
                        net->errw, T.c, T.cs, hw, T.w, T.readers);
         } else if (T.dtype == T_I8 && !delta) {
-            const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
-            launch_seq(transpose_i8_kernel<false>, dim3(ptiles * ctiles * T.n), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, T.c, T.cs, hw,
-                       ptiles, ctiles, 0ll, 0ll);
+            const TileGrid tg(T.cs / 32, T.n, 1);
+            launch_seq(transpose_i8_kernel<false>, tg.grid(ceil_div(hw, 128)), dim3(256), 0, st, (const int8_t*)frame, (int8_t*)X, T.c, T.cs, hw, tg, 0ll, 0ll);
         } else if (T.dtype == T_F32) {
             auto kd = import_nchw_kernel<float, true>;
             auto kn = import_nchw_kernel<float, false>;
@@ -1877,13 +1894,12 @@ int launch_export_tensor(rrm_net* net, int t, void* dst, bool stateless, cudaStr
     const long long total = (long long)T.n * T.c * hw;
     const int blocks = (int)((total + 255) / 256);
     if (T.dtype == T_I8 && T.cs % 32 == 0) {
-        const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
-        launch_seq(transpose_i8_kernel<true>, dim3(ptiles * ctiles * T.n), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, ptiles, ctiles, 0ll, 0ll);
+        const TileGrid tg(T.cs / 32, T.n, 1);
+        launch_seq(transpose_i8_kernel<true>, tg.grid(ceil_div(hw, 128)), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, tg, 0ll, 0ll);
     } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, dim3(blocks), dim3(256), 0, st, (const int8_t*)X, (int8_t*)dst, T.c, T.cs, hw, total, 0ll, 0ll);
     else {
-        const unsigned ptiles = ceil_div(hw, 32), ctiles = ceil_div(T.c, 32);
-        launch_seq(export_nchw_tiled_kernel, dim3(ptiles * ctiles * T.n), dim3(32, 8), 0, st, (const uint32_t*)X, (uint32_t*)dst,
-                   T.c, T.cs, hw, ptiles, ctiles, 0ll, 0ll);
+        const TileGrid tg(ceil_div(T.c, 32), T.n, 1);
+        launch_seq(export_nchw_tiled_kernel, tg.grid(ceil_div(hw, 32)), dim3(32, 8), 0, st, (const uint32_t*)X, (uint32_t*)dst, T.c, T.cs, hw, tg, 0ll, 0ll);
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
@@ -1902,15 +1918,15 @@ int launch_export_seq(rrm_net* net, int frames, void* dst, cudaStream_t st)
     const long long total = (long long)T.n * T.c * hw;
     const dim3 grid((unsigned)((total + 255) / 256), (unsigned)frames);
     if (T.dtype == T_I8 && T.cs % 32 == 0) {
-        const unsigned ptiles = ceil_div(hw, 128), ctiles = T.cs / 32;
-        launch_seq(transpose_i8_kernel<true>, dim3(ptiles * ctiles * T.n, 1, frames), dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, ptiles, ctiles,
+        const TileGrid tg(T.cs / 32, T.n, frames);
+        launch_seq(transpose_i8_kernel<true>, tg.grid(ceil_div(hw, 128)), dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, tg,
                    (long long)T.bytes(), total);
     } else if (T.dtype == T_I8) launch_seq(export_nchw_kernel<int8_t>, grid, dim3(256), 0, st, (const int8_t*)T.Xfull, (int8_t*)dst, T.c, T.cs, hw, total,
                                     (long long)T.bytes(), total);
     else {
-        const unsigned ptiles = ceil_div(hw, 32), ctiles = ceil_div(T.c, 32);
-        launch_seq(export_nchw_tiled_kernel, dim3(ptiles * ctiles * T.n, 1, frames), dim3(32, 8), 0, st, (const uint32_t*)T.Xfull, (uint32_t*)dst,
-                   T.c, T.cs, hw, ptiles, ctiles, (long long)T.bytes() / 4, total);
+        const TileGrid tg(ceil_div(T.c, 32), T.n, frames);
+        launch_seq(export_nchw_tiled_kernel, tg.grid(ceil_div(hw, 32)), dim3(32, 8), 0, st, (const uint32_t*)T.Xfull, (uint32_t*)dst, T.c, T.cs, hw, tg,
+                   (long long)T.bytes() / 4, total);
     }
     RRM_CUDA_TRY(cudaGetLastError());
     return RRM_OK;
