@@ -54,7 +54,7 @@ constexpr int WN_FILL = 256;                  // threads that fill windows and d
 constexpr int WN_THREADS = WN_FILL + 64;
 constexpr int WN_MAX_STAGES = 8, WN_MAX_ABUF = 4, WN_MAX_MT = 2;
 constexpr int WN_MAX_SPAN = 1152;             // pixels of one plane of a window
-constexpr int WN_TURN = 36;                  // words per row where a warp turns 32 rows x 32 columns around (16-byte aligned, staggered over the banks)
+constexpr int WN_TURN = 64;                  // columns of its 32 rows that a warp turns around at a time
 constexpr int WN_PROMOTE = 32;                // fp32: K steps the leading product accumulates before it is promoted
 constexpr size_t WN_SMEM_LIMIT = 227 * 1024;
 
@@ -319,6 +319,17 @@ __device__ __forceinline__ uint32_t wn_f8(const WinParams& p, int c, const int (
 {
     if (p.bn_scale) return wn_f8_bn(p, c, x[0], x[1], x[2], x[3], res);
     return wn_f8_plain(x, res, p.shift > 0 ? 1 << (p.shift - 1) : 0, p.shift, p.act_fn == RRM_ACT_RELU ? 0 : -127, p.res != nullptr);
+}
+
+// fp32 f of 4 neighbouring channels with the explicit affine or a shortcut (out of line like wn_f8_bn)
+__device__ __noinline__ float4 wn_f32_slow(const WinParams& p, int ch, int live, size_t at, float4 v)
+{
+    const float x[4] = {v.x, v.y, v.z, v.w};
+    float res[4] = {0.f, 0.f, 0.f, 0.f}, y[4];
+    #pragma unroll
+    for (int j = 0; j < 4; ++j) if (p.res && j < live) res[j] = reinterpret_cast<const float*>(p.res)[at + j];
+    wn_f<T_F32, T_F32, float>(p, ch, x, res, y);
+    return make_float4(y[0], y[1], y[2], y[3]);
 }
 
 // fp32, the way out of windows with infinities, NaNs or values beyond bf16: one row's share of the sums, columns c_lo to
@@ -773,6 +784,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     const bool halves = p.mt > 1 && p.bn > 64;               // two tiles: 64 columns at a time, so that both fit
     const int cw = halves ? 64 : p.bn;                       // columns per pass
     const int ldr = cw + 4;                                  // words per staged row (16-byte aligned, staggered over the banks)
+    const int ldt = min(p.bn, WN_TURN) + 4;                  // ... where a warp turns its rows around by itself
     const bool vec = (p.c_out & 3) == 0;
     const bool adds = !DENSE && !p.store;                    // delta: onto the stored projection
     const bool bulk_add = adds && vec && !p.cluster;         // ... by the copy engine, a row per thread (exact in any order for integers,
@@ -802,15 +814,12 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         const int r = m_own * TC_M + (warp & 3) * 32 + lane;
         const int q = S->q[r];
         const bool keep = q >= p.keep_from;                  // (q >= 0 then)
-        uint32_t* row = staged + (size_t)r * ldr;
-        int32_t* dstP = reinterpret_cast<int32_t*>(P) + (size_t)(keep ? q - p.keep_from : 0) * p.c_out + n0;
-        // (a loop, not unrolled: every CTA runs this code once, so its length is instruction fetches.  64 columns per turn of the
-        // row buffer, 32 per turn of the accumulator)
-        #pragma unroll 1
-        for (int cb = c_lo; cb < c_hi; cb += 64) {
-            if (keep && cb > c_lo) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        uint32_t* mine = staged + (size_t)warp * 32 * ldt;   // (the warp's rows, where projections are kept)
+        const bool any_keep = __any_sync(0xffffffffu, keep);
+        // (a loop, not unrolled: every CTA runs this code once, so its length is instruction fetches)
+        {
             #pragma unroll 1
-            for (int cc = cb; cc < min(cb + 64, c_hi); cc += 32) {
+            for (int cc = c_lo; cc < c_hi; cc += 32) {
                 const bool inside = q >= 0 && n0 + cc < (p.bits ? p.cs * 32 : p.cs);
                 uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
                 if (p.res && inside) {
@@ -825,20 +834,26 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     const int4 b = *reinterpret_cast<const int4*>(S->bias + cc + j);
                     v[j] += (uint32_t)b.x; v[j + 1] += (uint32_t)b.y; v[j + 2] += (uint32_t)b.z; v[j + 3] += (uint32_t)b.w;
                 }
-                if (keep) {                                  // (before f: the fence waits for this thread's stores, the output's too)
-                    if (vec) {
-                        uint32_t* at = row + (cc - cb) + (halves ? 0 : cb);
-                        #pragma unroll
-                        for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(at + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                        const int cols = min(32, ncols - cc);
-                        fence_async_smem();
-                        if (cols > 0)
-                            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                                         ::"l"(dstP + cc), "r"(smem_u32(at)), "r"((uint32_t)cols * 4u) : "memory");
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    } else {
-                        #pragma unroll
-                        for (int j = 0; j < 32; ++j) if (cc + j < ncols) dstP[cc + j] = (int32_t)v[j];
+                if (any_keep) {
+                    // the projection leaves as whole lines, eight lanes a row.  (Row by row through the copy engine, 128 bytes a copy:
+                    // 9 to 18 clocks each, 4.6 to 9.4 k of a keyframe CTA's 14 to 38 k)
+                    #pragma unroll
+                    for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(mine + lane * ldt + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    __syncwarp();
+                    const int c4 = (lane & 7) * 4, left = ncols - cc - c4;
+                    #pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = i * 4 + (lane >> 3), qq = __shfl_sync(0xffffffffu, q, rr);
+                        if (qq < p.keep_from || left <= 0) continue;
+                        const uint4 t = *reinterpret_cast<const uint4*>(mine + rr * ldt + c4);
+                        uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(qq - p.keep_from) * p.c_out + n0 + cc + c4;
+                        if (vec) *reinterpret_cast<uint4*>(dst) = t;
+                        else {
+                            dst[0] = t.x;
+                            if (left > 1) dst[1] = t.y;
+                            if (left > 2) dst[2] = t.z;
+                            if (left > 3) dst[3] = t.w;
+                        }
                     }
                 }
                 if (!inside) continue;
@@ -875,7 +890,6 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 }
             }
         }
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the row buffers may be released
     }
     // one value group of 4 neighbouring channels (c: column of the tile) of projection pixel q leaves: f and the output row
     // (ACT), the projection where it is kept.  Every lane of a warp comes here (signs are put together by shuffles).
@@ -899,26 +913,21 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         } else if (ACT) {
             if (q >= 0 && c < ncols) {
                 const size_t at = (size_t)q * p.cs + ch;
-                float x[4], res[4] = {0.f, 0.f, 0.f, 0.f}, y[4];
-                #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    x[j] = __uint_as_float(o[j]);
-                    if (p.res && c + j < ncols) res[j] = reinterpret_cast<const float*>(p.res)[at + j];
-                }
-                if (p.bn_scale) wn_f<T_F32, T_F32, float>(p, ch, x, res, y);
-                else {
-                    #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        y[j] = x[j] + res[j];
-                        if (p.act_fn == RRM_ACT_RELU) y[j] = y[j] > 0 ? y[j] : 0;
-                        else if (p.act_fn == RRM_ACT_LEAKY) y[j] = y[j] > 0 ? y[j] : 0.1f * y[j];
-                    }
+                float4 y = make_float4(__uint_as_float(o[0]), __uint_as_float(o[1]), __uint_as_float(o[2]), __uint_as_float(o[3]));
+                if (p.bn_scale || p.res) y = wn_f32_slow(p, ch, ncols - c, at, y);
+                else if (p.act_fn != RRM_ACT_NONE) {
+                    const float leak = 0.1f;
+                    const bool relu = p.act_fn == RRM_ACT_RELU;
+                    y.x = y.x > 0 ? y.x : (relu ? 0.f : leak * y.x); y.y = y.y > 0 ? y.y : (relu ? 0.f : leak * y.y);
+                    y.z = y.z > 0 ? y.z : (relu ? 0.f : leak * y.z); y.w = y.w > 0 ? y.w : (relu ? 0.f : leak * y.w);
                 }
                 float* dst = reinterpret_cast<float*>(p.X) + at;
-                if (vec) *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
+                if (vec) *reinterpret_cast<float4*>(dst) = y;
                 else {
-                    #pragma unroll
-                    for (int j = 0; j < 4; ++j) if (c + j < ncols) dst[j] = y[j];
+                    dst[0] = y.x;
+                    if (c + 1 < ncols) dst[1] = y.y;
+                    if (c + 2 < ncols) dst[2] = y.z;
+                    if (c + 3 < ncols) dst[3] = y.w;
                 }
             }
         }
@@ -942,53 +951,60 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             for (int j = 0; j < 4; ++j) if (c + j < ncols) o[j] = from[j];
         }
     };
-    // 32 columns of this thread's accumulator row, from column cc of the tile on (k: index into the promoted sums)
-    auto take32 = [&](int cc, int k, uint32_t (&v)[32]) {
-        __syncwarp();
-        if (DT == T_F32) {
-            wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + cc), v);
+    // this thread's accumulator row, up to 64 columns from column cb of the tile on, into shared memory.  (fp32: all of the
+    // thread's columns, completed from the promoted sums and the two accumulators of small products)
+    auto put_row = [&](int cb, uint32_t* row) {
+        #pragma unroll (DT == T_F32 ? 2 : 1)
+        for (int k = 0; k < 64; k += 32) {
+            const int cc = cb + k;
+            if (cc >= c_hi) continue;                        // (the same in all lanes)
+            uint32_t v[32];
+            __syncwarp();
+            if (DT == T_F32) {
+                wn_ld32(tmem + lane_base + (uint32_t)(3 * p.bn + cc), v);
+                #pragma unroll
+                for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? k + j : 0] = fmaf(__uint_as_float(v[j]), 1.f / (WN_SCALE * WN_SCALE), facc[DT == T_F32 ? k + j : 0]);
+            }
+            wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + cc), v);
+            if (DT == T_F32) {
+                #pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaf(__uint_as_float(v[j]), 1.f / WN_SCALE, facc[DT == T_F32 ? k + j : 0]));
+            }
             #pragma unroll
-            for (int j = 0; j < 32; ++j) facc[DT == T_F32 ? k + j : 0] = fmaf(__uint_as_float(v[j]), 1.f / (WN_SCALE * WN_SCALE), facc[DT == T_F32 ? k + j : 0]);
-        }
-        wn_ld32(tmem + lane_base + (uint32_t)((DT == T_F32 ? 2 : m_own) * p.bn + cc), v);
-        if (DT == T_F32) {
-            #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaf(__uint_as_float(v[j]), 1.f / WN_SCALE, facc[DT == T_F32 ? k + j : 0]));
+            for (int j = 0; j < 32; j += 4) if (cc + j < c_hi) *reinterpret_cast<uint4*>(row + k + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         }
     };
     if (!direct && !p.cluster && !bulk_add) {
-        // one share: a warp turns its 32 rows x 32 columns around in shared memory of its own (eight lanes a row, whole
-        // lines), without a barrier of the CTA
+        // one share: a warp turns its 32 rows around in shared memory of its own, 64 columns at a time (16 lanes a row, or 8
+        // where the tile has no more columns: whole lines), without a barrier of the CTA.  The loop over the rows is short on
+        // purpose: every CTA runs this code once, and an unrolled form cost its length in instruction fetches
         if (warp < 8 && ok) {
-            uint32_t* mine = staged + (size_t)warp * 32 * WN_TURN;
+            uint32_t* mine = staged + (size_t)warp * 32 * ldt;
             const int q_own = S->q[m_own * TC_M + (warp & 3) * 32 + lane];
-            const int sub = lane >> 3, c4 = (lane & 7) * 4;
-            #pragma unroll (DT == T_F32 ? 2 : 1)
-            for (int k = 0; k < (DT == T_F32 ? 64 : 128); k += 32) {
-                const int cc = c_lo + k;
-                if (cc >= c_hi) continue;                    // (the same in all lanes)
-                uint32_t v[32];
-                take32(cc, k, v);
-                #pragma unroll
-                for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(mine + lane * WN_TURN + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            const bool narrow = p.bn <= 32;
+            const int sub = narrow ? lane >> 3 : lane >> 4, step = narrow ? 4 : 2, c4 = (narrow ? lane & 7 : lane & 15) * 4;
+            #pragma unroll 1
+            for (int cb = c_lo; cb < c_hi; cb += WN_TURN) {
+                put_row(cb, mine + lane * ldt);
                 __syncwarp();
-                uint32_t base4[4];
-                if (!adds) base_of(0, cc + c4, base4);       // (the bias: the same for every row)
-                #pragma unroll
-                for (int half = 0; half < 2; ++half) {
+                uint32_t base4[4] = {0, 0, 0, 0};
+                if (!adds) base_of(0, cb + c4, base4);       // (the bias: the same for every row)
+                #pragma unroll 1
+                for (int r0 = sub; r0 < 32; r0 += 4 * step) {
                     uint32_t o[4][4];
                     int q[4];
                     #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        q[i] = __shfl_sync(0xffffffffu, q_own, (half * 4 + i) * 4 + sub);
-                        if (adds) base_of(q[i], cc + c4, o[i]);
+                        q[i] = __shfl_sync(0xffffffffu, q_own, r0 + i * step);
+                        if (cb + c4 >= c_hi) q[i] = -1;
+                        if (adds) base_of(q[i], cb + c4, o[i]);
                         else { o[i][0] = base4[0]; o[i][1] = base4[1]; o[i][2] = base4[2]; o[i][3] = base4[3]; }
                     }
                     #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const uint4 t = *reinterpret_cast<const uint4*>(mine + ((half * 4 + i) * 4 + sub) * WN_TURN + c4);
+                        const uint4 t = *reinterpret_cast<const uint4*>(mine + (r0 + i * step) * ldt + c4);
                         o[i][0] = plus(o[i][0], t.x); o[i][1] = plus(o[i][1], t.y); o[i][2] = plus(o[i][2], t.z); o[i][3] = plus(o[i][3], t.w);
-                        emit(q[i], cc + c4, o[i]);
+                        emit(q[i], cb + c4, o[i]);
                     }
                 }
                 __syncwarp();
@@ -1003,15 +1019,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 const int r = m_own * TC_M + (warp & 3) * 32 + lane;
                 uint32_t* row = staged + (size_t)r * ldr;
                 const int lo = halves ? p0 : c_lo, hi = halves ? min(p0 + 64, c_hi) : c_hi;
-                #pragma unroll (DT == T_F32 ? 2 : 1)
-                for (int k = 0; k < 64; k += 32) {
-                    const int cc = lo + k;
-                    if (cc >= hi) continue;
-                    uint32_t v[32];
-                    take32(cc, k, v);
-                    #pragma unroll
-                    for (int j = 0; j < 32; j += 4) if (cc + j < hi) *reinterpret_cast<uint4*>(row + cc + j - p0) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                }
+                for (int cb = lo; cb < hi; cb += 64) put_row(cb, row + cb - p0);
                 const int q = S->q[r], end = min(hi, ncols);
                 fence_async_smem();                          // this thread's part of the row -> visible to the copy engine
                 if (q >= 0 && end > lo) {
@@ -1029,62 +1037,51 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         }
     } else if (p.cluster) {
         if (warp < 8 && ok) {
-            uint32_t* row = staged + (size_t)((warp & 3) * 32 + lane) * ldr;
-            #pragma unroll (DT == T_F32 ? 2 : 1)
-            for (int k = 0; k < 64; k += 32) {
-                const int cc = c_lo + k;
-                if (cc >= c_hi) continue;
-                uint32_t v[32];
-                take32(cc, k, v);
-                #pragma unroll
-                for (int j = 0; j < 32; j += 4) if (cc + j < c_hi) *reinterpret_cast<uint4*>(row + cc + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-            }
-            // rows split, split + ks, ... of the tile, a few at a time per warp (half a warp where the tile has up to 64
-            // columns), all shares' reads of a turn in flight together; what they are added to is on its way before the
-            // shares meet
+            if (c_lo < c_hi) put_row(c_lo, staged + (size_t)((warp & 3) * 32 + lane) * ldr + c_lo);
+            // rows split, split + ks, ... of the tile, two at a time per warp (half a warp where the tile has up to 64
+            // columns); of four shares' rows at a time all reads are in flight together, added in the order of the shares
             const bool wide = p.bn > 64;
             const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
             const int c = (wide ? lane : lane & 15) * 4;
-            auto close = [&](auto nr, auto ns) {
-                constexpr int NR = decltype(nr)::value, NS = decltype(ns)::value;
+            constexpr int NR = 2, NS = 4;
+            uint32_t base4[4] = {0, 0, 0, 0};
+            if (!adds) base_of(0, c, base4);                 // (the bias: the same for every row)
+            wn_cluster_meet();                               // every share's partial tile is in its shared memory
+            #pragma unroll 1
+            for (int k0 = team * NR; split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M; k0 += teams * NR) {      // (whole warps stay together)
                 uint32_t o[NR][4];
                 int q[NR];
-                auto begin = [&](int k0) {
-                    #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
-                        const int r = split + (k0 + u) * p.ks;
-                        q[u] = r < TC_M ? S->q[r] : -1;
-                        base_of(q[u], c, o[u]);
-                    }
-                };
-                begin(team * NR);
-                wn_cluster_meet();                           // every share's partial tile is in its shared memory
-                for (int k0 = team * NR; split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M;) {      // (whole warps stay together)
+                #pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const int r = split + (k0 + u) * p.ks;
+                    q[u] = r < TC_M ? S->q[r] : -1;
+                    if (adds) base_of(q[u], c, o[u]);
+                    else { o[u][0] = base4[0]; o[u][1] = base4[1]; o[u][2] = base4[2]; o[u][3] = base4[3]; }
+                }
+                #pragma unroll 1
+                for (int s0 = 0; s0 < p.ks; s0 += NS) {
                     uint4 t[NS][NR];
                     #pragma unroll
                     for (int s = 0; s < NS; ++s)
                         #pragma unroll
                         for (int u = 0; u < NR; ++u) {
                             t[s][u] = make_uint4(0, 0, 0, 0);
-                            if (s < p.ks && q[u] >= 0 && c < p.bn) t[s][u] = wn_ld_remote(smem_u32(staged + (size_t)(split + (k0 + u) * p.ks) * ldr + c), (uint32_t)s);
+                            if (s0 + s < p.ks && q[u] >= 0 && c < p.bn)
+                                t[s][u] = wn_ld_remote(smem_u32(staged + (size_t)(split + (k0 + u) * p.ks) * ldr + c), (uint32_t)(s0 + s));
                         }
                     #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
+                    for (int s = 0; s < NS; ++s) {
+                        if (s0 + s >= p.ks) break;
                         #pragma unroll
-                        for (int s = 0; s < NS; ++s) {
-                            if (s >= p.ks) break;
+                        for (int u = 0; u < NR; ++u) {
                             o[u][0] = plus(o[u][0], t[s][u].x); o[u][1] = plus(o[u][1], t[s][u].y);
                             o[u][2] = plus(o[u][2], t[s][u].z); o[u][3] = plus(o[u][3], t[s][u].w);
                         }
-                        emit(q[u], c, o[u]);
                     }
-                    k0 += teams * NR;
-                    if (split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M) begin(k0);
                 }
-            };
-            using std::integral_constant;
-            if (p.ks <= 4) close(integral_constant<int, 2>{}, integral_constant<int, 4>{});
-            else close(integral_constant<int, 2>{}, integral_constant<int, 8>{});
+                #pragma unroll
+                for (int u = 0; u < NR; ++u) emit(q[u], c, o[u]);
+            }
         } else wn_cluster_meet();
         wn_cluster_meet();                                   // nobody's shared memory goes away while it is read
     }
@@ -1297,8 +1294,9 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
         p.span = base_span + (mt - 1) * TC_M;
         if (p.span > WN_MAX_SPAN) continue;                  // (the tables hold no wider window: one tile, which win_geometry has checked)
         p.L = slots(p.span);
-        // drained rows: a tile's (64 columns of it where there are two), or 32 rows x 32 columns per warp
-        const size_t whole = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4, turned = (size_t)8 * 32 * WN_TURN * 4;
+        // drained rows: a tile's (64 columns of it where there are two), or 32 rows x up to 64 columns per warp
+        const size_t whole = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4;
+        const size_t turned = (size_t)8 * 32 * ((p.bn < WN_TURN ? p.bn : WN_TURN) + 4) * 4;
         const size_t staging = whole > turned ? whole : turned;
         int gblk = xcol ? p.groups : (p.groups < 4 ? p.groups : 4);
         if (f32 && !xcol) while (gblk > 1 && gblk * plane_taps > 18) gblk = (gblk + 1) / 2;
