@@ -216,6 +216,7 @@ struct Layer {
     // window kernel (rrm_conv_win.cu)
     bool win_ready = false;
     void* win_Wimg = nullptr;               // [n_tiles][tap][K group][pieces][2][bn][16 bytes] operand tiles of the filters
+    void* win_Wnarrow = nullptr;            // integers: the same as tiles of 32 columns (launches of few tiles)
     int win_bn = 0, win_ntiles = 0;
     int win_tiles = 0;                      // accumulator tiles of 128 rows that cover the layer once
     void* Apre = nullptr;                   // pooled integer layers: f before the pool window, a row per projection pixel (keyframes)

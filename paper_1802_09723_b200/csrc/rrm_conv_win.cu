@@ -56,6 +56,7 @@ constexpr int WN_MAX_STAGES = 8, WN_MAX_ABUF = 4, WN_MAX_MT = 2;
 constexpr int WN_MAX_SPAN = 1152;             // pixels of one plane of a window
 constexpr int WN_TURN = 64;                  // columns of its 32 rows that a warp turns around at a time
 constexpr int WN_PROMOTE = 32;                // fp32: K steps the leading product accumulates before it is promoted
+constexpr int WN_NARROW = 32;                 // integers: columns of a tile where the wide ones are too few
 constexpr size_t WN_SMEM_LIMIT = 227 * 1024;
 
 // One plane's taps: first filter row / column and their numbers, the remainders of its pixels, the first tap's shift.
@@ -88,6 +89,7 @@ struct WinParams {
     int tsplit;               // > 1: a share is one block's taps, cut into so many parts (ks = nblk * tsplit)
     int cluster;              // the shares of a tile form a cluster that adds them up (0: each adds onto the projection by itself)
     int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
+    int ntiles, narrow;       // column tiles, and whether they are the narrow ones
     int tps, stages, abuf;    // taps per filter stage, stages, window buffers
     int xarr;                 // first layers: arrays of an image row's chunks (0: the chunks of every column side by side)
     unsigned a_step, a_lbo;   // 16-byte slots between a pixel's K groups, and between the two chunks of a group
@@ -1039,16 +1041,17 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         if (warp < 8 && ok) {
             if (c_lo < c_hi) put_row(c_lo, staged + (size_t)((warp & 3) * 32 + lane) * ldr + c_lo);
             // rows split, split + ks, ... of the tile, two at a time per warp (half a warp where the tile has up to 64
-            // columns); of four shares' rows at a time all reads are in flight together, added in the order of the shares
-            const bool wide = p.bn > 64;
-            const int team = wide ? warp : warp * 2 + (lane >> 4), teams = wide ? 8 : 16;
-            const int c = (wide ? lane : lane & 15) * 4;
+            // columns, a quarter up to 32); of four shares' rows at a time all reads are in flight together, added in the
+            // order of the shares
+            const int lpr = p.bn > 64 ? 5 : (p.bn > 32 ? 4 : 3);                 // (log2 of the lanes of a row)
+            const int team = lane >> lpr, c = (lane & ((1 << lpr) - 1)) * 4;
             constexpr int NR = 2, NS = 4;
             uint32_t base4[4] = {0, 0, 0, 0};
             if (!adds) base_of(0, c, base4);                 // (the bias: the same for every row)
             wn_cluster_meet();                               // every share's partial tile is in its shared memory
             #pragma unroll 1
-            for (int k0 = team * NR; split + (wide ? k0 : k0 & ~(2 * NR - 1)) * p.ks < TC_M; k0 += teams * NR) {      // (whole warps stay together)
+            for (int kb = warp * (32 >> lpr) * NR; split + kb * p.ks < TC_M; kb += 8 * (32 >> lpr) * NR) {
+                const int k0 = kb + team * NR;
                 uint32_t o[NR][4];
                 int q[NR];
                 #pragma unroll
@@ -1274,9 +1277,19 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
 {
     const bool f32 = L.d.dtype == RRM_F32;
     const int pieces = f32 ? 3 : 1;
-    p.bn = L.win_bn;
     const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
-    const long long tiles = (rows + TC_M - 1) / TC_M * L.win_ntiles * frames;
+    const long long row_tiles = (rows + TC_M - 1) / TC_M * frames;
+    // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
+    // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
+    const bool clustered = dense || store || f32 || (p.c_out & 3) != 0;
+    // Integers whose shares would form a cluster, and whose tiles leave half of the wave idle: tiles of 32 columns first.  A
+    // cluster's way out (two meetings, rows read from the other shares) takes 8 to 10 k clocks with 128 columns, an MMA of 32
+    // columns two thirds of one of 128 (77 clocks: the reads of its rows).  256 -> 256 3x3 at 14 x 14, 4 images: 16.0 -> 14.0 k
+    // clocks a CTA; 96 -> 256 5x5 at 27 x 27: 16.6 -> 13.0 k.  Shares that add by themselves are as fast with wide tiles.
+    p.narrow = clustered && L.win_Wnarrow && row_tiles * L.win_ntiles * 2 <= wave;
+    p.bn = p.narrow ? WN_NARROW : L.win_bn;
+    p.ntiles = p.narrow ? L.win_ntiles * L.win_bn / WN_NARROW : L.win_ntiles;
+    const long long tiles = row_tiles * p.ntiles;
     const int base_span = p.span, planes = p.planes;
     const int plane_taps = ceil_div(p.kh, p.stride) * (xcol ? 1 : ceil_div(p.kw, p.stride));
     const size_t unit = (size_t)p.bn * 32 * pieces, tail = sizeof(WinTail) + 128;
@@ -1284,11 +1297,11 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     // two accumulator tiles per CTA share every filter stage (what bounds a full machine is the filters' way from L2),
     // once that leaves a CTA per SM
     int mt = !f32 && tiles >= 2ll * 148 && rows > TC_M ? 2 : 1;
-    // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
-    // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
-    const bool clustered = dense || store || f32 || (p.c_out & 3) != 0;
+    // (a cluster of narrow tiles is worth it for shares of some 48 K steps)
+    const int steps = p.groups * p.kh * (xcol ? 1 : p.kw);
+    const int most = !clustered ? 16 : (!p.narrow ? 8 : (steps < 96 ? 1 : (steps / 48 < 8 ? steps / 48 : 8)));
     int want = 1;
-    while (mt == 1 && want < (clustered ? 8 : 16) && tiles * (want + 1) <= wave) ++want;
+    while (mt == 1 && want < most && tiles * (want + 1) <= wave) ++want;
     for (; mt >= 1; mt /= 2) {
         p.mt = mt;
         p.span = base_span + (mt - 1) * TC_M;
@@ -1373,14 +1386,18 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     const int taps = xcol ? d.kh : d.kh * d.kw;
     const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
     const size_t bytes = chunks * 16 * (f32 ? 3 : 1);
+    const bool narrow = !f32 && L.win_bn > WN_NARROW;        // (the same filters once more, as tiles of 32 columns)
     void* img = nullptr;
-    if (cudaMalloc(&img, bytes + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
+    if (cudaMalloc(&img, bytes * (narrow ? 2 : 1) + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
     net->allocs.push_back(img);
     const unsigned grid = (unsigned)((chunks + 255) / 256);
     unsigned char* im = reinterpret_cast<unsigned char*>(img);
-    int* beyond = reinterpret_cast<int*>(im + bytes);
+    int* beyond = reinterpret_cast<int*>(im + bytes * (narrow ? 2 : 1));
     RRM_CUDA_TRY(cudaMemset(beyond, 0, 4));
-    auto pack = [&](auto kernel) { kernel<<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles, beyond); };
+    auto pack = [&](auto kernel) {
+        kernel<<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles, beyond);
+        if (narrow) kernel<<<grid, 256>>>(W_dev, im + bytes, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, WN_NARROW, L.win_ntiles * L.win_bn / WN_NARROW, beyond);
+    };
     if (f32) { if (xcol) pack(pack_weights_win_kernel<T_F32, true>); else pack(pack_weights_win_kernel<T_F32, false>); }
     else if (xcol) pack(pack_weights_win_kernel<T_I8, true>);
     else pack(pack_weights_win_kernel<T_I8, false>);
@@ -1395,6 +1412,7 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
         }
     }
     L.win_Wimg = img;
+    if (narrow) L.win_Wnarrow = im + bytes;
     RRM_TRY((win_allow<T_F32, true>())); RRM_TRY((win_allow<T_F32, false>()));
     RRM_TRY((win_allow<T_I8, true>())); RRM_TRY((win_allow<T_I8, false>()));
     RRM_TRY((win_allow<T_BIN, false>()));
@@ -1428,7 +1446,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     p.A = bin ? in.D : (dense ? X : in.D);
     p.Anew = (!dense && !stateless && in.Xn_cur) ? in.Xn_cur : X;    // (chunks of frames: this frame's copy of the new rows)
     p.in_act = in.act; p.oact = L.oact; p.ocount = L.ocount;
-    p.Wimg = reinterpret_cast<const unsigned char*>(L.win_Wimg); p.bias = L.bias;
+    p.Wimg = reinterpret_cast<const unsigned char*>(p.narrow ? L.win_Wnarrow : L.win_Wimg); p.bias = L.bias;
     p.P = P_dst && !dense ? P_dst : (stateless ? L.P2 : L.P);
     p.errw = net->errw;
     p.wait_limit = net->opt.wait_limit;
@@ -1442,7 +1460,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
         p.P = out->P; p.keep_from = out->P ? out->keep_from : INT_MAX;
     }
     const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
-    const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)L.win_ntiles, (unsigned)(nf * p.ks));
+    const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)p.ntiles, (unsigned)(nf * p.ks));
     const size_t smem = win_smem(p);
     cudaError_t e;
     if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, out, grid, smem, st) : win_launch<T_F32, false>(p, dense, out, grid, smem, st);

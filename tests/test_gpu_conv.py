@@ -274,6 +274,20 @@ def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
     net.close()
 
 
+@pytest.mark.parametrize("dtype", ["i8", "bin"])
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [
+    (64, 70, (14, 13), 3, 1, 1, 1), (320, 200, (13, 13), 3, 1, 1, 1),         # one share (18 and 90 K steps), ragged columns
+    (352, 130, (9, 11), 3, 1, 1, 2), (512, 64, (7, 7), 3, 1, 1, 4), (96, 96, (17, 18), 5, 2, 2, 3),      # clusters of 2 and 3, strides
+    (3, 96, (60, 61), 11, 4, 0, 1), (32, 33, (8, 8), 1, 1, 0, 1)])
+def test_dense_passes_of_few_tiles_take_narrow_ones(dtype, c_in, c_out, hw, k, s, p, n):
+    """Keyframes and dense passes whose tiles would leave the machine idle run as tiles of 32 columns; with f in the kernel
+    (int8, signs), as raw projections, and with delta steps in between."""
+    rng = np.random.default_rng(c_in + c_out)
+    for kw in ((dict(act="sign", theta=1), dict(shift=-1, act="none")) if dtype == "bin" else (dict(act="relu", shift=8), dict(shift=-1, act="none"))):
+        sp = _spec(dtype, c_in, hw, c_out, k, s, p, rng, **kw)
+        _run([sp], _video(dtype, c_in, hw, 4, n, rng), n=n, stats=True, keyframe_at=(1, 3))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p,pool", [
     (24, 20, (5, 700), 3, 1, 1, (3, 2, 0)),  # wider than 510 pixels
