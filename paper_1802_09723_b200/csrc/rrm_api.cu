@@ -336,7 +336,10 @@ int build_graph(rrm_net* net, int kind, unsigned long long mask)
     if (stateless) RRM_TRY(ensure_stateless(net));           // allocations cannot happen inside a capture
     if (!net->cap_stream) RRM_CUDA_TRY(cudaStreamCreateWithFlags(&net->cap_stream, cudaStreamNonBlocking));
     RRM_CUDA_TRY(cudaStreamBeginCapture(net->cap_stream, cudaStreamCaptureModeThreadLocal));
-    const int s = launch_sequence(net, net->frame_buf, net->out_buf, net->cap_stream, dense, stateless, mask);
+    const int s = [&] {
+        const OverlapLaunches overlap(dense);
+        return launch_sequence(net, net->frame_buf, net->out_buf, net->cap_stream, dense, stateless, mask);
+    }();
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(net->cap_stream, &g);
     if (s != RRM_OK || e != cudaSuccess || !g) { if (g) cudaGraphDestroy(g); cudaGetLastError(); return s != RRM_OK ? s : RRM_ERR_CUDA; }
@@ -704,6 +707,7 @@ static int build_dense_batch_graph(rrm_net* net, int kind, int T)
     int status = RRM_OK;
     auto fail = [&](int s) { if (status == RRM_OK && s != RRM_OK) status = s; };
     RRM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    const OverlapLaunches overlap;
     if (cudaMemsetAsync(net->chunk_arena[0], 0, net->cleared_bytes, st) != cudaSuccess) fail(RRM_ERR_CUDA);
     for (int m0 = 0; m0 < T && status == RRM_OK; m0 += per) {
         const int F = T - m0 < per ? T - m0 : per;

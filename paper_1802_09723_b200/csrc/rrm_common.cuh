@@ -31,18 +31,33 @@ namespace rrm {
 
 // ---- programmatic dependent launch between the kernels of a per-frame sequence --------------------------------
 // Every kernel of the sequence lets its successor start launching at once (launch_dependents at its top) and waits
-// for its predecessor's results (pdl_wait) only when it first needs global memory: thread-block scheduling, barrier
-// initialisation and tensor-memory allocation of kernel k+1 then overlap the tail of kernel k.  Without the launch
-// attribute both instructions do nothing.  Measured on B200 inside replayed graphs the attribute moves a step by
-// -8 % .. +27 % depending on the stack (the graph's own launch gaps are already small), so it is opt-in:
-// RRM_PDL=1 in the environment launches with the attribute.
+// for its predecessor's results (pdl_wait) only when it first needs what a predecessor writes: thread-block scheduling,
+// barrier initialisation, tensor-memory allocation, window tables and first filter copies of kernel k+1 then overlap the tail
+// of kernel k.  Some thread of every grid waits, so a grid ends after its predecessors, and a wait covers them all.  What a
+// predecessor wrote is read with ordinary loads (not through the read-only path).  Without the launch attribute both
+// instructions do nothing.  The attribute is set (OverlapLaunches) while a dense
+// pass, a keyframe or a dense chunk is captured: there most of a kernel's set-up needs nothing of its predecessor, and a pass
+// of 25 launches went from 206 to 189 us (4 ResNet-18-shaped streams), one of 12 from 104 to 97 (24 AlexNet-shaped keyframes).
+// Delta steps, whose kernels start with their predecessor's bitmaps, gained nothing or lost (one int8 frame 63.7 -> 65.3
+// us), and graphs whose frames overlap have their own edges and fill the machine by themselves.  RRM_PDL=1 in the
+// environment sets it everywhere, RRM_PDL=0 nowhere.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The launches of this thread overlap their predecessors while an object of this kind lives.
+struct OverlapLaunches {
+    static int& depth() { static thread_local int d = 0; return d; }
+    const int by;
+    explicit OverlapLaunches(bool on = true) : by(on ? 1 : 0) { depth() += by; }
+    ~OverlapLaunches() { depth() -= by; }
+    OverlapLaunches(const OverlapLaunches&) = delete;
+    OverlapLaunches& operator=(const OverlapLaunches&) = delete;
+};
+
 inline bool pdl_enabled()
 {
-    static const bool on = [] { const char* e = getenv("RRM_PDL"); return e && e[0] == '1'; }();
-    return on;
+    static const char asked = [] { const char* e = getenv("RRM_PDL"); return e ? e[0] : '\0'; }();
+    return asked == '1' || (asked != '0' && OverlapLaunches::depth() > 0);
 }
 
 // cluster_z > 1: the CTAs that differ only in blockIdx.z form one thread-block cluster (they can read each other's

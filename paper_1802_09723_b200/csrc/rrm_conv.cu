@@ -58,10 +58,10 @@ struct ConvParams {
 };
 
 // The number of set bits of bm[0 .. words) -> *out, by one CTA (the activity of a layer that is evaluated densely).
-__device__ __forceinline__ void count_bits_cta(const uint32_t* __restrict__ bm, int words, int* out, int* s_scratch)
+__device__ __forceinline__ void count_bits_cta(const uint32_t* bm, int words, int* out, int* s_scratch)
 {
     int c = 0;
-    for (int i = threadIdx.x; i < words; i += blockDim.x) c += __popc(__ldg(bm + i));
+    for (int i = threadIdx.x; i < words; i += blockDim.x) c += __popc(bm[i]);
     #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0) s_scratch[threadIdx.x >> 5] = c;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(CONV_THREADS) conv_gemm_kernel(ConvParams p)
             for (int g = tid >> 5; g < nfr; g += CONV_THREADS / 32) {
                 const uint32_t* bm = reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(p.oact) + (long long)g * p.arena_stride);
                 int c = 0;
-                for (int i = lane; i < words; i += 32) c += __popc(__ldg(bm + i));
+                for (int i = lane; i < words; i += 32) c += __popc(bm[i]);
                 c = __reduce_add_sync(0xffffffffu, c);
                 if (lane == 0) s_fcnt[g] = c;
             }
@@ -902,7 +902,7 @@ struct TileGrid {
 // 30 frames of 45 x 45: export of 80 channels 24 -> 6.2 us against a thread per element, import of 48 channels 10.8 -> 7.0
 // against the 32-pixel tiles.
 template <bool EXPORT>
-__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* __restrict__ src, int8_t* dst, int c, int cs, int hw, TileGrid tg,
+__global__ void __launch_bounds__(256) transpose_i8_kernel(const int8_t* src, int8_t* dst, int c, int cs, int hw, TileGrid tg,
                                                           long long src_stride, long long dst_stride)
 {
     __shared__ __align__(16) int8_t tile[32][132];
@@ -1352,7 +1352,7 @@ __global__ void __launch_bounds__(256) epilogue_kernel(EpiParams p)
 // Exports to the boundary layout.
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void export_nchw_kernel(const T* __restrict__ src, T* dst, int c, int cs, int hw, long long total,
+__global__ void export_nchw_kernel(const T* src, T* dst, int c, int cs, int hw, long long total,
                                    long long src_stride = 0, long long dst_stride = 0)   // elements between frames (frame = blockIdx.y)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1369,7 +1369,7 @@ __global__ void export_nchw_kernel(const T* __restrict__ src, T* dst, int c, int
 
 // The same through a 32 x 32 tile in shared memory (4-byte elements): rows read along the channels, planes written
 // along the pixels, both coalesced.  block = (32, 8).
-__global__ void __launch_bounds__(256) export_nchw_tiled_kernel(const uint32_t* __restrict__ src, uint32_t* dst, int c, int cs, int hw,
+__global__ void __launch_bounds__(256) export_nchw_tiled_kernel(const uint32_t* src, uint32_t* dst, int c, int cs, int hw,
                                                                 TileGrid tg, long long src_stride, long long dst_stride)
 {
     __shared__ uint32_t tile[32][33];

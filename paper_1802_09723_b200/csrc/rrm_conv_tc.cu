@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) conv_tc_kernel(TcParams p)
     if (DENSE && p.count_bitmap && tile == 0 && ntile == 0 && split == 0) {
         // (uniform for the whole CTA) the layer's activity is still measured while it is evaluated densely
         int c = 0;
-        for (int i = tid; i < ((p.opixels + 31) >> 5); i += TC_THREADS) c += __popc(__ldg(p.count_bitmap + i));
+        for (int i = tid; i < ((p.opixels + 31) >> 5); i += TC_THREADS) c += __popc(p.count_bitmap[i]);
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
         if (lane == 0) s_tmp[warp] = c;

@@ -241,8 +241,9 @@ __device__ __forceinline__ bool wn_bf16_nan(uint32_t a) { return (a & 0x7fffu) >
 __device__ __forceinline__ uint32_t wn_spread4(uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; }
 __device__ __forceinline__ int wn_div(int x, const WinDiv& d) { return (int)((unsigned long long)(unsigned)x * d.m >> d.sh); }
 
-// The windows' table for one plane: where each window pixel lies in the input.
-template <bool DENSE, bool XCOL>
+// The windows' table for one plane: where each window pixel lies in the input.  EARLY: without a look at the activity (the
+// pixel's number is kept for wn_table_active, which the same threads run over their entries later).
+template <bool DENSE, bool XCOL, bool EARLY = false>
 __device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_act, WinTail* S, int lin0, int plane)
 {
     const int ry = p.plane[plane].ry, rx = p.plane[plane].rx;
@@ -263,12 +264,21 @@ __device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_
                 const int ix = X * p.stride + rx;
                 if (img < p.n && iy < p.h && ix < p.w) {
                     const int pix = (img * p.h + iy) * p.w + ix;
-                    if (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u)) off = pix * p.row_units;
+                    if (EARLY || DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u)) off = pix * p.row_units;
+                    if (EARLY) x0 = pix;
                 }
             }
         }
         S->src[i] = off;
-        if (XCOL) S->x0[i] = x0;
+        if (XCOL || EARLY) S->x0[i] = x0;
+    }
+}
+__device__ __forceinline__ void wn_table_active(const WinParams& p, const uint32_t* in_act, WinTail* S)
+{
+    #pragma unroll 2
+    for (int i = threadIdx.x; i < p.span; i += WN_FILL) {
+        const int pix = S->x0[i];
+        if (S->src[i] >= 0 && !((in_act[pix >> 5] >> (pix & 31)) & 1u)) S->src[i] = -1;
     }
 }
 
@@ -419,26 +429,40 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&S->bfull[s]), 1); mbar_init(smem_u32(&S->bempty[s]), 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // ---- the tile's rows, and the first plane's table
-    int active;
+    // ---- the tile's rows, and the first plane's table.  All that is no predecessor's work comes before the wait for them: a
+    // launch that overlaps its predecessor's tail then has its barriers, tensor memory, tables and, in dense passes, its
+    // first filters at hand when the inputs arrive
+    int active = 0;
     {
         int q = -1;
-        bool bit = false;
         if (tid < WN_FILL) {
-            pdl_wait();                                      // bitmaps and inputs are the predecessors' work
             if (tid < p.mt * TC_M) {
                 const int hwq = p.Hq * p.Wq;
                 const int lin = lin0 + tid, img = wn_div(lin, p.div_img), rem = lin - img * hwq, oy = wn_div(rem, p.div_row), ox = rem - oy * p.Wq;
                 if (img < p.n && oy < p.oh && ox < p.ow) q = (img * p.oh + oy) * p.ow + ox;
-                if (!DENSE && q >= 0 && !((oact[q >> 5] >> (q & 31)) & 1u)) q = -1;
-                bit = DENSE ? (p.count_bitmap && q >= 0 && ((p.count_bitmap[q >> 5] >> (q & 31)) & 1u)) : q >= 0;
-                S->q[tid] = q;
+                if (DENSE) S->q[tid] = q;
             }
-            wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane0);
+            wn_table<DENSE, XCOL, !DENSE && !XCOL>(p, in_act, S, lin0, plane0);
             if (ACT && tid < p.bn) S->bias[tid] = p.bias && ntile * p.bn + tid < p.c_out ? reinterpret_cast<const int*>(p.bias)[ntile * p.bn + tid] : 0;
         }
-        tc_fence_before();
-        active = __syncthreads_count(bit);
+        if (!DENSE || p.count_bitmap) {
+            bool bit = false;
+            if (tid < WN_FILL) {
+                pdl_wait();                                  // bitmaps and inputs are the predecessors' work
+                if (q >= 0) {
+                    const uint32_t* bits = DENSE ? p.count_bitmap : oact;
+                    bit = (bits[q >> 5] >> (q & 31)) & 1u;
+                }
+                if (!DENSE && tid < p.mt * TC_M) S->q[tid] = bit ? q : -1;
+                if (!DENSE && !XCOL) wn_table_active(p, in_act, S);
+            }
+            tc_fence_before();
+            active = __syncthreads_count(bit);
+        } else {
+            tc_fence_before();
+            __syncthreads();
+            if (warp != 9) pdl_wait();                       // (the filters are constants: their warp waits when the ring is full)
+        }
         tc_fence_after();
         if (active && tid == 0 && ntile == 0 && split == 0) {
             int* oc = shift_bytes(p.ocount, arena_off);
@@ -687,6 +711,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 const unsigned char* src = p.Wimg + ((size_t)ntile * (row_taps * p.kh) * p.groups + g0) * unit_b +
                                            (size_t)((p.plane[plane].ky0 + jy * p.stride) * row_taps + p.plane[plane].kx0 + jx * p.stride) * tap_bytes;
                 while (lt < t_end) {
+                    if (DENSE && issued == p.stages) pdl_wait();      // (bounded waits are for this launch's own work, not for its predecessors')
                     if (!mbar_wait(smem_u32(&S->bempty[stage]), phase, p.wait_limit) || *(volatile int*)&S->fail) { ok = false; break; }
                     const int tn = min(p.tps, t_end - lt);
                     const uint32_t bar = smem_u32(&S->bfull[stage]);
@@ -1103,7 +1128,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
 // (the sign of a maximum is the OR of the signs).  Bound by its reads; the int32 projections it would otherwise read are
 // four times as many bytes.
 template <int KW, bool BITS>
-__global__ void __launch_bounds__(256) pool_window_kernel(const void* __restrict__ A, void* X, int oh, int ow, int th, int tw, int units, int s,
+__global__ void __launch_bounds__(256) pool_window_kernel(const void* A, void* X, int oh, int ow, int th, int tw, int units, int s,
                                                           int pad, int total)
 {
     using T = typename std::conditional<BITS, uint32_t, uint4>::type;

@@ -59,7 +59,7 @@ __device__ __forceinline__ int fc_apply_f(int v, int shift, int act)
 // One filter row at a time: its usable taps are a run of consecutive input pixels, whose activity bits come out of
 // one or two bitmap words together; filters wider than 32 taps go tap by tap, 8 bitmap loads in flight.
 template <bool DENSE>
-__device__ __forceinline__ void row_tap_masks(const uint32_t* __restrict__ in_act, int pix0, int y0, int x0, int h, int w, int kh, int kw,
+__device__ __forceinline__ void row_tap_masks(const uint32_t* in_act, int pix0, int y0, int x0, int h, int w, int kh, int kw,
                                               unsigned long long& m0, unsigned long long& m1)
 {
     m0 = 0; m1 = 0;

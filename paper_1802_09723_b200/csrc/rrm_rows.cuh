@@ -89,14 +89,14 @@ __device__ __forceinline__ void scatter_changed_warp(const Readers& R, int ns, i
 // every row which thread's share holds its bit, and the row walks that share (a few words) itself:
 // all TM rows are located in parallel.
 template <int TM>
-__device__ int select_rows(const uint32_t* __restrict__ bm, int words, int tile, int* s_q, int* s_pref)
+__device__ int select_rows(const uint32_t* bm, int words, int tile, int* s_q, int* s_pref)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nwarps = (nt + 31) >> 5;
     int* s_warp = s_pref + 257;
     const int nper = (words + nt - 1) / nt;
     const int lo = min(words, tid * nper), hi = min(words, lo + nper);
     int mine = 0;
-    for (int i = lo; i < hi; ++i) mine += __popc(__ldg(bm + i));
+    for (int i = lo; i < hi; ++i) mine += __popc(bm[i]);
     int incl = mine;
     #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -123,7 +123,7 @@ __device__ int select_rows(const uint32_t* __restrict__ bm, int words, int tile,
                 if (t + step < nt && s_pref[t + step] <= rank) t += step;
             int k = rank - s_pref[t];
             for (int i = t * nper; i < words; ++i) {
-                const uint32_t w = __ldg(bm + i);
+                const uint32_t w = bm[i];
                 const int c = __popc(w);
                 if (k < c) { q = i * 32 + (int)__fns(w, 0, k + 1); break; }
                 k -= c;
