@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             mbar_arrive(smem_u32(&S->dempty[pb]));
             return true;
         };
-        const bool lag = DT == T_I8 && !XCOL && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
+        const bool lag = DT == T_I8 && !XCOL && !DENSE && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
         int plane = plane0, chb = b0 - plane0 * p.nchb, ib = 0, buf = -1;
         uint32_t phase = 0;                                  // of aempty: the ring's first filling waits for nobody
         for (int b = b0; b < b1; ++b, ++ib) {
@@ -533,7 +533,32 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const uint32_t piece = (uint32_t)(arrays * p.L) * 16u;              // bytes between the fp32 pieces' windows
             const unsigned magic = cl > 1 ? (unsigned)(((1ull << 32) + cl - 1) / cl) : 0u;
             const int items = p.span * cl;
-            if (DT == T_I8 && !XCOL) {
+            if (DT == T_I8 && !XCOL && DENSE) {
+                // Dense blocks are many and full: through registers, a turn's loads all on their way before its first store.
+                // (Asynchronous copies, handed over when the next block's were on their way, took 2.3 to 3 k clocks a block: 24
+                // AlexNet-shaped keyframes 97.2 -> 93.2 us, 4 ResNet-18-shaped streams 188.9 -> 181.8.)
+                const unsigned char* src0 = reinterpret_cast<const unsigned char*>(A) + g0 * 32;
+                constexpr int TURN = 6;
+                #pragma unroll 1
+                for (int idx = tid; idx < items; idx += TURN * WN_FILL) {
+                    uint4 v[TURN];
+                    #pragma unroll
+                    for (int u = 0; u < TURN; ++u) {
+                        const int id = idx + u * WN_FILL, i = magic ? (int)__umulhi((unsigned)id, magic) : id, c = id - i * cl;
+                        const int off = id < items ? S->src[i] : -1;
+                        v[u] = make_uint4(0, 0, 0, 0);
+                        if (off >= 0) v[u] = __ldcg(reinterpret_cast<const uint4*>(src0 + off + c * 16));
+                    }
+                    #pragma unroll
+                    for (int u = 0; u < TURN; ++u) {
+                        const int id = idx + u * WN_FILL, i = magic ? (int)__umulhi((unsigned)id, magic) : id, c = id - i * cl;
+                        if (id < items) *reinterpret_cast<uint4*>(Ap + (size_t)(c * p.L + i) * 16) = v[u];
+                    }
+                }
+                fence_async_smem();
+                mbar_arrive(smem_u32(&S->afull[buf]));
+            } else if (DT == T_I8 && !XCOL) {
+                // delta rows: asynchronous copies (one frame's steps, one small block per CTA: 64.2 us against 65.8 through registers)
                 const unsigned char* src0 = reinterpret_cast<const unsigned char*>(A) + g0 * 32;
                 #pragma unroll 4
                 for (int idx = tid; idx < items; idx += WN_FILL) {
@@ -686,7 +711,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 // (a warp whose wait ran out says so when the warps meet at the next block)
             }
         }
-        if (DT == T_I8 && !XCOL) {
+        if (DT == T_I8 && !XCOL && !DENSE) {
             cp_async_wait<0>();
             fence_async_smem();
             if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[buf]));
