@@ -81,7 +81,7 @@ struct WinParams {
     int row_units;            // units per input pixel: bytes, words or floats
     int Wq, Hq;               // pitches of the linear output space
     int min_shift, span, L;   // window: first pixel relative to the tile's first, pixels, 16-byte slots per K chunk
-    int planes;
+    int planes, all_tables;   // (all_tables: the planes' tables have room side by side)
     WinPlane plane[WN_MAX_PLANES];
     WinDiv div_img, div_row;  // by Hq * Wq and by Wq
     int groups, gblk, nchb, nblk;   // 32-byte K groups per tap, groups per block, channel blocks per plane, blocks
@@ -114,8 +114,10 @@ struct WinTail {
     int exact;                                // fp32: a window holds a value whose pieces are no finite numbers
     alignas(16) int bias[128];                // of the CTA's columns (f in the kernel)
     int q[WN_MAX_MT * TC_M];                  // projection pixel of the row (-1: none, or not to be updated)
-    int src[WN_MAX_SPAN];                     // input pixel's offset in units (first layers: of its image row's first pixel, in pixels), -1: zero
-    int x0[WN_MAX_SPAN];                      // first layers: first input column under the filter row * 256 + input rows from the tap's first on (at most 255)
+    // the windows' tables, one behind the other: per window pixel of a plane its offset in the input in units, -1: zero (first
+    // layers: of its image row's first pixel, in pixels; and behind them, in the second half, the first input column under the
+    // filter row * 256 + the input rows from the tap's first on, at most 255)
+    int tab[2 * WN_MAX_SPAN];
 };
 
 // ---- small device helpers
@@ -241,10 +243,9 @@ __device__ __forceinline__ bool wn_bf16_nan(uint32_t a) { return (a & 0x7fffu) >
 __device__ __forceinline__ uint32_t wn_spread4(uint32_t x) { return ((x & 0xfu) * 0x00204081u) & 0x01010101u; }
 __device__ __forceinline__ int wn_div(int x, const WinDiv& d) { return (int)((unsigned long long)(unsigned)x * d.m >> d.sh); }
 
-// The windows' table for one plane: where each window pixel lies in the input.  EARLY: without a look at the activity (the
-// pixel's number is kept for wn_table_active, which the same threads run over their entries later).
-template <bool DENSE, bool XCOL, bool EARLY = false>
-__device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_act, WinTail* S, int lin0, int plane)
+// The windows' table for one plane: where each window pixel lies in the input.
+template <bool DENSE, bool XCOL>
+__device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_act, int* tab, int lin0, int plane)
 {
     const int ry = p.plane[plane].ry, rx = p.plane[plane].rx;
     const int hwq = p.Hq * p.Wq;
@@ -264,21 +265,12 @@ __device__ __forceinline__ void wn_table(const WinParams& p, const uint32_t* in_
                 const int ix = X * p.stride + rx;
                 if (img < p.n && iy < p.h && ix < p.w) {
                     const int pix = (img * p.h + iy) * p.w + ix;
-                    if (EARLY || DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u)) off = pix * p.row_units;
-                    if (EARLY) x0 = pix;
+                    if (DENSE || ((in_act[pix >> 5] >> (pix & 31)) & 1u)) off = pix * p.row_units;
                 }
             }
         }
-        S->src[i] = off;
-        if (XCOL || EARLY) S->x0[i] = x0;
-    }
-}
-__device__ __forceinline__ void wn_table_active(const WinParams& p, const uint32_t* in_act, WinTail* S)
-{
-    #pragma unroll 2
-    for (int i = threadIdx.x; i < p.span; i += WN_FILL) {
-        const int pix = S->x0[i];
-        if (S->src[i] >= 0 && !((in_act[pix >> 5] >> (pix & 31)) & 1u)) S->src[i] = -1;
+        tab[i] = off;
+        if (XCOL) tab[WN_MAX_SPAN + i] = x0;
     }
 }
 
@@ -435,6 +427,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
     int active = 0;
     {
         int q = -1;
+        uint32_t word = 0;                                   // of the layer's update bitmap
         if (tid < WN_FILL) {
             if (tid < p.mt * TC_M) {
                 const int hwq = p.Hq * p.Wq;
@@ -442,20 +435,21 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 if (img < p.n && oy < p.oh && ox < p.ow) q = (img * p.oh + oy) * p.ow + ox;
                 if (DENSE) S->q[tid] = q;
             }
-            wn_table<DENSE, XCOL, !DENSE && !XCOL>(p, in_act, S, lin0, plane0);
+            if (!DENSE) {
+                pdl_wait();                                  // bitmaps and inputs are the predecessors' work
+                if (q >= 0) word = oact[q >> 5];             // (on its way together with the table's words)
+            }
+            wn_table<DENSE, XCOL>(p, in_act, S->tab, lin0, plane0);
+            if (!XCOL && p.all_tables) for (int b = plane0 + 1; b * p.nchb < b1; ++b) wn_table<DENSE, XCOL>(p, in_act, S->tab + (b - plane0) * p.span, lin0, b);
             if (ACT && tid < p.bn) S->bias[tid] = p.bias && ntile * p.bn + tid < p.c_out ? reinterpret_cast<const int*>(p.bias)[ntile * p.bn + tid] : 0;
         }
         if (!DENSE || p.count_bitmap) {
-            bool bit = false;
-            if (tid < WN_FILL) {
-                pdl_wait();                                  // bitmaps and inputs are the predecessors' work
-                if (q >= 0) {
-                    const uint32_t* bits = DENSE ? p.count_bitmap : oact;
-                    bit = (bits[q >> 5] >> (q & 31)) & 1u;
-                }
-                if (!DENSE && tid < p.mt * TC_M) S->q[tid] = bit ? q : -1;
-                if (!DENSE && !XCOL) wn_table_active(p, in_act, S);
+            if (DENSE && tid < WN_FILL) {
+                pdl_wait();
+                if (q >= 0) word = p.count_bitmap[q >> 5];
             }
+            const bool bit = q >= 0 && (word >> (q & 31) & 1u);
+            if (!DENSE && tid < p.mt * TC_M) S->q[tid] = bit ? q : -1;
             tc_fence_before();
             active = __syncthreads_count(bit);
         } else {
@@ -509,6 +503,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             return true;
         };
         const bool lag = DT == T_I8 && !XCOL && !DENSE && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
+        const int* src = S->tab;                             // the plane's table
+        const int* const xcol0 = S->tab + WN_MAX_SPAN;
         int plane = plane0, chb = b0 - plane0 * p.nchb, ib = 0, buf = -1;
         uint32_t phase = 0;                                  // of aempty: the ring's first filling waits for nobody
         for (int b = b0; b < b1; ++b, ++ib) {
@@ -520,10 +516,13 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const bool new_plane = ib > 0 && chb == p.nchb;
             if (chb == p.nchb) { chb = 0; ++plane; }
             const int g0 = chb * p.gblk, gn = min(p.gblk, p.groups - g0), ry = XCOL ? p.plane[plane].ry : 0;
-            if (new_plane && !XCOL) {
-                wn_meet();                                   // (everyone is done with the last plane's)
-                wn_table<DENSE, XCOL>(p, in_act, S, lin0, plane);
-                wn_meet();
+            if (!XCOL && new_plane) {
+                if (p.all_tables) src += p.span;
+                else {
+                    wn_meet();                               // (everyone is done with the last plane's)
+                    wn_table<DENSE, XCOL>(p, in_act, S->tab, lin0, plane);
+                    wn_meet();
+                }
             }
             ++chb;
             const uint32_t Ab = base_u32 + buf * p.abytes;
@@ -545,7 +544,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     #pragma unroll
                     for (int u = 0; u < TURN; ++u) {
                         const int id = idx + u * WN_FILL, i = magic ? (int)__umulhi((unsigned)id, magic) : id, c = id - i * cl;
-                        const int off = id < items ? S->src[i] : -1;
+                        const int off = id < items ? src[i] : -1;
                         v[u] = make_uint4(0, 0, 0, 0);
                         if (off >= 0) v[u] = __ldcg(reinterpret_cast<const uint4*>(src0 + off + c * 16));
                     }
@@ -563,7 +562,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 #pragma unroll 4
                 for (int idx = tid; idx < items; idx += WN_FILL) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
-                    const int off = S->src[i];
+                    const int off = src[i];
                     cp_async16(Ab + (uint32_t)(c * p.L + i) * 16u, off >= 0 ? src0 + off + c * 16 : src0, off >= 0 ? 16u : 0u);
                 }
                 cp_async_commit();
@@ -581,7 +580,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 const uint32_t* Aw = reinterpret_cast<const uint32_t*>(A);
                 auto fetch = [&](int idx, uint32_t (&v)[4]) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
-                    const int row0 = S->src[i], xl = S->x0[i], row = row0 + ry * p.w, x = (xl >> 8) + 4 * c;
+                    const int row0 = src[i], xl = xcol0[i], row = row0 + ry * p.w, x = (xl >> 8) + 4 * c;
                     v[0] = v[1] = v[2] = v[3] = 0u;
                     if (row0 < 0 || ry >= (xl & 255)) return;
                     unsigned bits = 0xfu;                    // which of the four pixels count
@@ -622,7 +621,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                     #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int id = idx + u * WN_FILL, i = (int)__umulhi((unsigned)id, magic), c = id - i * cl;      // (cl >= 2)
-                        off[u] = id < items ? S->src[i] : -1;
+                        off[u] = id < items ? src[i] : -1;
                         if (off[u] >= 0) {
                             nw[u] = Nu[off[u] + (c >> 1)];
                             if (!DENSE) cw4[u] = Cu[off[u] + (c >> 1)];
@@ -658,12 +657,12 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 uint32_t thirds = 0;                         // sums of the third pieces
                 auto fetch = [&](int idx, float (&x)[8]) {
                     const int i = magic ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - i * cl;
-                    const int off = S->src[i];
+                    const int off = src[i];
                     #pragma unroll
                     for (int j = 0; j < 8; ++j) x[j] = 0.f;
                     if (XCOL) {
                         // two neighbouring pixels x 4 channels
-                        const int xl = S->x0[i], xx = (xl >> 8) + 2 * (g0 * 2 + c);
+                        const int xl = xcol0[i], xx = (xl >> 8) + 2 * (g0 * 2 + c);
                         if (off < 0 || ry >= (xl & 255)) return;
                         #pragma unroll
                         for (int e = 0; e < 2; ++e) {
@@ -1347,9 +1346,11 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     // two accumulator tiles per CTA share every filter stage (what bounds a full machine is the filters' way from L2),
     // once that leaves a CTA per SM
     int mt = !f32 && tiles >= 2ll * 148 && rows > TC_M ? 2 : 1;
-    // (a cluster of narrow tiles is worth it for shares of some 48 K steps)
+    // (a cluster of narrow tiles is worth it for shares of some 48 K steps; with several planes, whose blocks are small and cost
+    // some 2.5 k clocks each for their windows, as soon as it leaves a block out: 256 -> 512 3x3 of stride 2 at 14 x 14, 4 images,
+    // 27.9 -> 14.4 k clocks a CTA)
     const int steps = p.groups * p.kh * (xcol ? 1 : p.kw);
-    const int most = !clustered ? 16 : (!p.narrow ? 8 : (steps < 96 ? 1 : (steps / 48 < 8 ? steps / 48 : 8)));
+    const int most = !clustered ? 16 : (!p.narrow || planes > 1 ? 8 : (steps < 96 ? 1 : (steps / 48 < 8 ? steps / 48 : 8)));
     int want = 1;
     while (mt == 1 && want < most && tiles * (want + 1) <= wave) ++want;
     for (; mt >= 1; mt /= 2) {
@@ -1357,6 +1358,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
         p.span = base_span + (mt - 1) * TC_M;
         if (p.span > WN_MAX_SPAN) continue;                  // (the tables hold no wider window: one tile, which win_geometry has checked)
         p.L = slots(p.span);
+        p.all_tables = !xcol && planes * p.span <= 2 * WN_MAX_SPAN;
         // drained rows: a tile's (64 columns of it where there are two), or 32 rows x up to 64 columns per warp
         const size_t whole = (size_t)mt * TC_M * ((mt > 1 && p.bn > 64 ? 64 : p.bn) + 4) * 4;
         const size_t turned = (size_t)8 * 32 * ((p.bn < WN_TURN ? p.bn : WN_TURN) + 4) * 4;
