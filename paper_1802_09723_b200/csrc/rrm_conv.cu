@@ -862,23 +862,51 @@ __global__ void __launch_bounds__(256, 4) import_f32_px_kernel(const float* __re
     }
 }
 
-// Dense int8 frames of at most 4 channels: four pixels of a thread's reads in flight together.
+// Dense int8 frames of at most 4 channels: a thread turns four neighbouring pixels around.  Bound by its reads, which are words
+// (byte by byte: 9.5 us for 32 frames of 3 x 227 x 227; the chunk that holds them 128.4 -> 126.1 us): a plane's four bytes start anywhere, so they are cut out of the two
+// words they lie in.  Pixels of two images, and words that reach beyond the frames, go byte by byte.
 __global__ void __launch_bounds__(256) import_i8_word_dense_kernel(const int8_t* __restrict__ src, uint32_t* X, int c, int hw, int pixels)
 {
-    const int base = blockIdx.x * 1024 + threadIdx.x;
+    const int gp = (blockIdx.x * 256 + threadIdx.x) * 4;
     pdl_launch_dependents();
     pdl_wait();
-    uint32_t v[4] = {0, 0, 0, 0};
-    #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int gp = base + 256 * k;
-        if (gp >= pixels) continue;
-        const int ns = gp / hw, pix = gp - ns * hw;
+    if (gp >= pixels) return;
+    const int ns = gp / hw, pix = gp - ns * hw;
+    const int8_t* const end = src + (size_t)(pixels / hw) * c * hw;
+    uint32_t r[4] = {0, 0, 0, 0};                            // channel ch of the four pixels
+    if (pix + 4 <= hw) {
         #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) if (ch < c) v[k] |= ((uint32_t)(uint8_t)src[((size_t)ns * c + ch) * hw + pix]) << (8 * ch);
+        for (int ch = 0; ch < 4; ++ch) {
+            if (ch >= c) break;
+            const int8_t* const a = src + ((size_t)ns * c + ch) * hw + pix;
+            const unsigned off = (unsigned)(uintptr_t)a & 3u;
+            const int8_t* const lo = a - off;
+            if (lo >= src && lo + (off ? 8 : 4) <= end) {
+                const uint32_t w0 = *reinterpret_cast<const uint32_t*>(lo), w1 = off ? *reinterpret_cast<const uint32_t*>(lo + 4) : 0u;
+                r[ch] = __funnelshift_r(w0, w1, 8u * off);
+            } else {
+                #pragma unroll
+                for (int j = 0; j < 4; ++j) r[ch] |= (uint32_t)(uint8_t)a[j] << (8 * j);
+            }
+        }
+    } else {
+        #pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int g = gp + j, ms = g / hw;
+            if (g >= pixels) break;
+            #pragma unroll
+            for (int ch = 0; ch < 4; ++ch) if (ch < c) r[ch] |= (uint32_t)(uint8_t)src[((size_t)ms * c + ch) * hw + g - ms * hw] << (8 * j);
+        }
     }
-    #pragma unroll
-    for (int k = 0; k < 4; ++k) if (base + 256 * k < pixels) X[base + 256 * k] = v[k];
+    const uint32_t lo01 = __byte_perm(r[0], r[1], 0x5140), hi01 = __byte_perm(r[0], r[1], 0x7362);
+    const uint32_t lo23 = __byte_perm(r[2], r[3], 0x5140), hi23 = __byte_perm(r[2], r[3], 0x7362);
+    const uint4 v = make_uint4(__byte_perm(lo01, lo23, 0x5410), __byte_perm(lo01, lo23, 0x7632), __byte_perm(hi01, hi23, 0x5410), __byte_perm(hi01, hi23, 0x7632));
+    if (gp + 4 <= pixels) *reinterpret_cast<uint4*>(X + gp) = v;
+    else {
+        X[gp] = v.x;
+        if (gp + 1 < pixels) X[gp + 1] = v.y;
+        if (gp + 2 < pixels) X[gp + 2] = v.z;
+    }
 }
 
 // Tiles of `ptiles` pixel tiles x (channel tiles x images) x frames as a grid: y holds at most 65535 of the middle product,

@@ -243,6 +243,23 @@ def test_boundary_layouts(dtype, c_in, c_out, hw, n):
     net.close()
 
 
+@pytest.mark.parametrize("c_in,hw,n", [(1, (9, 7), 1), (2, (5, 5), 3), (3, (7, 9), 4), (3, (33, 41), 3), (4, (6, 11), 2), (3, (2, 1), 5)])
+def test_dense_frames_of_few_channels_start_anywhere(c_in, hw, n):
+    """Keyframes of int8 frames of up to 4 channels, at every alignment of the frame's first byte: pixels of two images in one
+    thread, planes whose bytes straddle words, the first and last words."""
+    rng = np.random.default_rng(c_in * hw[1])
+    sp = _spec("i8", c_in, hw, 8, 1, 1, 0, rng, act="relu", shift=6)
+    net = _rrm().net_from_specs([sp], n=n)
+    for off in range(4):
+        x = rng.integers(-127, 128, size=(n, c_in) + hw).astype(np.int8)
+        raw = torch.zeros(x.size + 4, dtype=torch.int8, device="cuda")
+        frame = raw[off:off + x.size].view(n, c_in, *hw)
+        frame.copy_(torch.from_numpy(x))
+        net.keyframe(frame)
+        _compare([sp], net, x, off)
+    net.close()
+
+
 @pytest.mark.parametrize("dtype,n,T", [("i8", 512, 1), ("i8", 16, 32), ("f32", 512, 1), ("f32", 16, 32)])
 def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
     """Channel tiles x streams x frames of a launch at 65536, one more than a grid has along y: 4096 channels in (int8) and out."""
