@@ -37,11 +37,11 @@
 // and a dense pass needs no zeroed projection).  Every wait on an mbarrier is bounded; one that runs out sets
 // ERRW_TIMEOUT and the CTA leaves through the common exit.
 //
-// What bounds it: in a long K loop the MMAs' operand reads from shared memory (an MMA of 128 columns reads 8 KB, the 64
-// clocks it takes), beside which the filter copies write another quarter (fp32 step of 768 MMA clocks: 1064 measured); in a
-// launch of a few tiles a chain of ~7 us (rows and table 2.2, window 1.2, MMAs 1.5, accumulators out 1.7).  AlexNet-shaped
-// stack at 227 x 227 against kernels that gather rows tap by tap (fp32: on the CUDA cores): 8 fp32 streams 546 -> 191 us, 32
-// fp32 frames 1630 -> 469, one int8 frame 83 -> 64, 32 int8 frames 266 -> 144.
+// What bounds it: in a long K loop the MMAs' operand reads from shared memory (an MMA of 128 columns reads 8 KB and takes 97 to
+// 118 clocks instead of 64, one of 32 columns 77; fp32: 413 clocks a K step of 16, 384 of them MMAs, 126 bytes of shared memory
+// a clock); in a launch of a few tiles a chain (clocks: set-up 1.8 k, first window 2.2 k, MMAs 3 to 6 k, way out 1.2 to 2.3 k, 7 k
+// for 64 KB of fp32 rows).  AlexNet-shaped stack at 227 x 227: 8 fp32 streams 187 us, 32 fp32 frames 465, one int8 frame 64, 32
+// int8 frames 126; 4 ResNet-18-shaped int8 streams 171.
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
