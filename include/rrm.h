@@ -337,6 +337,21 @@ int64_t rrm_net_tensor_bytes(const rrm_net* net, int t);
 int rrm_fc_step_noalloc(const int8_t* Wt_dev, const int8_t* Xt_dev, int8_t* Xprev_dev, int32_t* P_dev,
                         void* Y_dev, int n, int c_in, int c_out, int shift, int act, void* stream);
 
+/* ---- how a convolution launch is cut ------------------------------------------------
+ * (No counterpart in the paper: a reporting aid, host arithmetic that touches no device.)  What the tensor-core kernel
+ * that most convolutions run on makes of a layer: columns (output channels) and accumulator tiles of 128 projection
+ * pixels per thread block, the thread blocks that share a tile's K loop, and whether those add up as one cluster.
+ * desc as for rrm_layer_create; frames: that many frames in one launch (RRM_PLAN_DENSE: a dense chunk batched over its
+ * frames, RRM_PLAN_SEQ: a delta chunk taken layer by layer; 1 otherwise).  Layers of the other kernels: all zero. */
+enum { RRM_PLAN_DELTA = 0, RRM_PLAN_DENSE = 1, RRM_PLAN_SEQ = 2, RRM_PLAN_PIPELINED = 3 /* a delta step among overlapping frames */ };
+typedef struct {
+    int32_t columns, tiles_per_cta, shares, clustered;
+    int64_t ctas;
+    int32_t narrow_filters;    /* the filters are held as tiles of 32 columns too */
+    int32_t reserved;
+} rrm_conv_plan;
+int rrm_plan_conv(const rrm_layer_desc* desc, int form, int frames, rrm_conv_plan* out);
+
 /* ---- measured ALU peaks -------------------------------------------------------------
  * (No counterpart in the paper: a reporting aid.)  Runs a register-only loop of independent operations on every
  * SM of the current device and returns the best of four timings as multiply-accumulates per second:

@@ -11,6 +11,7 @@ from . import build as _build
 KIND = {"conv": 0, "fc": 1}
 DTYPE = {"f32": 0, "i8": 1, "bin": 2}
 ACT = {"none": 0, "relu": 1, "sign": 2, "leaky": 3}
+PLAN = {"delta": 0, "dense": 1, "seq": 2, "pipelined": 3}
 VARIANT = {"auto": 0, "gather": 1, "tensor": 2, "dense": 3, "sparse_w": 4}
 
 
@@ -38,6 +39,11 @@ class Options(ctypes.Structure):
                 ("layer_delta_activity", ctypes.c_float), ("stack_dense_activity", ctypes.c_float),
                 ("stack_reprobe", ctypes.c_int32), ("fc_dense_rows", ctypes.c_float), ("fc_dense_density", ctypes.c_float),
                 ("chunk_dense_activity", ctypes.c_float)]
+
+
+class ConvPlan(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("columns", "tiles_per_cta", "shares", "clustered")] + [
+        ("ctas", ctypes.c_int64), ("narrow_filters", ctypes.c_int32), ("reserved", ctypes.c_int32)]
 
 
 _lib = None
@@ -110,6 +116,8 @@ def lib():
     L.rrm_aecs_predict.restype = ctypes.c_double
     L.rrm_net_tensor_bytes.argtypes = [_P, ctypes.c_int]
     L.rrm_net_tensor_bytes.restype = ctypes.c_int64
+    L.rrm_plan_conv.argtypes = [ctypes.POINTER(LayerDesc), ctypes.c_int, ctypes.c_int, ctypes.POINTER(ConvPlan)]
+    L.rrm_plan_conv.restype = ctypes.c_int
     L.rrm_measure_alu_peak.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
     L.rrm_measure_alu_peak.restype = ctypes.c_int
     L.rrm_strerror.argtypes = [ctypes.c_int]
@@ -326,6 +334,13 @@ def measure_alu_peak(kind):
     v = ctypes.c_double()
     _check(lib().rrm_measure_alu_peak({"ffma": 0, "dp4a": 1, "popc": 2}[kind], ctypes.byref(v)), "rrm_measure_alu_peak")
     return v.value
+
+
+def plan_conv(desc, form="delta", frames=1):
+    """rrm_plan_conv: how a launch of the described convolution is cut (all zero: another kernel's layer).  Needs no GPU."""
+    p = ConvPlan()
+    _check(lib().rrm_plan_conv(ctypes.byref(desc), PLAN[form], frames, ctypes.byref(p)), "rrm_plan_conv")
+    return {n: getattr(p, n) for n, _ in p._fields_ if n != "reserved"}
 
 
 def aecs_predict(mu, e_t):

@@ -1,6 +1,7 @@
 // C ABI of the RRM library: object construction, validation and the per-frame launch sequences.
 #include "rrm_common.cuh"
 #include <new>
+#include <climits>
 #include <cstring>
 #include <cstdlib>
 
@@ -70,6 +71,20 @@ void set_tensor(Tensor& T, int dtype, int n, int c, int h, int w)
     else { T.cs = c; T.unit_bytes = 4; }
 }
 
+void set_conv_size(Layer& L)
+{
+    L.oh = (L.d.h + 2 * L.d.pad - L.d.kh) / L.d.stride + 1;
+    L.ow = (L.d.w + 2 * L.d.pad - L.d.kw) / L.d.stride + 1;
+}
+
+int check_capacity(const Layer& L, const Tensor& in)
+{
+    const rrm_layer_desc& d = L.d;
+    if ((long long)d.n * L.oh * L.ow * (long long)d.c_out > (1ll << 31) - 1) return RRM_ERR_CAPACITY;
+    if ((long long)d.n * d.h * d.w * (long long)in.cs > (1ll << 31) - 1) return RRM_ERR_CAPACITY;
+    return RRM_OK;
+}
+
 // Points every activity bitmap and per-step counter at an arena (one memset clears it): tensors' activity bitmaps,
 // layers' update bitmaps, then the counters.  A net has one arena for frame-by-frame stepping and, for pipelined
 // chunks of frames, one per frame in flight.
@@ -130,8 +145,7 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
         if (!W[l]) return RRM_ERR_INVALID_ARG;
         Layer& L = net->layers[l];
         L.d = d;
-        L.oh = (d.h + 2 * d.pad - d.kh) / d.stride + 1;
-        L.ow = (d.w + 2 * d.pad - d.kw) / d.stride + 1;
+        set_conv_size(L);
         L.th = L.oh; L.tw = L.ow;
         if (d.pool_k > 0) {
             if (L.oh + 2 * d.pool_p < d.pool_k || L.ow + 2 * d.pool_p < d.pool_k) return RRM_ERR_SHAPE;
@@ -152,8 +166,7 @@ int build_net(rrm_net* net, const rrm_layer_desc* descs, int n_layers, const voi
             const Tensor& r = net->tensors[d.res];
             if (r.dtype != ot || r.c != d.c_out || r.h != L.th || r.w != L.tw) return RRM_ERR_SHAPE;
         }
-        if ((long long)n * L.oh * L.ow * (long long)d.c_out > (1ll << 31) - 1) return RRM_ERR_CAPACITY;
-        if ((long long)n * d.h * d.w * (long long)in.cs > (1ll << 31) - 1) return RRM_ERR_CAPACITY;
+        RRM_TRY(check_capacity(L, in));
     }
     // the fused FC kernel serves a lone int8 FC layer that reads the external input
     bool fused = false;
@@ -1417,6 +1430,28 @@ int64_t rrm_net_tensor_bytes(const rrm_net* net, int t)
     int64_t b = 0;
     tensor_bytes_boundary(net->tensors[t], &b);
     return b;
+}
+
+int rrm_plan_conv(const rrm_layer_desc* desc, int form, int frames, rrm_conv_plan* out)
+{
+    if (!desc || !out || form < RRM_PLAN_DELTA || form > RRM_PLAN_PIPELINED || frames < 1) return RRM_ERR_INVALID_ARG;
+    RRM_TRY(validate_desc(*desc, desc->src > 0 ? desc->src : 0, 1));
+    if ((long long)desc->n * frames > INT_MAX) return RRM_ERR_CAPACITY;
+    try {
+        rrm_net net;
+        net.tensors.resize(1);
+        Tensor& in = net.tensors[0];
+        set_tensor(in, desc->dtype == RRM_F32 ? T_F32 : (desc->dtype == RRM_I8 ? T_I8 : T_BIN), desc->n, desc->c_in, desc->h, desc->w);
+        Layer L;
+        L.d = *desc;
+        L.d.src = 0;
+        set_conv_size(L);
+        RRM_TRY(check_capacity(L, in));
+        *out = rrm_conv_plan{};
+        return conv_win_asked(L) ? conv_win_query(net, L, form, frames, out) : RRM_OK;
+    } catch (const std::bad_alloc&) {
+        return RRM_ERR_ALLOC;
+    }
 }
 
 const char* rrm_strerror(int status)

@@ -232,6 +232,7 @@ struct Layer {
     bool win_ready = false;
     void* win_Wimg = nullptr;               // [n_tiles][tap][K group][pieces][2][bn][16 bytes] operand tiles of the filters
     void* win_Wnarrow = nullptr;            // integers: the same as tiles of 32 columns (launches of few tiles)
+    bool win_narrow = false;                // such tiles may be taken
     int win_bn = 0, win_ntiles = 0;
     int win_tiles = 0;                      // accumulator tiles of 128 rows that cover the layer once
     void* Apre = nullptr;                   // pooled integer layers: f before the pool window, a row per projection pixel (keyframes)
@@ -397,6 +398,7 @@ int launch_conv_tc(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool st
 int zero_projection(void* P, long long words, cudaStream_t st);
 
 // ---- rrm_conv_win.cu
+inline bool conv_win_asked(const Layer& L) { return L.d.variant != RRM_VARIANT_GATHER && L.d.kh * L.d.kw <= 128; }
 int conv_win_create(rrm_net* net, Layer& L, const void* W_dev);
 // f applied by the convolution kernel (dense passes): where its result goes (the output tensor's rows, or for a pooled
 // layer a row per projection pixel), the shortcut, and the projection to keep (nullptr: none) from pixel keep_from on.
@@ -404,6 +406,7 @@ struct WinOutput { void* X; const void* res; int cs, bits; void* P; int keep_fro
 int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool stateless, cudaStream_t st,
                     const uint32_t* count_bitmap = nullptr, void* P_dst = nullptr, int frames = 1, long long arena_stride = 0,
                     const WinOutput* out = nullptr);
+int conv_win_query(const rrm_net& net, Layer& L, int form, int frames, rrm_conv_plan* out);
 int launch_pool_window(const Layer& L, const Tensor& out, const void* A, void* X, cudaStream_t st);
 
 // ---- rrm_conv.cu

@@ -1517,7 +1517,7 @@ int conv_layer_create(rrm_net* net, Layer& L, const void* W_dev, const void* bia
     RRM_TRY(dev_alloc(net, &L.P, (size_t)L.opixels() * d.c_out * 4));
     if (bias_dev) RRM_CUDA_TRY(cudaMemcpy(L.bias, bias_dev, (size_t)d.c_out * 4, cudaMemcpyDeviceToDevice));
     if (d.kh * d.kw > 128) return RRM_ERR_UNSUPPORTED;       // the kernels keep a row's usable taps in a 128-bit mask
-    if (d.variant != RRM_VARIANT_GATHER) {
+    if (conv_win_asked(L)) {
         // the window kernel where it takes the layer, else the kernel that gathers compacted rows (int8 and binary)
         const int s = conv_win_create(net, L, W_dev);
         if (s != RRM_ERR_UNSUPPORTED) return s;

@@ -1335,7 +1335,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     // cluster's way out (two meetings, rows read from the other shares) takes 8 to 10 k clocks with 128 columns, an MMA of 32
     // columns two thirds of one of 128 (77 clocks: the reads of its rows).  256 -> 256 3x3 at 14 x 14, 4 images: 16.0 -> 14.0 k
     // clocks a CTA; 96 -> 256 5x5 at 27 x 27: 16.6 -> 13.0 k.  Shares that add by themselves are as fast with wide tiles.
-    p.narrow = clustered && L.win_Wnarrow && row_tiles * L.win_ntiles * 2 <= wave;
+    p.narrow = clustered && L.win_narrow && row_tiles * L.win_ntiles * 2 <= wave;
     p.bn = p.narrow ? WN_NARROW : L.win_bn;
     p.ntiles = p.narrow ? L.win_ntiles * L.win_bn / WN_NARROW : L.win_ntiles;
     const long long tiles = row_tiles * p.ntiles;
@@ -1423,22 +1423,40 @@ static int win_allow()
     return RRM_OK;
 }
 
-// Packs the filters of a layer the window kernel takes; RRM_ERR_UNSUPPORTED: the layer keeps the other kernels.
-int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
+// Whether the window kernel takes the layer, and the widths of its column tiles.  Every launch of a layer that is taken has
+// to find a plan: whether a window and three filter stages fit shared memory depends on the width alone (a plan falls back to
+// one accumulator tile, one K group per block and one window buffer, whatever it was first cut for), so one plan of each width
+// decides.  The narrow tiles are no easier to fit than the wide ones: tiles of 96 columns have stages of 12 KB, narrow
+// ones of 16 (first layers of wide windows fit only the former).
+static bool win_choose(const rrm_net* net, Layer& L)
 {
     const rrm_layer_desc& d = L.d;
-    WinParams p{};
-    if (!win_geometry(net, L, p)) return RRM_ERR_UNSUPPORTED;
+    WinParams wide{}, narrow{};
+    if (!win_geometry(net, L, wide)) return false;
+    narrow = wide;                                           // (win_plan widens the window it is given)
     const bool xcol = win_xcol(net, L), f32 = d.dtype == RRM_F32;
     L.win_ntiles = ceil_div(d.c_out, 128);
     // (integer layers: whole groups of 32 columns, so that a padded output row is covered by the column tiles)
     L.win_bn = round_up(ceil_div(d.c_out, L.win_ntiles), f32 ? 16 : 32);
     L.win_ntiles = ceil_div(d.c_out, L.win_bn);
-    if (!win_plan(L, p, xcol, true, false, 1, 148)) return RRM_ERR_UNSUPPORTED;
+    L.win_narrow = false;
+    if (!win_plan(L, wide, xcol, true, false, 1, 148)) return false;
+    L.win_narrow = !f32 && L.win_bn > WN_NARROW;
+    L.win_narrow = L.win_narrow && win_plan(L, narrow, xcol, true, false, 1, INT_MAX);       // (a wave that makes any launch one of few tiles)
+    return true;
+}
+
+// Packs the filters of a layer the window kernel takes; RRM_ERR_UNSUPPORTED: the layer keeps the other kernels.
+int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
+{
+    const rrm_layer_desc& d = L.d;
+    WinParams p{};
+    if (!win_choose(net, L) || !win_geometry(net, L, p)) return RRM_ERR_UNSUPPORTED;
+    const bool xcol = win_xcol(net, L), f32 = d.dtype == RRM_F32;
     const int taps = xcol ? d.kh : d.kh * d.kw;
     const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
     const size_t bytes = chunks * 16 * (f32 ? 3 : 1);
-    const bool narrow = !f32 && L.win_bn > WN_NARROW;        // (the same filters once more, as tiles of 32 columns)
+    const bool narrow = L.win_narrow;                        // (the same filters once more, as tiles of 32 columns)
     void* img = nullptr;
     if (cudaMalloc(&img, bytes * (narrow ? 2 : 1) + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
     net->allocs.push_back(img);
@@ -1470,6 +1488,23 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     RRM_TRY((win_allow<T_BIN, false>()));
     L.win_tiles = ceil_div((int)(((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow), TC_M);
     L.win_ready = true;
+    return RRM_OK;
+}
+
+// How a launch of the layer is cut (host arithmetic; the layer's sizes are set, nothing else).
+int conv_win_query(const rrm_net& net, Layer& L, int form, int frames, rrm_conv_plan* out)
+{
+    *out = rrm_conv_plan{};
+    WinParams p{};
+    if (!win_choose(&net, L)) return RRM_OK;
+    const bool xcol = win_xcol(&net, L), dense = form == RRM_PLAN_DENSE, seq = form == RRM_PLAN_SEQ;
+    if (dense) L.d.n *= frames;                              // (a batch of dense frames is that many more images)
+    if (!win_geometry(&net, L, p) || !win_plan(L, p, xcol, dense, seq, seq ? frames : 1, form == RRM_PLAN_PIPELINED ? 74 : 148))
+        return RRM_ERR_UNSUPPORTED;                          // (never: win_choose takes no such layer)
+    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    out->columns = p.bn; out->tiles_per_cta = p.mt; out->shares = p.ks; out->clustered = p.cluster;
+    out->ctas = (rows + p.mt * TC_M - 1) / (p.mt * TC_M) * p.ntiles * p.ks * (seq ? frames : 1);
+    out->narrow_filters = L.win_narrow;
     return RRM_OK;
 }
 

@@ -1,0 +1,45 @@
+"""How convolution launches are cut, by host arithmetic (no GPU): every layer that the tensor-core kernel takes has a plan
+for every launch it can come to."""
+import random
+
+import paper_1802_09723_b200 as rrm
+
+FORMS = (("delta", 1), ("pipelined", 1), ("dense", 1), ("dense", 7), ("dense", 32), ("seq", 2), ("seq", 32))
+
+
+def desc(dtype, c_in, h, w, c_out, kh, kw, stride, pad, n):
+    d = rrm.LayerDesc()
+    d.kind, d.dtype, d.n, d.c_in, d.h, d.w, d.c_out = 0, rrm.DTYPE[dtype], n, c_in, h, w, c_out
+    d.kh, d.kw, d.stride, d.pad, d.shift, d.res = kh, kw, stride, pad, -1, -1
+    return d
+
+
+def test_layers_of_wide_windows_have_a_plan_for_every_launch():
+    """First layers whose window leaves room for the filter stages of one tile width only: stages are 12 KB for tiles of 96
+    columns and 16 KB for those of 128 and of 32."""
+    taken = 0
+    for shape in (("i8", 4, 19, 77, 162, 11, 11, 1, 3, 2), ("i8", 3, 64, 1110, 64, 9, 9, 3, 0, 1), ("i8", 3, 64, 1110, 96, 9, 9, 3, 0, 1),
+                  ("i8", 4, 31, 87, 96, 11, 11, 1, 5, 1), ("i8", 3, 40, 91, 70, 11, 11, 1, 0, 1)):
+        for form, frames in FORMS:
+            taken += rrm.plan_conv(desc(*shape), form, frames)["columns"] > 0      # (raises if a launch has no plan)
+    assert taken > 0
+
+
+def test_every_layer_that_is_taken_has_a_plan_for_every_launch():
+    r = random.Random(1)
+    taken = 0
+    for _ in range(6000):
+        k = r.randint(1, 11)
+        kw = k if r.random() < 0.6 else r.randint(1, min(16, 128 // k))
+        dtype = r.choice(("i8", "i8", "i8", "bin", "f32"))
+        c_in = r.randint(1, 4) if r.random() < 0.5 else r.randint(5, 300)
+        h, w = r.randint(k, 90), r.randint(kw, 1200)
+        d = desc(dtype, c_in, h, w, r.randint(1, 512), k, kw, r.randint(1, 4), r.randint(0, min(k, kw) - 1), r.randint(1, 3))
+        for form, frames in FORMS:
+            try:
+                p = rrm.plan_conv(d, form, frames)
+            except rrm.RRMError as e:
+                assert "(-5)" in str(e), (str(e), form, frames, [getattr(d, f) for f, _ in d._fields_])     # (more than 2^31 elements)
+                continue
+            taken += p["columns"] > 0
+    assert taken > 10000

@@ -291,6 +291,22 @@ def test_boundary_layouts_of_many_streams_of_many_channels(dtype, n, T):
     net.close()
 
 
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [(4, 162, (19, 77), 11, 1, 3, 2), (3, 64, (64, 1110), 9, 3, 0, 1)])
+def test_first_layers_whose_window_leaves_room_for_one_tile_width(c_in, c_out, hw, k, s, p, n):
+    """A window beside which only the stages of 96 columns fit, and one beside which only those of 32 do: keyframes, steps and dense
+    chunks."""
+    rng = np.random.default_rng(c_out)
+    sp = _spec("i8", c_in, hw, c_out, k, s, p, rng, act="relu", shift=9)
+    video = _video("i8", c_in, hw, 4, n, rng)
+    _run([sp], video, n=n, keyframe_at=(1,))
+    net = _rrm().net_from_specs([sp], n=n)
+    outs = net.new_output(frames=4)
+    net.dense_seq(torch.from_numpy(video).cuda(), outs)
+    for t in range(4):
+        np.testing.assert_array_equal(outs[t].cpu().numpy().astype(np.int64), orc.dense_forward([sp], video[t])[0][1], err_msg=f"frame {t}")
+    net.close()
+
+
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [
     (64, 70, (14, 13), 3, 1, 1, 1), (320, 200, (13, 13), 3, 1, 1, 1),         # one share (18 and 90 K steps), ragged columns
