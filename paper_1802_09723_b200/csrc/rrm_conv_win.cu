@@ -1318,7 +1318,13 @@ static bool win_xcol(const rrm_net* net, const Layer& L)
     return L.d.dtype == RRM_F32 ? L.d.c_in <= 4 : (L.d.dtype == RRM_I8 && net->tensors[L.d.src].cs == 4);
 }
 
+// Rows of the linear space that accumulator tiles cover, per frame.
+static long long win_rows(const WinParams& p) { return ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow; }
+
 static int slots(int span) { return round_up(span, 8) + 1; }    // (neighbouring chunks of a pixel fall into different banks)
+
+// Wide tiles that leave half of the wave idle.
+static bool win_few_tiles(const Layer& L, long long row_tiles, int wave) { return row_tiles * L.win_ntiles * 2 <= wave; }
 
 // How a launch cuts the work: accumulator tiles and shares of K per CTA, window blocks, filter stages.  `wave`: CTAs that
 // are to be kept busy.
@@ -1326,7 +1332,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
 {
     const bool f32 = L.d.dtype == RRM_F32;
     const int pieces = f32 ? 3 : 1;
-    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    const long long rows = win_rows(p);
     const long long row_tiles = (rows + TC_M - 1) / TC_M * frames;
     // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
     // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
@@ -1335,9 +1341,9 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     // cluster's way out (two meetings, rows read from the other shares) takes 8 to 10 k clocks with 128 columns, an MMA of 32
     // columns two thirds of one of 128 (77 clocks: the reads of its rows).  256 -> 256 3x3 at 14 x 14, 4 images: 16.0 -> 14.0 k
     // clocks a CTA; 96 -> 256 5x5 at 27 x 27: 16.6 -> 13.0 k.  Shares that add by themselves are as fast with wide tiles.
-    p.narrow = clustered && L.win_narrow && row_tiles * L.win_ntiles * 2 <= wave;
+    p.narrow = clustered && L.win_narrow && win_few_tiles(L, row_tiles, wave);
     p.bn = p.narrow ? WN_NARROW : L.win_bn;
-    p.ntiles = p.narrow ? L.win_ntiles * L.win_bn / WN_NARROW : L.win_ntiles;
+    p.ntiles = p.narrow ? ceil_div(p.c_out, WN_NARROW) : L.win_ntiles;
     const long long tiles = row_tiles * p.ntiles;
     const int base_span = p.span, planes = p.planes;
     const int plane_taps = ceil_div(p.kh, p.stride) * (xcol ? 1 : ceil_div(p.kw, p.stride));
@@ -1441,7 +1447,8 @@ static bool win_choose(const rrm_net* net, Layer& L)
     L.win_ntiles = ceil_div(d.c_out, L.win_bn);
     L.win_narrow = false;
     if (!win_plan(L, wide, xcol, true, false, 1, 148)) return false;
-    L.win_narrow = !f32 && L.win_bn > WN_NARROW;
+    // (more frames are only more tiles, and 148 is the larger wave: with too many tiles in one frame no launch takes narrow ones)
+    L.win_narrow = !f32 && L.win_bn > WN_NARROW && win_few_tiles(L, (win_rows(wide) + TC_M - 1) / TC_M, 148);
     L.win_narrow = L.win_narrow && win_plan(L, narrow, xcol, true, false, 1, INT_MAX);       // (a wave that makes any launch one of few tiles)
     return true;
 }
@@ -1456,17 +1463,24 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     const int taps = xcol ? d.kh : d.kh * d.kw;
     const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
     const size_t bytes = chunks * 16 * (f32 ? 3 : 1);
-    const bool narrow = L.win_narrow;                        // (the same filters once more, as tiles of 32 columns)
-    void* img = nullptr;
-    if (cudaMalloc(&img, bytes * (narrow ? 2 : 1) + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
+    void *img = nullptr, *few = nullptr;
+    if (cudaMalloc(&img, bytes + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
     net->allocs.push_back(img);
-    const unsigned grid = (unsigned)((chunks + 255) / 256);
-    unsigned char* im = reinterpret_cast<unsigned char*>(img);
-    int* beyond = reinterpret_cast<int*>(im + bytes * (narrow ? 2 : 1));
+    // the same filters once more, as tiles of 32 columns; where there is no room for them the layer goes without
+    const int few_ntiles = ceil_div(d.c_out, WN_NARROW);
+    const size_t few_chunks = (size_t)few_ntiles * taps * p.groups * 2 * WN_NARROW;
+    if (L.win_narrow) {
+        if (cudaMalloc(&few, few_chunks * 16) == cudaSuccess) net->allocs.push_back(few);
+        else { cudaGetLastError(); few = nullptr; L.win_narrow = false; }
+    }
+    int* beyond = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(img) + bytes);
     RRM_CUDA_TRY(cudaMemset(beyond, 0, 4));
     auto pack = [&](auto kernel) {
-        kernel<<<grid, 256>>>(W_dev, im, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, L.win_bn, L.win_ntiles, beyond);
-        if (narrow) kernel<<<grid, 256>>>(W_dev, im + bytes, d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, WN_NARROW, L.win_ntiles * L.win_bn / WN_NARROW, beyond);
+        auto go = [&](void* to, size_t n, int bn, int ntiles) {
+            kernel<<<(unsigned)((n + 255) / 256), 256>>>(W_dev, reinterpret_cast<unsigned char*>(to), d.c_in, d.c_out, d.kh, d.kw, taps, p.groups, bn, ntiles, beyond);
+        };
+        go(img, chunks, L.win_bn, L.win_ntiles);
+        if (few) go(few, few_chunks, WN_NARROW, few_ntiles);
     };
     if (f32) { if (xcol) pack(pack_weights_win_kernel<T_F32, true>); else pack(pack_weights_win_kernel<T_F32, false>); }
     else if (xcol) pack(pack_weights_win_kernel<T_I8, true>);
@@ -1482,11 +1496,11 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
         }
     }
     L.win_Wimg = img;
-    if (narrow) L.win_Wnarrow = im + bytes;
+    L.win_Wnarrow = few;
     RRM_TRY((win_allow<T_F32, true>())); RRM_TRY((win_allow<T_F32, false>()));
     RRM_TRY((win_allow<T_I8, true>())); RRM_TRY((win_allow<T_I8, false>()));
     RRM_TRY((win_allow<T_BIN, false>()));
-    L.win_tiles = ceil_div((int)(((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow), TC_M);
+    L.win_tiles = ceil_div((int)win_rows(p), TC_M);
     L.win_ready = true;
     return RRM_OK;
 }
@@ -1501,7 +1515,7 @@ int conv_win_query(const rrm_net& net, Layer& L, int form, int frames, rrm_conv_
     if (dense) L.d.n *= frames;                              // (a batch of dense frames is that many more images)
     if (!win_geometry(&net, L, p) || !win_plan(L, p, xcol, dense, seq, seq ? frames : 1, form == RRM_PLAN_PIPELINED ? 74 : 148))
         return RRM_ERR_UNSUPPORTED;                          // (never: win_choose takes no such layer)
-    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    const long long rows = win_rows(p);
     out->columns = p.bn; out->tiles_per_cta = p.mt; out->shares = p.ks; out->clustered = p.cluster;
     out->ctas = (rows + p.mt * TC_M - 1) / (p.mt * TC_M) * p.ntiles * p.ks * (seq ? frames : 1);
     out->narrow_filters = L.win_narrow;
@@ -1546,7 +1560,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
         p.bn_scale = L.bn_scale; p.bn_shift = L.bn_shift; p.shift = d.shift; p.act_fn = d.act; p.theta = d.theta;
         p.P = out->P; p.keep_from = out->P ? out->keep_from : INT_MAX;
     }
-    const long long rows = ((long long)(p.n - 1) * p.Hq + p.oh - 1) * p.Wq + p.ow;
+    const long long rows = win_rows(p);
     const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)p.ntiles, (unsigned)(nf * p.ks));
     const size_t smem = win_smem(p);
     cudaError_t e;

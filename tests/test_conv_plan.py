@@ -43,3 +43,19 @@ def test_every_layer_that_is_taken_has_a_plan_for_every_launch():
                 continue
             taken += p["columns"] > 0
     assert taken > 10000
+
+
+def test_filters_are_held_as_narrow_tiles_only_where_a_launch_can_take_them():
+    """A dense pass takes 32-column tiles while twice the wide tiles (128 pixels x up to 128 channels) fit 148 CTAs; a layer with more
+    of them in one frame, of 32 columns anyway, or of floats holds its filters once."""
+    for shape, want in ((("i8", 64, 14, 14, 256, 3, 3, 1, 1, 1), 1),
+                        (("i8", 64, 96, 97, 64, 3, 3, 1, 1, 1), 1),          # 74 tiles
+                        (("i8", 64, 97, 97, 64, 3, 3, 1, 1, 1), 0),          # 75
+                        (("bin", 64, 97, 97, 64, 3, 3, 1, 1, 1), 0),
+                        (("i8", 64, 56, 56, 256, 3, 3, 1, 1, 24), 0),
+                        (("i8", 64, 14, 14, 32, 3, 3, 1, 1, 1), 0), (("f32", 64, 14, 14, 256, 3, 3, 1, 1, 1), 0)):
+        d = desc(*shape)
+        assert rrm.plan_conv(d, "dense")["narrow_filters"] == want, shape
+        for form, frames in FORMS:
+            p = rrm.plan_conv(d, form, frames)
+            assert want or p["columns"] != 32 or shape[4] <= 32
