@@ -32,8 +32,8 @@ namespace rrm {
 // ---- programmatic dependent launch between the kernels of a per-frame sequence --------------------------------
 // Every kernel of the sequence lets its successor start launching at once (launch_dependents at its top) and waits
 // for its predecessor's results (pdl_wait) only when it first needs what a predecessor writes: thread-block scheduling,
-// barrier initialisation, tensor-memory allocation, window tables and first filter copies of kernel k+1 then overlap the tail
-// of kernel k.  Some thread of every grid waits, so a grid ends after its predecessors, and a wait covers them all.  What a
+// barrier initialisation, tensor-memory allocation and, in dense passes, window tables and first filter copies of kernel k+1
+// then overlap the tail of kernel k.  Some thread of every grid waits, so a grid ends after its predecessors, and a wait covers them all.  What a
 // predecessor wrote is read with ordinary loads (not through the read-only path).  Without the launch attribute both
 // instructions do nothing.  The attribute is set (OverlapLaunches) while a dense
 // pass, a keyframe or a dense chunk is captured: there most of a kernel's set-up needs nothing of its predecessor, and a pass

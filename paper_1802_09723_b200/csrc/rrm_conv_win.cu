@@ -421,10 +421,14 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&S->bfull[s]), 1); mbar_init(smem_u32(&S->bempty[s]), 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // ---- the tile's rows, and the first plane's table.  All that is no predecessor's work comes before the wait for them: a
-    // launch that overlaps its predecessor's tail then has its barriers, tensor memory, tables and, in dense passes, its
-    // first filters at hand when the inputs arrive
+    // ---- the tile's rows, and the windows' tables.  All that is no predecessor's work comes before the wait for them: a dense
+    // pass that overlaps its predecessor's tail then has its barriers, tensor memory, all planes' tables and first filters at
+    // hand when the inputs arrive.  Delta tables are made of the input's activity bitmap: here the first plane's, on its way
+    // together with the update bitmap, and the others' once the tile has work
     int active = 0;
+    auto other_tables = [&] {
+        if (!XCOL && p.all_tables) for (int b = plane0 + 1; b * p.nchb < b1; ++b) wn_table<DENSE, XCOL>(p, in_act, S->tab + (b - plane0) * p.span, lin0, b);
+    };
     {
         int q = -1;
         uint32_t word = 0;                                   // of the layer's update bitmap
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 if (q >= 0) word = oact[q >> 5];             // (on its way together with the table's words)
             }
             wn_table<DENSE, XCOL>(p, in_act, S->tab, lin0, plane0);
-            if (!XCOL && p.all_tables) for (int b = plane0 + 1; b * p.nchb < b1; ++b) wn_table<DENSE, XCOL>(p, in_act, S->tab + (b - plane0) * p.span, lin0, b);
+            if (DENSE) other_tables();
             if (ACT && tid < p.bn) S->bias[tid] = p.bias && ntile * p.bn + tid < p.c_out ? reinterpret_cast<const int*>(p.bias)[ntile * p.bn + tid] : 0;
         }
         if (!DENSE || p.count_bitmap) {
@@ -502,6 +506,10 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             mbar_arrive(smem_u32(&S->dempty[pb]));
             return true;
         };
+        if (!DENSE && !XCOL && p.all_tables && (plane0 + 1) * p.nchb < b1) {   // (now that the tile has work)
+            other_tables();
+            wn_meet();
+        }
         const bool lag = DT == T_I8 && !XCOL && !DENSE && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
         const int* src = S->tab;                             // the plane's table
         const int* const xcol0 = S->tab + WN_MAX_SPAN;
