@@ -1334,22 +1334,20 @@ static int slots(int span) { return round_up(span, 8) + 1; }    // (neighbouring
 // Wide tiles that leave half of the wave idle.
 static bool win_few_tiles(const Layer& L, long long row_tiles, int wave) { return row_tiles * L.win_ntiles * 2 <= wave; }
 
-// How a launch cuts the work: accumulator tiles and shares of K per CTA, window blocks, filter stages.  `wave`: CTAs that
-// are to be kept busy.
-static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool store, int frames, int wave)
+// Shares of K form a cluster (at most 8 CTAs); integer delta passes add theirs onto the projection one by one.
+static bool win_clustered(const Layer& L, bool dense, bool store) { return dense || store || L.d.dtype == RRM_F32 || (L.d.c_out & 3) != 0; }
+
+// How a launch with column tiles of one width cuts the work: accumulator tiles and shares of K per CTA, window blocks, filter
+// stages.  `wave`: CTAs that are to be kept busy.
+static bool win_cut(const Layer& L, WinParams& p, bool xcol, bool dense, bool store, int frames, int wave, bool narrow)
 {
     const bool f32 = L.d.dtype == RRM_F32;
     const int pieces = f32 ? 3 : 1;
     const long long rows = win_rows(p);
     const long long row_tiles = (rows + TC_M - 1) / TC_M * frames;
-    // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave.  Integer delta passes add
-    // their shares onto the projection one by one; otherwise the shares form a cluster (at most 8 CTAs)
-    const bool clustered = dense || store || f32 || (p.c_out & 3) != 0;
-    // Integers whose shares would form a cluster, and whose tiles leave half of the wave idle: tiles of 32 columns first.  A
-    // cluster's way out (two meetings, rows read from the other shares) takes 8 to 10 k clocks with 128 columns, an MMA of 32
-    // columns two thirds of one of 128 (77 clocks: the reads of its rows).  256 -> 256 3x3 at 14 x 14, 4 images: 16.0 -> 14.0 k
-    // clocks a CTA; 96 -> 256 5x5 at 27 x 27: 16.6 -> 13.0 k.  Shares that add by themselves are as fast with wide tiles.
-    p.narrow = clustered && L.win_narrow && win_few_tiles(L, row_tiles, wave);
+    // shares of K: whole blocks, or parts of one block's taps, until the tiles fill one wave
+    const bool clustered = win_clustered(L, dense, store);
+    p.narrow = narrow;
     p.bn = p.narrow ? WN_NARROW : L.win_bn;
     p.ntiles = p.narrow ? ceil_div(p.c_out, WN_NARROW) : L.win_ntiles;
     const long long tiles = row_tiles * p.ntiles;
@@ -1418,6 +1416,40 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     return false;
 }
 
+// What a CTA of an integer launch takes, in clocks, apart from what is the same for all cuts: its blocks one after the other
+// (the window's way into shared memory, or the MMAs, whichever is longer; the shorter once more where nothing hides it) and the
+// cluster's way out (meetings, rows read from the other shares; as far as the tile's rows are projection pixels).  The
+// figures are fitted to 1200 timed cuts of 132 layers: of both widths and all numbers of shares, 1x1 to 7x7, strides 1 to 4.
+static long long win_clocks(const WinParams& p, bool xcol, int frames)
+{
+    const long long rows = (win_rows(p) + TC_M - 1) / TC_M * TC_M * frames, pixels = (long long)p.n * p.oh * p.ow * frames;
+    const long long fill = 1500 + 300ll * ceil_div(p.span * (p.xarr ? p.xarr : p.gblk * 2), WN_FILL);
+    const long long steps = (long long)p.groups * p.kh * (xcol ? 1 : p.kw);
+    const long long mmas = steps * (32 + p.bn) * p.mt / ((long long)p.nblk * p.tsplit);
+    long long clocks = p.per * (fill > mmas ? fill : mmas) + (fill > mmas ? mmas : fill);
+    if (p.cluster) clocks += 4000 + 300ll * p.ks + 32ll * p.bn * pixels / rows;
+    return clocks;
+}
+
+// Integers whose shares would form a cluster, and whose tiles leave half of the wave idle, may take tiles of 32 columns
+// instead.  That saves the cluster's way out (8 to 10 k clocks with 128 columns) or most of it, and an MMA of 32 columns is
+// shorter than one of 128; but every column tile lays out the windows of all its blocks, which shares of K divide.  Few blocks:
+// narrow (us, wide / narrow: 28 -> 239 5x5 at 23 x 26 14.3 / 8.4; 96 -> 256 5x5 at 27 x 27 12.8 / 10.8).  Many blocks, of several
+// planes or of 1x1 filters: wide (409 -> 85 3x3 of stride 3 at 112 x 120, 3 images, 36 blocks: 35.4 / 71.9; 1024 -> 256 1x1 at
+// 14 x 14, 2 images: 12.0 / 16.9).  Over 109 such layers the estimate's choice is 11 % ahead of wide tiles alone, at worst
+// 2 % behind; narrow tiles alone are 8 % ahead, at worst 103 % behind.
+static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool store, int frames, int wave)
+{
+    if (win_clustered(L, dense, store) && L.win_narrow && win_few_tiles(L, (win_rows(p) + TC_M - 1) / TC_M * frames, wave)) {
+        WinParams few = p;
+        const bool narrow = win_cut(L, few, xcol, dense, store, frames, wave, true);
+        if (!win_cut(L, p, xcol, dense, store, frames, wave, false)) return false;
+        if (narrow && win_clocks(few, xcol, frames) <= win_clocks(p, xcol, frames)) p = few;
+        return true;
+    }
+    return win_cut(L, p, xcol, dense, store, frames, wave, false);
+}
+
 // Shared memory of a launch.  At least as large a part of an SM's as the CTA's share of the 512 tensor-memory columns: CTAs
 // that fit an SM together can then always allocate their columns together.  (A CTA that waits for columns while the rest
 // of its cluster waits for it, beside another cluster in the mirrored state, would wait forever.)
@@ -1447,7 +1479,7 @@ static bool win_choose(const rrm_net* net, Layer& L)
     const rrm_layer_desc& d = L.d;
     WinParams wide{}, narrow{};
     if (!win_geometry(net, L, wide)) return false;
-    narrow = wide;                                           // (win_plan widens the window it is given)
+    narrow = wide;                                           // (a plan widens the window it is given)
     const bool xcol = win_xcol(net, L), f32 = d.dtype == RRM_F32;
     L.win_ntiles = ceil_div(d.c_out, 128);
     // (integer layers: whole groups of 32 columns, so that a padded output row is covered by the column tiles)
@@ -1457,7 +1489,7 @@ static bool win_choose(const rrm_net* net, Layer& L)
     if (!win_plan(L, wide, xcol, true, false, 1, 148)) return false;
     // (more frames are only more tiles, and 148 is the larger wave: with too many tiles in one frame no launch takes narrow ones)
     L.win_narrow = !f32 && L.win_bn > WN_NARROW && win_few_tiles(L, (win_rows(wide) + TC_M - 1) / TC_M, 148);
-    L.win_narrow = L.win_narrow && win_plan(L, narrow, xcol, true, false, 1, INT_MAX);       // (a wave that makes any launch one of few tiles)
+    L.win_narrow = L.win_narrow && win_cut(L, narrow, xcol, true, false, 1, 148, true);
     return true;
 }
 

@@ -59,3 +59,16 @@ def test_filters_are_held_as_narrow_tiles_only_where_a_launch_can_take_them():
         for form, frames in FORMS:
             p = rrm.plan_conv(d, form, frames)
             assert want or p["columns"] != 32 or shape[4] <= 32
+
+
+def test_narrow_tiles_are_taken_where_every_one_lays_out_few_windows():
+    """Few blocks of the K loop: 32 columns; many, of several planes or of 1x1 filters: wide tiles whose shares divide them.  The
+    same for the deltas whose shares form a cluster (channels that are no multiple of 4)."""
+    for shape, form, want in ((("i8", 28, 23, 26, 239, 5, 5, 1, 0, 2), "dense", 32), (("i8", 96, 27, 27, 256, 5, 5, 1, 2, 1), "dense", 32),
+                              (("i8", 256, 14, 14, 512, 3, 3, 2, 1, 4), "dense", 32), (("bin", 127, 13, 9, 185, 1, 1, 3, 0, 2), "dense", 32),
+                              (("i8", 3, 227, 227, 96, 11, 11, 4, 0, 1), "dense", 32),
+                              (("i8", 409, 112, 120, 85, 3, 3, 3, 0, 3), "dense", 96), (("bin", 414, 96, 74, 84, 3, 3, 2, 1, 3), "dense", 96),
+                              (("i8", 1024, 14, 14, 256, 1, 1, 1, 0, 2), "dense", 128), (("i8", 455, 47, 30, 57, 3, 3, 2, 1, 8), "dense", 64),
+                              (("bin", 272, 67, 103, 481, 3, 3, 2, 1, 1), "delta", 128), (("i8", 104, 8, 11, 170, 3, 3, 1, 0, 11), "delta", 32)):
+        p = rrm.plan_conv(desc(*shape), form)
+        assert p["columns"] == want and (p["clustered"] or p["shares"] == 1), (shape, p)
