@@ -348,7 +348,7 @@ typedef struct {
     int32_t columns, tiles_per_cta, shares, clustered;
     int64_t ctas;
     int32_t narrow_filters;    /* the filters are held as tiles of 32 columns too */
-    int32_t reserved;
+    int32_t async_windows;     /* int8: the input windows go to shared memory by asynchronous copies, not through registers */
 } rrm_conv_plan;
 int rrm_plan_conv(const rrm_layer_desc* desc, int form, int frames, rrm_conv_plan* out);
 

@@ -43,7 +43,7 @@ class Options(ctypes.Structure):
 
 class ConvPlan(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int32) for n in ("columns", "tiles_per_cta", "shares", "clustered")] + [
-        ("ctas", ctypes.c_int64), ("narrow_filters", ctypes.c_int32), ("reserved", ctypes.c_int32)]
+        ("ctas", ctypes.c_int64), ("narrow_filters", ctypes.c_int32), ("async_windows", ctypes.c_int32)]
 
 
 _lib = None
@@ -340,7 +340,7 @@ def plan_conv(desc, form="delta", frames=1):
     """rrm_plan_conv: how a launch of the described convolution is cut (all zero: another kernel's layer).  Needs no GPU."""
     p = ConvPlan()
     _check(lib().rrm_plan_conv(ctypes.byref(desc), PLAN[form], frames, ctypes.byref(p)), "rrm_plan_conv")
-    return {n: getattr(p, n) for n, _ in p._fields_ if n != "reserved"}
+    return {n: getattr(p, n) for n, _ in p._fields_}
 
 
 def aecs_predict(mu, e_t):

@@ -91,6 +91,7 @@ struct WinParams {
     int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
     int ntiles, narrow;       // column tiles, and whether they are the narrow ones
     int tps, stages, abuf;    // taps per filter stage, stages, window buffers
+    int async_windows;        // int8: windows by asynchronous copies, not through registers
     int xarr;                 // first layers: arrays of an image row's chunks (0: the chunks of every column side by side)
     unsigned a_step, a_lbo;   // 16-byte slots between a pixel's K groups, and between the two chunks of a group
     unsigned stage_bytes, abytes, tail_off, tmem_cols;    // (tail_off: barriers and tables, behind windows, stages and drained rows)
@@ -510,7 +511,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             other_tables();
             wn_meet();
         }
-        const bool lag = DT == T_I8 && !XCOL && !DENSE && p.abuf > 1;  // asynchronous copies: a block is handed over when the next one is on its way
+        const bool async = DT == T_I8 && !XCOL && (!DENSE || p.async_windows);
+        const bool lag = async && p.abuf > 1;                // asynchronous copies: a block is handed over when the next one is on its way
         const int* src = S->tab;                             // the plane's table
         const int* const xcol0 = S->tab + WN_MAX_SPAN;
         int plane = plane0, chb = b0 - plane0 * p.nchb, ib = 0, buf = -1;
@@ -540,10 +542,10 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const uint32_t piece = (uint32_t)(arrays * p.L) * 16u;              // bytes between the fp32 pieces' windows
             const unsigned magic = cl > 1 ? (unsigned)(((1ull << 32) + cl - 1) / cl) : 0u;
             const int items = p.span * cl;
-            if (DT == T_I8 && !XCOL && DENSE) {
-                // Dense blocks are many and full: through registers, a turn's loads all on their way before its first store.
-                // (Asynchronous copies, handed over when the next block's were on their way, took 2.3 to 3 k clocks a block: 24
-                // AlexNet-shaped keyframes 97.2 -> 93.2 us, 4 ResNet-18-shaped streams 188.9 -> 181.8.)
+            if (DT == T_I8 && !XCOL && DENSE && !async) {
+                // Dense blocks are full: through registers, a turn's loads all on their way before its first store.  (Asynchronous
+                // copies, handed over when the next block's are on their way, take 2.3 to 3 k clocks a block: 24 AlexNet-shaped
+                // keyframes 97.2 -> 93.2 us, 4 ResNet-18-shaped streams 188.9 -> 181.8.)
                 const unsigned char* src0 = reinterpret_cast<const unsigned char*>(A) + g0 * 32;
                 constexpr int TURN = 6;
                 #pragma unroll 1
@@ -565,7 +567,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 fence_async_smem();
                 mbar_arrive(smem_u32(&S->afull[buf]));
             } else if (DT == T_I8 && !XCOL) {
-                // delta rows: asynchronous copies (one frame's steps, one small block per CTA: 64.2 us against 65.8 through registers)
+                // asynchronous copies: delta rows (one frame's steps, one small block per CTA: 64.2 us against 65.8 through
+                // registers), and dense passes of many short blocks (win_async_windows)
                 const unsigned char* src0 = reinterpret_cast<const unsigned char*>(A) + g0 * 32;
                 #pragma unroll 4
                 for (int idx = tid; idx < items; idx += WN_FILL) {
@@ -718,7 +721,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 // (a warp whose wait ran out says so when the warps meet at the next block)
             }
         }
-        if (DT == T_I8 && !XCOL && !DENSE) {
+        if (async) {
             cp_async_wait<0>();
             fence_async_smem();
             if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[buf]));
@@ -1416,6 +1419,19 @@ static bool win_cut(const Layer& L, WinParams& p, bool xcol, bool dense, bool st
     return false;
 }
 
+// Clocks of a block of an integer launch: of its window's way into shared memory, and of its MMAs.
+static long long win_fill_clocks(const WinParams& p) { return 1500 + 300ll * ceil_div(p.span * (p.xarr ? p.xarr : p.gblk * 2), WN_FILL); }
+static long long win_mma_clocks(const WinParams& p, bool xcol)
+{
+    return (long long)p.groups * p.kh * (xcol ? 1 : p.kw) * (32 + p.bn) * p.mt / ((long long)p.nblk * p.tsplit);
+}
+
+// Dense int8 windows by asynchronous copies: with three buffers or more two blocks' copies are under way at a time, which pays
+// where the MMAs are too short to hide a block's way through registers (9 x 36 short blocks, 409 -> 85 3x3 of stride 3 at
+// 112 x 120, 12 images: 133.9 us through registers, 103.4 so; 31 of 340 timed launches fall under the rule, 5 % faster on
+// average, at worst level but for one of 17.6 us, 4 % slower).  The others are up to 15 % slower so.
+static bool win_async_windows(const WinParams& p, bool xcol) { return p.abuf >= 3 && win_mma_clocks(p, xcol) * 5 < win_fill_clocks(p) * 2; }
+
 // What a CTA of an integer launch takes, in clocks, apart from what is the same for all cuts: its blocks one after the other
 // (the window's way into shared memory, or the MMAs, whichever is longer; the shorter once more where nothing hides it) and the
 // cluster's way out (meetings, rows read from the other shares; as far as the tile's rows are projection pixels).  The
@@ -1425,9 +1441,7 @@ static bool win_cut(const Layer& L, WinParams& p, bool xcol, bool dense, bool st
 static long long win_clocks(const WinParams& p, bool xcol, bool dense, int frames)
 {
     const long long rows = (win_rows(p) + TC_M - 1) / TC_M * TC_M * frames, pixels = (long long)p.n * p.oh * p.ow * frames;
-    const long long fill = 1500 + 300ll * ceil_div(p.span * (p.xarr ? p.xarr : p.gblk * 2), WN_FILL);
-    const long long steps = (long long)p.groups * p.kh * (xcol ? 1 : p.kw);
-    const long long mmas = steps * (32 + p.bn) * p.mt / ((long long)p.nblk * p.tsplit);
+    const long long fill = win_fill_clocks(p), mmas = win_mma_clocks(p, xcol);
     long long clocks = p.per * (fill > mmas ? fill : mmas) + (fill > mmas ? mmas : fill);
     if (p.cluster) clocks += 300ll * p.ks + (dense ? 4000 + 32ll * p.bn * pixels / rows : 2500);
     return clocks;
@@ -1561,6 +1575,7 @@ int conv_win_query(const rrm_net& net, Layer& L, int form, int frames, rrm_conv_
     out->columns = p.bn; out->tiles_per_cta = p.mt; out->shares = p.ks; out->clustered = p.cluster;
     out->ctas = (rows + p.mt * TC_M - 1) / (p.mt * TC_M) * p.ntiles * p.ks * (seq ? frames : 1);
     out->narrow_filters = L.win_narrow;
+    out->async_windows = L.d.dtype == RRM_I8 && !xcol && (!dense || win_async_windows(p, xcol));
     return RRM_OK;
 }
 
@@ -1585,6 +1600,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     const int nf = batched ? frames : 1;
     if (!win_plan(L, p, xcol, dense, batched, nf, net->many_in_flight ? 74 : 148)) return RRM_ERR_UNSUPPORTED;
     if (p.span > WN_MAX_SPAN) return RRM_ERR_CAPACITY;       // (never: win_plan takes no such window)
+    p.async_windows = win_async_windows(p, xcol);
     const void* X = stateless ? in.X2 : in.X;
     p.A = bin ? in.D : (dense ? X : in.D);
     p.Anew = (!dense && !stateless && in.Xn_cur) ? in.Xn_cur : X;    // (chunks of frames: this frame's copy of the new rows)

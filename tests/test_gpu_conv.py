@@ -321,6 +321,20 @@ def test_dense_passes_of_few_tiles_take_narrow_ones(dtype, c_in, c_out, hw, k, s
         _run([sp], _video(dtype, c_in, hw, 4, n, rng), n=n, stats=True, keyframe_at=(1, 3))
 
 
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n,plan", [
+    (420, 33, (20, 19), 3, 3, 0, 3, (32, 1, 8)),             # clusters; a last block of two of four groups
+    (70, 128, (34, 31), 3, 2, 1, 8, (32, 1, 1)), (512, 70, (14, 13), 1, 1, 0, 2, (32, 1, 1)),      # narrow tiles; one plane
+    (260, 40, (61, 60), 3, 3, 1, 9, (64, 1, 4)), (32, 64, (41, 40), 3, 2, 1, 92, (64, 2, 1))])     # two accumulator tiles
+def test_dense_windows_of_many_short_blocks(c_in, c_out, hw, k, s, p, n, plan):
+    """Dense int8 passes whose windows come by asynchronous copies, as outputs and as raw projections, delta steps in between."""
+    rng = np.random.default_rng(c_in + c_out)
+    for kw in (dict(act="relu", shift=8), dict(shift=-1, act="none")):
+        sp = _spec("i8", c_in, hw, c_out, k, s, p, rng, **kw)
+        got = _rrm().plan_conv(_rrm().desc_from_spec(sp, n), "dense")
+        assert got["async_windows"] and (got["columns"], got["tiles_per_cta"], got["shares"]) == plan, got
+        _run([sp], _video("i8", c_in, hw, 4, n, rng), n=n, keyframe_at=(1, 3))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "i8", "bin"])
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p,pool", [
     (24, 20, (5, 700), 3, 1, 1, (3, 2, 0)),  # wider than 510 pixels
