@@ -44,12 +44,12 @@ namespace rrm {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The launches of this thread overlap their predecessors while an object of this kind lives.
+// While an object of this kind lives the launches of this thread overlap their predecessors, or do not.
 struct OverlapLaunches {
-    static int& depth() { static thread_local int d = 0; return d; }
-    const int by;
-    explicit OverlapLaunches(bool on = true) : by(on ? 1 : 0) { depth() += by; }
-    ~OverlapLaunches() { depth() -= by; }
+    static bool& on() { static thread_local bool o = false; return o; }
+    const bool before;
+    explicit OverlapLaunches(bool now = true) : before(on()) { on() = now; }
+    ~OverlapLaunches() { on() = before; }
     OverlapLaunches(const OverlapLaunches&) = delete;
     OverlapLaunches& operator=(const OverlapLaunches&) = delete;
 };
@@ -57,7 +57,7 @@ struct OverlapLaunches {
 inline bool pdl_enabled()
 {
     static const char asked = [] { const char* e = getenv("RRM_PDL"); return e ? e[0] : '\0'; }();
-    return asked == '1' || (asked != '0' && OverlapLaunches::depth() > 0);
+    return asked == '1' || (asked != '0' && OverlapLaunches::on());
 }
 
 // cluster_z > 1: the CTAs that differ only in blockIdx.z form one thread-block cluster (they can read each other's

@@ -1476,6 +1476,22 @@ static size_t win_smem(const WinParams& p)
     return need > share ? need : share;
 }
 
+// Launches that overlap their predecessors (dense passes) are placed while those still hold some of the SMs: two CTAs of an
+// integer launch then come to lie on one SM and leave others idle.  Launches of fewer CTAs than SMs, but of many, ask for more than
+// half of an SM's shared memory, so that each has one to itself (411 -> 22 3x3 of stride 2, binary, 56 images of 27 x 37, 132
+// CTAs: 37.3 us without overlap, 42.5 with, 36.3 so; dense chunks of 32 AlexNet-shaped frames 124.7 -> 119.2, 4 ResNet-18-shaped
+// streams 172.2 -> 168.8).  Below 90 CTAs they find room beside each other, and the next launch's wait beside them (24
+// AlexNet-shaped keyframes, two launches of 81 CTAs: 90.9, 92.0 with an SM each).
+constexpr int WN_ALONE = 90;
+constexpr size_t WN_ALONE_SMEM = 116 * 1024;
+
+static bool win_alone(const WinParams& p, int dtype, long long ctas) { return dtype != RRM_F32 && !p.cluster && ctas >= WN_ALONE && ctas <= 148; }
+
+// Clusters cannot be placed so: their CTAs also have to lie in one part of the machine (one CTA an SM is up to 1.6 times as slow).
+// Binary clusters of long chains, whose windows keep an SM's ALUs busy, are not launched early instead (457 -> 69 3x3 of stride 3 at
+// 84 x 68, 11 images, 112 CTAs of 18 blocks each: 47.2 us without overlap, 53.9 with).
+constexpr long long WN_LONG_CHAIN = 18000;                   // clocks of a CTA's windows
+
 template <int DT, bool XCOL>
 static int win_allow()
 {
@@ -1620,7 +1636,9 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     }
     const long long rows = win_rows(p);
     const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)p.ntiles, (unsigned)(nf * p.ks));
-    const size_t smem = win_smem(p);
+    size_t smem = win_smem(p);
+    if (dense && pdl_enabled() && win_alone(p, d.dtype, (long long)grid.x * grid.y * grid.z) && smem < WN_ALONE_SMEM) smem = WN_ALONE_SMEM;
+    const OverlapLaunches early(OverlapLaunches::on() && !(dense && bin && p.cluster && p.per * win_fill_clocks(p) >= WN_LONG_CHAIN));
     cudaError_t e;
     if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, out, grid, smem, st) : win_launch<T_F32, false>(p, dense, out, grid, smem, st);
     else if (d.dtype == RRM_I8) e = xcol ? win_launch<T_I8, true>(p, dense, out, grid, smem, st) : win_launch<T_I8, false>(p, dense, out, grid, smem, st);

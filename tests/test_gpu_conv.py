@@ -1,6 +1,10 @@
 """GPU parity of the convolution path (single layers and layer stacks) against the CPU oracle.
 Integer and binary layers must match bit for bit; fp32 layers within 1e-4 * max|P_dense| per
 frame (the accumulated projection is compared at every frame, so drift would show)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -333,6 +337,45 @@ def test_dense_windows_of_many_short_blocks(c_in, c_out, hw, k, s, p, n, plan):
         got = _rrm().plan_conv(_rrm().desc_from_spec(sp, n), "dense")
         assert got["async_windows"] and (got["columns"], got["tiles_per_cta"], got["shares"]) == plan, got
         _run([sp], _video("i8", c_in, hw, 4, n, rng), n=n, keyframe_at=(1, 3))
+
+
+def _dense_outputs(path):
+    """Keyframes, dense passes and dense chunks of three stacks and of layers whose launches lie alone on their SMs or are not
+    launched early; every call twice in a row, so that a pass starts while the last one ends."""
+    rrm, got = _rrm(), {}
+    rng = np.random.default_rng(8)
+    nets = [("f32", wl.alexnet_convs("f32", hw=67), 2, (3, 67, 67)), ("i8", wl.alexnet_convs("i8", hw=67), 3, (3, 67, 67)),
+            ("bin", wl.xnor_alexnet_convs(hw=67), 2, (3, 67, 67)), ("res", wl.resnet18_convs(hw=64), 2, (3, 64, 64))]
+    for i, (dtype, c_in, c_out, hw, k, s, p, n) in enumerate((("bin", 411, 22, (27, 37), 3, 2, 1, 56), ("bin", 457, 69, (84, 68), 3, 3, 0, 11),
+                                                              ("i8", 64, 64, (56, 56), 3, 1, 1, 4))):
+        nets.append((f"{dtype}{i}", [_spec(dtype, c_in, hw, c_out, k, s, p, rng, **(dict(act="sign", theta=1) if dtype == "bin" else dict(act="relu", shift=9)))],
+                     n, (c_in,) + hw))
+    for name, specs, n, shape in nets:
+        net = rrm.net_from_specs(specs, n=n)
+        x = _frame_to_dev(specs, _video(specs[0].dtype, shape[0], shape[1:], 4, n, rng)[0])
+        y = x.flip(0).contiguous()
+        out, outs = net.new_output(), net.new_output(frames=3)
+        for what in ("keyframe", "dense"):
+            getattr(net, what)(x, out)
+            getattr(net, what)(y, out)
+            got[f"{name} {what}"] = out.cpu().numpy()
+        for _ in range(2):
+            net.dense_seq(torch.stack((x, y, x)), outs)
+        got[f"{name} chunk"] = outs.cpu().numpy()
+        net.close()
+    np.savez(path, **got)
+
+
+def test_dense_launches_that_overlap_give_the_same_bits(tmp_path):
+    """With the launches of dense passes overlapping their predecessors, and (in a process of its own: the switch is read once)
+    without."""
+    _dense_outputs(tmp_path / "overlapping.npz")
+    code = f"import sys; sys.path[:0] = [{os.path.dirname(__file__)!r}, {os.path.dirname(os.path.dirname(__file__))!r}]; import test_gpu_conv as t; t._dense_outputs({str(tmp_path / 'apart.npz')!r})"
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=600, env=dict(os.environ, RRM_PDL="0"))
+    a, b = np.load(tmp_path / "overlapping.npz"), np.load(tmp_path / "apart.npz")
+    assert sorted(a.files) == sorted(b.files) and len(a.files) == 21
+    for name in a.files:
+        np.testing.assert_array_equal(a[name], b[name], err_msg=name)
 
 
 @pytest.mark.parametrize("dtype", ["f32", "i8", "bin"])
