@@ -1535,17 +1535,16 @@ int conv_win_create(rrm_net* net, Layer& L, const void* W_dev)
     const int taps = xcol ? d.kh : d.kh * d.kw;
     const size_t chunks = (size_t)L.win_ntiles * taps * p.groups * 2 * L.win_bn;
     const size_t bytes = chunks * 16 * (f32 ? 3 : 1);
-    void *img = nullptr, *few = nullptr;
-    if (cudaMalloc(&img, bytes + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
-    net->allocs.push_back(img);
-    // the same filters once more, as tiles of 32 columns; where there is no room for them the layer goes without
+    // the same filters once more, as tiles of 32 columns; where there is no room for both the layer goes without (one block
+    // for both: an allocation costs some 60 us)
     const int few_ntiles = ceil_div(d.c_out, WN_NARROW);
     const size_t few_chunks = (size_t)few_ntiles * taps * p.groups * 2 * WN_NARROW;
-    if (L.win_narrow) {
-        if (cudaMalloc(&few, few_chunks * 16) == cudaSuccess) net->allocs.push_back(few);
-        else { cudaGetLastError(); few = nullptr; L.win_narrow = false; }
-    }
+    void *img = nullptr, *few = nullptr;
+    if (L.win_narrow && cudaMalloc(&img, bytes + 16 + few_chunks * 16) != cudaSuccess) { cudaGetLastError(); img = nullptr; L.win_narrow = false; }
+    if (!img && cudaMalloc(&img, bytes + 16) != cudaSuccess) { cudaGetLastError(); return RRM_ERR_ALLOC; }
+    net->allocs.push_back(img);
     int* beyond = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(img) + bytes);
+    if (L.win_narrow) few = beyond + 4;
     RRM_CUDA_TRY(cudaMemset(beyond, 0, 4));
     auto pack = [&](auto kernel) {
         auto go = [&](void* to, size_t n, int bn, int ntiles) {
