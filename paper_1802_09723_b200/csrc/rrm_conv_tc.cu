@@ -83,6 +83,7 @@ constexpr int TC_LAG = 1;                     // a slab is handed to the tensor 
                                               // copies in flight too, left the stage's MMAs too little time to commit before the
                                               // producers want the stage back (measured: 3-5 % slower steps)
 constexpr int TC_ROW_WORDS = TC_MAX_BN + 4;   // epilogue row buffers: 16-byte aligned rows, staggered over the banks
+static_assert(TC_SMEM_BYTES >= tmem_share(TC_MAX_BN), "CTAs that fit an SM together must find their columns together");
 static_assert((size_t)TC_M * TC_ROW_WORDS * 4 <= TC_STAGES * TC_STAGE_BYTES, "epilogue rows reuse the stage buffers");
 
 template <bool BIN, bool DENSE>

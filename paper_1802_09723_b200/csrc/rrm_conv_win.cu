@@ -1466,13 +1466,10 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
     return win_cut(L, p, xcol, dense, store, frames, wave, false);
 }
 
-// Shared memory of a launch.  At least as large a part of an SM's as the CTA's share of the 512 tensor-memory columns: CTAs
-// that fit an SM together can then always allocate their columns together.  (A CTA that waits for columns while the rest
-// of its cluster waits for it, beside another cluster in the mirrored state, would wait forever.)
+// Shared memory of a launch: at least the CTA's share of tensor memory.
 static size_t win_smem(const WinParams& p)
 {
-    const size_t need = p.tail_off + sizeof(WinTail) + 128;
-    const size_t share = (size_t)p.tmem_cols * 228 * 1024 / 512 - 1024;
+    const size_t need = p.tail_off + sizeof(WinTail) + 128, share = tmem_share(p.tmem_cols);
     return need > share ? need : share;
 }
 

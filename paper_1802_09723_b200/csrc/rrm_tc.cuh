@@ -9,6 +9,14 @@ namespace rrm {
 constexpr unsigned WAIT_LIMIT_DEFAULT = 1u << 20;   // polls of one bounded wait before it gives up (rrm_options.wait_limit)
 constexpr int TC_M = 128;                       // accumulator rows of one MMA tile
 
+// The dynamic shared memory a CTA that allocates `cols` columns of tensor memory asks for at least: as large a part of an SM's 228
+// KB (of which the system keeps 1 KB per CTA) as the columns are of the SM's 512.  CTAs that fit an SM together can then always
+// allocate their columns together, whichever kernels and launches they belong to: a dense pass's launches overlap, and those
+// of two or three layers meet on an SM.  (A CTA that waits for columns while the rest of its cluster waits for it, beside
+// another cluster in the mirrored state, would wait forever; and one that waits for the columns of a launch before it only
+// waits for CTAs that are running already, since a launch begins once all CTAs of the one before it have.)
+constexpr size_t tmem_share(unsigned cols) { return (size_t)cols * 228 * 1024 / 512 - 1024; }
+
 // ---- raw PTX wrappers ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
