@@ -26,10 +26,12 @@
  *   - One object may be used from one stream at a time.
  *   - Environment switches, read when an object is created (debugging aids): RRM_NO_GRAPH=1 launches every
  *     kernel of a stack step on its own instead of replaying a captured CUDA graph; RRM_DEBUG=1 names a failing
- *     CUDA call (file, line, error string) on stderr and prints the shape of captured chunk graphs; RRM_PDL=1
- *     launches all kernels of a stack with programmatic dependent launch (each kernel's set-up overlaps its
- *     predecessor's tail), RRM_PDL=0 none (by default the dense passes, keyframes and dense chunks use it: delta steps
- *     gain nothing from it; the kernels of a lone FC layer, which are plain launches, always do); RRM_CHUNK_INPLACE=1
+ *     CUDA call (file, line, error string) on stderr and prints the shape of captured chunk graphs; RRM_PDL=1 (this
+ *     one is read once per process) launches all kernels of a stack with programmatic dependent launch (each kernel's set-up
+ *     overlaps its predecessor's tail), RRM_PDL=0 none (by default the captured dense passes and keyframes and the dense chunks
+ *     batched over their frames use it, but for kernels that lose by it: delta steps gain nothing from it, dense passes under
+ *     RRM_NO_GRAPH=1 and dense chunks of overlapping frames go without; the kernels of a lone FC layer, which are plain
+ *     launches, always do); RRM_CHUNK_INPLACE=1
  *     makes the delta chunks of a stack (rrm_net_step_seq) add each frame's product straight onto the stored
  *     projection, as single steps do, instead of keeping it in a per-frame buffer that the epilogue merges (the
  *     default, which lets the convolution of frame t+1 run beside the epilogue of frame t; same results).
