@@ -312,17 +312,28 @@ def test_first_layers_whose_window_leaves_room_for_one_tile_width(c_in, c_out, h
 
 
 @pytest.mark.parametrize("dtype", ["i8", "bin"])
-@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n", [
-    (64, 70, (14, 13), 3, 1, 1, 1), (320, 200, (13, 13), 3, 1, 1, 1),         # one share (18 and 90 K steps), ragged columns
-    (352, 130, (9, 11), 3, 1, 1, 2), (512, 64, (7, 7), 3, 1, 1, 4), (96, 96, (17, 18), 5, 2, 2, 3),      # clusters of 2 and 3, strides
-    (3, 96, (60, 61), 11, 4, 0, 1), (32, 33, (8, 8), 1, 1, 0, 1)])
-def test_dense_passes_of_few_tiles_take_narrow_ones(dtype, c_in, c_out, hw, k, s, p, n):
+@pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n,dense,delta", [
+    # (columns, accumulator tiles per CTA, shares): one share (18 and 90 K steps), ragged columns
+    (64, 70, (14, 13), 3, 1, 1, 1, (32, 1, 1), (32, 1, 1)), (320, 200, (13, 13), 3, 1, 1, 1, (32, 1, 1), (128, 1, 10)),
+    # clusters of 2, strides, deltas in clusters; a layer whose shares of wide tiles are ahead
+    (352, 130, (9, 11), 3, 1, 1, 2, (32, 1, 2), (96, 1, 6)), (96, 96, (17, 18), 5, 2, 2, 3, (32, 1, 8), (96, 1, 12)),
+    (512, 64, (7, 7), 3, 1, 1, 4, (64, 1, 8), (64, 1, 16)), (32, 33, (8, 8), 1, 1, 0, 1, (32, 1, 1), (32, 1, 1)),
+    # 74 and 75 wide tiles; 74 of 128 columns are 296 narrow ones, of which a CTA takes two
+    (32, 64, (96, 97), 3, 1, 1, 1, (32, 1, 1), (64, 1, 2)), (32, 64, (97, 97), 3, 1, 1, 1, (64, 1, 1), (64, 1, 1)),
+    (32, 256, (12, 12), 3, 1, 1, 28, (32, 2, 1), (128, 1, 2)), (32, 250, (12, 12), 3, 1, 1, 28, (32, 2, 1), (32, 2, 1)),
+    # first layers (binary ones are not), of wide windows too
+    (3, 96, (60, 61), 11, 4, 0, 1, {"i8": (32, 1, 4), "bin": (32, 1, 8)}, {"i8": (96, 1, 4), "bin": (96, 1, 16)}),
+    (3, 96, (24, 500), 7, 2, 3, 1, {"i8": (32, 1, 2), "bin": (96, 1, 4)}, {"i8": (96, 1, 2), "bin": (96, 1, 4)})])
+def test_dense_passes_of_few_tiles_take_narrow_ones(dtype, c_in, c_out, hw, k, s, p, n, dense, delta):
     """Keyframes and dense passes whose tiles would leave the machine idle run as tiles of 32 columns; with f in the kernel
     (int8, signs), as raw projections, and with delta steps in between."""
     rng = np.random.default_rng(c_in + c_out)
     for kw in ((dict(act="sign", theta=1), dict(shift=-1, act="none")) if dtype == "bin" else (dict(act="relu", shift=8), dict(shift=-1, act="none"))):
         sp = _spec(dtype, c_in, hw, c_out, k, s, p, rng, **kw)
-        _run([sp], _video(dtype, c_in, hw, 4, n, rng), n=n, stats=True, keyframe_at=(1, 3))
+        for form, want in (("dense", dense), ("delta", delta)):
+            got = _rrm().plan_conv(_rrm().desc_from_spec(sp, n), form)
+            assert (got["columns"], got["tiles_per_cta"], got["shares"]) == (want[dtype] if isinstance(want, dict) else want), (form, got)
+        _run([sp], _video(dtype, c_in, hw, 4, n, rng), n=n, stats=n < 28, keyframe_at=(1, 3))
 
 
 @pytest.mark.parametrize("c_in,c_out,hw,k,s,p,n,plan", [
