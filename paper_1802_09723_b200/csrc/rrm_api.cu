@@ -920,13 +920,13 @@ int run_chunk(rrm_net* net, const void* frames, void* outs, int T, cudaStream_t 
             // Chunks have a batched dense form that needs no change detection, marking or prefix sums and stores no
             // projections but the last frame's: on tensor-core stacks it is ahead from a lower activity on than the
             // whole-stack switch of single steps.  What a delta chunk can save is accumulator tiles without any pixel to
-            // update, so those are what its activity counts.  Measured, us per frame, delta as the library chooses /
-            // dense: AlexNet int8 on the quiet video (a third of the pixels) 1 stream x 16 frames 12.1 / 9.2, 32 frames
-            // 7.1 / 6.4, 8 streams x 4 frames 57 / 51; busy 13.7 / 9.1; a lone int8 layer, 3 streams x 8 frames 17 / 9.8.
-            // fp32, delta / dense: AlexNet busy 18.5 / 14.1, quiet 16.4 / 14.1 (1 stream x 32), 13.8 / 14.2 (2 x 16); lone 3x3
-            // layers, us per chunk: 2 x 16 frames of 64 x 112 x 112 with 0.05 and 0.2 % of the pixels, or 5 % of the 8 x 8 patches, changing
-            // 495, 586, 652 / 512; 4 x 16 of 256 x 28 x 28 460-522 / 361.  (Chunks of fewer than 8 frames stay on the delta path below the whole-stack threshold: their callers
-            // read counters frame by frame.)
+            // update, so those are what its activity counts.  Measured, us per chunk, delta / dense, at 227 x 227 (streams x
+            // frames): AlexNet int8, quiet video (a third of the pixels) 1 x 16 169 / 86, 1 x 32 195 / 109, 8 x 4 211 / 114, busy 198
+            // / 86, 247 / 109, 273 / 114; binary within 5 % of these; fp32 quiet 306 / 313, 524 / 439, 2 x 16 432 / 442, 8 x 4 410 /
+            // 450, busy 399 / 315, 584 / 439, 589 / 441, 551 / 451.  Lone layers: int8 48 -> 80 5x5 at 45 x 45, 3 x 8, 104 / 33; fp32
+            // 3x3, 2 x 16 frames of 64 x 112 x 112 with 0.05 and 0.2 % of the pixels, or 10 % in 8 x 8 patches, changing 502, 584, 724 / 474,
+            // 4 x 16 of 256 x 28 x 28 530 / 344.  (Chunks of fewer than 8 frames stay on the delta path below the whole-stack
+            // threshold: their callers read counters frame by frame.)
             const bool go_dense = (net->auto_switch && net->activity >= net->opt.stack_dense_activity) ||
                                   (long_chunk && net->chunk_activity >= net->opt.chunk_dense_activity);
             if (go_dense && net->dense_streak < net->opt.stack_reprobe) {

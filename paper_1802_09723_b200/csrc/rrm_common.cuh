@@ -33,11 +33,12 @@ namespace rrm {
 // Every kernel of the sequence lets its successor start launching at once (launch_dependents at its top) and waits
 // for its predecessor's results (pdl_wait) only when it first needs what a predecessor writes: thread-block scheduling,
 // barrier initialisation, tensor-memory allocation and, in dense passes, window tables and first filter copies of kernel k+1
-// then overlap the tail of kernel k.  Some thread of every grid waits, so a grid ends after its predecessors, and a wait covers them all.  What a
-// predecessor wrote is read with ordinary loads (not through the read-only path).  Without the launch attribute both
-// instructions do nothing.  The attribute is set (OverlapLaunches) while a dense
-// pass, a keyframe or a dense chunk is captured: there most of a kernel's set-up needs nothing of its predecessor, and a pass
-// of 25 launches went from 206 to 189 us (4 ResNet-18-shaped streams), one of 12 from 104 to 97 (24 AlexNet-shaped keyframes).
+// then overlap the tail of kernel k.  Some thread of every grid waits, so a grid ends after its predecessors, and a wait covers
+// them all.  What a predecessor wrote is read with ordinary loads (not through the read-only path).  Without the launch
+// attribute both instructions do nothing.  The attribute is set (OverlapLaunches) while a dense pass, a keyframe or a dense
+// chunk is captured: there most of a kernel's set-up needs nothing of its predecessor, and a pass of 25 launches went from 206
+// to 189 us (4 ResNet-18-shaped streams), one of 12 from 104 to 97 (24 AlexNet-shaped keyframes).  Launches that lose by an early
+// start (they are placed around what their predecessor still holds) go without it; the rules stand where they are launched.
 // Delta steps, whose kernels start with their predecessor's bitmaps, gained nothing or lost (one int8 frame 63.7 -> 65.3
 // us), and graphs whose frames overlap have their own edges and fill the machine by themselves.  RRM_PDL=1 in the
 // environment sets it everywhere, RRM_PDL=0 nowhere.

@@ -40,8 +40,8 @@
 // What bounds it: in a long K loop the MMAs' operand reads from shared memory (an MMA of 128 columns reads 8 KB and takes 97 to
 // 118 clocks instead of 64, one of 32 columns 77; fp32: 413 clocks a K step of 16, 384 of them MMAs, 126 bytes of shared memory
 // a clock); in a launch of a few tiles a chain (clocks: set-up 1.8 k, first window 2.2 k, MMAs 3 to 6 k, way out 1.2 to 2.3 k, 7 k
-// for 64 KB of fp32 rows).  AlexNet-shaped stack at 227 x 227: 8 fp32 streams 187 us, 32 fp32 frames 465, one int8 frame 64, 32
-// int8 frames 126; 4 ResNet-18-shaped int8 streams 171.
+// for 64 KB of fp32 rows).  AlexNet-shaped stack at 227 x 227: 8 fp32 streams 187 us, 32 fp32 frames 462, one int8 frame 65, 32
+// int8 frames 121; 4 ResNet-18-shaped int8 streams 168.
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
@@ -879,77 +879,75 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
         uint32_t* mine = staged + (size_t)warp * 32 * ldt;   // (the warp's rows, where projections are kept)
         const bool any_keep = __any_sync(0xffffffffu, keep);
         // (a loop, not unrolled: every CTA runs this code once, so its length is instruction fetches)
-        {
-            #pragma unroll 1
-            for (int cc = c_lo; cc < c_hi; cc += 32) {
-                const bool inside = q >= 0 && n0 + cc < (p.bits ? p.cs * 32 : p.cs);
-                uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-                if (p.res && inside) {
-                    const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const int8_t*>(p.res) + (size_t)q * p.cs + n0 + cc);
-                    rw[0] = src[0]; rw[1] = src[1];
-                }
-                uint32_t v[32];
-                __syncwarp();
-                wn_ld32(tmem + lane_base + (uint32_t)(m_own * p.bn + cc), v);
+        #pragma unroll 1
+        for (int cc = c_lo; cc < c_hi; cc += 32) {
+            const bool inside = q >= 0 && n0 + cc < (p.bits ? p.cs * 32 : p.cs);
+            uint4 rw[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+            if (p.res && inside) {
+                const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const int8_t*>(p.res) + (size_t)q * p.cs + n0 + cc);
+                rw[0] = src[0]; rw[1] = src[1];
+            }
+            uint32_t v[32];
+            __syncwarp();
+            wn_ld32(tmem + lane_base + (uint32_t)(m_own * p.bn + cc), v);
+            #pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const int4 b = *reinterpret_cast<const int4*>(S->bias + cc + j);
+                v[j] += (uint32_t)b.x; v[j + 1] += (uint32_t)b.y; v[j + 2] += (uint32_t)b.z; v[j + 3] += (uint32_t)b.w;
+            }
+            if (any_keep) {
+                // the projection leaves as whole lines, eight lanes a row.  (Row by row through the copy engine, 128 bytes a copy:
+                // 9 to 18 clocks each, 4.6 to 9.4 k of a keyframe CTA's 14 to 38 k)
                 #pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                    const int4 b = *reinterpret_cast<const int4*>(S->bias + cc + j);
-                    v[j] += (uint32_t)b.x; v[j + 1] += (uint32_t)b.y; v[j + 2] += (uint32_t)b.z; v[j + 3] += (uint32_t)b.w;
-                }
-                if (any_keep) {
-                    // the projection leaves as whole lines, eight lanes a row.  (Row by row through the copy engine, 128 bytes a copy:
-                    // 9 to 18 clocks each, 4.6 to 9.4 k of a keyframe CTA's 14 to 38 k)
-                    #pragma unroll
-                    for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(mine + lane * ldt + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                    __syncwarp();
-                    const int c4 = (lane & 7) * 4, left = ncols - cc - c4;
-                    #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int rr = i * 4 + (lane >> 3), qq = __shfl_sync(0xffffffffu, q, rr);
-                        if (qq < p.keep_from || left <= 0) continue;
-                        const uint4 t = *reinterpret_cast<const uint4*>(mine + rr * ldt + c4);
-                        uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(qq - p.keep_from) * p.c_out + n0 + cc + c4;
-                        if (vec) *reinterpret_cast<uint4*>(dst) = t;
-                        else {
-                            dst[0] = t.x;
-                            if (left > 1) dst[1] = t.y;
-                            if (left > 2) dst[2] = t.z;
-                            if (left > 3) dst[3] = t.w;
-                        }
+                for (int j = 0; j < 32; j += 4) *reinterpret_cast<uint4*>(mine + lane * ldt + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                __syncwarp();
+                const int c4 = (lane & 7) * 4, left = ncols - cc - c4;
+                #pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3), qq = __shfl_sync(0xffffffffu, q, rr);
+                    if (qq < p.keep_from || left <= 0) continue;
+                    const uint4 t = *reinterpret_cast<const uint4*>(mine + rr * ldt + c4);
+                    uint32_t* dst = reinterpret_cast<uint32_t*>(P) + (size_t)(qq - p.keep_from) * p.c_out + n0 + cc + c4;
+                    if (vec) *reinterpret_cast<uint4*>(dst) = t;
+                    else {
+                        dst[0] = t.x;
+                        if (left > 1) dst[1] = t.y;
+                        if (left > 2) dst[2] = t.z;
+                        if (left > 3) dst[3] = t.w;
                     }
                 }
-                if (!inside) continue;
-                if (p.bits) {
-                    uint32_t word = 0;
-                    #pragma unroll
-                    for (int j = 0; j < 32; ++j) word |= (uint32_t)((int)v[j] >= p.theta) << j;
-                    if (ncols - cc < 32) word &= (1u << max(ncols - cc, 0)) - 1u;
-                    reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + ((n0 + cc) >> 5)] = word;
-                } else {
-                    const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
-                    uint32_t o[8];
-                    if (!p.bn_scale) {
-                        const int rnd = p.shift > 0 ? 1 << (p.shift - 1) : 0, sh = p.shift, lo = p.act_fn == RRM_ACT_RELU ? 0 : -127;
-                        if (!p.res) {
-                            #pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                o[j] = wn_pack4(max(((int)v[4 * j] + rnd) >> sh, lo), max(((int)v[4 * j + 1] + rnd) >> sh, lo),
-                                                max(((int)v[4 * j + 2] + rnd) >> sh, lo), max(((int)v[4 * j + 3] + rnd) >> sh, lo));
-                        } else {
-                            #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
-                                o[j] = wn_f8_plain(x, rr[j], rnd, sh, lo, true);
-                            }
-                        }
+            }
+            if (!inside) continue;
+            if (p.bits) {
+                uint32_t word = 0;
+                #pragma unroll
+                for (int j = 0; j < 32; ++j) word |= (uint32_t)((int)v[j] >= p.theta) << j;
+                if (ncols - cc < 32) word &= (1u << max(ncols - cc, 0)) - 1u;
+                reinterpret_cast<uint32_t*>(p.X)[(size_t)q * p.cs + ((n0 + cc) >> 5)] = word;
+            } else {
+                const uint32_t rr[8] = {rw[0].x, rw[0].y, rw[0].z, rw[0].w, rw[1].x, rw[1].y, rw[1].z, rw[1].w};
+                uint32_t o[8];
+                if (!p.bn_scale) {
+                    const int rnd = p.shift > 0 ? 1 << (p.shift - 1) : 0, sh = p.shift, lo = p.act_fn == RRM_ACT_RELU ? 0 : -127;
+                    if (!p.res) {
+                        #pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            o[j] = wn_pack4(max(((int)v[4 * j] + rnd) >> sh, lo), max(((int)v[4 * j + 1] + rnd) >> sh, lo),
+                                            max(((int)v[4 * j + 2] + rnd) >> sh, lo), max(((int)v[4 * j + 3] + rnd) >> sh, lo));
                     } else {
                         #pragma unroll
-                        for (int j = 0; j < 8; ++j) o[j] = wn_f8_bn(p, n0 + cc + 4 * j, (int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3], rr[j]);
+                        for (int j = 0; j < 8; ++j) {
+                            const int x[4] = {(int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3]};
+                            o[j] = wn_f8_plain(x, rr[j], rnd, sh, lo, true);
+                        }
                     }
-                    uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
-                    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                } else {
+                    #pragma unroll
+                    for (int j = 0; j < 8; ++j) o[j] = wn_f8_bn(p, n0 + cc + 4 * j, (int)v[4 * j], (int)v[4 * j + 1], (int)v[4 * j + 2], (int)v[4 * j + 3], rr[j]);
                 }
+                uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(p.X) + (size_t)q * p.cs + n0 + cc);
+                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
         }
     }
