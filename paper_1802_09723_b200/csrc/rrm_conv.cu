@@ -476,9 +476,10 @@ static void launch_gemm(const ConvParams& p_in, dim3 grid, cudaStream_t st)
 {
     ConvParams p = p_in;
     const int cluster_z = (DT == T_F32 && p.ksplit > 1) ? p.ksplit : 1;       // fp32 shares of a tile: one cluster
-    // Dense passes of shares that take more than one CTA an SM are not launched early: placed around what their predecessor still
-    // holds they take a quarter longer (fp32 138 -> 128 7x7 at 14 x 31, 32 images, 400 CTAs in clusters of 2: 442 us, 550 early)
-    const OverlapLaunches early(OverlapLaunches::on() && !(p.ksplit > 1 && (long long)grid.x * grid.y * grid.z > 148));
+    // Dense passes of shares are not launched early: placed around what their predecessor still holds, clusters take a quarter
+    // longer (fp32 138 -> 128 7x7 at 14 x 31, 32 images, 400 CTAs in clusters of 2: 442 us, 550 early), large ones up to 1.6 times
+    // as long (162 -> 105 7x7 of stride 3 at 18 x 20, 6 images, 64 CTAs in clusters of 16: 55, 91); none gained more than 5 %
+    const OverlapLaunches early(OverlapLaunches::on() && p.ksplit <= 1);
     // (exact while the dividend stays below 2^32 / divisor: K units and taps are far below that)
     p.magic_u = p.u_in > 1 ? (unsigned)(((1ull << 32) + p.u_in - 1) / p.u_in) : 0u;
     p.magic_kw = p.kw > 1 ? (unsigned)(((1ull << 32) + p.kw - 1) / p.kw) : 0u;

@@ -1485,7 +1485,12 @@ static bool win_alone(const WinParams& p, int dtype, long long ctas) { return dt
 // Clusters cannot be placed so: their CTAs also have to lie in one part of the machine (one CTA an SM is up to 1.6 times as slow).
 // Binary clusters of long chains, whose windows keep an SM's ALUs busy, are not launched early instead (457 -> 69 3x3 of stride 3 at
 // 84 x 68, 11 images, 112 CTAs of 18 blocks each: 47.2 us without overlap, 53.9 with).
-constexpr long long WN_LONG_CHAIN = 18000;                   // clocks of a CTA's windows
+constexpr long long WN_LONG_CHAIN = 18000;                   // clocks of a CTA's blocks
+static bool win_long_binary(const WinParams& p)
+{
+    const long long fill = win_fill_clocks(p), mmas = win_mma_clocks(p, false);
+    return p.cluster && p.per * (fill > mmas ? fill : mmas) >= WN_LONG_CHAIN;
+}
 
 template <int DT, bool XCOL>
 static int win_allow()
@@ -1632,7 +1637,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)p.ntiles, (unsigned)(nf * p.ks));
     size_t smem = win_smem(p);
     if (dense && pdl_enabled() && win_alone(p, d.dtype, (long long)grid.x * grid.y * grid.z) && smem < WN_ALONE_SMEM) smem = WN_ALONE_SMEM;
-    const OverlapLaunches early(OverlapLaunches::on() && !(dense && bin && p.cluster && p.per * win_fill_clocks(p) >= WN_LONG_CHAIN));
+    const OverlapLaunches early(OverlapLaunches::on() && !(dense && bin && win_long_binary(p)));
     cudaError_t e;
     if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, out, grid, smem, st) : win_launch<T_F32, false>(p, dense, out, grid, smem, st);
     else if (d.dtype == RRM_I8) e = xcol ? win_launch<T_I8, true>(p, dense, out, grid, smem, st) : win_launch<T_I8, false>(p, dense, out, grid, smem, st);

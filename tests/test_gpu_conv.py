@@ -359,7 +359,7 @@ def _dense_outputs(path):
             ("bin", wl.xnor_alexnet_convs(hw=67), 2, (3, 67, 67)), ("res", wl.resnet18_convs(hw=64), 2, (3, 64, 64))]
     for i, (dtype, c_in, c_out, hw, k, s, p, n) in enumerate((
             ("bin", 411, 22, (27, 37), 3, 2, 1, 56), ("bin", 457, 69, (84, 68), 3, 3, 0, 11), ("i8", 64, 64, (56, 56), 3, 1, 1, 4),
-            ("i8", 212, 163, (15, 15), 9, 2, 0, 12), ("i8", 73, 296, (17, 9), 7, 1, 0, 1), ("f32", 130, 150, (22, 15), 7, 1, 0, 7))):
+            ("i8", 212, 163, (15, 15), 9, 2, 0, 12), ("i8", 73, 296, (17, 9), 7, 1, 0, 1), ("f32", 130, 150, (22, 15), 7, 1, 0, 7), ("f32", 162, 105, (18, 20), 7, 3, 0, 6))):
         nets.append((f"{dtype}{i}", [_spec(dtype, c_in, hw, c_out, k, s, p, rng, **(dict(act="sign", theta=1) if dtype == "bin" else dict(act="relu", shift=9)))],
                      n, (c_in,) + hw))
     for name, specs, n, shape in nets:
@@ -385,7 +385,7 @@ def test_dense_launches_that_overlap_give_the_same_bits(tmp_path):
     code = f"import sys; sys.path[:0] = [{os.path.dirname(__file__)!r}, {os.path.dirname(os.path.dirname(__file__))!r}]; import test_gpu_conv as t; t._dense_outputs({str(tmp_path / 'apart.npz')!r})"
     subprocess.run([sys.executable, "-c", code], check=True, timeout=600, env=dict(os.environ, RRM_PDL="0"))
     a, b = np.load(tmp_path / "overlapping.npz"), np.load(tmp_path / "apart.npz")
-    assert sorted(a.files) == sorted(b.files) and len(a.files) == 30
+    assert sorted(a.files) == sorted(b.files) and len(a.files) == 33
     for name in a.files:
         np.testing.assert_array_equal(a[name], b[name], err_msg=name)
 
