@@ -1435,7 +1435,9 @@ int64_t rrm_net_tensor_bytes(const rrm_net* net, int t)
 int rrm_plan_conv(const rrm_layer_desc* desc, int form, int frames, rrm_conv_plan* out)
 {
     if (!desc || !out || form < RRM_PLAN_DELTA || form > RRM_PLAN_PIPELINED || frames < 1) return RRM_ERR_INVALID_ARG;
-    RRM_TRY(validate_desc(*desc, desc->src > 0 ? desc->src : 0, 1));
+    rrm_layer_desc d = *desc;
+    d.src = 0; d.res = -1;                                   // (where a stack's layer reads its input and shortcut does not matter here)
+    RRM_TRY(validate_desc(d, 0, 1));
     if ((long long)desc->n * frames > INT_MAX) return RRM_ERR_CAPACITY;
     try {
         rrm_net net;
@@ -1443,8 +1445,7 @@ int rrm_plan_conv(const rrm_layer_desc* desc, int form, int frames, rrm_conv_pla
         Tensor& in = net.tensors[0];
         set_tensor(in, desc->dtype == RRM_F32 ? T_F32 : (desc->dtype == RRM_I8 ? T_I8 : T_BIN), desc->n, desc->c_in, desc->h, desc->w);
         Layer L;
-        L.d = *desc;
-        L.d.src = 0;
+        L.d = d;
         set_conv_size(L);
         RRM_TRY(check_capacity(L, in));
         *out = rrm_conv_plan{};

@@ -2,6 +2,7 @@
 for every launch it can come to."""
 import random
 
+import workloads as wl
 import paper_1802_09723_b200 as rrm
 
 FORMS = (("delta", 1), ("pipelined", 1), ("dense", 1), ("dense", 7), ("dense", 32), ("seq", 2), ("seq", 32))
@@ -73,3 +74,9 @@ def test_narrow_tiles_are_taken_where_every_one_lays_out_few_windows():
                               (("bin", 59, 50, 46, 91, 3, 3, 2, 0, 12), "delta", 96), (("bin", 59, 50, 46, 91, 3, 3, 2, 0, 12), "dense", 32)):
         p = rrm.plan_conv(desc(*shape), form)
         assert p["columns"] == want and (p["clustered"] or p["shares"] == 1), (shape, p)
+
+
+def test_layers_of_stacks_are_planned_like_lone_ones():
+    for s in wl.resnet18_convs(hw=64):
+        d = rrm.desc_from_spec(s, 2)
+        assert rrm.plan_conv(d, "dense") == rrm.plan_conv(desc(s.dtype, s.c_in, s.h, s.w, s.c_out, s.kh, s.kw, s.stride, s.pad, 2), "dense")
