@@ -91,7 +91,6 @@ struct WinParams {
     int bn, mt;               // columns and accumulator tiles (of 128 rows) per CTA
     int ntiles, narrow;       // column tiles, and whether they are the narrow ones
     int tps, stages, abuf;    // taps per filter stage, stages, window buffers
-    int async_windows;        // int8: windows by asynchronous copies, not through registers
     int xarr;                 // first layers: arrays of an image row's chunks (0: the chunks of every column side by side)
     unsigned a_step, a_lbo;   // 16-byte slots between a pixel's K groups, and between the two chunks of a group
     unsigned stage_bytes, abytes, tail_off, tmem_cols;    // (tail_off: barriers and tables, behind windows, stages and drained rows)
@@ -377,8 +376,10 @@ __device__ __noinline__ void wn_exact_row(const WinParams& p, const float* A, co
 }
 
 // DT: T_F32, T_I8 or T_BIN.  XCOL: the first-layer form.  ACT (dense passes): f is applied here and the output written,
-// instead of the projection by this kernel and f by another; the projection is stored only where a state needs it.
-template <int DT, bool DENSE, bool XCOL, bool ACT>
+// instead of the projection by this kernel and f by another; the projection is stored only where a state needs it.  ASYNC: int8
+// windows by asynchronous copies (a kernel of its own for dense passes: every CTA runs the code once, so the other way's
+// instructions would cost each launch some 0.15 us).
+template <int DT, bool DENSE, bool XCOL, bool ACT, bool ASYNC>
 __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kernel(const __grid_constant__ WinParams p)
 {
     constexpr int PIECES = DT == T_F32 ? 3 : 1;
@@ -511,8 +512,8 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             other_tables();
             wn_meet();
         }
-        const bool async = DT == T_I8 && !XCOL && (!DENSE || p.async_windows);
-        const bool lag = async && p.abuf > 1;                // asynchronous copies: a block is handed over when the next one is on its way
+        static_assert(!ASYNC || (DT == T_I8 && !XCOL));
+        const bool lag = ASYNC && p.abuf > 1;                // asynchronous copies: a block is handed over when the next one is on its way
         const int* src = S->tab;                             // the plane's table
         const int* const xcol0 = S->tab + WN_MAX_SPAN;
         int plane = plane0, chb = b0 - plane0 * p.nchb, ib = 0, buf = -1;
@@ -542,7 +543,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
             const uint32_t piece = (uint32_t)(arrays * p.L) * 16u;              // bytes between the fp32 pieces' windows
             const unsigned magic = cl > 1 ? (unsigned)(((1ull << 32) + cl - 1) / cl) : 0u;
             const int items = p.span * cl;
-            if (DT == T_I8 && !XCOL && DENSE && !async) {
+            if (DT == T_I8 && !XCOL && !ASYNC) {
                 // Dense blocks are full: through registers, a turn's loads all on their way before its first store.  (Asynchronous
                 // copies, handed over when the next block's are on their way, take 2.3 to 3 k clocks a block: 24 AlexNet-shaped
                 // keyframes 97.2 -> 93.2 us, 4 ResNet-18-shaped streams 188.9 -> 181.8.)
@@ -721,7 +722,7 @@ __global__ void __launch_bounds__(WN_THREADS, DT == T_F32 ? 1 : 2) conv_win_kern
                 // (a warp whose wait ran out says so when the warps meet at the next block)
             }
         }
-        if (async) {
+        if (ASYNC) {
             cp_async_wait<0>();
             fence_async_smem();
             if (ok && lag && ib > 0) mbar_arrive(smem_u32(&S->afull[buf]));
@@ -1495,9 +1496,15 @@ static bool win_long_binary(const WinParams& p)
 template <int DT, bool XCOL>
 static int win_allow()
 {
-    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, false, XCOL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
-    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
-    RRM_CUDA_TRY(cudaFuncSetAttribute(conv_win_kernel<DT, true, XCOL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT));
+    constexpr bool COPIES = DT == T_I8 && !XCOL;             // (delta rows always, dense windows by win_async_windows)
+    auto allow = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WN_SMEM_LIMIT); };
+    RRM_CUDA_TRY(allow(conv_win_kernel<DT, false, XCOL, false, COPIES>));
+    RRM_CUDA_TRY(allow(conv_win_kernel<DT, true, XCOL, false, false>));
+    RRM_CUDA_TRY(allow(conv_win_kernel<DT, true, XCOL, true, false>));
+    if constexpr (COPIES) {
+        RRM_CUDA_TRY(allow(conv_win_kernel<DT, true, XCOL, false, true>));
+        RRM_CUDA_TRY(allow(conv_win_kernel<DT, true, XCOL, true, true>));
+    }
     return RRM_OK;
 }
 
@@ -1597,10 +1604,12 @@ int conv_win_query(const rrm_net& net, Layer& L, int form, int frames, rrm_conv_
 template <int DT, bool XCOL>
 static cudaError_t win_launch(const WinParams& p, bool dense, bool act, dim3 grid, size_t smem, cudaStream_t st)
 {
-    const int cl = p.cluster ? p.ks : 1;
-    if (act) return launch_seq_cluster(conv_win_kernel<DT, true, XCOL, true>, grid, dim3(WN_THREADS), smem, st, cl, p);
-    return dense ? launch_seq_cluster(conv_win_kernel<DT, true, XCOL, false>, grid, dim3(WN_THREADS), smem, st, cl, p)
-                 : launch_seq_cluster(conv_win_kernel<DT, false, XCOL, false>, grid, dim3(WN_THREADS), smem, st, cl, p);
+    auto go = [&](auto kernel) { return launch_seq_cluster(kernel, grid, dim3(WN_THREADS), smem, st, p.cluster ? p.ks : 1, p); };
+    constexpr bool COPIES = DT == T_I8 && !XCOL;
+    if (!dense) return go(conv_win_kernel<DT, false, XCOL, false, COPIES>);
+    if constexpr (COPIES)
+        if (win_async_windows(p, XCOL)) return act ? go(conv_win_kernel<DT, true, XCOL, true, true>) : go(conv_win_kernel<DT, true, XCOL, false, true>);
+    return act ? go(conv_win_kernel<DT, true, XCOL, true, false>) : go(conv_win_kernel<DT, true, XCOL, false, false>);
 }
 
 // F*dI (dense: F*X + b); arguments as for launch_conv_tc.
@@ -1615,7 +1624,6 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     const int nf = batched ? frames : 1;
     if (!win_plan(L, p, xcol, dense, batched, nf, net->many_in_flight ? 74 : 148)) return RRM_ERR_UNSUPPORTED;
     if (p.span > WN_MAX_SPAN) return RRM_ERR_CAPACITY;       // (never: win_plan takes no such window)
-    p.async_windows = win_async_windows(p, xcol);
     const void* X = stateless ? in.X2 : in.X;
     p.A = bin ? in.D : (dense ? X : in.D);
     p.Anew = (!dense && !stateless && in.Xn_cur) ? in.Xn_cur : X;    // (chunks of frames: this frame's copy of the new rows)
