@@ -1433,16 +1433,17 @@ static bool win_async_windows(const WinParams& p, bool xcol) { return p.abuf >= 
 
 // What a CTA of an integer launch takes, in clocks, apart from what is the same for all cuts: its blocks one after the other
 // (the window's way into shared memory, or the MMAs, whichever is longer; the shorter once more where nothing hides it) and the
-// cluster's way out (meetings, rows read from the other shares; as far as the tile's rows are projection pixels).  The
+// cluster's way out (meetings, rows read from the other shares; as far as the fullest tile's rows are projection pixels).  The
 // figures are fitted to 1200 timed cuts of 132 layers: of both widths and all numbers of shares, 1x1 to 7x7, strides 1 to 4.
 // Deltas update few of a tile's rows, so their clusters close early (59 -> 91 3x3 of stride 2 at 50 x 46, binary, 12 images, 1 % of
 // the pixels changing: 18.7 us as clusters of 2, 20.7 as narrow tiles, which a dense pass is as fast with).
-static long long win_clocks(const WinParams& p, bool xcol, bool dense, int frames)
+static long long win_clocks(const WinParams& p, bool xcol, bool dense)
 {
-    const long long rows = (win_rows(p) + TC_M - 1) / TC_M * TC_M * frames, pixels = (long long)p.n * p.oh * p.ow * frames;
+    const long long rows = win_rows(p), full = rows < TC_M ? rows : TC_M;                     // (of the fullest tile)
+    const long long pixels = (long long)p.n * p.oh * p.ow * full / rows;
     const long long fill = win_fill_clocks(p), mmas = win_mma_clocks(p, xcol);
     long long clocks = p.per * (fill > mmas ? fill : mmas) + (fill > mmas ? mmas : fill);
-    if (p.cluster) clocks += 300ll * p.ks + (dense ? 4000 + 32ll * p.bn * pixels / rows : 2500);
+    if (p.cluster) clocks += 300ll * p.ks + (dense ? 4000 + 32ll * p.bn * pixels / TC_M : 2500);
     return clocks;
 }
 
@@ -1459,7 +1460,7 @@ static bool win_plan(const Layer& L, WinParams& p, bool xcol, bool dense, bool s
         WinParams few = p;
         const bool narrow = win_cut(L, few, xcol, dense, store, frames, wave, true);
         if (!win_cut(L, p, xcol, dense, store, frames, wave, false)) return false;
-        if (narrow && win_clocks(few, xcol, dense, frames) <= win_clocks(p, xcol, dense, frames)) p = few;
+        if (narrow && win_clocks(few, xcol, dense) <= win_clocks(p, xcol, dense)) p = few;
         return true;
     }
     return win_cut(L, p, xcol, dense, store, frames, wave, false);
