@@ -41,7 +41,7 @@
 // 118 clocks instead of 64, one of 32 columns 77; fp32: 413 clocks a K step of 16, 384 of them MMAs, 126 bytes of shared memory
 // a clock); in a launch of a few tiles a chain (clocks: set-up 1.8 k, first window 2.2 k, MMAs 3 to 6 k, way out 1.2 to 2.3 k, 7 k
 // for 64 KB of fp32 rows).  AlexNet-shaped stack at 227 x 227: 8 fp32 streams 187 us, 32 fp32 frames 462, one int8 frame 65, 32
-// int8 frames 121; 4 ResNet-18-shaped int8 streams 168.
+// int8 frames 121; 4 ResNet-18-shaped int8 streams 171.
 #include "rrm_common.cuh"
 #include "rrm_tc.cuh"
 #include "rrm_dev.cuh"
@@ -1476,13 +1476,18 @@ static size_t win_smem(const WinParams& p)
 // Launches that overlap their predecessors (dense passes) are placed while those still hold some of the SMs: two CTAs of an
 // integer launch then come to lie on one SM and leave others idle.  Launches of fewer CTAs than SMs, but of many, ask for more than
 // half of an SM's shared memory, so that each has one to itself (411 -> 22 3x3 of stride 2, binary, 56 images of 27 x 37, 132
-// CTAs: 37.3 us without overlap, 42.5 with, 36.3 so; dense chunks of 32 AlexNet-shaped frames 124.7 -> 119.2, 4 ResNet-18-shaped
-// streams 172.2 -> 168.8).  Below 90 CTAs they find room beside each other, and the next launch's wait beside them (24
-// AlexNet-shaped keyframes, two launches of 81 CTAs: 90.9, 92.0 with an SM each).
+// CTAs: 37.3 us without overlap, 42.5 with, 36.3 so; dense chunks of 32 AlexNet-shaped frames 124.7 -> 119.2, of 2 x 8
+// ResNet-18-shaped ones at 183 x 183 181 -> 172).  Below 90 CTAs they find room beside each other, and the next launch's wait beside
+// them (24 AlexNet-shaped keyframes, two launches of 81 CTAs: 90.9, 92.0 with an SM each); short chains lose more by the wait for an
+// SM than by sharing one (5 ResNet-18-shaped frames at 160 x 160, four launches of 132 CTAs of some 4 k clocks: 130.4, 133.4).
 constexpr int WN_ALONE = 90;
+constexpr long long WN_ALONE_CHAIN = 8200;                   // clocks of a CTA's blocks
 constexpr size_t WN_ALONE_SMEM = 116 * 1024;
 
-static bool win_alone(const WinParams& p, int dtype, long long ctas) { return dtype != RRM_F32 && !p.cluster && ctas >= WN_ALONE && ctas <= 148; }
+static bool win_alone(const WinParams& p, int dtype, bool xcol, long long ctas)
+{
+    return dtype != RRM_F32 && !p.cluster && ctas >= WN_ALONE && ctas <= 148 && win_clocks(p, xcol, true) >= WN_ALONE_CHAIN;
+}
 
 // Clusters cannot be placed so: their CTAs also have to lie in one part of the machine (one CTA an SM is up to 1.6 times as slow).
 // Binary clusters of long chains, whose windows keep an SM's ALUs busy, are not launched early instead (457 -> 69 3x3 of stride 3 at
@@ -1645,7 +1650,7 @@ int launch_conv_win(rrm_net* net, Layer& L, const Tensor& in, bool dense, bool s
     const long long rows = win_rows(p);
     const dim3 grid((unsigned)((rows + p.mt * TC_M - 1) / (p.mt * TC_M)), (unsigned)p.ntiles, (unsigned)(nf * p.ks));
     size_t smem = win_smem(p);
-    if (dense && pdl_enabled() && win_alone(p, d.dtype, (long long)grid.x * grid.y * grid.z) && smem < WN_ALONE_SMEM) smem = WN_ALONE_SMEM;
+    if (dense && pdl_enabled() && win_alone(p, d.dtype, xcol, (long long)grid.x * grid.y * grid.z) && smem < WN_ALONE_SMEM) smem = WN_ALONE_SMEM;
     const OverlapLaunches early(OverlapLaunches::on() && !(dense && bin && win_long_binary(p)));
     cudaError_t e;
     if (d.dtype == RRM_F32) e = xcol ? win_launch<T_F32, true>(p, dense, out, grid, smem, st) : win_launch<T_F32, false>(p, dense, out, grid, smem, st);
